@@ -4,7 +4,7 @@
 // that the tick reads. Its cost does not depend on the history length.
 //
 // Per call:  embed -> n_layers x [ RMSNorm+QKV (tcgen05 GEMM) -> rotary
-//            embedding + cache-row writes -> causal attention over
+//            embedding, cache-row writes and causal attention over
 //            [cached rows ; new rows] -> W_o + residual -> RMSNorm+gate/up+SiLU
 //            -> W_d + residual ] -> residual stream out.
 // The four projections reuse the tensor-core GEMM of the tick (gemm_tc.cu):
@@ -16,6 +16,7 @@
 #include <cuda_runtime.h>
 
 #include <algorithm>
+#include <cmath>
 #include <cstdarg>
 #include <cstdio>
 #include <thread>
@@ -59,14 +60,18 @@ __device__ __forceinline__ int status_set(const int* status) {
 }
 
 // ---- token rows in: x (fp32 residual stream), its fp16 copy and the per-token
-// sums of x^2 over each 128-column group (the RMSNorm input of the QKV GEMM).
-// Block 0 also checks the offsets and destination rows.
+// sums of x^2 over each 128-column group (the RMSNorm input of the QKV GEMM), and the
+// cosines and sines of the token's rotary angles, which depend on its position only:
+// formed once per call (fp64 angles) and read by every layer. Block 0 also checks the
+// offsets and destination rows, its threads sharing the B (B - 1) / 2 pairs of ranges.
 struct EmbedArgsA {
   const __nv_bfloat16* x_new;  // [M, d]
   const int64_t* offsets;      // [B + 1]
   const int64_t* dst;          // [B]
   int B, n_new, d;
   long long max_rows;
+  const double* inv_freq;      // [64] base^(-2 j / 128)
+  float2* rot;                 // [M][64] (cos, sin) of position * inv_freq
   float* x;
   __half* x16;
   float* ss;
@@ -76,16 +81,25 @@ struct EmbedArgsA {
 
 __global__ void __launch_bounds__(128) append_embed_kernel(const EmbedArgsA a) {
   const int m = blockIdx.x;
-  if (m == 0 && threadIdx.x == 0) {
+  if (m == 0) {
     const int64_t* off = a.offsets;
     bool ok = off[0] >= 0 && off[a.B] <= a.max_rows;
-    for (int b = 0; b < a.B && ok; ++b) ok = off[b + 1] >= off[b];
-    for (int b = 0; b < a.B && ok; ++b) {
-      const int64_t lo = a.dst[b], hi = a.dst[b] + a.n_new;
-      ok = lo >= 0 && hi <= a.max_rows && (hi <= off[0] || lo >= off[a.B]);
-      for (int c = 0; c < b && ok; ++c) ok = hi <= a.dst[c] || lo >= a.dst[c] + a.n_new;
+    for (int b = threadIdx.x; b < a.B; b += blockDim.x) {
+      const int64_t lo = a.dst[b], hi = lo + a.n_new;
+      ok = ok && off[b + 1] >= off[b] && lo >= 0 && hi <= a.max_rows && (hi <= off[0] || lo >= off[a.B]);
+      for (int c = 0; c < b; ++c) {
+        const int64_t o = a.dst[c];
+        ok = ok && (hi <= o || lo >= o + a.n_new);
+      }
     }
     if (!ok) fsx::set_status(a.status, fsx::kStatusDeviceArg);
+  }
+  if (threadIdx.x < kRopePairs) {
+    const int b = m / a.n_new;
+    const long long pos = (a.offsets[b + 1] - a.offsets[b]) + (m - b * a.n_new);
+    double sd, cd;
+    sincos(static_cast<double>(pos) * a.inv_freq[threadIdx.x], &sd, &cd);
+    a.rot[static_cast<size_t>(m) * kRopePairs + threadIdx.x] = make_float2(static_cast<float>(cd), static_cast<float>(sd));
   }
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   for (int g = warp; g < a.d / 128; g += 4) {
@@ -100,56 +114,32 @@ __global__ void __launch_bounds__(128) append_embed_kernel(const EmbedArgsA a) {
   }
 }
 
-// ---- rotary embedding of q and k at the new tokens' positions; k (rotated) and v
-// written to the layer's cache rows dst[b] + i as bf16; q rotated in place.
-struct RopeArgsA {
-  __half* qkv;  // [M, 3 HD]: q | k | v
+// ---- rotary embedding, cache-row writes and causal attention of the new tokens of
+// vehicle b, head h, in one launch. The CTA rotates the new queries and keys itself
+// (cos / sin from the embed kernel) and rounds the new keys and values to bf16 in shared
+// memory; rank 0 of the cluster writes them to the cache rows dst[b] + i. The keys are the
+// vehicle's cached rows (positions 0 .. L_b-1) in 32-key chunks, then one chunk of its new
+// rows; new token i sees every cached row and new rows 0 .. i. Everything is fp32.
+//
+// The keys are few and every row is read once, so the kernel is bound by load latency:
+// a warp issues the loads of its chunk's K rows and half of its V rows (12 KB) before the first use,
+// the chunks go round robin over the 4 warps of `cluster` CTAs (as many as keep two CTAs
+// per SM for the batch), and the score step moves no key through shared memory: 4 lanes
+// share a key row (full 32-byte sectors), 4 keys per lane, and a transposed reduction over
+// the 4 lanes leaves key 8 j + g with lane 4 g + j. Both products use packed fp32 FMAs.
+// The CTAs of a cluster exchange their (max, sum, output) through distributed shared memory,
+// each merging its share of the n_new x 128 outputs.
+// Measured (two-layer append, 4 tokens a vehicle): one vehicle with 224 rows 392 -> 311 us a
+// call, 16 vehicles with 96-480 rows 552 -> 370 us, against separate rotary (fp64 pow and
+// sincos per pair and layer) and attention launches (a lane per key, one 32-key chunk's loads
+// dependent on the previous one's), which took 55 and 130 us of a layer.
+struct AttnArgsA {
+  const __half* qkv;   // [M, 3 HD]: q | k | v before the rotation
   int ld;
   int HD;
-  const int64_t* offsets;
-  const int64_t* dst;
-  int n_new;
-  double base;
+  const float2* rot;   // [M][64]
   __nv_bfloat16* k_cache;  // this layer's rows
   __nv_bfloat16* v_cache;
-  int* status;
-};
-
-__global__ void __launch_bounds__(kRopePairs) append_rope_kernel(const RopeArgsA r) {
-  if (status_set(r.status)) return;
-  const int m = blockIdx.x, h = blockIdx.y, j = threadIdx.x;  // pair (j, j + 64) of head h
-  const int b = m / r.n_new, i = m - b * r.n_new;
-  const long long pos = (r.offsets[b + 1] - r.offsets[b]) + i;
-  const long long row = r.dst[b] + i;
-  double sd, cd;
-  sincos(static_cast<double>(pos) * pow(r.base, -2.0 * j / kHeadDim), &sd, &cd);
-  const float s = static_cast<float>(sd), c = static_cast<float>(cd);
-  __half* q = r.qkv + static_cast<size_t>(m) * r.ld + h * kHeadDim;
-  const __half* k = q + r.HD;
-  const __half* v = q + 2 * r.HD;
-  const float q0 = __half2float(q[j]), q1 = __half2float(q[j + kRopePairs]);
-  const float k0 = __half2float(k[j]), k1 = __half2float(k[j + kRopePairs]);
-  q[j] = __float2half_rn(q0 * c - q1 * s);
-  q[j + kRopePairs] = __float2half_rn(q0 * s + q1 * c);
-  const size_t o = static_cast<size_t>(row) * r.HD + h * kHeadDim;
-  r.k_cache[o + j] = __float2bfloat16_rn(k0 * c - k1 * s);
-  r.k_cache[o + j + kRopePairs] = __float2bfloat16_rn(k0 * s + k1 * c);
-  r.v_cache[o + j] = __float2bfloat16_rn(__half2float(v[j]));
-  r.v_cache[o + j + kRopePairs] = __float2bfloat16_rn(__half2float(v[j + kRopePairs]));
-}
-
-// ---- causal attention of the new tokens of vehicle b, head h: keys are the
-// vehicle's cached rows (positions 0 .. L_b-1) then its new rows (positions
-// L_b ..); new token i sees every cached row and new rows 0 .. i. Warp w takes
-// 32-key chunks w, w + 4, ...: lane l scores key 32c + l against every query
-// (online softmax per query across the chunk), then owns value dims 4l..4l+3
-// of the output. The four warps merge their states at the end.
-struct AttnArgsA {
-  const __half* qkv;  // rotated q at column h * 128 of row m
-  int ld;
-  int HD;
-  const __nv_bfloat16* k_cache;
-  const __nv_bfloat16* v_cache;
   const int64_t* offsets;
   const int64_t* dst;
   int n_new;
@@ -157,113 +147,253 @@ struct AttnArgsA {
   int* status;
 };
 
-__device__ __forceinline__ const __nv_bfloat16* key_row(const __nv_bfloat16* base, long long lo, long long L,
-                                                        long long d0, int key, int HD, int h) {
-  const long long row = key < L ? lo + key : d0 + (key - L);
-  return base + static_cast<size_t>(row) * HD + h * kHeadDim;
+constexpr int kNewStride = kHeadDim + 8;  // bf16 row stride of the new keys / values in shared memory
+constexpr int kMaxSplit = 8;              // CTAs of a cluster
+
+// d += a * b on two packed fp32 values
+__device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
+  asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(d) : "l"(a), "l"(b));
+}
+__device__ __forceinline__ uint64_t mul2(uint64_t a, uint64_t b) {
+  uint64_t d;
+  asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(a), "l"(b));
+  return d;
+}
+__device__ __forceinline__ uint64_t pack2(float lo, float hi) {
+  uint64_t d;
+  asm("mov.b64 %0, {%1, %2};" : "=l"(d) : "f"(lo), "f"(hi));
+  return d;
+}
+__device__ __forceinline__ float2 unpack2(uint64_t v) {
+  float2 f;
+  asm("mov.b64 {%0, %1}, %2;" : "=f"(f.x), "=f"(f.y) : "l"(v));
+  return f;
+}
+__device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t v) {
+  return pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+}
+__device__ __forceinline__ uint32_t peer_addr(const void* local, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(fsx::smem_addr(local)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, float v) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
-__global__ void __launch_bounds__(kAttnWarps * 32) append_attn_kernel(const AttnArgsA a) {
-  if (status_set(a.status)) return;
-  __shared__ float qs[kMaxNew][kHeadDim];
-  __shared__ float sm_m[kAttnWarps][kMaxNew], sm_l[kAttnWarps][kMaxNew];
-  __shared__ float sm_o[kAttnWarps][kMaxNew][kHeadDim];
-  const int b = blockIdx.x, h = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// NQ: query slots (4 or 8) for n_new <= NQ new tokens
+template <int NQ>
+__global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const AttnArgsA a) {
+  __shared__ __align__(16) float qs[NQ][kHeadDim];
+  __shared__ __align__(16) __nv_bfloat16 kn[kMaxNew][kNewStride], vn[kMaxNew][kNewStride];
+  __shared__ float sm_m[kAttnWarps][NQ], sm_l[kAttnWarps][NQ];
+  __shared__ __align__(16) float sm_o[kAttnWarps][NQ][kHeadDim];
+  __shared__ float rv_o[NQ * kHeadDim];                       // [split][this rank's share of the outputs]
+  __shared__ float rv_m[kMaxSplit][NQ], rv_l[kMaxSplit][NQ];  // every split's running maxima and sums
+  fsx::pdl_launch_dependents();
+  fsx::pdl_wait();
+  if (status_set(a.status)) return;  // set before this launch or not at all: the same for the whole cluster
+  const int S = gridDim.x, rank = blockIdx.x;  // the cluster spans the grid's x extent
+  const int h = blockIdx.y, b = blockIdx.z;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nq = a.n_new;
+  if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this CTA runs
   const long long lo = a.offsets[b];
-  const long long L = a.offsets[b + 1] - lo;
+  const int L = static_cast<int>(a.offsets[b + 1] - lo);
   const long long d0 = a.dst[b];
-  const int N = static_cast<int>(L) + nq;
+  const int n_chunks = (L + 31) / 32 + 1;  // the last one: the new rows
+
+  const int g = lane >> 2, j = lane & 3;    // scores: key group lane, 16-byte unit lane
+  const int hv = lane >> 4, u = lane & 15;  // values: key parity, 16-byte unit
+  uint4 kraw[4][4], vraw[8];
+  // row loads of chunk c (zeros past the vehicle's rows): all K rows and V rows 0-15, then
+  // V rows 16-31 once the scores have released the registers of K
+  auto chunk_keys = [&](int c) { return c == n_chunks - 1 ? nq : min(32, L - 32 * c); };
+  auto chunk_base = [&](int c, __nv_bfloat16* cache, __nv_bfloat16* fresh) -> const __nv_bfloat16* {
+    if (c == n_chunks - 1) return fresh;
+    return cache + (static_cast<size_t>(lo) + 32 * static_cast<size_t>(c)) * a.HD + h * kHeadDim;
+  };
+  auto load_v = [&](int c, int half) {
+    const int n = chunk_keys(c);
+    const size_t stride = c == n_chunks - 1 ? kNewStride : static_cast<size_t>(a.HD);
+    const __nv_bfloat16* vb = chunk_base(c, a.v_cache, &vn[0][0]);
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      const int key = 16 * half + 2 * kk + hv;
+      vraw[kk] = key < n ? *reinterpret_cast<const uint4*>(vb + key * stride + u * 8) : make_uint4(0u, 0u, 0u, 0u);
+    }
+  };
+  auto load_chunk = [&](int c) {
+    const int n = chunk_keys(c);
+    const size_t stride = c == n_chunks - 1 ? kNewStride : static_cast<size_t>(a.HD);
+    const __nv_bfloat16* kb = chunk_base(c, a.k_cache, &kn[0][0]);
+#pragma unroll
+    for (int t = 0; t < 4; ++t)
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+        kraw[t][i] = 8 * t + g < n ? *reinterpret_cast<const uint4*>(kb + (8 * t + g) * stride + (4 * i + j) * 8)
+                                   : make_uint4(0u, 0u, 0u, 0u);
+    load_v(c, 0);
+  };
+  const int step = S * kAttnWarps;
+  int c = rank * kAttnWarps + warp;
+  if (c < n_chunks - 1) load_chunk(c);  // in flight while the new rows are rotated
+
   const float scale = 1.4426950408889634f * rsqrtf(static_cast<float>(kHeadDim));  // log2(e) / sqrt(128)
-  for (int t = threadIdx.x; t < nq * kHeadDim; t += blockDim.x) {
-    const int qi = t / kHeadDim, dd = t - qi * kHeadDim;
-    qs[qi][dd] = __half2float(a.qkv[static_cast<size_t>(b * nq + qi) * a.ld + h * kHeadDim + dd]) * scale;
+  for (int t = tid; t < NQ * kRopePairs; t += kAttnWarps * 32) {
+    const int i = t / kRopePairs, jj = t - i * kRopePairs;
+    if (i >= nq) {
+      qs[i][jj] = qs[i][jj + kRopePairs] = 0.f;
+      continue;
+    }
+    const int m = b * nq + i;
+    const float2 cs = a.rot[static_cast<size_t>(m) * kRopePairs + jj];
+    const __half* q = a.qkv + static_cast<size_t>(m) * a.ld + h * kHeadDim + jj;
+    const __half* k = q + a.HD;
+    const __half* v = q + 2 * a.HD;
+    const float q0 = __half2float(q[0]), q1 = __half2float(q[kRopePairs]);
+    const float k0 = __half2float(k[0]), k1 = __half2float(k[kRopePairs]);
+    qs[i][jj] = (q0 * cs.x - q1 * cs.y) * scale;
+    qs[i][jj + kRopePairs] = (q0 * cs.y + q1 * cs.x) * scale;
+    kn[i][jj] = __float2bfloat16_rn(k0 * cs.x - k1 * cs.y);
+    kn[i][jj + kRopePairs] = __float2bfloat16_rn(k0 * cs.y + k1 * cs.x);
+    vn[i][jj] = __float2bfloat16_rn(__half2float(v[0]));
+    vn[i][jj + kRopePairs] = __float2bfloat16_rn(__half2float(v[kRopePairs]));
   }
   __syncthreads();
+  if (rank == 0)  // the new cache rows, 16 bytes a thread
+    for (int t = tid; t < nq * (kHeadDim / 8); t += kAttnWarps * 32) {
+      const int i = t / (kHeadDim / 8), uu = t - i * (kHeadDim / 8);
+      const size_t o = static_cast<size_t>(d0 + i) * a.HD + h * kHeadDim + uu * 8;
+      *reinterpret_cast<uint4*>(a.k_cache + o) = *reinterpret_cast<const uint4*>(&kn[i][uu * 8]);
+      *reinterpret_cast<uint4*>(a.v_cache + o) = *reinterpret_cast<const uint4*>(&vn[i][uu * 8]);
+    }
 
-  float m_run[kMaxNew], l_run[kMaxNew], o[kMaxNew][4];
+  float m_run[NQ], l_run[NQ];  // l_run: this lane's keys only
+  uint64_t o[NQ][4];           // this half warp's keys, value dims 8 u .. 8 u + 7
 #pragma unroll
-  for (int qi = 0; qi < kMaxNew; ++qi) {
+  for (int qi = 0; qi < NQ; ++qi) {
     m_run[qi] = -INFINITY;
     l_run[qi] = 0.f;
 #pragma unroll
-    for (int e = 0; e < 4; ++e) o[qi][e] = 0.f;
+    for (int e = 0; e < 4; ++e) o[qi][e] = 0ull;
   }
-  for (int c0 = warp * 32; c0 < N; c0 += kAttnWarps * 32) {
-    const int key = c0 + lane;
-    float s[kMaxNew];
+  bool loaded = c < n_chunks - 1;
+  for (; c < n_chunks; c += step) {
+    if (!loaded) load_chunk(c);
+    loaded = false;
+    const bool own = c == n_chunks - 1;
+    const int n = chunk_keys(c);
+    uint64_t acc[4][NQ];
 #pragma unroll
-    for (int qi = 0; qi < kMaxNew; ++qi) s[qi] = 0.f;
-    if (key < N) {
-      const uint4* kr = reinterpret_cast<const uint4*>(key_row(a.k_cache, lo, L, d0, key, a.HD, h));
-#pragma unroll 4
-      for (int u = 0; u < kHeadDim / 8; ++u) {
-        const uint4 raw = kr[u];
-        float kv[8];
-        kv[0] = __uint_as_float(raw.x << 16);
-        kv[1] = __uint_as_float(raw.x & 0xffff0000u);
-        kv[2] = __uint_as_float(raw.y << 16);
-        kv[3] = __uint_as_float(raw.y & 0xffff0000u);
-        kv[4] = __uint_as_float(raw.z << 16);
-        kv[5] = __uint_as_float(raw.z & 0xffff0000u);
-        kv[6] = __uint_as_float(raw.w << 16);
-        kv[7] = __uint_as_float(raw.w & 0xffff0000u);
+    for (int t = 0; t < 4; ++t)
 #pragma unroll
-        for (int qi = 0; qi < kMaxNew; ++qi)
-          if (qi < nq)
+      for (int qi = 0; qi < NQ; ++qi) acc[t][qi] = 0ull;
 #pragma unroll
-            for (int e = 0; e < 8; ++e) s[qi] = fmaf(qs[qi][u * 8 + e], kv[e], s[qi]);
+    for (int i = 0; i < 4; ++i) {
+      uint64_t kv[4][4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        kv[t][0] = bf16x2_to_f32x2(kraw[t][i].x);
+        kv[t][1] = bf16x2_to_f32x2(kraw[t][i].y);
+        kv[t][2] = bf16x2_to_f32x2(kraw[t][i].z);
+        kv[t][3] = bf16x2_to_f32x2(kraw[t][i].w);
+      }
+#pragma unroll
+      for (int qi = 0; qi < NQ; ++qi) {
+        const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&qs[qi][(4 * i + j) * 8]);
+        const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(&qs[qi][(4 * i + j) * 8 + 4]);
+#pragma unroll
+        for (int t = 0; t < 4; ++t) {
+          fma2(acc[t][qi], kv[t][0], qa.x);
+          fma2(acc[t][qi], kv[t][1], qa.y);
+          fma2(acc[t][qi], kv[t][2], qb.x);
+          fma2(acc[t][qi], kv[t][3], qb.y);
+        }
       }
     }
-    float p[kMaxNew];
+    // transposed sum over the 4 lanes of a key row: lane 4 g + j keeps key 8 j + g
+    float p[NQ];
 #pragma unroll
-    for (int qi = 0; qi < kMaxNew; ++qi) {
-      // visible: a real key that is a cached row or a new row j <= qi
-      const bool vis = qi < nq && key < N && (key < L || key - L <= qi);
-      const float sv = vis ? s[qi] : -INFINITY;
+    for (int qi = 0; qi < NQ; ++qi) {
+      float s[4];
+#pragma unroll
+      for (int t = 0; t < 4; ++t) {
+        const float2 f = unpack2(acc[t][qi]);
+        s[t] = f.x + f.y;
+      }
+      const bool up2 = (j & 2) != 0, up1 = (j & 1) != 0;
+      const float a0 = (up2 ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, up2 ? s[0] : s[2], 2);
+      const float a1 = (up2 ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, up2 ? s[1] : s[3], 2);
+      p[qi] = (up1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up1 ? a0 : a1, 1);
+    }
+    const int key = 8 * j + g;
+#pragma unroll
+    for (int qi = 0; qi < NQ; ++qi) {
+      // visible: a real key that is a cached row or a new row <= qi
+      const bool vis = qi < nq && key < n && (!own || key <= qi);
+      const float sv = vis ? p[qi] : -INFINITY;
       float mx = sv;
 #pragma unroll
       for (int sh = 16; sh > 0; sh >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, sh));
       const float m_new = fmaxf(m_run[qi], mx);
-      if (m_new == -INFINITY) {  // nothing visible yet for this query
+      if (m_new == -INFINITY) {  // an unused query slot
         p[qi] = 0.f;
         continue;
       }
       const float alpha = exp2f(m_run[qi] - m_new);
       p[qi] = vis ? exp2f(sv - m_new) : 0.f;
-      l_run[qi] = l_run[qi] * alpha + fsx::warp_sum(p[qi]);
+      l_run[qi] = l_run[qi] * alpha + p[qi];
       m_run[qi] = m_new;
+      const uint64_t al = pack2(alpha, alpha);
 #pragma unroll
-      for (int e = 0; e < 4; ++e) o[qi][e] *= alpha;
+      for (int e = 0; e < 4; ++e) o[qi][e] = mul2(o[qi][e], al);
     }
-    const int n_chunk = min(32, N - c0);
-    for (int kk = 0; kk < n_chunk; ++kk) {
-      const uint2 raw = *reinterpret_cast<const uint2*>(key_row(a.v_cache, lo, L, d0, c0 + kk, a.HD, h) + lane * 4);
-      const float v0 = __uint_as_float(raw.x << 16), v1 = __uint_as_float(raw.x & 0xffff0000u);
-      const float v2 = __uint_as_float(raw.y << 16), v3 = __uint_as_float(raw.y & 0xffff0000u);
+    auto attend = [&](int half) {
 #pragma unroll
-      for (int qi = 0; qi < kMaxNew; ++qi) {
-        const float pk = __shfl_sync(0xffffffffu, p[qi], kk);
-        o[qi][0] = fmaf(pk, v0, o[qi][0]);
-        o[qi][1] = fmaf(pk, v1, o[qi][1]);
-        o[qi][2] = fmaf(pk, v2, o[qi][2]);
-        o[qi][3] = fmaf(pk, v3, o[qi][3]);
+      for (int kk = 0; kk < 8; ++kk) {
+        const uint64_t v0 = bf16x2_to_f32x2(vraw[kk].x), v1 = bf16x2_to_f32x2(vraw[kk].y);
+        const uint64_t v2 = bf16x2_to_f32x2(vraw[kk].z), v3 = bf16x2_to_f32x2(vraw[kk].w);
+        const int kv = 16 * half + 2 * kk + hv;  // its probability is with lane 4 (kv mod 8) + kv / 8
+#pragma unroll
+        for (int qi = 0; qi < NQ; ++qi) {
+          const float pk = __shfl_sync(0xffffffffu, p[qi], ((kv & 7) << 2) | (kv >> 3));
+          const uint64_t pp = pack2(pk, pk);
+          fma2(o[qi][0], pp, v0);
+          fma2(o[qi][1], pp, v1);
+          fma2(o[qi][2], pp, v2);
+          fma2(o[qi][3], pp, v3);
+        }
       }
-    }
+    };
+    attend(0);
+    load_v(c, 1);
+    attend(1);
   }
 #pragma unroll
-  for (int qi = 0; qi < kMaxNew; ++qi) {
+  for (int qi = 0; qi < NQ; ++qi) {
+    float ov[8];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+      const float2 f = unpack2(o[qi][e]);
+      ov[2 * e] = f.x + __shfl_xor_sync(0xffffffffu, f.x, 16);
+      ov[2 * e + 1] = f.y + __shfl_xor_sync(0xffffffffu, f.y, 16);
+    }
+    *reinterpret_cast<float4*>(&sm_o[warp][qi][u * 8 + hv * 4]) =
+        hv == 0 ? make_float4(ov[0], ov[1], ov[2], ov[3]) : make_float4(ov[4], ov[5], ov[6], ov[7]);
+    const float l = fsx::warp_sum(l_run[qi]);
     if (lane == 0) {
       sm_m[warp][qi] = m_run[qi];
-      sm_l[warp][qi] = l_run[qi];
+      sm_l[warp][qi] = l;
     }
-#pragma unroll
-    for (int e = 0; e < 4; ++e) sm_o[warp][qi][lane * 4 + e] = o[qi][e];
   }
   __syncthreads();
-  for (int t = threadIdx.x; t < nq * kHeadDim; t += blockDim.x) {
-    const int qi = t / kHeadDim, dd = t - qi * kHeadDim;
+  // the CTA's four warps, then (S > 1) the cluster's CTAs: output element e = query * 128 + dim
+  // belongs to rank e / (n_new * 128 / S)
+  if (S > 1) asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every peer runs
+  const int share = nq * kHeadDim / S;
+  for (int e = tid; e < nq * kHeadDim; e += kAttnWarps * 32) {
+    const int qi = e / kHeadDim, dd = e - qi * kHeadDim;
     float mm = -INFINITY;
 #pragma unroll
     for (int w = 0; w < kAttnWarps; ++w) mm = fmaxf(mm, sm_m[w][qi]);
@@ -274,8 +404,40 @@ __global__ void __launch_bounds__(kAttnWarps * 32) append_attn_kernel(const Attn
       num += f * sm_o[w][qi][dd];
       den += f * sm_l[w][qi];
     }
+    if (S == 1) {
+      a.out[static_cast<size_t>(b * nq + qi) * a.HD + h * kHeadDim + dd] = __float2half_rn(den > 0.f ? num / den : 0.f);
+      continue;
+    }
+    const int owner = e / share;
+    st_peer(peer_addr(&rv_o[rank * share + (e - owner * share)], owner), num);
+    if (dd < S) {  // this split's maximum and sum of the query, to every rank
+      st_peer(peer_addr(&rv_m[rank][qi], dd), mm);
+      st_peer(peer_addr(&rv_l[rank][qi], dd), den);
+    }
+  }
+  if (S == 1) return;
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  for (int t = tid; t < share; t += kAttnWarps * 32) {
+    const int e = rank * share + t;
+    const int qi = e / kHeadDim, dd = e - qi * kHeadDim;
+    float mm = -INFINITY;
+    for (int r = 0; r < S; ++r) mm = fmaxf(mm, rv_m[r][qi]);
+    float num = 0.f, den = 0.f;
+    for (int r = 0; r < S; ++r) {  // a split without keys has the maximum -inf
+      const float f = rv_m[r][qi] == -INFINITY ? 0.f : exp2f(rv_m[r][qi] - mm);
+      num += f * rv_o[r * share + t];
+      den += f * rv_l[r][qi];
+    }
     a.out[static_cast<size_t>(b * nq + qi) * a.HD + h * kHeadDim + dd] = __float2half_rn(den > 0.f ? num / den : 0.f);
   }
+}
+
+// CTAs per (vehicle, head): the largest power of two up to 8 that keeps the batch's CTAs
+// within two per SM
+int append_attn_splits(int B, int n_heads, int sm_count) {
+  int s = kMaxSplit;
+  while (s > 1 && static_cast<long long>(B) * n_heads * s > 2ll * sm_count) s >>= 1;
+  return s;
 }
 
 }  // namespace
@@ -297,6 +459,8 @@ struct fsx_append_s {
   __half* qkv = nullptr;
   __half* o = nullptr;
   __half* hbuf = nullptr;
+  double* inv_freq = nullptr;  // [64] rotary frequencies
+  float2* rot = nullptr;       // [n_new * max_batch][64] (cos, sin) of the current call's positions
   float* gemm_part = nullptr;
   int* tile_count = nullptr;
   int* status = nullptr;
@@ -308,7 +472,8 @@ void free_append(fsx_append_s* h) {
   if (!h) return;
   cudaSetDevice(h->device);
   cudaDeviceSynchronize();
-  void* bufs[] = {h->w_arena, h->x, h->x16, h->ss, h->qkv, h->o, h->hbuf, h->gemm_part, h->tile_count, h->status};
+  void* bufs[] = {h->w_arena, h->x, h->x16, h->ss, h->qkv, h->o, h->hbuf,
+                  h->inv_freq, h->rot, h->gemm_part, h->tile_count, h->status};
   for (void* p : bufs)
     if (p) cudaFree(p);
   delete h;
@@ -460,6 +625,13 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
           !fsx::encode_act_map(&h->map_h[i], h->hbuf, m_pad, F, boxes[i]))
         return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
   }
+  {
+    double inv_freq[kRopePairs];
+    for (int j = 0; j < kRopePairs; ++j) inv_freq[j] = std::pow(static_cast<double>(cfg->rope_base), -2.0 * j / kHeadDim);
+    FSX_CUDA_H(cudaMalloc(&h->inv_freq, sizeof(inv_freq)));
+    FSX_CUDA_H(cudaMemcpy(h->inv_freq, inv_freq, sizeof(inv_freq), cudaMemcpyHostToDevice));
+  }
+  FSX_CUDA_H(cudaMalloc(&h->rot, static_cast<size_t>(cfg->n_new) * cfg->max_batch * kRopePairs * sizeof(float2)));
   FSX_CUDA_H(cudaMalloc(&h->gemm_part, fsx::gemm_tc_part_bytes(h->sm_count)));
   FSX_CUDA_H(cudaMalloc(&h->tile_count, sizeof(int) * h->sm_count));
   FSX_CUDA_H(cudaMemset(h->tile_count, 0, sizeof(int) * h->sm_count));
@@ -504,6 +676,8 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
   ea.n_new = c.n_new;
   ea.d = d;
   ea.max_rows = c.max_cache_rows;
+  ea.inv_freq = h->inv_freq;
+  ea.rot = h->rot;
   ea.x = h->x;
   ea.x16 = h->x16;
   ea.ss = h->ss;
@@ -512,6 +686,7 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
   append_embed_kernel<<<M, 128, 0, st>>>(ea);
   FSX_CUDA(cudaGetLastError());
 
+  const int attn_splits = append_attn_splits(B, c.n_heads, h->sm_count);
   for (int l = 0; l < c.n_layers; ++l) {
     fsx::TcGemmArgs g{};
     g.M = M;
@@ -526,33 +701,23 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     g.ss_stride = h->ss_stride;
     FSX_CUDA(fsx::launch_gemm_tc(h->map_x16[bn_i], g, bn, fsx::kEpiStore, true, st, false));
 
-    RopeArgsA ra{};
-    ra.qkv = h->qkv;
-    ra.ld = 3 * HD;
-    ra.HD = HD;
-    ra.offsets = d_offsets;
-    ra.dst = d_dst_rows;
-    ra.n_new = c.n_new;
-    ra.base = static_cast<double>(c.rope_base);
-    ra.k_cache = static_cast<__nv_bfloat16*>(k_cache[l]);
-    ra.v_cache = static_cast<__nv_bfloat16*>(v_cache[l]);
-    ra.status = h->status;
-    append_rope_kernel<<<dim3(M, c.n_heads), kRopePairs, 0, st>>>(ra);
-    FSX_CUDA(cudaGetLastError());
-
     AttnArgsA aa{};
     aa.qkv = h->qkv;
     aa.ld = 3 * HD;
     aa.HD = HD;
-    aa.k_cache = static_cast<const __nv_bfloat16*>(k_cache[l]);
-    aa.v_cache = static_cast<const __nv_bfloat16*>(v_cache[l]);
+    aa.rot = h->rot;
+    aa.k_cache = static_cast<__nv_bfloat16*>(k_cache[l]);
+    aa.v_cache = static_cast<__nv_bfloat16*>(v_cache[l]);
     aa.offsets = d_offsets;
     aa.dst = d_dst_rows;
     aa.n_new = c.n_new;
     aa.out = h->o;
     aa.status = h->status;
-    append_attn_kernel<<<dim3(B, c.n_heads), kAttnWarps * 32, 0, st>>>(aa);
-    FSX_CUDA(cudaGetLastError());
+    void* attn_args[] = {&aa};
+    FSX_CUDA(fsx::launch_ex(c.n_new <= 4 ? reinterpret_cast<const void*>(&append_attn_kernel<4>)
+                                         : reinterpret_cast<const void*>(&append_attn_kernel<kMaxNew>),
+                            dim3(attn_splits, c.n_heads, B), dim3(kAttnWarps * 32), 0, st, false, attn_args, 1,
+                            attn_splits));
 
     fsx::TcGemmArgs go{};
     go.M = M;

@@ -1,0 +1,61 @@
+"""The append's rotary embedding and attention at the edges of their tiling, against the fp64 append oracle:
+cached lengths around the 32-key chunks and around the 128 keys that one CTA's four warps take in turn, 1 to 8 new
+tokens (both query-slot variants), and batches whose (vehicle, head) pairs run on 8, 4, 2 and 1 CTAs.
+
+Tolerance per row (one token's hidden state or one appended cache row), as a share of the row's largest entry: the
+new keys and values are rounded to bf16 (2^-9 = 2.0e-3 of an entry), the GEMM operands to fp16 (2^-11 = 4.9e-4 each,
+three GEMMs deep for a hidden state): below 2^-9 + 4 * 2^-11 = 4e-3; 6e-3 is asked."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from oracle import append_oracle
+from paper_2607_15621_gb300 import fsx, synth
+
+pytestmark = pytest.mark.gpu
+TOL = 6e-3
+
+
+def row_err(got, ref):
+    ref = np.asarray(ref, np.float64)
+    ref = ref.reshape(-1, ref.shape[-1])
+    got = np.asarray(got, np.float64).reshape(ref.shape)
+    return (np.abs(got - ref).max(-1) / np.maximum(np.abs(ref).max(-1), 1e-30)).max()
+
+
+@pytest.mark.parametrize("n_new,lengths", [
+    (4, [0]), (4, [31]), (1, [32]), (3, [33]), (8, [128]), (5, [1025]),
+    (4, [127, 0]), (8, [129, 32, 257]), (4, [1, 64, 31, 300, 0]), (7, [5, 0, 97, 128, 33]),
+])
+def test_append_attention_edges(n_new, lengths):
+    dims = synth.BackboneDims(n_layers=1, d_model=256, d_ff=256, n_new=n_new)
+    H, D, B = dims.n_heads, dims.head_dim, len(lengths)
+    w = synth.make_backbone_weights(dims, 5, "bf16")
+    off = np.concatenate([[0], np.cumsum(lengths)]).astype(np.int64)
+    total = int(off[-1])
+    dst = np.array([total + n_new * (B - 1 - b) for b in range(B)], dtype=np.int64)  # not in vehicle order
+    rows = total + n_new * B + 1
+    g = torch.Generator().manual_seed(n_new * 100 + B)
+    kc = (torch.randn(rows, H, D, generator=g) * torch.exp(0.5 * torch.randn(H, D, generator=g))).bfloat16()
+    vc = torch.randn(rows, H, D, generator=g).bfloat16()
+    x = synth.make_append_tokens(dims, B, seed=6)
+    kg, vg = kc.cuda(), vc.cuda()
+    hidden = torch.empty(B, n_new, dims.d_model, device="cuda")
+    ap = fsx.Append(dims, w, B, rows)
+    try:
+        ap.append([kg], [vg], torch.as_tensor(off).cuda(), torch.as_tensor(dst).cuda(), x.cuda(), hidden)
+        assert ap.status() == fsx.FSX_OK
+    finally:
+        ap.close()
+    h_ref, k_ref, v_ref = append_oracle.backbone_append(w, [kc[:total].float().numpy()], [vc[:total].float().numpy()],
+                                                        off, x.float().numpy(), H, D)
+    written = np.concatenate([np.arange(d0, d0 + n_new) for d0 in dst])
+    assert row_err(hidden.cpu().numpy().reshape(B * n_new, -1), np.asarray(h_ref).reshape(B * n_new, -1)) <= TOL
+    for got, was, ref in ((kg, kc, k_ref), (vg, vc, v_ref)):
+        got = got.cpu()
+        assert row_err(got[written].float().numpy().reshape(B * n_new, -1),
+                       np.asarray(ref[0]).reshape(B * n_new, -1)) <= TOL
+        keep = np.setdiff1d(np.arange(rows), written)
+        assert torch.equal(got[keep], was[keep])
