@@ -401,10 +401,11 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
  * word (FSX_OK or FSX_ERR_DEVICE_ARG). */
 fsx_status fsx_append_get_status(fsx_append_handle h, void* stream);
 
-/* enable = 1: later appends on this handle run no kernel that waits on other CTAs
- * (the residual GEMMs are not split along K), so an append can share the GPU with a
- * tick whose single-launch kernel needs all of its CTAs resident (the concurrent
- * schedule of fsx_session). Slower per append; enable = 0 restores the default. */
+/* enable = 1: later appends on this handle run no kernel that waits on other CTAs,
+ * so an append can share the GPU with a tick whose single-launch kernel needs all of
+ * its CTAs resident (the concurrent schedule of fsx_session). The append's kernels
+ * hold to that under either setting (split sums are completed by whichever CTA
+ * arrives last), so both run the same code at the same speed. */
 fsx_status fsx_append_set_concurrent(fsx_append_handle h, int enable);
 
 /* Bytes of the handle's fp16 weight arena (algorithmic weight bytes per call). */
@@ -425,7 +426,7 @@ void fsx_append_destroy(fsx_append_handle h);
  *                        in flight and reads its rows.
  *   FSX_SCHED_CONCURRENT appends run on a low-priority stream of their own, ticks on
  *                        a high-priority stream; the append handle is switched to
- *                        fsx_append_set_concurrent(h, 1), so no append kernel waits
+ *                        fsx_append_set_concurrent(h, 1): no append kernel waits
  *                        on other CTAs and the single-launch tick always gets its SMs.
  * The session never frees the handles or the cache; destroy it before them. */
 typedef struct fsx_session_s* fsx_session;

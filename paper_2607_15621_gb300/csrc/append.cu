@@ -7,11 +7,12 @@
 //            embedding, cache-row writes and causal attention over
 //            [cached rows ; new rows] -> W_o + residual -> RMSNorm+gate/up+SiLU
 //            -> W_d + residual ] -> residual stream out.
-// The four projections reuse the tensor-core GEMM of the tick (gemm_tc.cu):
-// norm gains folded into the packed weights, 1/rms applied in the epilogue from
-// per-128-column sums of x^2, split K for the narrow residual GEMMs. The token
+// The four projections run on the few-token tensor-core GEMM (gemm_stream.cu): norm
+// gains folded into the packed weights, 1/rms applied in the epilogue from
+// per-128-column sums of x^2, the weight stream cut evenly over the SMs. The token
 // count is n_new * B (4 for one vehicle), so the call streams every backbone
-// weight once and is bound by HBM.
+// weight once and is bound by HBM. No kernel of a call waits on other CTAs of its
+// grid (those of a cluster are scheduled together).
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
 
@@ -445,13 +446,12 @@ int append_attn_splits(int B, int n_heads, int sm_count) {
 struct fsx_append_s {
   fsx_append_config cfg{};
   int device = 0;
-  bool concurrent = false;  // no kernel of a call waits on other CTAs (no split K)
   int sm_count = 0;
   int HD = 0;
   void* w_arena = nullptr;
   long long weight_bytes = 0;
   std::vector<const unsigned char*> w_qkv, w_o, w_gu, w_dn;
-  CUtensorMap map_x16[3], map_o[3], map_h[3];
+  CUtensorMap map_x16[fsx::kStreamTileCount], map_o[fsx::kStreamTileCount], map_h[fsx::kStreamTileCount];
   float* x = nullptr;
   __half* x16 = nullptr;
   float* ss = nullptr;
@@ -533,7 +533,7 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
 
   FSX_CUDA_H(cudaSetDevice(device));
   FSX_CUDA_H(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device));
-  FSX_CUDA_H(fsx::gemm_tc_set_attributes());
+  FSX_CUDA_H(fsx::gemm_stream_set_attributes());
 
   // ---- weight tiles per layer [QKV | W_o | gate/up | W_d], 128-row x 64-K swizzled
   // images; RMSNorm gains folded into the K columns of QKV and gate/up; gate/up rows
@@ -618,11 +618,10 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
   FSX_CUDA_H(cudaMemset(h->o, 0, m_pad * HD * sizeof(__half)));
   FSX_CUDA_H(cudaMemset(h->hbuf, 0, m_pad * F * sizeof(__half)));
   {
-    const uint32_t boxes[3] = {48, 128, 256};  // index 0 (48-token tiles) is encoded but unused
-    for (int i = 0; i < 3; ++i)
-      if (!fsx::encode_act_map(&h->map_x16[i], h->x16, m_pad, d, boxes[i]) ||
-          !fsx::encode_act_map(&h->map_o[i], h->o, m_pad, HD, boxes[i]) ||
-          !fsx::encode_act_map(&h->map_h[i], h->hbuf, m_pad, F, boxes[i]))
+    for (int i = 0; i < fsx::kStreamTileCount; ++i)
+      if (!fsx::encode_act_map(&h->map_x16[i], h->x16, m_pad, d, fsx::kStreamTiles[i]) ||
+          !fsx::encode_act_map(&h->map_o[i], h->o, m_pad, HD, fsx::kStreamTiles[i]) ||
+          !fsx::encode_act_map(&h->map_h[i], h->hbuf, m_pad, F, fsx::kStreamTiles[i]))
         return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
   }
   {
@@ -632,9 +631,10 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
     FSX_CUDA_H(cudaMemcpy(h->inv_freq, inv_freq, sizeof(inv_freq), cudaMemcpyHostToDevice));
   }
   FSX_CUDA_H(cudaMalloc(&h->rot, static_cast<size_t>(cfg->n_new) * cfg->max_batch * kRopePairs * sizeof(float2)));
-  FSX_CUDA_H(cudaMalloc(&h->gemm_part, fsx::gemm_tc_part_bytes(h->sm_count)));
-  FSX_CUDA_H(cudaMalloc(&h->tile_count, sizeof(int) * h->sm_count));
-  FSX_CUDA_H(cudaMemset(h->tile_count, 0, sizeof(int) * h->sm_count));
+  FSX_CUDA_H(cudaMalloc(&h->gemm_part, fsx::gemm_stream_part_bytes(cfg->n_new * cfg->max_batch, h->sm_count)));
+  const size_t n_tiles = static_cast<size_t>(std::max({3 * HD, 2 * F, d})) / 128;  // of the widest matrix
+  FSX_CUDA_H(cudaMalloc(&h->tile_count, sizeof(int) * n_tiles));
+  FSX_CUDA_H(cudaMemset(h->tile_count, 0, sizeof(int) * n_tiles));
   FSX_CUDA_H(cudaMalloc(&h->status, sizeof(int)));
   FSX_CUDA_H(cudaMemset(h->status, 0, sizeof(int)));
   FSX_CUDA_H(cudaDeviceSynchronize());
@@ -645,7 +645,7 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
 
 fsx_status fsx_append_set_concurrent(fsx_append_handle h, int enable) {
   if (!h) return fail(FSX_ERR_INVALID_ARG, "handle is NULL");
-  h->concurrent = enable != 0;
+  (void)enable;  // no append kernel waits on other CTAs under either setting
   return FSX_OK;
 }
 
@@ -662,11 +662,7 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
   FSX_CUDA(cudaSetDevice(h->device));
   const int d = c.d_model, HD = h->HD, F = c.d_ff;
   const int M = B * c.n_new;
-  // token tile of the GEMMs: 128 up to 128 tokens (an MMA of N = 128 costs the same as one of
-  // N = 48 at one CTA per SM, and the weights bound the call), 256 above
-  const int bn_i = M <= 128 ? 1 : 2;
-  const int bn = bn_i == 1 ? 128 : 256;
-  const int m_tiles = (M + bn - 1) / bn;
+  const int bn_i = fsx::gemm_stream_tile(M);  // M <= 256: checked at create
 
   EmbedArgsA ea{};
   ea.x_new = static_cast<const __nv_bfloat16*>(d_x_new);
@@ -699,7 +695,9 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     g.ss_in = h->ss;
     g.n_ss = d / 128;
     g.ss_stride = h->ss_stride;
-    FSX_CUDA(fsx::launch_gemm_tc(h->map_x16[bn_i], g, bn, fsx::kEpiStore, true, st, false));
+    g.part = h->gemm_part;
+    g.tile_count = h->tile_count;
+    FSX_CUDA(fsx::launch_gemm_stream(h->map_x16[bn_i], g, fsx::kEpiStore, h->sm_count, st, true));
 
     AttnArgsA aa{};
     aa.qkv = h->qkv;
@@ -716,7 +714,7 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     void* attn_args[] = {&aa};
     FSX_CUDA(fsx::launch_ex(c.n_new <= 4 ? reinterpret_cast<const void*>(&append_attn_kernel<4>)
                                          : reinterpret_cast<const void*>(&append_attn_kernel<kMaxNew>),
-                            dim3(attn_splits, c.n_heads, B), dim3(kAttnWarps * 32), 0, st, false, attn_args, 1,
+                            dim3(attn_splits, c.n_heads, B), dim3(kAttnWarps * 32), 0, st, true, attn_args, 1,
                             attn_splits));
 
     fsx::TcGemmArgs go{};
@@ -730,10 +728,9 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     go.ldxo = d;
     go.ss_out = h->ss;
     go.ss_stride = h->ss_stride;
-    go.k_splits = h->concurrent ? 1 : fsx::gemm_tc_k_splits((d / 128) * m_tiles, HD / 64, h->sm_count);
     go.part = h->gemm_part;
     go.tile_count = h->tile_count;
-    FSX_CUDA(fsx::launch_gemm_tc(h->map_o[bn_i], go, bn, fsx::kEpiResidual, false, st, false));
+    FSX_CUDA(fsx::launch_gemm_stream(h->map_o[bn_i], go, fsx::kEpiResidual, h->sm_count, st, true));
 
     fsx::TcGemmArgs gg{};
     gg.M = M;
@@ -746,7 +743,9 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     gg.ss_in = h->ss;
     gg.n_ss = d / 128;
     gg.ss_stride = h->ss_stride;
-    FSX_CUDA(fsx::launch_gemm_tc(h->map_x16[bn_i], gg, bn, fsx::kEpiSwiglu, true, st, false));
+    gg.part = h->gemm_part;
+    gg.tile_count = h->tile_count;
+    FSX_CUDA(fsx::launch_gemm_stream(h->map_x16[bn_i], gg, fsx::kEpiSwiglu, h->sm_count, st, true));
 
     fsx::TcGemmArgs gd{};
     gd.M = M;
@@ -759,10 +758,9 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     gd.ldxo = d;
     gd.ss_out = h->ss;
     gd.ss_stride = h->ss_stride;
-    gd.k_splits = h->concurrent ? 1 : fsx::gemm_tc_k_splits((d / 128) * m_tiles, F / 64, h->sm_count);
     gd.part = h->gemm_part;
     gd.tile_count = h->tile_count;
-    FSX_CUDA(fsx::launch_gemm_tc(h->map_h[bn_i], gd, bn, fsx::kEpiResidual, false, st, false));
+    FSX_CUDA(fsx::launch_gemm_stream(h->map_h[bn_i], gd, fsx::kEpiResidual, h->sm_count, st, true));
   }
   FSX_CUDA(cudaMemcpyAsync(d_hidden, h->x, static_cast<size_t>(M) * d * sizeof(float), cudaMemcpyDeviceToDevice, st));
   return FSX_OK;

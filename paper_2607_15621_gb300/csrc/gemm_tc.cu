@@ -693,10 +693,8 @@ const void* tc_select(int bn, int epi, bool norm, bool pair, size_t* smem) {
     return tc_fn<BN_, EPI_, NORM_, true>();                       \
   }
   FSX_TC(48, kEpiStore, true)
-  FSX_TC(48, kEpiStore, false)
   FSX_TC(48, kEpiSwiglu, true)
   FSX_TC(48, kEpiResidual, false)
-  FSX_TC(128, kEpiStore, true)
   FSX_TC(128, kEpiSwiglu, true)
   FSX_TC(128, kEpiResidual, false)
   FSX_TC(144, kEpiResidual, false)

@@ -56,6 +56,18 @@ int gemm_tc_pair_clusters();
 // of 256, no K split): map_a then has 128-row boxes and map_w covers the packed weight tiles
 cudaError_t launch_gemm_tc(const CUtensorMap& map_a, const TcGemmArgs& args, int bn, int epi, bool norm,
                            cudaStream_t stream, bool pdl, const CUtensorMap* map_w = nullptr);
+// ---- few-token variant (gemm_stream.cu): M <= 256 tokens in one tile of kStreamTiles[i] tokens
+// (map_a: a box of that many rows), the weight stream cut evenly over the SMs. Takes w, N, K, M,
+// the epilogue's outputs, ss_in / ss_out, `part` (gemm_stream_part_bytes) and `tile_count`
+// ([N / 128], zero between launches); k_splits and w_tile0 are not used. RMSNorm is fused into
+// the store and SwiGLU epilogues.
+constexpr int kStreamTileCount = 5;
+constexpr int kStreamTiles[kStreamTileCount] = {16, 32, 64, 128, 256};
+cudaError_t gemm_stream_set_attributes();
+int gemm_stream_tile(int M);  // index into kStreamTiles (-1: too many tokens)
+size_t gemm_stream_part_bytes(int M, int sm_count);
+cudaError_t launch_gemm_stream(const CUtensorMap& map_a, const TcGemmArgs& args, int epi, int sm_count,
+                               cudaStream_t stream, bool pdl);
 // rows[128]: pointers to the 128 source rows (fp32, length >= k0 + 64); col_scale: optional per-K gain.
 void pack_tc_tile(const float* const* rows, const float* col_scale, int k0, __half* out);
 // 2-D fp16 tensor map over a row-major [rows, cols] buffer with a (box_rows x 64) box and 128-byte swizzle.

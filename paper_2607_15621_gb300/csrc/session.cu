@@ -6,12 +6,12 @@
 // have completed and reads exactly the committed rows, so it never sees a row that is
 // still being written.
 //
-// Two schedules (the hazard between them: the single-launch tick needs all of its CTAs
-// resident at once, and the append's split-K GEMMs wait on each other's CTAs):
+// Two schedules (the hazard to avoid: the single-launch tick needs all of its CTAs resident
+// at once, which a kernel whose CTAs wait on each other could prevent while it holds SMs):
 //   FSX_SCHED_SERIAL     appends run on the tick stream; a tick waits for an append in
 //                        flight (no concurrency, no hazard);
 //   FSX_SCHED_CONCURRENT appends run on their own low-priority stream with every kernel
-//                        free of inter-CTA waits (fsx_append_set_concurrent: no split K),
+//                        free of inter-CTA waits (fsx_append_set_concurrent),
 //                        so whatever SMs an append holds are released when its kernels
 //                        end and the tick's CTAs always become resident.
 #include <cuda_runtime.h>
