@@ -81,6 +81,7 @@ struct EmbedArgsA {
 };
 
 __global__ void __launch_bounds__(128) append_embed_kernel(const EmbedArgsA a) {
+  fsx::pdl_launch_dependents();  // the first GEMM fills its weight ring meanwhile
   const int m = blockIdx.x;
   if (m == 0) {
     const int64_t* off = a.offsets;
@@ -760,9 +761,9 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     gd.ss_stride = h->ss_stride;
     gd.part = h->gemm_part;
     gd.tile_count = h->tile_count;
+    gd.x_copy = l == c.n_layers - 1 ? d_hidden : nullptr;  // the residual stream after the last layer
     FSX_CUDA(fsx::launch_gemm_stream(h->map_h[bn_i], gd, fsx::kEpiResidual, h->sm_count, st, true));
   }
-  FSX_CUDA(cudaMemcpyAsync(d_hidden, h->x, static_cast<size_t>(M) * d * sizeof(float), cudaMemcpyDeviceToDevice, st));
   return FSX_OK;
 }
 

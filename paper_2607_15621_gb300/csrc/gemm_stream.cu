@@ -11,8 +11,8 @@
 // the CTA that arrives last on the tile's counter adds the segments in range order and runs
 // the epilogue. No CTA ever waits for another one, so the kernel may share the GPU with
 // kernels whose CTAs must all be resident, and the result does not depend on who is last.
-// Up to 12 steps (216 KB) are in flight per SM, requested before the previous kernel has
-// finished (programmatic dependent launch): they depend on no activation.
+// The first steps are requested before the previous kernel has finished (programmatic
+// dependent launch): weights depend on no activation.
 //   warp 0: producer (one bulk copy of the packed weight image and one 2-D TMA token box a
 //           step); warp 1: MMA issue (M = 128, N = BN, two accumulators in tensor memory);
 //   warps 2-9: epilogue, two groups of four warps (one per tensor-memory lane quadrant)
@@ -43,17 +43,34 @@ template <int BN>
 __host__ __device__ constexpr int stage_bytes() {
   return kWBytes + BN * kTcTileK * 2;
 }
+// With 16-token tiles a CTA takes half an SM, so that the next GEMM of the stream is resident and
+// fills its ring while the last steps and the split sums of this one run (two-layer append of 4
+// tokens: 237 -> 218 us a call together with the last GEMM writing the call's result itself).
+// From 32 tokens on the sums of the split tiles weigh more than the fill, and one CTA per SM with
+// a deeper ring and more registers for the sums is faster (64 tokens: 359 us a call with two CTAs
+// of 4 stages, 333 us with one of 9).
 template <int BN>
-__host__ __device__ constexpr int n_stages() {  // as many as the shared memory holds, at most 12
-  return BN <= 16 ? 12 : (BN <= 32 ? 11 : (BN <= 64 ? 9 : (BN <= 128 ? 6 : 4)));
+__host__ __device__ constexpr int ctas_per_sm() {
+  return BN <= 16 ? 2 : 1;
+}
+template <int BN>
+__host__ __device__ constexpr int n_stages() {  // as many as that share of the shared memory holds
+  return BN <= 16 ? 6 : (BN <= 32 ? 10 : (BN <= 64 ? 9 : (BN <= 128 ? 6 : 4)));
+}
+template <int BN>
+__host__ __device__ constexpr int sum_batch() {  // segments of a split tile in flight at once
+  return ctas_per_sm<BN>() == 2 ? 4 : 8;
 }
 template <int BN>
 __host__ __device__ constexpr int smem_bytes() {
   return 1024 /* alignment of the ring */ + kHeader + n_stages<BN>() * stage_bytes<BN>();
 }
-static_assert(smem_bytes<16>() <= 232448 && smem_bytes<32>() <= 232448 && smem_bytes<64>() <= 232448 &&
-                  smem_bytes<128>() <= 232448 && smem_bytes<256>() <= 232448,
-              "shared memory of a token tile exceeds the per-block limit");
+template <int BN>
+__host__ __device__ constexpr bool smem_fits() {  // 228 KB per SM, 1 KB of it reserved per CTA
+  return ctas_per_sm<BN>() * (smem_bytes<BN>() + 1024) <= 228 * 1024;
+}
+static_assert(smem_fits<16>() && smem_fits<32>() && smem_fits<64>() && smem_fits<128>() && smem_fits<256>(),
+              "shared memory of a token tile exceeds its share of an SM");
 
 __device__ __forceinline__ void tma_tokens(void* dst, const CUtensorMap* map, int k, uint64_t* bar) {
   asm volatile(
@@ -83,11 +100,12 @@ __device__ __forceinline__ void epi_sync() {
 }
 
 template <int BN, int EPI, bool NORM>
-__global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_constant__ CUtensorMap map_a,
+__global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kernel(const __grid_constant__ CUtensorMap map_a,
                                                                  const TcGemmArgs p) {
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int kStages = n_stages<BN>();
   constexpr int kStageBytes = stage_bytes<BN>();
+  constexpr int kBatch = sum_batch<BN>();
   constexpr uint32_t kTmemCols = 2 * BN <= 32 ? 32 : 2 * BN;  // two accumulators of BN fp32 columns
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -242,6 +260,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
             x[j] += v[j];
             p.xo[idx + static_cast<size_t>(j) * p.ldxo] = x[j];
             p.xo16[idx + static_cast<size_t>(j) * p.ldxo] = __float2half_rn(x[j]);
+            if (p.x_copy != nullptr) p.x_copy[idx + static_cast<size_t>(j) * p.ldxo] = x[j];
           }
 #pragma unroll
         for (int j = 0; j < kChunk; ++j) {
@@ -314,10 +333,10 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
             float v[kChunk];
 #pragma unroll
             for (int j = 0; j < kChunk; ++j) v[j] = 0.f;
-            for (int sg = 0; sg < n_seg; sg += 8) {  // in range order, 8 segments in flight
-              float4 w4[8][2];
+            for (int sg = 0; sg < n_seg; sg += kBatch) {  // in range order
+              float4 w4[kBatch][2];
 #pragma unroll
-              for (int e = 0; e < 8; ++e) {
+              for (int e = 0; e < kBatch; ++e) {
                 const int c = first + sg + e;
                 const float4* d = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(2 * c + (sg + e == 0 ? 1 : 0)) * kSlot) +
                                   static_cast<size_t>(c0 / 4) * kRows + row;
@@ -326,7 +345,7 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_stream_kernel(const __grid_c
                   w4[e][hh] = sg + e < n_seg ? __ldcg(d + hh * kRows) : make_float4(0.f, 0.f, 0.f, 0.f);
               }
 #pragma unroll
-              for (int e = 0; e < 8; ++e)
+              for (int e = 0; e < kBatch; ++e)
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
                   v[4 * hh] += w4[e][hh].x;

@@ -40,6 +40,8 @@ struct TcGemmArgs {
   int k_splits;
   float* part;
   int* tile_count;
+  // gemm_stream, kEpiResidual: optional second copy of the updated rows (layout of xo)
+  float* x_copy;
   // pair variant: index of the tile at `w` in the weight map (tiles of 16 KB from the map's base)
   int w_tile0;
 };
