@@ -120,21 +120,23 @@ __global__ void __launch_bounds__(128) append_embed_kernel(const EmbedArgsA a) {
 // vehicle b, head h, in one launch. The CTA rotates the new queries and keys itself
 // (cos / sin from the embed kernel) and rounds the new keys and values to bf16 in shared
 // memory; rank 0 of the cluster writes them to the cache rows dst[b] + i. The keys are the
-// vehicle's cached rows (positions 0 .. L_b-1) in 32-key chunks, then one chunk of its new
+// vehicle's cached rows (positions 0 .. L_b-1) in 16-key units, then one unit of its new
 // rows; new token i sees every cached row and new rows 0 .. i. Everything is fp32.
 //
 // The keys are few and every row is read once, so the kernel is bound by load latency:
-// a warp issues the loads of its chunk's K rows and half of its V rows (12 KB) before the first use,
-// the chunks go round robin over the 4 warps of `cluster` CTAs (as many as keep two CTAs
-// per SM for the batch), and the score step moves no key through shared memory: 4 lanes
-// share a key row (full 32-byte sectors), 4 keys per lane, and a transposed reduction over
-// the 4 lanes leaves key 8 j + g with lane 4 g + j. Both products use packed fp32 FMAs.
-// The CTAs of a cluster exchange their (max, sum, output) through distributed shared memory,
-// each merging its share of the n_new x 128 outputs.
-// Measured (two-layer append, 4 tokens a vehicle): one vehicle with 224 rows 392 -> 311 us a
-// call, 16 vehicles with 96-480 rows 552 -> 370 us, against separate rotary (fp64 pow and
-// sincos per pair and layer) and attention launches (a lane per key, one 32-key chunk's loads
-// dependent on the previous one's), which took 55 and 130 us of a layer.
+// a warp works on 16-key units, holds one unit's K and V rows (8 KB) in registers and issues
+// the next unit's K loads as soon as the scores are formed and its V loads after P V; four
+// CTAs share an SM (16 units in flight), and the units go round robin over the 4 warps of
+// `cluster` CTAs (as many as keep four CTAs per SM for the batch). No key moves through
+// shared memory: in the score step 4 lanes share a key row (full 32-byte sectors), 2 keys per
+// lane, and a transposed reduction over the 4 lanes leaves lane 4 g + 2 t + i with half i of
+// the queries of key 8 t + g. Both products use packed fp32 FMAs. The CTAs of a cluster
+// exchange their (max, sum, output) through distributed shared memory, each merging its share
+// of the n_new x 128 outputs.
+// Measured per layer (ncu, 4 tokens a vehicle): one vehicle with 224 rows 8.9 us a launch, 16
+// vehicles with 96-480 rows 31 us; the separate rotary (fp64 pow and sincos per pair and layer)
+// and attention (a lane per key) launches before took 55 and 130 us, and 32-key units with two
+// CTAs per SM 12.3 and 41 us.
 struct AttnArgsA {
   const __half* qkv;   // [M, 3 HD]: q | k | v before the rotation
   int ld;
@@ -151,6 +153,8 @@ struct AttnArgsA {
 
 constexpr int kNewStride = kHeadDim + 8;  // bf16 row stride of the new keys / values in shared memory
 constexpr int kMaxSplit = 8;              // CTAs of a cluster
+constexpr int kUnit = 16;                 // keys of a warp's unit of work
+static_assert(kMaxNew <= kUnit, "the new rows are one unit");
 
 // d += a * b on two packed fp32 values
 __device__ __forceinline__ void fma2(uint64_t& d, uint64_t a, uint64_t b) {
@@ -174,6 +178,13 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
 __device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t v) {
   return pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
+// 16 bytes of shared memory, read where it stands: hoisted out of the loop over the units, the
+// query values would take 32 registers per query
+__device__ __forceinline__ ulonglong2 ld_shared2(uint32_t addr) {
+  ulonglong2 v;
+  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(addr));
+  return v;
+}
 __device__ __forceinline__ uint32_t peer_addr(const void* local, int rank) {
   uint32_t r;
   asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(fsx::smem_addr(local)), "r"(rank));
@@ -185,82 +196,83 @@ __device__ __forceinline__ void st_peer(uint32_t addr, float v) {
 
 // NQ: query slots (4 or 8) for n_new <= NQ new tokens
 template <int NQ>
-__global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const AttnArgsA a) {
+__global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_kernel(const AttnArgsA a) {
   __shared__ __align__(16) float qs[NQ][kHeadDim];
   __shared__ __align__(16) __nv_bfloat16 kn[kMaxNew][kNewStride], vn[kMaxNew][kNewStride];
   __shared__ float sm_m[kAttnWarps][NQ], sm_l[kAttnWarps][NQ];
   __shared__ __align__(16) float sm_o[kAttnWarps][NQ][kHeadDim];
   __shared__ float rv_o[NQ * kHeadDim];                       // [split][this rank's share of the outputs]
   __shared__ float rv_m[kMaxSplit][NQ], rv_l[kMaxSplit][NQ];  // every split's running maxima and sums
+  constexpr int NH = NQ / 2;  // queries whose scores a lane keeps
   fsx::pdl_launch_dependents();
   fsx::pdl_wait();
-  if (status_set(a.status)) return;  // set before this launch or not at all: the same for the whole cluster
   const int S = gridDim.x, rank = blockIdx.x;  // the cluster spans the grid's x extent
   const int h = blockIdx.y, b = blockIdx.z;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nq = a.n_new;
+  const long long lo = a.offsets[b], hi = a.offsets[b + 1], d0 = a.dst[b];
+  if (status_set(a.status)) return;  // set before this launch or not at all: the same for the whole cluster
   if (S > 1) asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this CTA runs
-  const long long lo = a.offsets[b];
-  const int L = static_cast<int>(a.offsets[b + 1] - lo);
-  const long long d0 = a.dst[b];
-  const int n_chunks = (L + 31) / 32 + 1;  // the last one: the new rows
+  const int L = static_cast<int>(hi - lo);
+  const int n_units = (L + kUnit - 1) / kUnit + 1;  // the last one: the new rows
 
-  const int g = lane >> 2, j = lane & 3;    // scores: key group lane, 16-byte unit lane
+  const int g = lane >> 2, j = lane & 3;    // scores: key within a group of 8, 16-byte unit
   const int hv = lane >> 4, u = lane & 15;  // values: key parity, 16-byte unit
-  uint4 kraw[4][4], vraw[8];
-  // row loads of chunk c (zeros past the vehicle's rows): all K rows and V rows 0-15, then
-  // V rows 16-31 once the scores have released the registers of K
-  auto chunk_keys = [&](int c) { return c == n_chunks - 1 ? nq : min(32, L - 32 * c); };
-  auto chunk_base = [&](int c, __nv_bfloat16* cache, __nv_bfloat16* fresh) -> const __nv_bfloat16* {
-    if (c == n_chunks - 1) return fresh;
-    return cache + (static_cast<size_t>(lo) + 32 * static_cast<size_t>(c)) * a.HD + h * kHeadDim;
+  uint4 kraw[2][4], vraw[8];
+  // row loads of unit c (zeros past the vehicle's rows)
+  auto unit_keys = [&](int c) { return c == n_units - 1 ? nq : min(kUnit, L - kUnit * c); };
+  auto unit_base = [&](int c, const __nv_bfloat16* cache, const __nv_bfloat16* fresh) {
+    return c == n_units - 1 ? fresh : cache + (static_cast<size_t>(lo) + kUnit * static_cast<size_t>(c)) * a.HD + h * kHeadDim;
   };
-  auto load_v = [&](int c, int half) {
-    const int n = chunk_keys(c);
-    const size_t stride = c == n_chunks - 1 ? kNewStride : static_cast<size_t>(a.HD);
-    const __nv_bfloat16* vb = chunk_base(c, a.v_cache, &vn[0][0]);
+  auto load_k = [&](int c) {
+    const int n = unit_keys(c);
+    const size_t stride = c == n_units - 1 ? kNewStride : static_cast<size_t>(a.HD);
+    const __nv_bfloat16* kb = unit_base(c, a.k_cache, &kn[0][0]);
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
-      const int key = 16 * half + 2 * kk + hv;
-      vraw[kk] = key < n ? *reinterpret_cast<const uint4*>(vb + key * stride + u * 8) : make_uint4(0u, 0u, 0u, 0u);
-    }
-  };
-  auto load_chunk = [&](int c) {
-    const int n = chunk_keys(c);
-    const size_t stride = c == n_chunks - 1 ? kNewStride : static_cast<size_t>(a.HD);
-    const __nv_bfloat16* kb = chunk_base(c, a.k_cache, &kn[0][0]);
-#pragma unroll
-    for (int t = 0; t < 4; ++t)
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
       for (int i = 0; i < 4; ++i)
         kraw[t][i] = 8 * t + g < n ? *reinterpret_cast<const uint4*>(kb + (8 * t + g) * stride + (4 * i + j) * 8)
                                    : make_uint4(0u, 0u, 0u, 0u);
-    load_v(c, 0);
+  };
+  auto load_v = [&](int c) {
+    const int n = unit_keys(c);
+    const size_t stride = c == n_units - 1 ? kNewStride : static_cast<size_t>(a.HD);
+    const __nv_bfloat16* vb = unit_base(c, a.v_cache, &vn[0][0]);
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk)
+      vraw[kk] = 2 * kk + hv < n ? *reinterpret_cast<const uint4*>(vb + (2 * kk + hv) * stride + u * 8)
+                                 : make_uint4(0u, 0u, 0u, 0u);
   };
   const int step = S * kAttnWarps;
   int c = rank * kAttnWarps + warp;
-  if (c < n_chunks - 1) load_chunk(c);  // in flight while the new rows are rotated
+  if (c < n_units - 1) {  // in flight while the new rows are rotated
+    load_k(c);
+    load_v(c);
+  }
 
   const float scale = 1.4426950408889634f * rsqrtf(static_cast<float>(kHeadDim));  // log2(e) / sqrt(128)
-  for (int t = tid; t < NQ * kRopePairs; t += kAttnWarps * 32) {
-    const int i = t / kRopePairs, jj = t - i * kRopePairs;
-    if (i >= nq) {
+#pragma unroll
+  for (int t0 = 0; t0 < NQ * kRopePairs; t0 += kAttnWarps * 32) {
+    const int i = (t0 + tid) / kRopePairs, jj = tid % kRopePairs;
+    if (i < nq) {
+      const int m = b * nq + i;
+      const float2 cs = a.rot[static_cast<size_t>(m) * kRopePairs + jj];
+      const __half* q = a.qkv + static_cast<size_t>(m) * a.ld + h * kHeadDim + jj;
+      const __half* k = q + a.HD;
+      const __half* v = q + 2 * a.HD;
+      const float q0 = __half2float(q[0]), q1 = __half2float(q[kRopePairs]);
+      const float k0 = __half2float(k[0]), k1 = __half2float(k[kRopePairs]);
+      const float v0 = __half2float(v[0]), v1 = __half2float(v[kRopePairs]);
+      qs[i][jj] = (q0 * cs.x - q1 * cs.y) * scale;
+      qs[i][jj + kRopePairs] = (q0 * cs.y + q1 * cs.x) * scale;
+      kn[i][jj] = __float2bfloat16_rn(k0 * cs.x - k1 * cs.y);
+      kn[i][jj + kRopePairs] = __float2bfloat16_rn(k0 * cs.y + k1 * cs.x);
+      vn[i][jj] = __float2bfloat16_rn(v0);
+      vn[i][jj + kRopePairs] = __float2bfloat16_rn(v1);
+    } else {
       qs[i][jj] = qs[i][jj + kRopePairs] = 0.f;
-      continue;
     }
-    const int m = b * nq + i;
-    const float2 cs = a.rot[static_cast<size_t>(m) * kRopePairs + jj];
-    const __half* q = a.qkv + static_cast<size_t>(m) * a.ld + h * kHeadDim + jj;
-    const __half* k = q + a.HD;
-    const __half* v = q + 2 * a.HD;
-    const float q0 = __half2float(q[0]), q1 = __half2float(q[kRopePairs]);
-    const float k0 = __half2float(k[0]), k1 = __half2float(k[kRopePairs]);
-    qs[i][jj] = (q0 * cs.x - q1 * cs.y) * scale;
-    qs[i][jj + kRopePairs] = (q0 * cs.y + q1 * cs.x) * scale;
-    kn[i][jj] = __float2bfloat16_rn(k0 * cs.x - k1 * cs.y);
-    kn[i][jj + kRopePairs] = __float2bfloat16_rn(k0 * cs.y + k1 * cs.x);
-    vn[i][jj] = __float2bfloat16_rn(__half2float(v[0]));
-    vn[i][jj + kRopePairs] = __float2bfloat16_rn(__half2float(v[kRopePairs]));
   }
   __syncthreads();
   if (rank == 0)  // the new cache rows, 16 bytes a thread
@@ -271,31 +283,38 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const A
       *reinterpret_cast<uint4*>(a.v_cache + o) = *reinterpret_cast<const uint4*>(&vn[i][uu * 8]);
     }
 
-  float m_run[NQ], l_run[NQ];  // l_run: this lane's keys only
-  uint64_t o[NQ][4];           // this half warp's keys, value dims 8 u .. 8 u + 7
+  const uint32_t q_addr = fsx::smem_addr(&qs[0][8 * j]);  // unit 4 i + j of query qi: 128 qi + 32 i values on
+  const int q_lane = (j & 1) * NH;  // this lane's queries q_lane .. q_lane + NH - 1
+  float m_run[NH], l_run[NH];       // l_run: this lane's keys only
+  uint64_t o[NQ][4];                // this half warp's keys, value dims 8 u .. 8 u + 7
 #pragma unroll
-  for (int qi = 0; qi < NQ; ++qi) {
-    m_run[qi] = -INFINITY;
-    l_run[qi] = 0.f;
+  for (int qq = 0; qq < NH; ++qq) {
+    m_run[qq] = -INFINITY;
+    l_run[qq] = 0.f;
+  }
+#pragma unroll
+  for (int qi = 0; qi < NQ; ++qi)
 #pragma unroll
     for (int e = 0; e < 4; ++e) o[qi][e] = 0ull;
+  if (c == n_units - 1) {  // a warp whose first unit is the new rows
+    load_k(c);
+    load_v(c);
   }
-  bool loaded = c < n_chunks - 1;
-  for (; c < n_chunks; c += step) {
-    if (!loaded) load_chunk(c);
-    loaded = false;
-    const bool own = c == n_chunks - 1;
-    const int n = chunk_keys(c);
-    uint64_t acc[4][NQ];
+#pragma unroll 1
+  for (; c < n_units; c += step) {
+    const bool own = c == n_units - 1;
+    const int n = unit_keys(c);
+    const int next = c + step;
+    uint64_t acc[2][NQ];
 #pragma unroll
-    for (int t = 0; t < 4; ++t)
+    for (int t = 0; t < 2; ++t)
 #pragma unroll
       for (int qi = 0; qi < NQ; ++qi) acc[t][qi] = 0ull;
 #pragma unroll
     for (int i = 0; i < 4; ++i) {
-      uint64_t kv[4][4];
+      uint64_t kv[2][4];
 #pragma unroll
-      for (int t = 0; t < 4; ++t) {
+      for (int t = 0; t < 2; ++t) {
         kv[t][0] = bf16x2_to_f32x2(kraw[t][i].x);
         kv[t][1] = bf16x2_to_f32x2(kraw[t][i].y);
         kv[t][2] = bf16x2_to_f32x2(kraw[t][i].z);
@@ -303,10 +322,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const A
       }
 #pragma unroll
       for (int qi = 0; qi < NQ; ++qi) {
-        const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&qs[qi][(4 * i + j) * 8]);
-        const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(&qs[qi][(4 * i + j) * 8 + 4]);
+        const ulonglong2 qa = ld_shared2(q_addr + (qi * kHeadDim + 32 * i) * 4);
+        const ulonglong2 qb = ld_shared2(q_addr + (qi * kHeadDim + 32 * i + 4) * 4);
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
+        for (int t = 0; t < 2; ++t) {
           fma2(acc[t][qi], kv[t][0], qa.x);
           fma2(acc[t][qi], kv[t][1], qa.y);
           fma2(acc[t][qi], kv[t][2], qb.x);
@@ -314,63 +333,64 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const A
         }
       }
     }
-    // transposed sum over the 4 lanes of a key row: lane 4 g + j keeps key 8 j + g
-    float p[NQ];
+    if (next < n_units) load_k(next);
+    // transposed sum over the 4 lanes of a key row: first the key group, then the query half
+    const bool up2 = (j & 2) != 0, up1 = (j & 1) != 0;
+    float r[NQ], p[NH];
 #pragma unroll
     for (int qi = 0; qi < NQ; ++qi) {
-      float s[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const float2 f = unpack2(acc[t][qi]);
-        s[t] = f.x + f.y;
-      }
-      const bool up2 = (j & 2) != 0, up1 = (j & 1) != 0;
-      const float a0 = (up2 ? s[2] : s[0]) + __shfl_xor_sync(0xffffffffu, up2 ? s[0] : s[2], 2);
-      const float a1 = (up2 ? s[3] : s[1]) + __shfl_xor_sync(0xffffffffu, up2 ? s[1] : s[3], 2);
-      p[qi] = (up1 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up1 ? a0 : a1, 1);
+      const float2 f0 = unpack2(acc[0][qi]), f1 = unpack2(acc[1][qi]);
+      const float a0 = f0.x + f0.y, a1 = f1.x + f1.y;
+      r[qi] = (up2 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up2 ? a0 : a1, 2);
     }
-    const int key = 8 * j + g;
 #pragma unroll
-    for (int qi = 0; qi < NQ; ++qi) {
-      // visible: a real key that is a cached row or a new row <= qi
+    for (int qq = 0; qq < NH; ++qq)
+      p[qq] = (up1 ? r[NH + qq] : r[qq]) + __shfl_xor_sync(0xffffffffu, up1 ? r[qq] : r[NH + qq], 1);
+    const int key = 8 * (j >> 1) + g;
+    float alpha[NH];
+    bool moved = false;
+#pragma unroll
+    for (int qq = 0; qq < NH; ++qq) {
+      // visible: a real key that is a cached row or a new row <= the query's
+      const int qi = q_lane + qq;
       const bool vis = qi < nq && key < n && (!own || key <= qi);
-      const float sv = vis ? p[qi] : -INFINITY;
-      float mx = sv;
+      const float sv = vis ? p[qq] : -INFINITY;
+      float mx = sv;  // over the 16 keys: the lanes with this lane's query half
 #pragma unroll
-      for (int sh = 16; sh > 0; sh >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, sh));
-      const float m_new = fmaxf(m_run[qi], mx);
-      if (m_new == -INFINITY) {  // an unused query slot
-        p[qi] = 0.f;
-        continue;
-      }
-      const float alpha = exp2f(m_run[qi] - m_new);
-      p[qi] = vis ? exp2f(sv - m_new) : 0.f;
-      l_run[qi] = l_run[qi] * alpha + p[qi];
-      m_run[qi] = m_new;
-      const uint64_t al = pack2(alpha, alpha);
-#pragma unroll
-      for (int e = 0; e < 4; ++e) o[qi][e] = mul2(o[qi][e], al);
+      for (int sh = 16; sh > 1; sh >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, sh));
+      const float m_new = fmaxf(m_run[qq], mx);
+      const bool none = m_new == -INFINITY;  // an unused query slot
+      alpha[qq] = none ? 1.f : exp2f(m_run[qq] - m_new);
+      p[qq] = vis && !none ? exp2f(sv - m_new) : 0.f;
+      l_run[qq] = l_run[qq] * alpha[qq] + p[qq];
+      moved = moved || alpha[qq] != 1.f;
+      m_run[qq] = m_new;
     }
-    auto attend = [&](int half) {
+    if (__any_sync(0xffffffffu, moved)) {
 #pragma unroll
-      for (int kk = 0; kk < 8; ++kk) {
-        const uint64_t v0 = bf16x2_to_f32x2(vraw[kk].x), v1 = bf16x2_to_f32x2(vraw[kk].y);
-        const uint64_t v2 = bf16x2_to_f32x2(vraw[kk].z), v3 = bf16x2_to_f32x2(vraw[kk].w);
-        const int kv = 16 * half + 2 * kk + hv;  // its probability is with lane 4 (kv mod 8) + kv / 8
+      for (int qi = 0; qi < NQ; ++qi) {
+        const float av = __shfl_sync(0xffffffffu, alpha[qi % NH], qi / NH);
+        const uint64_t al = pack2(av, av);
 #pragma unroll
-        for (int qi = 0; qi < NQ; ++qi) {
-          const float pk = __shfl_sync(0xffffffffu, p[qi], ((kv & 7) << 2) | (kv >> 3));
-          const uint64_t pp = pack2(pk, pk);
-          fma2(o[qi][0], pp, v0);
-          fma2(o[qi][1], pp, v1);
-          fma2(o[qi][2], pp, v2);
-          fma2(o[qi][3], pp, v3);
-        }
+        for (int e = 0; e < 4; ++e) o[qi][e] = mul2(o[qi][e], al);
       }
-    };
-    attend(0);
-    load_v(c, 1);
-    attend(1);
+    }
+#pragma unroll
+    for (int kk = 0; kk < 8; ++kk) {
+      const uint64_t v0 = bf16x2_to_f32x2(vraw[kk].x), v1 = bf16x2_to_f32x2(vraw[kk].y);
+      const uint64_t v2 = bf16x2_to_f32x2(vraw[kk].z), v3 = bf16x2_to_f32x2(vraw[kk].w);
+      const int kv = 2 * kk + hv;  // its probabilities are with lanes 4 (kv mod 8) + 2 (kv / 8) + query half
+#pragma unroll
+      for (int qi = 0; qi < NQ; ++qi) {
+        const float pk = __shfl_sync(0xffffffffu, p[qi % NH], ((kv & 7) << 2) | ((kv >> 3) << 1) | (qi / NH));
+        const uint64_t pp = pack2(pk, pk);
+        fma2(o[qi][0], pp, v0);
+        fma2(o[qi][1], pp, v1);
+        fma2(o[qi][2], pp, v2);
+        fma2(o[qi][3], pp, v3);
+      }
+    }
+    if (next < n_units) load_v(next);
   }
 #pragma unroll
   for (int qi = 0; qi < NQ; ++qi) {
@@ -383,10 +403,15 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const A
     }
     *reinterpret_cast<float4*>(&sm_o[warp][qi][u * 8 + hv * 4]) =
         hv == 0 ? make_float4(ov[0], ov[1], ov[2], ov[3]) : make_float4(ov[4], ov[5], ov[6], ov[7]);
-    const float l = fsx::warp_sum(l_run[qi]);
-    if (lane == 0) {
-      sm_m[warp][qi] = m_run[qi];
-      sm_l[warp][qi] = l;
+  }
+#pragma unroll
+  for (int qq = 0; qq < NH; ++qq) {
+    float l = l_run[qq];
+#pragma unroll
+    for (int sh = 16; sh > 1; sh >>= 1) l += __shfl_xor_sync(0xffffffffu, l, sh);
+    if (lane < 2) {
+      sm_m[warp][q_lane + qq] = m_run[qq];
+      sm_l[warp][q_lane + qq] = l;
     }
   }
   __syncthreads();
@@ -435,10 +460,10 @@ __global__ void __launch_bounds__(kAttnWarps * 32, 2) append_attn_kernel(const A
 }
 
 // CTAs per (vehicle, head): the largest power of two up to 8 that keeps the batch's CTAs
-// within two per SM
+// within the four that share an SM
 int append_attn_splits(int B, int n_heads, int sm_count) {
   int s = kMaxSplit;
-  while (s > 1 && static_cast<long long>(B) * n_heads * s > 2ll * sm_count) s >>= 1;
+  while (s > 1 && static_cast<long long>(B) * n_heads * s > 4ll * sm_count) s >>= 1;
   return s;
 }
 
