@@ -30,9 +30,11 @@
  *     magnitude that rounds past 65504, infinity or NaN) is a device-side error:
  *     the status becomes FSX_ERR_RANGE and the tick is abandoned like on bad
  *     offsets, writing no waypoint, instead of returning NaN waypoints. In the
- *     tensor-core attention the check is made on the scores: a key beyond the
+ *     bf16 tensor-core attention of batched ticks (one key split, five vehicles or
+ *     more at 32 heads) the check is made on the scores: a key beyond the
  *     range whose scores all fall to -inf has weight zero, as its exact value
- *     would, and is not reported.
+ *     would, and is not reported. With key splits (fewer vehicles) or fp32 caches
+ *     every cache value is checked, the values that stay bf16 too.
  */
 #ifndef FSX_H
 #define FSX_H

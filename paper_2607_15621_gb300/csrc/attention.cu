@@ -3,6 +3,9 @@
 // of that layer's backbone cache rows (read only) and the expert's own keys and
 // values. No mask, no rotary phase on the expert side, scale 1/sqrt(128).
 //
+// The general kernel, for calls outside the tensor-core kernel's range (attention_tc.cu: 1 to 64
+// own keys and at most 8 splits, which every tick meets): no own keys or more than 64, or more
+// than 8 splits.
 // Split-KV flash decoding: the L_b + T keys of a vehicle are cut into
 // n_splits near-equal ranges; one CTA (3 warps x 16 queries = 48 query rows)
 // streams its range in 32-key chunks. Each chunk is staged raw (bf16 / fp32 cache
@@ -136,27 +139,15 @@ __global__ void __launch_bounds__(kThreads, FSX_ATTN_MIN_CTAS) attn_splitkv_kern
 
   pdl_launch_dependents();
   pdl_wait();
-  const int b = p.order != nullptr ? p.order[blockIdx.z] : static_cast<int>(blockIdx.z);
+  const int b = static_cast<int>(blockIdx.z);
   // The CTAs of a merge cluster read each other's shared memory, so they must
   // all stay; a raised status is honoured per vehicle below instead.
   if (!CM && *reinterpret_cast<volatile int*>(p.status) != 0) return;
 
-  const CT* kc;
-  const CT* vc;
-  const int64_t* offs;
-  const int64_t* starts = nullptr;
-  if (p.targs != nullptr) {
-    kc = static_cast<const CT*>(p.targs->k_cache[p.layer]);
-    vc = static_cast<const CT*>(p.targs->v_cache[p.layer]);
-    offs = p.targs->offsets;
-    starts = p.targs->starts;
-  } else {
-    kc = static_cast<const CT*>(p.k_cache);
-    vc = static_cast<const CT*>(p.v_cache);
-    offs = p.offsets;
-  }
-  const long long o_lo = starts != nullptr ? starts[b] : offs[b];
-  const long long o_hi = o_lo + (offs[b + 1] - offs[b]);
+  const CT* kc = static_cast<const CT*>(p.k_cache);
+  const CT* vc = static_cast<const CT*>(p.v_cache);
+  const long long o_lo = p.offsets[b];
+  const long long o_hi = p.offsets[b + 1];
   if (o_lo < 0 || o_hi < o_lo || o_hi > p.max_total ||
       (o_hi > o_lo && (kc == nullptr || vc == nullptr))) {  // never read outside the caller's cache
     set_status(p.status, kStatusDeviceArg);
@@ -574,37 +565,47 @@ size_t attention_workspace_bytes(int B, int n_heads, int n_splits) {
 
 int attention_launch_count(int n_splits) { return n_splits > kMaxClusterSplits ? 2 : 1; }
 
-cudaError_t attention_set_attributes() {
-  const void* fns[4] = {reinterpret_cast<const void*>(&attn_splitkv_kernel<__nv_bfloat16, false>),
-                        reinterpret_cast<const void*>(&attn_splitkv_kernel<__nv_bfloat16, true>),
-                        reinterpret_cast<const void*>(&attn_splitkv_kernel<float, false>),
-                        reinterpret_cast<const void*>(&attn_splitkv_kernel<float, true>)};
-  const size_t bytes[4] = {attn_smem_bytes<__nv_bfloat16>(), attn_smem_bytes<__nv_bfloat16>(),
-                           attn_smem_bytes<float>(), attn_smem_bytes<float>()};
-  for (int i = 0; i < 4; ++i) {
-    cudaError_t e = cudaFuncSetAttribute(fns[i], cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(bytes[i]));
+namespace {
+// the mma.sync kernel for these arguments and its shared memory
+const void* splitkv_fn(int cache_dtype, bool cluster_merge, size_t* smem) {
+  if (cache_dtype == 1) {
+    *smem = attn_smem_bytes<__nv_bfloat16>();
+    return cluster_merge ? reinterpret_cast<const void*>(&attn_splitkv_kernel<__nv_bfloat16, true>)
+                         : reinterpret_cast<const void*>(&attn_splitkv_kernel<__nv_bfloat16, false>);
+  }
+  *smem = attn_smem_bytes<float>();
+  return cluster_merge ? reinterpret_cast<const void*>(&attn_splitkv_kernel<float, true>)
+                       : reinterpret_cast<const void*>(&attn_splitkv_kernel<float, false>);
+}
+bool merges_in_cluster(int n_splits) { return n_splits > 1 && n_splits <= kMaxClusterSplits; }
+}  // namespace
+
+cudaError_t attention_set_attributes(const AttnArgs& a, int cache_dtype) {
+  if (attention_tc_eligible(a, a.n_splits)) return attention_tc_set_attributes(cache_dtype, a.n_splits > 1);
+  size_t smem = 0;
+  const void* fn = splitkv_fn(cache_dtype, merges_in_cluster(a.n_splits), &smem);
+  return cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+}
+
+cudaError_t attention_set_attributes(int cache_dtype) {
+  for (int split = 0; split < 2; ++split) {
+    size_t smem = 0;
+    const void* fn = splitkv_fn(cache_dtype, split != 0, &smem);
+    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(smem));
+    if (e == cudaSuccess) e = attention_tc_set_attributes(cache_dtype, split != 0);
     if (e != cudaSuccess) return e;
   }
-  return attention_tc_set_attributes();
+  return cudaSuccess;
 }
 
 cudaError_t launch_attention(const AttnArgs& a_in, int B, int cache_dtype, cudaStream_t stream, bool pdl) {
-  if (attention_tc_eligible(a_in, cache_dtype)) return launch_attention_tc(a_in, B, stream, pdl);
+  if (attention_tc_eligible(a_in, a_in.n_splits)) return launch_attention_tc(a_in, B, cache_dtype, stream, pdl);
   AttnArgs a = a_in;
   void* kargs[] = {&a};
   const dim3 grid(a.n_splits, a.n_heads, B);
-  const bool cm = a.n_splits > 1 && a.n_splits <= kMaxClusterSplits;
-  const void* fn;
-  size_t smem;
-  if (cache_dtype == 1) {
-    fn = cm ? reinterpret_cast<const void*>(&attn_splitkv_kernel<__nv_bfloat16, true>)
-            : reinterpret_cast<const void*>(&attn_splitkv_kernel<__nv_bfloat16, false>);
-    smem = attn_smem_bytes<__nv_bfloat16>();
-  } else {
-    fn = cm ? reinterpret_cast<const void*>(&attn_splitkv_kernel<float, true>)
-            : reinterpret_cast<const void*>(&attn_splitkv_kernel<float, false>);
-    smem = attn_smem_bytes<float>();
-  }
+  const bool cm = merges_in_cluster(a.n_splits);
+  size_t smem = 0;
+  const void* fn = splitkv_fn(cache_dtype, cm, &smem);
   cudaError_t e = launch_ex(fn, grid, dim3(kThreads), smem, stream, pdl, kargs, 1, cm ? a.n_splits : 1);
   if (e != cudaSuccess || a.n_splits <= kMaxClusterSplits) return e;
   return launch_ex(reinterpret_cast<const void*>(&attn_combine_kernel), dim3(a.n_heads, B, (a.n_q + 7) / 8), dim3(256),

@@ -101,9 +101,6 @@ extern "C" fsx_status fsx_attention_noalloc(const void* d_q, long long q_stride,
   void* base = nullptr;
   const fsx_status bs = scratch_base(&base);
   if (bs != FSX_OK) return bs;
-  if (fsx::attention_set_attributes() != cudaSuccess)
-    return noalloc_fail(FSX_ERR_CUDA, "cudaFuncSetAttribute failed");
-
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   int* status = static_cast<int*>(base);
   float* part = reinterpret_cast<float*>(static_cast<unsigned char*>(base) + kStatusSlot);
@@ -132,6 +129,8 @@ extern "C" fsx_status fsx_attention_noalloc(const void* d_q, long long q_stride,
   a.part_o = part;
   a.part_lse = part + static_cast<size_t>(B) * n_heads * n_splits * fsx::kTokTile * fsx::kHeadDim;
   a.status = status;
+  if (fsx::attention_set_attributes(a, cache_dtype) != cudaSuccess)
+    return noalloc_fail(FSX_ERR_CUDA, "cudaFuncSetAttribute failed");
   e = fsx::launch_attention(a, B, cache_dtype, st, false);
   if (e != cudaSuccess) return noalloc_fail(FSX_ERR_CUDA, cudaGetErrorString(e));
   return FSX_OK;

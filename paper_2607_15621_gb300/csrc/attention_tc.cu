@@ -1,34 +1,48 @@
-// Eq. 1 of Sec. 3.1 on the 5th-generation tensor cores: one CTA per (vehicle,
-// head) computes softmax(Q [K_vlm ; K_ae]^T / sqrt(128)) [V_vlm ; V_ae] for the
-// expert's queries (at most 48, padded to an M = 64 tile) with a bf16 backbone
-// cache, one split, fp32 accumulation. S = Q K^T in fp16: the bf16 cache K rows are
-// converted in shared memory (exact for |x| in [2^-14, 65504]) by the warps that
-// stage them. P V keeps the cache V rows in bf16 and splits P into bf16 P_hi + P_lo
-// (16 significant bits, more than fp16's 11); the own chunk (fp16 V) splits P into
-// fp16 P_hi + P_lo instead.
+// Eq. 1 of Sec. 3.1 on the 5th-generation tensor cores: one CTA per (vehicle, head, key split)
+// computes softmax(Q [K_vlm ; K_ae]^T / sqrt(128)) [V_vlm ; V_ae] for the
+// expert's queries (at most 48, padded to an M = 64 tile) with a bf16 or fp32 backbone
+// cache, fp32 accumulation. S = Q K^T in fp16: the cache K rows are
+// converted in shared memory (exact for bf16 |x| in [2^-14, 65504]) by the warps that
+// stage them. P V keeps bf16 cache V rows in bf16 and splits P into bf16 P_hi + P_lo
+// (16 significant bits, more than fp16's 11); the own chunk (fp16 V) and fp32 cache rows
+// (converted to fp16) split P into fp16 P_hi + P_lo instead.
 //
-// Data path ("slot" = 64 keys; shared-memory operands 128-byte swizzled):
-//   Q             [64 q][128 d] fp16   smem, A of S          (K-major)
-//   K slot (x3)   [64 keys][128 d]     smem, B of S          (K-major)
-//   V slot (x3)   [64 keys][128 d]     smem, B of P V        (N = d contiguous, MN-major;
-//                                      bf16 cache rows, fp16 own rows)
-//   S (x2)        [64 q][64 keys] fp32 tensor memory, 64 columns each
-//   P_hi, P_lo    [64 q][64 keys]      tensor memory, A of P V, written over the
-//                                      S buffer they were computed from (32 columns each)
-//   O             [64 q][128 d] fp32   tensor memory, 128 columns
+// Data path ("slot" = 64 keys; shared-memory operands 128-byte swizzled; kSlots = 3, 2 for fp32):
+//   Q                [64 q][128 d] fp16   smem, A of S          (K-major)
+//   K slot (xkSlots) [64 keys][128 d]     smem, B of S          (K-major)
+//   V slot (xkSlots) [64 keys][128 d]     smem, B of P V        (N = d contiguous, MN-major;
+//                                         bf16 cache rows, fp16 own rows and fp32 caches)
+//   raw (x2, fp32)   [64 keys][128 d] fp32 smem, rows as they lie in the cache, per tensor
+//   S (x2)           [64 q][64 keys] fp32 tensor memory, 64 columns each
+//   P_hi, P_lo       [64 q][64 keys]      tensor memory, A of P V, written over the
+//                                         S buffer they were computed from (32 columns each)
+//   O                [64 q][128 d] fp32   tensor memory, 128 columns
 //   Row q of an M = 64 tile lives in lane (q mod 16) + 32 (q / 16).
-// Chunk 0 holds the expert's own keys (fp16 as produced), chunk 1 + j the cache keys
-// [64 j, 64 j + 64); chunk i sits in K / V slot i mod 3.
+// The vehicle's cache keys are cut into 64-key chunks and the chunks into near-equal runs, one
+// per split; split 0 (never the longest run) takes the expert's own keys (fp16 as produced) as
+// its chunk 0 before its cache chunks. Chunk i sits in K / V slot i mod kSlots.
 //
-// Warp roles (256 threads): warps 0-2 run the online softmax for query rows
+// Warp roles: warps 0-2 run the online softmax for query rows
 // 16 w .. 16 w + 15, two rows per thread; warp 3 lane 0 issues S and P V as their inputs become
-// ready; warps 4-5 stage (and convert) the K rows, warps 6-7 the V rows, two chunks ahead.
+// ready; then 2 warps (4 for fp32) stage and convert the K rows and as many the V rows, two
+// chunks ahead. bf16 caches: two CTAs per SM, whole chunks by TMA. fp32 caches: twice the bytes
+// a key, so one CTA per SM holds two raw chunks per tensor (128 KB) in flight by 16-byte copies;
+// a warp converts only rows that it copied.
+// Splits: the CTAs of one (vehicle, head) form a thread-block cluster and merge
+// (log-sum-exp weights) by pushing each split's normalised fp32 rows to the rank that owns them
+// through distributed shared memory. Split and fp32 launches check every cache value they stage
+// against the fp16 range.
+// Measured against the mma.sync kernel of attention.cu, which split and fp32 launches ran before: a
+// tick of 4 vehicles with 0-700 bf16 rows, 8 layers, 2 splits: 740 -> 452 us; one vehicle with 2048
+// rows, 8 splits, Eq. 1 alone: 34 -> 27 us a call; 24 vehicles with 16-1000 fp32 rows, Eq. 1
+// alone: 104 -> 81 us a call (4.1 TB/s).
 // Every wait is bounded; a timeout raises the status word and the CTA drains its
 // MMAs before it frees the tensor memory.
 #include <cuda.h>
 #include <math_constants.h>
 
 #include "device_util.cuh"
+#include "gemm_tc.h"
 #include "kernels.h"
 #include "tcgen05.cuh"
 
@@ -38,27 +52,46 @@ namespace {
 
 constexpr int kD = kHeadDim;           // 128
 constexpr int kSlotKeys = 64;          // keys per chunk
-constexpr int kThreadsTc = 256;
 constexpr int kSoftmaxWarps = 3;       // rows 0..47
 constexpr int kMmaWarp = 3;
-constexpr int kProdWarp0 = 4;     // warps 4-5 stage K, warps 6-7 stage V
-constexpr int kProdThreads = 64;  // per tensor
+constexpr int kProdWarp0 = 4;          // then the K staging warps, then the V staging warps
 constexpr int kTmemCols = 256;         // S[2] x 64 + O 128
 constexpr uint32_t kColS = 0;    // S / P buffers at columns 0 and 64
 constexpr uint32_t kColO = 128;
+constexpr int kMaxClusterSplits = 8;
 
 // shared-memory layout (bytes from the 1024-aligned base)
 constexpr int kQBytes = 64 * kD * 2;            // 16 KB
 constexpr int kSlotBytes = kSlotKeys * kD * 2;  // 16 KB
-constexpr int kSlots = 3;                       // per tensor
-constexpr int kOffQ = 0;
-constexpr int kOffK = kOffQ + kQBytes;
-constexpr int kOffV = kOffK + kSlots * kSlotBytes;
-constexpr int kOffBar = kOffV + kSlots * kSlotBytes;
+constexpr int kRawBytes = kSlotKeys * kD * 4;   // one fp32 chunk of a tensor
 // barriers: kfull[3], kempty[3], vfull[3], vempty[3], sfull[2], pfull[2], pvdone[2], drain, ktma[3], vtma[3]
 constexpr int kNumBars = 25;
-constexpr int kSmemTc = kOffBar + kNumBars * 8 + 8 /*tmem slot + abort*/;
-static_assert(kSmemTc + 1024 <= (228 * 1024) / 2, "two CTAs per SM");
+template <bool F32>
+struct CacheType {
+  using T = __nv_bfloat16;
+};
+template <>
+struct CacheType<true> {
+  using T = float;
+};
+template <bool F32>
+struct Shape {
+  static constexpr int kSlots = F32 ? 2 : 3;           // per tensor
+  static constexpr int kProdWarps = F32 ? 4 : 2;       // per tensor
+  static constexpr int kProdThreads = 32 * kProdWarps;
+  static constexpr int kThreads = 32 * (kProdWarp0 + 2 * kProdWarps);
+  static constexpr int kOffQ = 0;
+  static constexpr int kOffK = kOffQ + kQBytes;
+  static constexpr int kOffV = kOffK + kSlots * kSlotBytes;
+  static constexpr int kOffRaw = kOffV + kSlots * kSlotBytes;  // [K, V][2]
+  static constexpr int kOffBar = kOffRaw + (F32 ? 4 * kRawBytes : 0);
+  static constexpr int kSmem = kOffBar + kNumBars * 8 + 8 /*tmem slot + abort*/;
+  static constexpr int kCtas = F32 ? 1 : 2;            // per SM
+};
+static_assert(2 * (Shape<false>::kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(Shape<true>::kSmem + 1024 <= 228 * 1024, "one CTA per SM");
+// merge buffers at the start of the K slots: at most (48 + 7) rows of 128 fp32 values, then their log-sum-exps
+static_assert((48 + kMaxClusterSplits - 1) * (kD + 1) * 4 <= Shape<true>::kSlots * kSlotBytes, "merge buffers");
 
 // byte offset of 16-byte unit u (8 elements) of row r in a [rows][128] tile made of
 // 64-element swizzled column blocks (1024-byte atoms of 8 rows; blocks 8 KB apart
@@ -184,6 +217,27 @@ __device__ __forceinline__ void tmem_st_16x128b_x8(uint32_t taddr, const uint32_
 
 constexpr float kLazyRescale = 8.f;  // log2 units; P <= 2^8 between rescales
 
+// bits 15 / 31 set where a bf16 value lies outside the fp16 range (magnitude bits >= 0x4780)
+__device__ __forceinline__ uint32_t bf16x2_out_of_range(uint32_t v) {
+  return ((v & 0x7fff7fffu) + 0x38803880u) & 0x80008000u;
+}
+
+// arrive at and wait for the cluster's barrier (threads of a warp may come apart)
+__device__ __forceinline__ void cluster_barrier() {
+  asm volatile("barrier.cluster.arrive.release;\nbarrier.cluster.wait.acquire;" ::: "memory");
+}
+__device__ __forceinline__ uint32_t peer_addr(const void* local, int rank) {
+  uint32_t r;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(smem_addr(local)), "r"(rank));
+  return r;
+}
+__device__ __forceinline__ void st_peer2(uint32_t addr, float a, float b) {
+  asm volatile("st.shared::cluster.v2.f32 [%0], {%1, %2};" ::"r"(addr), "f"(a), "f"(b) : "memory");
+}
+__device__ __forceinline__ void st_peer(uint32_t addr, float a) {
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(a) : "memory");
+}
+
 // one 64-token x 64-dim box of a head of the cache (3-D map [rows, heads, 128], 128-byte swizzle)
 __device__ __forceinline__ void tma_load_cache(void* dst, const CUtensorMap* map, int x, int head, int row,
                                                uint64_t* bar) {
@@ -194,13 +248,23 @@ __device__ __forceinline__ void tma_load_cache(void* dst, const CUtensorMap* map
       : "memory");
 }
 
-__global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p) {
+// map_k, map_v: maps of the one layer's caches when p.cache_maps is NULL and p.param_maps is set
+template <bool F32, bool SPLIT>
+__global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
+    attn_tc_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
+  using SH = Shape<F32>;
+  using CT = typename CacheType<F32>::T;
+  constexpr int kSlots = SH::kSlots;
+  constexpr bool kCheck = F32 || SPLIT;  // every staged cache value against the fp16 range
   extern __shared__ __align__(1024) unsigned char smem[];
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
   const int h = blockIdx.y;
   const int H = p.n_heads;
+  const int S = SPLIT ? static_cast<int>(gridDim.x) : 1;     // the cluster spans the grid's x extent
+  const int rank = SPLIT ? static_cast<int>(blockIdx.x) : 0;
+  const int has_own = rank == 0 ? 1 : 0;                     // chunk 0 holds the own keys
 
   pdl_launch_dependents();
   pdl_wait();
@@ -212,23 +276,23 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
   // each at the latency of a loaded memory system. The batched tick hands every CTA row
   // its schedule entry (vehicle, first cache row, length: one load); the copies of the
   // vehicle's queries and own keys / values are then in flight while the rest is read.
-  const __nv_bfloat16* kc;
-  const __nv_bfloat16* vc;
+  const CT* kc;
+  const CT* vc;
   if (p.targs != nullptr) {
-    kc = static_cast<const __nv_bfloat16*>(p.targs->k_cache[p.layer]);
-    vc = static_cast<const __nv_bfloat16*>(p.targs->v_cache[p.layer]);
+    kc = static_cast<const CT*>(p.targs->k_cache[p.layer]);
+    vc = static_cast<const CT*>(p.targs->v_cache[p.layer]);
   } else {
-    kc = static_cast<const __nv_bfloat16*>(p.k_cache);
-    vc = static_cast<const __nv_bfloat16*>(p.v_cache);
+    kc = static_cast<const CT*>(p.k_cache);
+    vc = static_cast<const CT*>(p.v_cache);
   }
   AttnPlan plan_z{0, 0, 0};
   if (p.plan != nullptr) plan_z = p.plan[blockIdx.z];
   const int b = p.plan != nullptr ? plan_z.b : (p.order != nullptr ? p.order[blockIdx.z] : static_cast<int>(blockIdx.z));
 
-  unsigned char* qt = smem + kOffQ;
-  unsigned char* kslot = smem + kOffK;
-  unsigned char* vslot = smem + kOffV;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + kOffBar);
+  unsigned char* qt = smem + SH::kOffQ;
+  unsigned char* kslot = smem + SH::kOffK;
+  unsigned char* vslot = smem + SH::kOffV;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + SH::kOffBar);
   uint64_t* kfull = bars + 0;    // [3] K rows of a chunk staged
   uint64_t* kempty = bars + 3;   // [3] S done with a K slot
   uint64_t* vfull = bars + 6;    // [3] V rows staged
@@ -244,34 +308,56 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
 
   // ---- producers' staging of chunk i (own rows fp16, cache rows bf16 converted later)
   const bool is_prod = warp >= kProdWarp0;
-  const bool is_v = warp >= kProdWarp0 + 2;
-  const int pt = (warp & 1) * 32 + lane;  // thread within the tensor's two warps
-  const int pu = pt & 15;                 // 16-byte unit of a 256-byte row
-  const int pr0 = pt >> 4;                // rows pr0, pr0 + 4, ...
+  const bool is_v = warp >= kProdWarp0 + SH::kProdWarps;
+  const int pw = warp & (SH::kProdWarps - 1);  // warp within the tensor's staging warps
+  const int pt = pw * 32 + lane;               // thread within them
+  const int pu = pt & 15;                      // 16-byte unit of a 256-byte row
+  const int pr0 = pt >> 4;                     // rows pr0, pr0 + kRowStep, ...
+  constexpr int kRowStep = SH::kProdThreads / 16;
   const size_t tok = static_cast<size_t>(H) * kD;
   const __half* obase = (is_v ? p.v_own : p.k_own) + static_cast<size_t>(b) * p.n_own * p.own_stride + h * kD + pu * 8;
-  const __nv_bfloat16* cbase = nullptr;  // this CTA's first cache row of the tensor, set below
-  long long L = 0;
+  const CT* cbase = nullptr;             // this CTA's first cache row of the tensor (its head), set below
+  long long L = 0;                       // cache keys of this CTA
   long long row0 = 0;                    // this CTA's first cache row, set below
   unsigned char* pslots = is_v ? vslot : kslot;
   // Whole cache chunks (every cache chunk but a short last one) come by two TMA box loads
   // issued by one thread of the tensor's warps (when the batched tick supplies the cache
   // maps); the own keys and a short last chunk by 16-byte copies of every thread.
-  const CUtensorMap* tmap =
-      (p.cache_maps != nullptr && p.targs != nullptr) ? p.cache_maps + 2 * p.layer + (is_v ? 1 : 0) : nullptr;
+  const CUtensorMap* tmap = nullptr;
+  if (!F32) {
+    if (p.cache_maps != nullptr && p.targs != nullptr)
+      tmap = p.cache_maps + 2 * p.layer + (is_v ? 1 : 0);
+    else if (p.param_maps)
+      tmap = is_v ? &map_v : &map_k;
+  }
   uint64_t* tbar = is_v ? vtma : ktma;
-  auto by_tma = [&](int i) { return tmap != nullptr && i >= 1 && static_cast<long long>(i) * kSlotKeys <= L; };
-  // chunks 1 .. L / 64 are the TMA chunks, so slot s = i mod 3 sees them in order from its
-  // first one (i = 3 for slot 0): the phase of chunk i on its slot's barrier
-  auto tma_parity = [](int i) { return static_cast<uint32_t>((i / kSlots - (i % kSlots == 0 ? 1 : 0)) & 1); };
+  auto is_own = [&](int i) { return i < has_own; };
+  auto by_tma = [&](int i) {
+    return tmap != nullptr && i >= has_own && static_cast<long long>(i - has_own + 1) * kSlotKeys <= L;
+  };
+  // the TMA chunks follow the own chunk, so slot s = i mod kSlots sees them in order from its
+  // first one (i = kSlots for slot 0 behind an own chunk): the phase of chunk i on its slot's barrier
+  auto tma_parity = [&](int i) {
+    return static_cast<uint32_t>((i / kSlots - (has_own != 0 && i % kSlots == 0 ? 1 : 0)) & 1);
+  };
   auto chunk_rows = [&](int i) {
-    return i == 0 ? p.n_own
-                  : static_cast<int>(min(static_cast<long long>(kSlotKeys), L - (i - 1) * static_cast<long long>(kSlotKeys)));
+    return is_own(i) ? p.n_own
+                     : static_cast<int>(min(static_cast<long long>(kSlotKeys),
+                                            L - (i - has_own) * static_cast<long long>(kSlotKeys)));
   };
   auto issue = [&](int i) {
     unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
     const int rows = chunk_rows(i);
-    const long long c0 = (i - 1) * static_cast<long long>(kSlotKeys);
+    const long long c0 = (i - has_own) * static_cast<long long>(kSlotKeys);
+    if (F32 && !is_own(i)) {  // raw fp32 rows, one warp instruction a row; row r is this warp's for r mod kProdWarps == pw
+      const uint32_t raw = smem_addr(smem + SH::kOffRaw + ((is_v ? 2 : 0) + (i & 1)) * kRawBytes) + lane * 16;
+      const CT* src = cbase + static_cast<size_t>(c0) * tok + lane * 4;
+#pragma unroll 8
+      for (int r = pw; r < kSlotKeys; r += SH::kProdWarps)
+        if (r < rows) cp_async_16(raw + r * (kD * 4), src + static_cast<size_t>(r) * tok);
+      cp_async_commit();
+      return;
+    }
     if (by_tma(i)) {
       if (pt == 0) {
         uint64_t* bar = tbar + i % kSlots;
@@ -284,12 +370,12 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
       return;
     }
 #pragma unroll 8
-    for (int m = 0; m < kSlotKeys / 4; ++m) {
-      const int r = pr0 + 4 * m;
+    for (int m = 0; m < kSlotKeys / kRowStep; ++m) {
+      const int r = pr0 + kRowStep * m;
       unsigned char* dst = slot + tile128_off(r, pu);
       if (r < rows) {
-        const void* src = i == 0 ? static_cast<const void*>(obase + static_cast<size_t>(r) * p.own_stride)
-                                 : static_cast<const void*>(cbase + static_cast<size_t>(c0 + r) * tok);
+        const void* src = is_own(i) ? static_cast<const void*>(obase + static_cast<size_t>(r) * p.own_stride)
+                                    : static_cast<const void*>(cbase + static_cast<size_t>(c0 + r) * tok + pu * 8);
         cp_async_16(smem_addr(dst), src);
       } else {
         *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);  // keys past the range: finite zeros
@@ -298,7 +384,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
     cp_async_commit();
   };
   // queries: 64 rows x 16 units, rows >= n_q zero (one copy group per thread)
-  for (int i = tid; i < 64 * 16; i += kThreadsTc) {
+  for (int i = tid; i < 64 * 16; i += SH::kThreads) {
     const int r = i >> 4;
     const int u = i & 15;
     unsigned char* dst = qt + tile128_off(r, u);
@@ -308,7 +394,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
       *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
   }
   cp_async_commit();
-  if (is_prod) issue(0);  // own keys / values
+  if (is_prod && has_own != 0) issue(0);  // own keys / values
 
   long long o_lo, o_hi;
   if (p.plan != nullptr) {
@@ -327,14 +413,20 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
   }
   L = o_hi - o_lo;
   row0 = o_lo;
-  const int n_chunks = 1 + static_cast<int>((L + kSlotKeys - 1) / kSlotKeys);  // chunk 0: own keys
-  cbase = (is_v ? vc : kc) + (static_cast<size_t>(o_lo) * H + h) * kD + pu * 8;
+  if (SPLIT) {  // this split's run of whole chunks
+    const long long n_cc = (L + kSlotKeys - 1) / kSlotKeys;
+    const long long k_lo = n_cc * rank / S * kSlotKeys, k_hi = min(L, n_cc * (rank + 1) / S * kSlotKeys);
+    row0 = o_lo + k_lo;
+    L = k_hi > k_lo ? k_hi - k_lo : 0;
+  }
+  const int n_chunks = has_own + static_cast<int>((L + kSlotKeys - 1) / kSlotKeys);  // 0: a split without keys
+  cbase = (is_v ? vc : kc) + (static_cast<size_t>(row0) * H + h) * kD;
 
   if (tid == 0) {
     for (int i = 0; i < kSlots; ++i) {
-      mbar_init(kfull + i, kProdThreads);
+      mbar_init(kfull + i, SH::kProdThreads);
       mbar_init(kempty + i, 1);
-      mbar_init(vfull + i, kProdThreads);
+      mbar_init(vfull + i, SH::kProdThreads);
       mbar_init(vempty + i, 1);
       mbar_arrive(kempty + i);  // release 0 of every slot: free from the start
       mbar_arrive(vempty + i);
@@ -354,17 +446,19 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
   }
-  if (is_prod) {  // the first cache chunk; then wait for this thread's query copies
+  const int n_first = min(n_chunks, 2);  // chunks whose loads are issued up front
+  if (is_prod) {  // the first cache chunks; then wait for this thread's query copies
     if (pt == 0 && tmap != nullptr) {  // the TMA barriers, before the first TMA chunk; read after the CTA barrier
       for (int i = 0; i < kSlots; ++i) mbar_init(tbar + i, 1);
       fence_proxy_async();
     }
-    if (n_chunks > 1) {
-      issue(1);
+    for (int i = has_own; i < n_first; ++i) issue(i);
+    if (n_first == 2)
       cp_async_wait<2>();
-    } else {
+    else if (n_first == 1)
       cp_async_wait<1>();
-    }
+    else
+      cp_async_wait<0>();
   } else {
     cp_async_wait<0>();
   }
@@ -375,7 +469,13 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
   if (*abort) {  // the tick was abandoned before this kernel: no MMA was issued
     cp_async_wait<0>();
-    if (is_prod && pt == 0 && n_chunks > 1 && by_tma(1)) mbar_wait(tbar + 1, 0, p.status);  // chunk 1 landed
+    if (is_prod && pt == 0)
+      for (int i = has_own; i < n_first; ++i)  // the first chunks landed
+        if (by_tma(i)) mbar_wait(tbar + i % kSlots, tma_parity(i), p.status);
+    if (SPLIT) {  // the other splits may not have seen the status yet: they push their rows here
+      cluster_barrier();
+      cluster_barrier();
+    }
     if (warp == kMmaWarp)
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
     return;
@@ -402,7 +502,7 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
       auto issue_pv = [&](int i) {  // O (+)= P V of chunk i, P from tensor memory
         const uint32_t pa = tmem + kColS + (i & 1) * kSlotKeys;
         const uint32_t vb = smem_addr(vslot + (i % kSlots) * kSlotBytes);
-        const uint32_t idv = i == 0 ? id_pv_own : id_pv;
+        const uint32_t idv = F32 || is_own(i) ? id_pv_own : id_pv;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {  // 16 keys = 8 columns of packed fp16 pairs
           const uint64_t bd = sw128_desc_mn(vb + kk * 2048, 8192, 1024);
@@ -459,11 +559,45 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
     uint64_t* full = is_v ? vfull : kfull;
     uint64_t* empty = is_v ? vempty : kempty;
     bool ok = true;
-    int issued = n_chunks > 1 ? 2 : 1;  // chunks whose loads were issued
+    int issued = n_first;  // chunks whose loads were issued
+    uint32_t range = 0;    // a staged cache value lies outside the fp16 range
     int i = 0;
     for (; ok && i < n_chunks; ++i) {
       if (i + 1 < n_chunks) cp_async_wait<1>();
       else cp_async_wait<0>();
+      unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
+      if (F32) {
+        if (!is_own(i)) {  // raw rows -> fp16 slot, once its previous chunk is consumed
+          __syncwarp();    // the warp's copies of its rows
+          ok = wait_bar(empty + i % kSlots, (i / kSlots) & 1, p.status, abort);
+          if (!ok) break;
+          const unsigned char* raw = smem + SH::kOffRaw + ((is_v ? 2 : 0) + (i & 1)) * kRawBytes;
+          const int rows = chunk_rows(i);
+          const int u = lane & 15;
+          const int sw = (lane >> 2) & 1;  // the two 16-byte reads of a unit in an order that spreads the banks
+#pragma unroll
+          for (int m = 0; m < kSlotKeys / SH::kProdWarps; m += 2) {
+            const int r = pw + SH::kProdWarps * (m + (lane >> 4));
+            uint4 out = make_uint4(0u, 0u, 0u, 0u);  // keys past the range: finite zeros
+            if (r < rows) {
+              const float4 x = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + sw * 16);
+              const float4 y = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + (sw ^ 1) * 16);
+              const uint32_t x0 = f32x2_to_half2_sat(x.x, x.y, range), x1 = f32x2_to_half2_sat(x.z, x.w, range);
+              const uint32_t y0 = f32x2_to_half2_sat(y.x, y.y, range), y1 = f32x2_to_half2_sat(y.z, y.w, range);
+              out = sw == 0 ? make_uint4(x0, x1, y0, y1) : make_uint4(y0, y1, x0, x1);
+            }
+            *reinterpret_cast<uint4*>(slot + tile128_off(r, u)) = out;
+          }
+          __syncwarp();  // the raw rows are read before they are refilled
+        }
+        fence_proxy_async();
+        mbar_arrive(full + (i % kSlots));
+        if (i + 2 < n_chunks) {
+          issue(i + 2);
+          issued = i + 3;
+        }
+        continue;
+      }
       if (by_tma(i)) {
         ok = wait_bar(tbar + i % kSlots, tma_parity(i), p.status, abort);
         if (!ok) break;
@@ -477,16 +611,24 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
           issued = i + 3;
         }
       }
-      if (i > 0 && !is_v) {  // cache K rows -> fp16 (V stays bf16): every read before the first write
-        unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
-        uint4 v[kSlotKeys / 4];
+      if (!is_own(i) && (!is_v || kCheck)) {  // cache K rows -> fp16 (V stays bf16): every read before the first write
+        uint4 v[kSlotKeys / kRowStep];
 #pragma unroll
-        for (int m = 0; m < kSlotKeys / 4; ++m) v[m] = *reinterpret_cast<const uint4*>(slot + tile128_off(pr0 + 4 * m, pu));
+        for (int m = 0; m < kSlotKeys / kRowStep; ++m)
+          v[m] = *reinterpret_cast<const uint4*>(slot + tile128_off(pr0 + kRowStep * m, pu));
+        if (kCheck) {
 #pragma unroll
-        for (int m = 0; m < kSlotKeys / 4; ++m)
-          *reinterpret_cast<uint4*>(slot + tile128_off(pr0 + 4 * m, pu)) =
-              make_uint4(bf16x2_to_half2(v[m].x), bf16x2_to_half2(v[m].y), bf16x2_to_half2(v[m].z),
-                         bf16x2_to_half2(v[m].w));
+          for (int m = 0; m < kSlotKeys / kRowStep; ++m)
+            range |= bf16x2_out_of_range(v[m].x) | bf16x2_out_of_range(v[m].y) | bf16x2_out_of_range(v[m].z) |
+                     bf16x2_out_of_range(v[m].w);
+        }
+        if (!is_v) {
+#pragma unroll
+          for (int m = 0; m < kSlotKeys / kRowStep; ++m)
+            *reinterpret_cast<uint4*>(slot + tile128_off(pr0 + kRowStep * m, pu)) =
+                make_uint4(bf16x2_to_half2(v[m].x), bf16x2_to_half2(v[m].y), bf16x2_to_half2(v[m].z),
+                           bf16x2_to_half2(v[m].w));
+        }
       }
       fence_proxy_async();
       mbar_arrive(full + (i % kSlots));
@@ -498,11 +640,13 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
         }
       }
     }
+    if (kCheck) flag_range(p.status, range);
     cp_async_wait<0>();
     // after an abort: the TMA chunks issued but not consumed land before the CTA leaves
     if (pt == 0)
       for (int j = i; j < issued; ++j)
         if (by_tma(j)) mbar_wait(tbar + j % kSlots, tma_parity(j), p.status);
+    __syncwarp();
   } else {
     // ---------------------------------------------------------------- softmax rows
     // Warp w owns query rows 16 w .. 16 w + 15 (tensor-memory lanes 32 w .. + 15).
@@ -578,11 +722,11 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
           const float p1 = ex2_approx(fmaf(s[r][2 * g + 1], scale_log2, nm));
           r4[g & 3] += p0 + p1;
           uint32_t hi, lo;
-          if (i == 0) {  // own chunk: fp16 like its V rows
+          if (F32 || is_own(i)) {  // fp16 like the V rows
             hi = pack_half2(p0, p1);
             const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hi));
             lo = pack_half2(p0 - f.x, p1 - f.y);
-          } else {  // cache chunks: bf16 like the V rows
+          } else {  // bf16 cache chunks: bf16 like the V rows
             hi = pack_bf16x2(p0, p1);
             lo = pack_bf16x2(p0 - __uint_as_float(hi << 16), p1 - __uint_as_float(hi & 0xffff0000u));
           }
@@ -617,15 +761,48 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
       tc_fence_before();
       mbar_arrive(pfull + (i & 1));
     }
-    if (ok && wait_bar(drain, 0, p.status, abort)) {  // every P V done
-      tc_fence_after();
-      const float inv[2] = {l_run[0] > 0.f ? 1.f / l_run[0] : 0.f, l_run[1] > 0.f ? 1.f / l_run[1] : 0.f};
-      const bool va = ra < p.n_q;
-      const bool vb = rbw < p.n_q;
-      // A cache key beyond the fp16 range became an infinity here; where it raised a
-      // score to +inf (or NaN) the row's sum is NaN: report it, the tick is abandoned.
-      // (A key whose scores all fell to -inf carries weight 0, as the exact value would.)
-      if ((va && !(l_run[0] == l_run[0])) || (vb && !(l_run[1] == l_run[1]))) set_status(p.status, kStatusRange);
+    ok = ok && wait_bar(drain, 0, p.status, abort);  // every P V done
+    tc_fence_after();
+    const float inv[2] = {l_run[0] > 0.f ? 1.f / l_run[0] : 0.f, l_run[1] > 0.f ? 1.f / l_run[1] : 0.f};
+    const bool va = ra < p.n_q;
+    const bool vb = rbw < p.n_q;
+    // A cache key beyond the fp16 range became an infinity here; where it raised a
+    // score to +inf (or NaN) the row's sum is NaN: report it, the tick is abandoned.
+    // (A key whose scores all fell to -inf carries weight 0, as the exact value would.)
+    if (ok && ((va && !(l_run[0] == l_run[0])) || (vb && !(l_run[1] == l_run[1])))) set_status(p.status, kStatusRange);
+    if (SPLIT) {
+      // every CTA of the cluster is done with its slots; rows go to their owners' K slots
+      __syncwarp();
+      cluster_barrier();
+      const int rows_per = (p.n_q + S - 1) / S;
+      const int own_a = ra / rows_per, own_b = rbw / rows_per;
+      float* rows_o = reinterpret_cast<float*>(smem + SH::kOffK);  // [S][rows_per][128]
+      float* rows_l = rows_o + S * rows_per * kD;                  // [S][rows_per] log2-domain log-sum-exp
+      const int ia = rank * rows_per + ra - own_a * rows_per, ib = rank * rows_per + rbw - own_b * rows_per;
+      const uint32_t da = peer_addr(rows_o + ia * kD + 2 * t4, va ? own_a : 0);
+      const uint32_t db = peer_addr(rows_o + ib * kD + 2 * t4, vb ? own_b : 0);
+      if (ok) {
+#pragma unroll 1
+        for (int c = 0; c < kD; c += 64) {
+          uint32_t o[32];
+          __syncwarp();
+          tmem_ld_16x256b_x8(tmem + lane_base + kColO + c, o);
+          const bool any = n_chunks > 0;  // a split without keys pushes zeros (its accumulator was never written)
+#pragma unroll
+          for (int g = 0; g < 8; ++g) {
+            if (va) st_peer2(da + (c + 8 * g) * 4, any ? __uint_as_float(o[4 * g]) * inv[0] : 0.f,
+                             any ? __uint_as_float(o[4 * g + 1]) * inv[0] : 0.f);
+            if (vb) st_peer2(db + (c + 8 * g) * 4, any ? __uint_as_float(o[4 * g + 2]) * inv[1] : 0.f,
+                             any ? __uint_as_float(o[4 * g + 3]) * inv[1] : 0.f);
+          }
+        }
+        if (t4 == 0) {
+          if (va) st_peer(peer_addr(rows_l + ia, own_a), l_run[0] > 0.f ? m_run[0] + log2f(l_run[0]) : -CUDART_INF_F);
+          if (vb) st_peer(peer_addr(rows_l + ib, own_b), l_run[1] > 0.f ? m_run[1] + log2f(l_run[1]) : -CUDART_INF_F);
+        }
+      }
+      __syncwarp();
+    } else if (ok) {
       __half* oa = p.out + (static_cast<size_t>(b) * p.n_q + (va ? ra : 0)) * p.out_stride + h * kD + 2 * t4;
       __half* ob = p.out + (static_cast<size_t>(b) * p.n_q + (vb ? rbw : 0)) * p.out_stride + h * kD + 2 * t4;
 #pragma unroll 1
@@ -647,6 +824,42 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
       }
     }
   }
+  if (SPLIT) {
+    if (warp >= kSoftmaxWarps) {  // this warp is done with the slots (the softmax warps met this barrier above)
+      __syncwarp();
+      cluster_barrier();
+    }
+    cluster_barrier();  // every row pushed
+    const int rows_per = (p.n_q + S - 1) / S;
+    const float* rows_o = reinterpret_cast<const float*>(smem + SH::kOffK);
+    const float* rows_l = rows_o + S * rows_per * kD;
+    const int q_lo = rank * rows_per;
+    const int n_rows = min(p.n_q, q_lo + rows_per) - q_lo;
+    for (int t = tid; t < n_rows * (kD / 4); t += SH::kThreads) {
+      const int qq = t / (kD / 4), d = (t % (kD / 4)) * 4;
+      float mmax = -CUDART_INF_F;
+      for (int r = 0; r < S; ++r) mmax = fmaxf(mmax, rows_l[r * rows_per + qq]);
+      float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+      float wsum = 0.f;
+      if (mmax != -CUDART_INF_F)
+        for (int r = 0; r < S; ++r) {  // in split order
+          const float w = exp2f(rows_l[r * rows_per + qq] - mmax);
+          const float4 v = *reinterpret_cast<const float4*>(rows_o + (r * rows_per + qq) * kD + d);
+          wsum += w;
+          acc.x += w * v.x;
+          acc.y += w * v.y;
+          acc.z += w * v.z;
+          acc.w += w * v.w;
+        }
+      const float iw = wsum > 0.f ? 1.f / wsum : 0.f;
+      const int q = q_lo + qq;
+      *reinterpret_cast<uint2*>(p.out + (static_cast<size_t>(b) * p.n_q + q) * p.out_stride + h * kD + d) =
+          make_uint2(pack_half2(acc.x * iw, acc.y * iw), pack_half2(acc.z * iw, acc.w * iw));
+      if (p.lse != nullptr && d == 0)
+        p.lse[(static_cast<size_t>(b) * H + h) * p.n_q + q] =
+            wsum > 0.f ? (mmax + log2f(wsum)) * 0.6931471805599453f : -CUDART_INF_F;
+    }
+  }
 
   tc_fence_before();
   __syncthreads();
@@ -658,20 +871,41 @@ __global__ void __launch_bounds__(kThreadsTc, 2) attn_tc_kernel(const AttnArgs p
 
 }  // namespace
 
-bool attention_tc_eligible(const AttnArgs& a, int cache_dtype) {
-  return cache_dtype == 1 && a.n_splits == 1 && a.n_q >= 1 && a.n_q <= 48 && a.n_own >= 1 && a.n_own <= kSlotKeys;
+bool attention_tc_eligible(const AttnArgs& a, int n_splits) {
+  return n_splits >= 1 && n_splits <= kMaxClusterSplits && a.n_q >= 1 && a.n_q <= 48 && a.n_own >= 1 &&
+         a.n_own <= kSlotKeys;
 }
 
-cudaError_t attention_tc_set_attributes() {
-  return cudaFuncSetAttribute(reinterpret_cast<const void*>(&attn_tc_kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              kSmemTc);
+namespace {
+const void* tc_fn(int cache_dtype, bool split) {
+  if (cache_dtype == 1)
+    return split ? reinterpret_cast<const void*>(&attn_tc_kernel<false, true>)
+                 : reinterpret_cast<const void*>(&attn_tc_kernel<false, false>);
+  return split ? reinterpret_cast<const void*>(&attn_tc_kernel<true, true>)
+               : reinterpret_cast<const void*>(&attn_tc_kernel<true, false>);
+}
+int tc_smem(int cache_dtype) { return cache_dtype == 1 ? Shape<false>::kSmem : Shape<true>::kSmem; }
+}  // namespace
+
+cudaError_t attention_tc_set_attributes(int cache_dtype, bool split) {
+  return cudaFuncSetAttribute(tc_fn(cache_dtype, split), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              tc_smem(cache_dtype));
 }
 
-cudaError_t launch_attention_tc(const AttnArgs& a_in, int B, cudaStream_t stream, bool pdl) {
+cudaError_t launch_attention_tc(const AttnArgs& a_in, int B, int cache_dtype, cudaStream_t stream, bool pdl) {
   AttnArgs a = a_in;
-  void* kargs[] = {&a};
-  return launch_ex(reinterpret_cast<const void*>(&attn_tc_kernel), dim3(1, a.n_heads, B), dim3(kThreadsTc), kSmemTc,
-                   stream, pdl, kargs);
+  CUtensorMap map_k{}, map_v{};
+  a.param_maps = 0;
+  // one layer's caches outside a tick: maps by value (the row count is not known here; a chunk
+  // is loaded by TMA only when all of its rows are the vehicle's)
+  if (cache_dtype == 1 && a.targs == nullptr && a.k_cache != nullptr && a.v_cache != nullptr &&
+      encode_cache_map(&map_k, a.k_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)) &&
+      encode_cache_map(&map_v, a.v_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)))
+    a.param_maps = 1;
+  void* kargs[] = {&a, &map_k, &map_v};
+  const int threads = cache_dtype == 1 ? Shape<false>::kThreads : Shape<true>::kThreads;
+  return launch_ex(tc_fn(cache_dtype, a.n_splits > 1), dim3(a.n_splits, a.n_heads, B), dim3(threads),
+                   static_cast<size_t>(tc_smem(cache_dtype)), stream, pdl, kargs, 1, a.n_splits);
 }
 
 }  // namespace fsx

@@ -134,7 +134,7 @@ namespace {
 
 int attention_splits(const fsx_handle_s* h, int B) {
   const int work = B * h->cfg.n_heads;
-  int s = (2 * h->sm_count) / std::max(work, 1);
+  int s = (fsx::attention_ctas_per_sm(h->cfg.cache_dtype) * h->sm_count) / std::max(work, 1);  // one wave of CTAs
   return std::min(std::max(s, 1), 8);  // <= 8: the splits merge inside one thread-block cluster
 }
 
@@ -591,7 +591,7 @@ fsx_status fsx_create(const fsx_config* cfg, const fsx_weights* w, int device, f
   FSX_CUDA_H(cudaSetDevice(device));
   FSX_CUDA_H(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device));
   FSX_CUDA_H(fsx::gemm_tc_set_attributes());
-  FSX_CUDA_H(fsx::attention_set_attributes());
+  FSX_CUDA_H(fsx::attention_set_attributes(cfg->cache_dtype));
 
   // ---- tcgen05 weight tiles: per layer [QKV | W_o | gate/up | W_d], each matrix as
   // 128-row x 64-K tiles in the swizzled shared-memory image (n-tile major)
@@ -981,7 +981,6 @@ fsx_status fsx_attention(const void* d_q, long long q_stride, const void* d_k_ow
   int* status = static_cast<int*>(d_workspace);  // first 256 bytes: status word
   float* part = reinterpret_cast<float*>(static_cast<unsigned char*>(d_workspace) + 256);
   FSX_CUDA(cudaMemsetAsync(status, 0, sizeof(int), st));
-  FSX_CUDA(fsx::attention_set_attributes());
   fsx::AttnArgs a{};
   a.q = static_cast<const __half*>(d_q);
   a.q_stride = q_stride;
@@ -1004,6 +1003,7 @@ fsx_status fsx_attention(const void* d_q, long long q_stride, const void* d_k_ow
   a.part_o = part;
   a.part_lse = part + static_cast<size_t>(B) * n_heads * n_splits * fsx::kTokTile * fsx::kHeadDim;
   a.status = status;
+  FSX_CUDA(fsx::attention_set_attributes(a, cache_dtype));
   FSX_CUDA(fsx::launch_attention(a, B, cache_dtype, st, false));
   return FSX_OK;
 }

@@ -67,16 +67,21 @@ struct AttnArgs {
   // optional (tensor-core path, with targs): [2 n_layers] TMA maps of the layers' K and V caches
   // (bf16 [rows, n_heads, 128]); whole 64-key chunks are then loaded by TMA
   const CUtensorMap* cache_maps;
+  int param_maps;             // set by the launcher: maps of k_cache / v_cache are kernel arguments
   int* status;
 };
 
 size_t attention_workspace_bytes(int B, int n_heads, int n_splits);
 cudaError_t launch_attention(const AttnArgs& a, int B, int cache_dtype, cudaStream_t stream, bool pdl);
-cudaError_t attention_set_attributes();
-// tcgen05 path: bf16 cache, one split, n_q <= 48, 1 <= n_own <= 64
-bool attention_tc_eligible(const AttnArgs& a, int cache_dtype);
-cudaError_t launch_attention_tc(const AttnArgs& a, int B, cudaStream_t stream, bool pdl);
-cudaError_t attention_tc_set_attributes();
+// attributes of the kernel that launch_attention runs for these arguments / of every kernel of a dtype
+cudaError_t attention_set_attributes(const AttnArgs& a, int cache_dtype);
+cudaError_t attention_set_attributes(int cache_dtype);
+// tcgen05 path: up to 8 splits, n_q <= 48, 1 <= n_own <= 64
+bool attention_tc_eligible(const AttnArgs& a, int n_splits);
+cudaError_t launch_attention_tc(const AttnArgs& a, int B, int cache_dtype, cudaStream_t stream, bool pdl);
+cudaError_t attention_tc_set_attributes(int cache_dtype, bool split);
+// CTAs of the tcgen05 path that share an SM
+constexpr int attention_ctas_per_sm(int cache_dtype) { return cache_dtype == 1 ? 2 : 1; }
 int attention_launch_count(int n_splits);
 
 // --------------------------------------------------------- embed / head

@@ -1,0 +1,56 @@
+"""The tensor-core attention's key splits and fp32 caches at the edges of their tiling, through fsx_attention against
+the fp64 oracle: cache lengths around the 64-key chunks, splits without any cache key, one to 48 queries, one to 64 own
+keys, and the range check of every cache value that split and fp32 launches make.
+
+Tolerance, as a share of a row's largest entry. bf16 caches: q, k and the scores' operands are exact in fp16, P keeps 16
+bits, so the fp16 result's own rounding (2^-11 = 4.9e-4) dominates: 1e-3. fp32 caches: K and V are rounded to fp16 (2^-12
+relative on average); a score of size s moves by about 2^-12 s, at most ~4e-3 for the largest scores here (|s| < 16) but
+averaged over keys, plus 2^-12 of V: 3e-3."""
+from __future__ import annotations
+
+import numpy as np
+import pytest
+import torch
+
+from paper_2607_15621_gb300 import fsx
+
+from test_gpu_attention import D, H, gpu_attention, make, oracle_attention, row_err
+
+pytestmark = pytest.mark.gpu
+TOL = {"bf16": 1e-3, "fp32": 3e-3}
+
+
+@pytest.mark.parametrize("cache_dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("n_splits,lengths,n_q,n_own", [
+    (1, [64, 1, 0, 129], 42, 42), (1, [63], 48, 64), (1, [191, 320], 1, 1),
+    (2, [64], 42, 42), (2, [65, 0], 48, 48), (3, [128, 63], 33, 1), (4, [191, 192, 193], 10, 64),
+    (5, [64, 321], 42, 42), (7, [450], 5, 7), (8, [0], 42, 42), (8, [511, 513], 42, 10), (8, [1100], 48, 48),
+])
+def test_splits_and_dtypes(cache_dtype, n_splits, lengths, n_q, n_own):
+    c = make(lengths, n_q=n_q, n_own=n_own, cache_dtype=cache_dtype, seed=n_splits * 31 + len(lengths))
+    out, lse = gpu_attention(c, n_splits)
+    ref, ref_lse = oracle_attention(c)
+    assert row_err(out, ref).max() <= TOL[cache_dtype]
+    assert np.abs(lse - ref_lse).max() <= 2e-3
+
+
+@pytest.mark.parametrize("cache_dtype,n_splits", [("bf16", 2), ("bf16", 8), ("fp32", 1), ("fp32", 3)])
+@pytest.mark.parametrize("which,row,dim", [("kc", 0, 0), ("kc", 200, 127), ("vc", 63, 5), ("vc", 64, 64), ("vc", 200, 127)])
+def test_values_beyond_fp16_are_reported(cache_dtype, n_splits, which, row, dim):
+    c = make([201], cache_dtype=cache_dtype, seed=9)
+    dev = lambda t: t.to("cuda").contiguous()
+    off = torch.as_tensor(c["off"], device="cuda")
+    ws = torch.empty(fsx.attention_workspace_bytes(1, H, 42, n_splits), device="cuda", dtype=torch.uint8)
+    out = torch.empty(42, H * D, device="cuda", dtype=torch.float16)
+
+    def status():
+        fsx.attention(dev(c["q"]), H * D, dev(c["ko"]), dev(c["vo"]), H * D, 42, 42, dev(c["kc"]), dev(c["vc"]),
+                      cache_dtype, off, 1, H, n_splits, out, None, ws)
+        torch.cuda.synchronize()
+        return int(ws[:4].view(torch.int32).item())
+
+    c[which][row, 7, dim] = 65280.0  # the largest bf16 value below 65504
+    assert status() == fsx.FSX_OK
+    for bad in (65536.0, -1e30, float("inf"), float("nan")):
+        c[which][row, 7, dim] = bad
+        assert status() == fsx.FSX_ERR_RANGE, bad
