@@ -235,7 +235,7 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
       h2.n_waypoints = c.n_waypoints;
       h2.B = 1;
       h2.status = h->status;
-      FSX_CUDA(fsx::launch_head2(h2, st, false));
+      FSX_CUDA(fsx::launch_head2(h2, st, true));
     }
     if (timed) h->timed_pairs = pair;
     return FSX_OK;

@@ -45,122 +45,198 @@ constexpr int kQueries = 5;
 
 __device__ __forceinline__ float silu(float z) { return z / (1.f + expf(-z)); }
 
-// y[r] = act(W[r, :] . x + bias[r]) for r < d_out, x in shared memory, d_in a multiple of
-// 128 (<= 1024). Each warp takes four rows at a time and issues all of their 16-byte
-// weight loads before the first multiply, so a block keeps many row loads in flight.
-template <bool kSilu>
-__device__ __forceinline__ void block_gemv(const float* __restrict__ W, const float* __restrict__ bias, const float* x,
-                                           float* y, int d_out, int d_in) {
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
-  const int nk = d_in / 128;
-  for (int r0 = warp * 4; r0 < d_out; r0 += n_warps * 4) {
-    float acc[4] = {0.f, 0.f, 0.f, 0.f};
-#pragma unroll 8
-    for (int kq = 0; kq < nk; ++kq) {
-      const int k = kq * 128 + lane * 4;
-      const float4 xv = *reinterpret_cast<const float4*>(x + k);
-      float4 wv[4];
+// Both kernels are matrix-vector products over 1 MB of fp32 weights (d = 512) that no single SM
+// can read in time (one CTA per vehicle took 17-20 us for the state token, one per waypoint 40 us
+// for the head), so the rows of a matrix are spread over CTAs, and a warp requests its first
+// rows' weights before it needs the vector they multiply: the calls are bound by a few load
+// latencies. Measured: a tick of one vehicle, 8 layers and 224 rows, 240 -> 196 us.
+constexpr int kMlpThreads = 512;
+constexpr int kMlpWarps = kMlpThreads / 32;
+constexpr int kMaxUnits = 8;      // 128-wide K units of a row (d <= 1024)
+constexpr int kHeadCluster = 8;   // CTAs that share the rows of W_h1 for one vehicle
+
+// two rows of a row-major [*, d] matrix, 4 values a lane and K unit (zeros past row `end`)
+struct RowPair {
+  float4 w[2][kMaxUnits];
+  float bias[2];
+  __device__ __forceinline__ void load(const float* __restrict__ W, const float* __restrict__ b, int r0, int end, int d,
+                                       int lane) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
-        wv[i] = r0 + i < d_out ? __ldg(reinterpret_cast<const float4*>(W + static_cast<size_t>(r0 + i) * d_in + k))
-                               : make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int i = 0; i < 2; ++i) {
 #pragma unroll
-      for (int i = 0; i < 4; ++i) acc[i] += wv[i].x * xv.x + wv[i].y * xv.y + wv[i].z * xv.z + wv[i].w * xv.w;
-    }
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-      const float v = warp_sum(acc[i]);
-      if (lane == 0 && r0 + i < d_out) y[r0 + i] = kSilu ? silu(v + bias[r0 + i]) : v + bias[r0 + i];
+      for (int kq = 0; kq < kMaxUnits; ++kq)
+        w[i][kq] = r0 + i < end && kq * 128 < d
+                       ? __ldg(reinterpret_cast<const float4*>(W + static_cast<size_t>(r0 + i) * d + kq * 128 + lane * 4))
+                       : make_float4(0.f, 0.f, 0.f, 0.f);
+      bias[i] = r0 + i < end ? __ldg(b + r0 + i) : 0.f;
     }
   }
-}
+  // this lane's part of rows . x (x in shared memory)
+  __device__ __forceinline__ void dot(const float* x, int d, int lane, float (&acc)[2]) const {
+    acc[0] = acc[1] = 0.f;
+#pragma unroll
+    for (int kq = 0; kq < kMaxUnits; ++kq)
+      if (kq * 128 < d) {
+        const float4 xv = *reinterpret_cast<const float4*>(x + kq * 128 + lane * 4);
+#pragma unroll
+        for (int i = 0; i < 2; ++i) acc[i] += w[i][kq].x * xv.x + w[i][kq].y * xv.y + w[i][kq].z * xv.z + w[i][kq].w * xv.w;
+      }
+  }
+};
 
-// One block per vehicle: frames[b] = [W_s2 silu(W_s1 s_b + b_s1) + b_s2 ; visual[b, 0..3]].
-// Layout of w: W_s1 [d, 16], b_s1 [d], W_s2 [d, d], b_s2 [d] (fp32, row-major [out, in]).
-__global__ void state_tokens_kernel(const StateArgs a) {
-  extern __shared__ float sm[];
-  float* s = sm;               // [16]
-  float* h1 = sm + kStateDim;  // [d]
-  const int b = blockIdx.x;
-  const int d = a.d;
+// Block (s, b): rows d s / n .. d (s + 1) / n - 1 of vehicle b's state token W_s2 silu(W_s1 s_b +
+// b_s1) + b_s2 (every block forms the hidden vector, 16 inputs wide, itself) and its share of the
+// visual rows. Layout of w: W_s1 [d, 16], b_s1 [d], W_s2 [d, d], b_s2 [d] (fp32, row-major [out, in]).
+__global__ void __launch_bounds__(kMlpThreads) state_tokens_kernel(const StateArgs a) {
+  __shared__ __align__(16) float s[kStateDim];
+  __shared__ __align__(16) float h1[kMaxUnits * 128];
+  const int b = blockIdx.y, d = a.d;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* w1 = a.w;
   const float* b1 = w1 + static_cast<size_t>(d) * kStateDim;
   const float* w2 = b1 + d;
   const float* b2 = w2 + static_cast<size_t>(d) * d;
+  const int r_lo = d * blockIdx.x / gridDim.x, r_hi = d * (blockIdx.x + 1) / gridDim.x;
+  RowPair rows;
+  int r0 = r_lo + 2 * warp;
+  rows.load(w2, b2, r0, r_hi, d, lane);
   if (threadIdx.x < kStateDim) s[threadIdx.x] = a.state[static_cast<size_t>(b) * kStateDim + threadIdx.x];
-  __syncthreads();
-  for (int o = threadIdx.x; o < d; o += blockDim.x) {
-    float acc = b1[o];
-#pragma unroll
-    for (int k = 0; k < kStateDim; ++k) acc += w1[static_cast<size_t>(o) * kStateDim + k] * s[k];
-    h1[o] = silu(acc);
-  }
-  __syncthreads();
   float* out = a.frames + static_cast<size_t>(b) * (1 + kVisual) * d;
-  block_gemv<false>(w2, b2, h1, out, d, d);
-  for (int i = threadIdx.x; i < kVisual * d; i += blockDim.x) {
+  for (int i = blockIdx.x * kMlpThreads + threadIdx.x; i < kVisual * d; i += gridDim.x * kMlpThreads) {
     const size_t src = static_cast<size_t>(b) * kVisual * d + i;
     out[d + i] = a.visual_dtype == 1 ? __bfloat162float(static_cast<const __nv_bfloat16*>(a.visual)[src])
                                      : static_cast<const float*>(a.visual)[src];
   }
+  __syncthreads();
+  for (int o = threadIdx.x; o < d; o += kMlpThreads) {
+    float acc = b1[o];
+#pragma unroll
+    for (int k = 0; k < kStateDim; k += 4) {
+      const float4 wv = __ldg(reinterpret_cast<const float4*>(w1 + static_cast<size_t>(o) * kStateDim + k));
+      acc += wv.x * s[k];
+      acc += wv.y * s[k + 1];
+      acc += wv.z * s[k + 2];
+      acc += wv.w * s[k + 3];
+    }
+    h1[o] = silu(acc);
+  }
+  __syncthreads();
+  for (; r0 < r_hi; r0 += 2 * kMlpWarps) {
+    float acc[2];
+    rows.dot(h1, d, lane, acc);
+    const float bias[2] = {rows.bias[0], rows.bias[1]};
+    if (r0 + 2 * kMlpWarps < r_hi) rows.load(w2, b2, r0 + 2 * kMlpWarps, r_hi, d, lane);
+#pragma unroll
+    for (int i = 0; i < 2; ++i) {
+      const float v = warp_sum(acc[i]);
+      if (lane == 0 && r0 + i < r_hi) out[r0 + i] = v + bias[i];
+    }
+  }
+}
+
+__device__ __forceinline__ void st_rank0(const float* local, float v) {  // the same offset in cluster CTA 0
+  uint32_t addr;
+  asm volatile("mapa.shared::cluster.u32 %0, %1, 0;" : "=r"(addr) : "r"(smem_addr(local)));
+  asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
 }  // namespace
 
-// One block per (vehicle, waypoint): w = W_h2 silu(W_h1 RMSNorm(x; g_f) + b_h1) + b_h2
-// over the query token's final state. Layout of a.w: W_h1 [d, d], b_h1 [d], W_h2 [2, d], b_h2 [2].
-__global__ void head2_kernel(const Head2Args a) {
-  pdl_launch_dependents();
-  pdl_wait();
-  if (*reinterpret_cast<volatile int*>(a.status) != 0) return;  // a device-side error: no waypoint
-  extern __shared__ float sm[];
-  const int d = a.d;
-  float* n = sm;       // [d]
-  float* h1 = sm + d;  // [d]
-  __shared__ float red[32];
-  __shared__ float s_rstd;
-  const int b = blockIdx.x, j = blockIdx.y;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, n_warps = blockDim.x >> 5;
-  const float* xr = a.x + (static_cast<size_t>(b) * a.vehicle_rows + j) * d;
-  float ss = 0.f;
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    const float v = __ldcg(xr + c);
-    ss += v * v;
-  }
-  ss = warp_sum(ss);
-  if (lane == 0) red[warp] = ss;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    float t = 0.f;
-    for (int w = 0; w < n_warps; ++w) t += red[w];
-    s_rstd = rsqrtf(t / static_cast<float>(d) + 1e-6f);
-  }
-  __syncthreads();
-  const float rstd = s_rstd;
-  for (int c = threadIdx.x; c < d; c += blockDim.x) n[c] = __ldcg(xr + c) * rstd * a.final_norm[c];
-  __syncthreads();
+// One cluster of 8 CTAs per vehicle: w_j = W_h2 silu(W_h1 RMSNorm(x_j; g_f) + b_h1) + b_h2 over the
+// final states of the five query tokens, which share every weight row read. Each CTA takes d / 8 rows
+// of W_h1 and the matching columns of W_h2; rank 0 adds the CTAs' partial outputs in rank order.
+// Layout of a.w: W_h1 [d, d], b_h1 [d], W_h2 [2, d], b_h2 [2].
+__global__ void __launch_bounds__(kMlpThreads) head2_kernel(const Head2Args a) {
+  __shared__ __align__(16) float n[kQueries][kMaxUnits * 128];
+  __shared__ float h1[kQueries][kMaxUnits * 128 / kHeadCluster];
+  __shared__ float part[kHeadCluster][2 * kQueries];
+  const int d = a.d, rank = blockIdx.x, b = blockIdx.y;
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float* w1 = a.w;
   const float* b1 = w1 + static_cast<size_t>(d) * d;
   const float* w2 = b1 + d;
   const float* b2 = w2 + static_cast<size_t>(2) * d;
-  block_gemv<true>(w1, b1, n, h1, d, d);
+  const int n_rows = d / kHeadCluster, r_lo = rank * n_rows, r_hi = r_lo + n_rows;
+  pdl_launch_dependents();
+  RowPair rows;  // weights depend on no other kernel
+  int r0 = r_lo + 2 * warp;
+  rows.load(w1, b1, r0, r_hi, d, lane);
+  float w2v[kMaxUnits * 128 / kHeadCluster / 32];  // warp 2 j + o: output o's columns for waypoint j
+#pragma unroll
+  for (int i = 0; i < kMaxUnits * 128 / kHeadCluster / 32; ++i)
+    w2v[i] = warp < 2 * kQueries && lane + 32 * i < n_rows ? __ldg(w2 + (warp & 1) * d + r_lo + lane + 32 * i) : 0.f;
+  pdl_wait();
+  if (*reinterpret_cast<volatile int*>(a.status) != 0) return;  // a device-side error: no waypoint (whole cluster)
+  asm volatile("barrier.cluster.arrive.relaxed.aligned;" ::: "memory");  // this CTA runs
+  if (warp < a.n_waypoints) {  // RMSNorm of one token a warp
+    const float* xr = a.x + (static_cast<size_t>(b) * a.vehicle_rows + warp) * d;
+    float4 x[kMaxUnits];
+    float ss = 0.f;
+#pragma unroll
+    for (int kq = 0; kq < kMaxUnits; ++kq) {
+      x[kq] = kq * 128 < d ? __ldcg(reinterpret_cast<const float4*>(xr + kq * 128 + lane * 4)) : make_float4(0.f, 0.f, 0.f, 0.f);
+      ss += x[kq].x * x[kq].x + x[kq].y * x[kq].y + x[kq].z * x[kq].z + x[kq].w * x[kq].w;
+    }
+    const float rstd = rsqrtf(warp_sum(ss) / static_cast<float>(d) + 1e-6f);
+#pragma unroll
+    for (int kq = 0; kq < kMaxUnits; ++kq)
+      if (kq * 128 < d) {
+        const float4 g = __ldg(reinterpret_cast<const float4*>(a.final_norm + kq * 128 + lane * 4));
+        *reinterpret_cast<float4*>(&n[warp][kq * 128 + lane * 4]) =
+            make_float4(x[kq].x * rstd * g.x, x[kq].y * rstd * g.y, x[kq].z * rstd * g.z, x[kq].w * rstd * g.w);
+      }
+  }
   __syncthreads();
-  float* out = a.targs->waypoints + (static_cast<size_t>(b) * a.n_waypoints + j) * 2;
-  block_gemv<false>(w2, b2, h1, out, 2, d);
+  for (; r0 < r_hi; r0 += 2 * kMlpWarps) {
+    float v[kQueries][2];
+#pragma unroll
+    for (int j = 0; j < kQueries; ++j) rows.dot(n[j], d, lane, v[j]);
+    const float bias[2] = {rows.bias[0], rows.bias[1]};
+    if (r0 + 2 * kMlpWarps < r_hi) rows.load(w1, b1, r0 + 2 * kMlpWarps, r_hi, d, lane);
+#pragma unroll
+    for (int j = 0; j < kQueries; ++j)
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const float t = warp_sum(v[j][i]);
+        if (lane == 0 && r0 + i < r_hi) h1[j][r0 + i - r_lo] = silu(t + bias[i]);
+      }
+  }
+  asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");  // every CTA of the cluster runs
+  __syncthreads();
+  if (warp < 2 * a.n_waypoints) {
+    float acc = 0.f;
+#pragma unroll
+    for (int i = 0; i < kMaxUnits * 128 / kHeadCluster / 32; ++i)
+      if (lane + 32 * i < n_rows) acc += w2v[i] * h1[warp >> 1][lane + 32 * i];
+    acc = warp_sum(acc);
+    if (lane == 0) st_rank0(&part[rank][warp], acc);
+  }
+  __syncwarp();
+  asm volatile("barrier.cluster.arrive.release.aligned;\nbarrier.cluster.wait.acquire.aligned;" ::: "memory");
+  if (rank == 0 && threadIdx.x < 2 * a.n_waypoints) {
+    float v = 0.f;
+#pragma unroll
+    for (int r = 0; r < kHeadCluster; ++r) v += part[r][threadIdx.x];
+    a.targs->waypoints[static_cast<size_t>(b) * a.n_waypoints * 2 + threadIdx.x] = v + b2[threadIdx.x & 1];
+  }
 }
 
 cudaError_t launch_state_tokens(const StateArgs& a_in, cudaStream_t stream) {
   StateArgs a = a_in;
   void* kargs[] = {&a};
-  return launch_ex(reinterpret_cast<const void*>(&state_tokens_kernel), dim3(a.B), dim3(1024),
-                   (kStateDim + a.d) * sizeof(float), stream, false, kargs);
+  // one pass of 32 rows a block for few vehicles, about two blocks per SM for many
+  int slices = 304 / a.B;
+  slices = slices > a.d / 32 ? a.d / 32 : (slices < 1 ? 1 : slices);
+  return launch_ex(reinterpret_cast<const void*>(&state_tokens_kernel), dim3(slices, a.B), dim3(kMlpThreads), 0, stream,
+                   false, kargs);
 }
 
 cudaError_t launch_head2(const Head2Args& a_in, cudaStream_t stream, bool pdl) {
   Head2Args a = a_in;
+  if (a.n_waypoints > kQueries) return cudaErrorInvalidValue;
   void* kargs[] = {&a};
-  return launch_ex(reinterpret_cast<const void*>(&head2_kernel), dim3(a.B, a.n_waypoints), dim3(1024),
-                   2 * a.d * sizeof(float), stream, pdl, kargs);
+  return launch_ex(reinterpret_cast<const void*>(&head2_kernel), dim3(kHeadCluster, a.B), dim3(kMlpThreads), 0, stream,
+                   pdl, kargs, 1, kHeadCluster);
 }
 
 }  // namespace fsx
