@@ -563,8 +563,6 @@ size_t attention_workspace_bytes(int B, int n_heads, int n_splits) {
   return parts * kTokTile * kD * sizeof(float) + parts * kTokTile * sizeof(float);
 }
 
-int attention_launch_count(int n_splits) { return n_splits > kMaxClusterSplits ? 2 : 1; }
-
 namespace {
 // the mma.sync kernel for these arguments and its shared memory
 const void* splitkv_fn(int cache_dtype, bool cluster_merge, size_t* smem) {

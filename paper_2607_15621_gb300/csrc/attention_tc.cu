@@ -892,8 +892,21 @@ cudaError_t attention_tc_set_attributes(int cache_dtype, bool split) {
                               tc_smem(cache_dtype));
 }
 
+// The most splits, at least 2 and at most `wanted`, whose clusters are all resident at once: one
+// cluster in a second wave costs as much as the first wave (32 clusters of 8 against 30 that fit).
+// Split launches check every cache value, so a call that asks for splits keeps two.
+static int resident_splits(int wanted, int B, int n_heads, int cache_dtype) {
+  const int threads = cache_dtype == 1 ? Shape<false>::kThreads : Shape<true>::kThreads;
+  int s = wanted;
+  while (s > 2 && max_resident_clusters(tc_fn(cache_dtype, true), threads, static_cast<size_t>(tc_smem(cache_dtype)), s) <
+                      static_cast<long long>(B) * n_heads)
+    --s;
+  return s;
+}
+
 cudaError_t launch_attention_tc(const AttnArgs& a_in, int B, int cache_dtype, cudaStream_t stream, bool pdl) {
   AttnArgs a = a_in;
+  if (a.n_splits > 1) a.n_splits = resident_splits(a.n_splits, B, a.n_heads, cache_dtype);
   CUtensorMap map_k{}, map_v{};
   a.param_maps = 0;
   // one layer's caches outside a tick: maps by value (the row count is not known here; a chunk

@@ -69,6 +69,7 @@ struct fsx_handle_s {
   std::vector<const unsigned char*> w_qkv, w_o, w_gu, w_dn;  // tcgen05 tile images per layer
   // 2-D tensor maps of the activation buffers for the token tile sizes 48 / 128 / 256
   CUtensorMap map_x16[4], map_o[4], map_h[4];  // token boxes of 48, 128, 256, 144 rows
+  CUtensorMap map_o_res[fsx::kResTileCount], map_h_res[fsx::kResTileCount];  // boxes of kResTiles rows
   CUtensorMap map_w;                            // every packed weight tile (pair GEMM variant)
   bool pair_gemm = false;                       // QKV at 256-token tiles may run on CTA pairs (opt-in)
   // fp32 small parameters
@@ -83,10 +84,6 @@ struct fsx_handle_s {
   __half* qkv = nullptr;
   __half* o = nullptr;
   __half* hbuf = nullptr;
-  float* part = nullptr;
-  size_t part_bytes = 0;
-  float* gemm_part = nullptr;   // split-K partial tiles of the residual GEMMs
-  int* tile_count = nullptr;    // [sm_count] split arrivals per tile, zero between launches
   int* order = nullptr;         // [max_batch] vehicles by decreasing cache length (attention schedule)
   fsx::AttnPlan* plan = nullptr;  // [max_batch] the same schedule with each vehicle's cache range
   int* status = nullptr;
@@ -134,8 +131,8 @@ namespace {
 
 int attention_splits(const fsx_handle_s* h, int B) {
   const int work = B * h->cfg.n_heads;
-  int s = (fsx::attention_ctas_per_sm(h->cfg.cache_dtype) * h->sm_count) / std::max(work, 1);  // one wave of CTAs
-  return std::min(std::max(s, 1), 8);  // <= 8: the splits merge inside one thread-block cluster
+  const int s = (fsx::attention_ctas_per_sm(h->cfg.cache_dtype) * h->sm_count) / std::max(work, 1);  // one wave of CTAs
+  return std::min(std::max(s, 1), 8);  // the splits merge inside one thread-block cluster
 }
 
 fsx_status check_config(const fsx_config* c) {
@@ -268,11 +265,18 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
   // tcgen05.mma costs the same for any N up to 256) whenever M exceeds one 48-token tile
   const int bq_i = M <= 48 ? 0 : 2;
   const int bq = bq_i == 0 ? 48 : 256;
-  // The residual GEMMs (N = d) have only d / 128 weight tiles: with 256-token tiles they
-  // fill about half the SMs. 144-token tiles give one tile per SM up to 38 x 144 tokens.
+  // The residual GEMMs (N = d) have only d / 128 weight tiles. Where those leave SMs idle, K is
+  // cut over clusters (gemm_res.cu); with more tokens 144-token tiles give one tile per SM up to
+  // 38 x 144 tokens, against half the SMs for 256-token tiles.
   const int rtiles144 = (d / 128) * ((M + 143) / 144);
   const int rbn_i = (bn_i == 2 && rtiles144 <= h->sm_count) ? 3 : bn_i;
   const int rbn = rbn_i == 3 ? 144 : bn;
+  auto launch_residual = [&](const CUtensorMap* maps, const CUtensorMap* maps_res, const fsx::ResPlan& plan,
+                             const fsx::TcGemmArgs& g) {
+    if (plan.splits > 1) return fsx::launch_gemm_res(maps_res[plan.tile], g, plan, st, pdl);
+    return fsx::launch_gemm_tc(maps[rbn_i], g, rbn, fsx::kEpiResidual, false, st, pdl);
+  };
+  const fsx::ResPlan plan_o = fsx::gemm_res_plan(M, d, HD), plan_d = fsx::gemm_res_plan(M, d, F);
   // QKV on CTA pairs (M = 256 tcgen05.mma.cta_group::2, half the token rows staged per SM)
   // when opted in, from 2048 tokens on. With the TMA-store epilogue the single-CTA kernel is
   // the faster one (5376 tokens: 60.7 against 67.3 us per launch), so it is the default.
@@ -317,8 +321,6 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
     a.out = h->o;
     a.out_stride = HD;
     a.lse = nullptr;
-    a.part_o = h->part;
-    a.part_lse = h->part + static_cast<size_t>(B) * c.n_heads * S * fsx::kTokTile * fsx::kHeadDim;
     a.order = h->order;
     a.plan = h->plan;
     a.cache_maps = h->d_cache_maps;
@@ -343,11 +345,8 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
     go.ldxo = d;
     go.ss_out = h->ss;
     go.ss_stride = h->ss_stride;
-    go.k_splits = fsx::gemm_tc_k_splits((d / 128) * ((M + rbn - 1) / rbn), HD / 64, h->sm_count);
-    go.part = h->gemm_part;
-    go.tile_count = h->tile_count;
     FSX_CUDA(mark(kClassWo, true));
-    FSX_CUDA(fsx::launch_gemm_tc(h->map_o[rbn_i], go, rbn, fsx::kEpiResidual, false, st, pdl));
+    FSX_CUDA(launch_residual(h->map_o, h->map_o_res, plan_o, go));
     FSX_CUDA(mark(kClassWo, false));
 
     // h = silu(RMSNorm(x) W_g^T) * (RMSNorm(x) W_u^T)
@@ -378,11 +377,8 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
     gd.ldxo = d;
     gd.ss_out = h->ss;
     gd.ss_stride = h->ss_stride;
-    gd.k_splits = fsx::gemm_tc_k_splits((d / 128) * ((M + rbn - 1) / rbn), F / 64, h->sm_count);
-    gd.part = h->gemm_part;
-    gd.tile_count = h->tile_count;
     FSX_CUDA(mark(kClassDown, true));
-    FSX_CUDA(fsx::launch_gemm_tc(h->map_h[rbn_i], gd, rbn, fsx::kEpiResidual, false, st, pdl));
+    FSX_CUDA(launch_residual(h->map_h, h->map_h_res, plan_d, gd));
     FSX_CUDA(mark(kClassDown, false));
   }
 
@@ -511,8 +507,8 @@ void free_handle(fsx_handle_s* h) {
   if (h->cap_stream) cudaStreamDestroy(h->cap_stream);
   if (h->paper_params) cudaFree(h->paper_params);
   if (h->paper_frames) cudaFree(h->paper_frames);
-  void* bufs[] = {h->p_arena, h->p_x, h->p_counters, h->w_arena, h->params, h->x, h->x16, h->ss, h->qkv, h->o, h->hbuf, h->part,
-                  h->gemm_part, h->tile_count, h->order, h->plan, h->status, h->d_args, h->d_cache_maps,
+  void* bufs[] = {h->p_arena, h->p_x, h->p_counters, h->w_arena, h->params, h->x, h->x16, h->ss, h->qkv, h->o, h->hbuf,
+                  h->order, h->plan, h->status, h->d_args, h->d_cache_maps,
                   h->st_offsets, h->st_frames, h->st_waypoints};
   for (void* p : bufs)
     if (p) cudaFree(p);
@@ -591,6 +587,7 @@ fsx_status fsx_create(const fsx_config* cfg, const fsx_weights* w, int device, f
   FSX_CUDA_H(cudaSetDevice(device));
   FSX_CUDA_H(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device));
   FSX_CUDA_H(fsx::gemm_tc_set_attributes());
+  FSX_CUDA_H(fsx::gemm_res_set_attributes());
   FSX_CUDA_H(fsx::attention_set_attributes(cfg->cache_dtype));
 
   // ---- tcgen05 weight tiles: per layer [QKV | W_o | gate/up | W_d], each matrix as
@@ -784,15 +781,11 @@ fsx_status fsx_create(const fsx_config* cfg, const fsx_weights* w, int device, f
           !fsx::encode_act_map(&h->map_h[i], h->hbuf, m_pad, F, boxes[i]))
         return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
     }
+    for (int i = 0; i < fsx::kResTileCount; ++i)
+      if (!fsx::encode_act_map(&h->map_o_res[i], h->o, m_pad, HD, fsx::kResTiles[i]) ||
+          !fsx::encode_act_map(&h->map_h_res[i], h->hbuf, m_pad, F, fsx::kResTiles[i]))
+        return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
   }
-  size_t part = 0;
-  for (int B = 1; B <= cfg->max_batch; ++B)
-    part = std::max(part, fsx::attention_workspace_bytes(B, cfg->n_heads, attention_splits(h, B)));
-  h->part_bytes = part;
-  if (part) FSX_CUDA_H(cudaMalloc(&h->part, part));
-  FSX_CUDA_H(cudaMalloc(&h->gemm_part, fsx::gemm_tc_part_bytes(h->sm_count)));
-  FSX_CUDA_H(cudaMalloc(&h->tile_count, sizeof(int) * h->sm_count));
-  FSX_CUDA_H(cudaMemset(h->tile_count, 0, sizeof(int) * h->sm_count));
   FSX_CUDA_H(cudaMalloc(&h->order, sizeof(int) * cfg->max_batch));
   FSX_CUDA_H(cudaMalloc(&h->plan, sizeof(fsx::AttnPlan) * cfg->max_batch));
   FSX_CUDA_H(cudaMalloc(&h->status, sizeof(int)));
@@ -920,7 +913,7 @@ long long fsx_weight_bytes(fsx_handle h) { return h ? h->weight_bytes : 0; }
 int fsx_tick_launches(fsx_handle h, int B) {
   if (!h || B < 1) return 0;
   if (use_persistent(h, B)) return h->paper_head != nullptr ? 2 : 1;
-  return 2 + h->cfg.n_layers * (4 + fsx::attention_launch_count(attention_splits(h, B)));
+  return 2 + h->cfg.n_layers * 5;
 }
 
 fsx_status fsx_set_kernel_timing(fsx_handle h, int enable, int kclass) {

@@ -215,20 +215,17 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   const int KT = p.K / kTileK;
   const int tiles_n = p.N / kTileN;
   const int n_tiles = tiles_n * ((p.M + BN - 1) / BN);
-  const int KS = (EPI == kEpiResidual && p.k_splits > 1) ? p.k_splits : 1;
   uint32_t crank = 0;  // pair: this CTA's rank in the cluster (0 issues the MMAs)
   if (PAIR) asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(crank));
-  // unit u: tile tile_of(u), K steps [kt0(u), kt1(u)). Pair units are (weight tile pair,
+  // unit u: tile tile_of(u), all K steps. Pair units are (weight tile pair,
   // token block); the CTA of rank c takes the pair's weight tile 2 j + c.
   const int half_n = tiles_n / 2;
-  const int n_units = PAIR ? n_tiles / 2 : n_tiles * KS;
+  const int n_units = PAIR ? n_tiles / 2 : n_tiles;
   const int u_first = PAIR ? static_cast<int>(blockIdx.x >> 1) : static_cast<int>(blockIdx.x);
   const int u_step = PAIR ? static_cast<int>(gridDim.x >> 1) : static_cast<int>(gridDim.x);
   auto tile_of = [&](int u) {
-    return PAIR ? (u / half_n) * tiles_n + (u % half_n) * 2 + static_cast<int>(crank) : u / KS;
+    return PAIR ? (u / half_n) * tiles_n + (u % half_n) * 2 + static_cast<int>(crank) : u;
   };
-  auto kt0 = [&](int u) { return (u % KS) * KT / KS; };
-  auto kt1 = [&](int u) { return (u % KS + 1) * KT / KS; };
   constexpr int kAbytes = (PAIR ? BN / 2 : BN) * kTileK * 2;
   constexpr uint32_t kTmemCols = tc_tmem_cols<BN>();
   // bounded wait that gives up at once after an earlier timeout of this CTA
@@ -285,7 +282,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
     if (lane == 0) {
       int g = 0;
       for (int u = u_first; u < n_units && g < kStages; u += u_step)
-        for (int kt = kt0(u); kt < kt1(u) && g < kStages; ++kt, ++g) {
+        for (int kt = 0; kt < KT && g < kStages; ++kt, ++g) {
           if (PAIR) {
             if (crank == 0) mbar_arrive_expect_tx(full + g, kPairTx);
             tma_load_w_pair(stages + g * kStageBytes, &map_w, w_tile(u, kt), pair_bar(g));
@@ -300,7 +297,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
     int total = 0;
     for (int u = u_first; u < n_units; u += u_step) {
       const int m_tile = tile_of(u) / tiles_n;
-      for (int kt = kt0(u); kt < kt1(u); ++kt, ++total) {
+      for (int kt = 0; kt < KT; ++kt, ++total) {
         const int g = total;
         const int s = g % kStages;
         unsigned char* st = stages + s * kStageBytes;
@@ -360,8 +357,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
       }
       tc_fence_after();
       const uint32_t d = tmem + static_cast<uint32_t>(acc * BN);
-      const int k_first = kt0(u);
-      for (int kt = k_first; kt < kt1(u); ++kt, ++g) {
+      for (int kt = 0; kt < KT; ++kt, ++g) {
         const int s = g % kStages;
         wait(full + s, static_cast<uint32_t>((g / kStages) & 1));
         tc_fence_after();
@@ -372,10 +368,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
           for (int k = 0; k < kTileK / 16; ++k) {
             if (PAIR)
               umma_f16_pair(d, sw128_desc(a_base + k * 32), sw128_desc(b_base + k * 32), idesc,
-                            (kt > k_first || k > 0) ? 1u : 0u);
+                            (kt > 0 || k > 0) ? 1u : 0u);
             else
               umma_f16(d, sw128_desc(a_base + k * 32), sw128_desc(b_base + k * 32), idesc,
-                       (kt > k_first || k > 0) ? 1u : 0u);
+                       (kt > 0 || k > 0) ? 1u : 0u);
           }
           if (PAIR)
             umma_commit_pair(empty + s, 3);  // both CTAs' producers may refill the stage
@@ -452,7 +448,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
     for (int u = u_first; u < n_units; u += u_step, ++i) {
       const int acc = i & 1;
       const int tile = tile_of(u);
-      const int split = u % KS;
       const int t_n = tile % tiles_n;
       const int n0 = t_n * kTileN;
       const int m0 = (tile / tiles_n) * BN;
@@ -485,14 +480,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
 #pragma unroll
             for (int j = 16; j < 32; ++j) r[j] = 0u;
           }
-          if (KS == 1) {
-            residual_chunk(t_n, m0, c0, nc, r);
-          } else {  // this split's partial -> workspace ([tile][split][token][128 columns])
-            float* pp = p.part + (static_cast<size_t>(tile * KS + split) * BN + c0) * kTileN + row;
-#pragma unroll
-            for (int j = 0; j < 32; ++j)
-              if (j < nc) pp[static_cast<size_t>(j) * kTileN] = __uint_as_float(r[j]);
-          }
+          residual_chunk(t_n, m0, c0, nc, r);
         } else {
           // the chunk as accumulator fragments: ra = lanes 32q .. 32q + 15 of the quadrant
           // (weight rows), rb = lanes 32q + 16 .. 32q + 31; 32 token columns each (a short
@@ -579,79 +567,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
                        : "memory");
         else
           mbar_arrive(tmem_empty + acc);
-      }
-      if (EPI == kEpiResidual && KS > 1) {
-        // every split of the tile waits until all KS partials are written (the grid holds
-        // at most one CTA per SM and never more CTAs than SMs, so all splits are resident),
-        // then adds the partials of its own slice of tokens in split order
-        __threadfence();
-        epi_sync();
-        if (etid == 0 && *abort == 0) {
-          atomicAdd(p.tile_count + tile, 1);
-          const unsigned long long t0 = global_timer_ns();
-          for (uint32_t it = 0;; ++it) {
-            int v;
-            asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(p.tile_count + tile) : "memory");
-            if (v >= KS) break;
-            if ((it & 63u) == 63u && global_timer_ns() - t0 > kWaitLimitNs) {
-              set_status(p.status, kStatusTimeout);
-              *abort = 1;
-              break;
-            }
-          }
-        }
-        epi_sync();
-        __threadfence();
-        const int tk_lo = split * BN / KS;
-        const int tk_hi = (split + 1) * BN / KS;
-        // warp ew takes tokens tk_lo + ew, + 12, ...; lane = 4-column group of the tile's
-        // 128 columns; 4 tokens' loads in flight at once
-        const int ew = etid >> 5;
-        constexpr int kEW = kEpiThreads / 32;
-        for (int tk0 = tk_lo + ew; tk0 < tk_hi; tk0 += 4 * kEW) {
-          float4 acc4[4];
-#pragma unroll
-          for (int bb = 0; bb < 4; ++bb) acc4[bb] = make_float4(0.f, 0.f, 0.f, 0.f);
-          for (int sp = 0; sp < KS; ++sp) {
-            const float* pp = p.part + (static_cast<size_t>(tile * KS + sp) * BN) * kTileN + lane * 4;
-            float4 w4[4];
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb) {
-              const int tk = tk0 + bb * kEW;
-              w4[bb] = tk < tk_hi ? __ldcg(reinterpret_cast<const float4*>(pp + static_cast<size_t>(tk) * kTileN))
-                                  : make_float4(0.f, 0.f, 0.f, 0.f);
-            }
-#pragma unroll
-            for (int bb = 0; bb < 4; ++bb) {
-              acc4[bb].x += w4[bb].x;
-              acc4[bb].y += w4[bb].y;
-              acc4[bb].z += w4[bb].z;
-              acc4[bb].w += w4[bb].w;
-            }
-          }
-#pragma unroll
-          for (int bb = 0; bb < 4; ++bb) {
-            const int tk = tk0 + bb * kEW;
-            const int m = m0 + tk;
-            float4 x = make_float4(0.f, 0.f, 0.f, 0.f);
-            const size_t idx = static_cast<size_t>(m) * p.ldxo + n0 + lane * 4;
-            if (tk < tk_hi && m < p.M) {
-              const float4 x0 = __ldcg(reinterpret_cast<const float4*>(p.xo + idx));
-              x = make_float4(x0.x + acc4[bb].x, x0.y + acc4[bb].y, x0.z + acc4[bb].z, x0.w + acc4[bb].w);
-              *reinterpret_cast<float4*>(p.xo + idx) = x;
-              uint2 pk;
-              pk.x = pack_half2(x.x, x.y);
-              pk.y = pack_half2(x.z, x.w);
-              *reinterpret_cast<uint2*>(p.xo16 + idx) = pk;
-            }
-            const float ss = warp_sum(x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w);
-            if (lane == 0 && tk < tk_hi && m < p.M && p.ss_out != nullptr)
-              p.ss_out[static_cast<size_t>(t_n) * p.ss_stride + m] = ss;
-          }
-        }
-        // departures: the last split to leave resets the counter for the next launch
-        epi_sync();
-        if (etid == 0 && atomicAdd(p.tile_count + tile, 1) == 2 * KS - 1) p.tile_count[tile] = 0;
       }
     }
     // the output stores of this group complete before the CTA leaves
@@ -749,24 +664,13 @@ cudaError_t gemm_tc_set_attributes() {
 
 int gemm_tc_pair_clusters() { return g_pair_clusters; }
 
-int gemm_tc_k_splits(int tiles, int KT, int sm_count) {
-  if (tiles <= 0 || tiles >= sm_count) return 1;
-  int ks = sm_count / tiles;                // all units in one wave
-  const int max_ks = KT / 4;                // at least 4 K steps (16 MMAs) per unit
-  if (ks > max_ks) ks = max_ks;
-  return ks < 1 ? 1 : ks;
-}
-
-// tiles x splits <= sm_count whenever splits > 1, and a partial tile is at most 128 x 256 fp32
-size_t gemm_tc_part_bytes(int sm_count) { return static_cast<size_t>(sm_count) * kTileN * 256 * sizeof(float); }
-
 cudaError_t launch_gemm_tc(const CUtensorMap& map_a, const TcGemmArgs& args, int bn, int epi, bool norm,
                            cudaStream_t stream, bool pdl, const CUtensorMap* map_w) {
   const bool pair = map_w != nullptr;
   size_t smem = 0;
   const void* fn = tc_select(bn, epi, norm, pair, &smem);
   if (!fn || args.N % kTileN != 0 || args.K % kTileK != 0) return cudaErrorInvalidValue;
-  if (pair && ((args.N / kTileN) % 2 != 0 || args.k_splits > 1 || g_pair_clusters <= 0)) return cudaErrorInvalidValue;
+  if (pair && ((args.N / kTileN) % 2 != 0 || g_pair_clusters <= 0)) return cudaErrorInvalidValue;
   static int sm_count = 0;
   if (sm_count == 0) {
     int dev = 0;
@@ -789,8 +693,7 @@ cudaError_t launch_gemm_tc(const CUtensorMap& map_a, const TcGemmArgs& args, int
   }
   TcGemmArgs a = args;
   void* kargs[] = {&map, &mapw, &mapy, &a};
-  if (a.k_splits > 1 && (epi != kEpiResidual || a.part == nullptr || a.tile_count == nullptr)) return cudaErrorInvalidValue;
-  const int units = (args.N / kTileN) * ((args.M + bn - 1) / bn) * (a.k_splits > 1 ? a.k_splits : 1);
+  const int units = (args.N / kTileN) * ((args.M + bn - 1) / bn);
   if (pair) {  // one cluster of two CTAs per pair unit, at most as many as are co-resident
     const int pairs = units / 2;
     const int clusters = pairs < g_pair_clusters ? pairs : g_pair_clusters;

@@ -31,13 +31,7 @@ struct TcGemmArgs {
   int n_ss;
   int ss_stride;
   int* status;
-  // split K (kEpiResidual only): k_splits > 1 cuts each tile's K steps into k_splits
-  // near-equal ranges run by different CTAs (never more units than SMs, one CTA per
-  // SM, so all are resident); each writes its fp32 partial tile to `part`
-  // ([tile][split][BN tokens][128]), waits until the tile's k_splits partials are
-  // there (tile_count[tile], zero between launches), and adds them in split order
-  // for its 1/k_splits share of the tile's tokens.
-  int k_splits;
+  // gemm_stream: fp32 partials of the tiles that several CTAs share, and arrivals per tile
   float* part;
   int* tile_count;
   // gemm_stream, kEpiResidual: optional second copy of the updated rows (layout of xo)
@@ -46,22 +40,17 @@ struct TcGemmArgs {
   int w_tile0;
 };
 
-// k splits for a residual GEMM with `tiles` output tiles of KT k steps on `sm_count` SMs
-int gemm_tc_k_splits(int tiles, int KT, int sm_count);
-// bytes of the split-K partial workspace that covers every GEMM of a handle
-size_t gemm_tc_part_bytes(int sm_count);
-
 cudaError_t gemm_tc_set_attributes();
 // co-resident CTA pairs of the pair variant on this device (0: the variant is not available)
 int gemm_tc_pair_clusters();
 // map_w != nullptr selects the pair variant (bn 256, RMSNorm-fused store epilogue, N a multiple
-// of 256, no K split): map_a then has 128-row boxes and map_w covers the packed weight tiles
+// of 256): map_a then has 128-row boxes and map_w covers the packed weight tiles
 cudaError_t launch_gemm_tc(const CUtensorMap& map_a, const TcGemmArgs& args, int bn, int epi, bool norm,
                            cudaStream_t stream, bool pdl, const CUtensorMap* map_w = nullptr);
 // ---- few-token variant (gemm_stream.cu): M <= 256 tokens in one tile of kStreamTiles[i] tokens
 // (map_a: a box of that many rows), the weight stream cut evenly over the SMs. Takes w, N, K, M,
 // the epilogue's outputs, ss_in / ss_out, `part` (gemm_stream_part_bytes) and `tile_count`
-// ([N / 128], zero between launches); k_splits and w_tile0 are not used. RMSNorm is fused into
+// ([N / 128], zero between launches); w_tile0 is not used. RMSNorm is fused into
 // the store and SwiGLU epilogues.
 constexpr int kStreamTileCount = 5;
 constexpr int kStreamTiles[kStreamTileCount] = {16, 32, 64, 128, 256};
@@ -70,6 +59,18 @@ int gemm_stream_tile(int M);  // index into kStreamTiles (-1: too many tokens)
 size_t gemm_stream_part_bytes(int M, int sm_count);
 cudaError_t launch_gemm_stream(const CUtensorMap& map_a, const TcGemmArgs& args, int epi, int sm_count,
                                cudaStream_t stream, bool pdl);
+// ---- residual projections with K cut over the CTAs of a cluster (gemm_res.cu): takes w, N, K, M,
+// xo, xo16, ldxo, ss_out and ss_stride; map_a with a box of kResTiles[plan.tile] rows
+constexpr int kResTileCount = 6;
+constexpr int kResTiles[kResTileCount] = {48, 64, 96, 128, 144, 160};
+struct ResPlan {
+  int tile;    // index into kResTiles
+  int splits;  // K splits = cluster size (1: not for this kernel)
+};
+ResPlan gemm_res_plan(int M, int N, int K);  // for the current device
+cudaError_t gemm_res_set_attributes();
+cudaError_t launch_gemm_res(const CUtensorMap& map_a, const TcGemmArgs& args, const ResPlan& plan, cudaStream_t stream,
+                            bool pdl);
 // rows[128]: pointers to the 128 source rows (fp32, length >= k0 + 64); col_scale: optional per-K gain.
 void pack_tc_tile(const float* const* rows, const float* col_scale, int k0, __half* out);
 // 2-D fp16 tensor map over a row-major [rows, cols] buffer with a (box_rows x 64) box and 128-byte swizzle.

@@ -76,13 +76,12 @@ cudaError_t launch_attention(const AttnArgs& a, int B, int cache_dtype, cudaStre
 // attributes of the kernel that launch_attention runs for these arguments / of every kernel of a dtype
 cudaError_t attention_set_attributes(const AttnArgs& a, int cache_dtype);
 cudaError_t attention_set_attributes(int cache_dtype);
-// tcgen05 path: up to 8 splits, n_q <= 48, 1 <= n_own <= 64
+// tcgen05 path: up to 8 splits (run on as many as are resident at once), n_q <= 48, 1 <= n_own <= 64
 bool attention_tc_eligible(const AttnArgs& a, int n_splits);
 cudaError_t launch_attention_tc(const AttnArgs& a, int B, int cache_dtype, cudaStream_t stream, bool pdl);
 cudaError_t attention_tc_set_attributes(int cache_dtype, bool split);
 // CTAs of the tcgen05 path that share an SM
 constexpr int attention_ctas_per_sm(int cache_dtype) { return cache_dtype == 1 ? 2 : 1; }
-int attention_launch_count(int n_splits);
 
 // --------------------------------------------------------- embed / head
 struct EmbedArgs {
@@ -144,5 +143,11 @@ cudaError_t launch_state_tokens(const StateArgs& a, cudaStream_t stream);
 // attribute when `pdl` is set and a (cluster_x, cluster_y, 1) cluster when either exceeds 1.
 cudaError_t launch_ex(const void* fn, dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                       bool pdl, void** args, int cluster_y = 1, int cluster_x = 1);
+
+// Clusters of `cluster` CTAs (x) of kernel `fn` that are resident at once on the current device (0 on
+// failure). Clusters do not straddle GPCs, so large ones leave SMs idle: with one CTA per SM 152 SMs
+// held 76 pairs, but 46 clusters of 3, 36 of 4, 28 of 5, 23 of 6 and 15 of 7 or 8. The dynamic
+// shared-memory attribute of `fn` must be set.
+int max_resident_clusters(const void* fn, int threads, size_t smem, int cluster);
 
 }  // namespace fsx
