@@ -893,13 +893,16 @@ cudaError_t attention_tc_set_attributes(int cache_dtype, bool split) {
 }
 
 // The most splits, at least 2 and at most `wanted`, whose clusters are all resident at once: one
-// cluster in a second wave costs as much as the first wave (32 clusters of 8 against 30 that fit).
+// cluster in a second wave costs as much as the first wave. The occupancy counts clusters at one
+// CTA per SM; where two share an SM, s CTAs take the SMs of (s + 1) / 2 (32 clusters of 8 started
+// within 3.3 us of one another, against 15 that it counts for 8 and 36 for 4).
 // Split launches check every cache value, so a call that asks for splits keeps two.
 static int resident_splits(int wanted, int B, int n_heads, int cache_dtype) {
   const int threads = cache_dtype == 1 ? Shape<false>::kThreads : Shape<true>::kThreads;
+  const int per_sm = attention_ctas_per_sm(cache_dtype);
   int s = wanted;
-  while (s > 2 && max_resident_clusters(tc_fn(cache_dtype, true), threads, static_cast<size_t>(tc_smem(cache_dtype)), s) <
-                      static_cast<long long>(B) * n_heads)
+  while (s > 2 && max_resident_clusters(tc_fn(cache_dtype, true), threads, static_cast<size_t>(tc_smem(cache_dtype)),
+                                        (s + per_sm - 1) / per_sm) < static_cast<long long>(B) * n_heads)
     --s;
   return s;
 }
