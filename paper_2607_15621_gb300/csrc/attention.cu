@@ -92,7 +92,7 @@ __device__ __forceinline__ void cp_async_wait_n(int n) {
 template <typename CT>
 __device__ __forceinline__ void convert_unit(const unsigned char* raw, uint4* dst, bool own, uint32_t& range);
 
-// bf16 cache rows: 16 raw bytes = 8 values -> 8 fp16 (saturated, out-of-range values recorded)
+// bf16 cache rows: 16 raw bytes = 8 values -> 8 fp16 (their largest magnitudes kept)
 template <>
 __device__ __forceinline__ void convert_unit<__nv_bfloat16>(const unsigned char* raw, uint4* dst, bool own,
                                                             uint32_t& range) {
@@ -100,8 +100,8 @@ __device__ __forceinline__ void convert_unit<__nv_bfloat16>(const unsigned char*
   if (own) {
     *dst = v;
   } else {
-    *dst = make_uint4(bf16x2_to_half2_sat(v.x, range), bf16x2_to_half2_sat(v.y, range),
-                      bf16x2_to_half2_sat(v.z, range), bf16x2_to_half2_sat(v.w, range));
+    *dst = make_uint4(bf16x2_to_half2_peak(v.x, range), bf16x2_to_half2_peak(v.y, range),
+                      bf16x2_to_half2_peak(v.z, range), bf16x2_to_half2_peak(v.w, range));
   }
 }
 
@@ -113,8 +113,8 @@ __device__ __forceinline__ void convert_unit<float>(const unsigned char* raw, ui
   } else {
     const float4 a = *reinterpret_cast<const float4*>(raw);
     const float4 b = *reinterpret_cast<const float4*>(raw + 16);
-    *dst = make_uint4(f32x2_to_half2_sat(a.x, a.y, range), f32x2_to_half2_sat(a.z, a.w, range),
-                      f32x2_to_half2_sat(b.x, b.y, range), f32x2_to_half2_sat(b.z, b.w, range));
+    *dst = make_uint4(f32x2_to_half2_peak(a.x, a.y, range), f32x2_to_half2_peak(a.z, a.w, range),
+                      f32x2_to_half2_peak(b.x, b.y, range), f32x2_to_half2_peak(b.z, b.w, range));
   }
 }
 
@@ -258,7 +258,7 @@ __global__ void __launch_bounds__(kThreads, FSX_ATTN_MIN_CTAS) attn_splitkv_kern
 
   const int n_chunks = empty_range ? 0 : static_cast<int>((kend - kbeg + kChunk - 1) / kChunk);
   for (int i = 0; i < kRawStages && i < n_chunks; ++i) issue_chunk(i, i);
-  uint32_t range = 0;  // a cache value outside the fp16 range was saturated
+  uint32_t range = 0;  // largest magnitudes of the converted cache values
 
   for (int c = 0; c < n_chunks; ++c) {
     const int s = c % kRawStages;

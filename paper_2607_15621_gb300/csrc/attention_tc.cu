@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
     uint64_t* empty = is_v ? vempty : kempty;
     bool ok = true;
     int issued = n_first;  // chunks whose loads were issued
-    uint32_t range = 0;    // a staged cache value lies outside the fp16 range
+    uint32_t range = 0;    // fp32: largest magnitudes of the staged values; bf16: bits set by out-of-range ones
     int i = 0;
     for (; ok && i < n_chunks; ++i) {
       if (i + 1 < n_chunks) cp_async_wait<1>();
@@ -582,8 +582,8 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
             if (r < rows) {
               const float4 x = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + sw * 16);
               const float4 y = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + (sw ^ 1) * 16);
-              const uint32_t x0 = f32x2_to_half2_sat(x.x, x.y, range), x1 = f32x2_to_half2_sat(x.z, x.w, range);
-              const uint32_t y0 = f32x2_to_half2_sat(y.x, y.y, range), y1 = f32x2_to_half2_sat(y.z, y.w, range);
+              const uint32_t x0 = f32x2_to_half2_peak(x.x, x.y, range), x1 = f32x2_to_half2_peak(x.z, x.w, range);
+              const uint32_t y0 = f32x2_to_half2_peak(y.x, y.y, range), y1 = f32x2_to_half2_peak(y.z, y.w, range);
               out = sw == 0 ? make_uint4(x0, x1, y0, y1) : make_uint4(y0, y1, x0, x1);
             }
             *reinterpret_cast<uint4*>(slot + tile128_off(r, u)) = out;
@@ -640,7 +640,8 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
         }
       }
     }
-    if (kCheck) flag_range(p.status, range);
+    if (F32) flag_range(p.status, range);
+    else if (SPLIT && range != 0) set_status(p.status, kStatusRange);
     cp_async_wait<0>();
     // after an abort: the TMA chunks issued but not consumed land before the CTA leaves
     if (pt == 0)

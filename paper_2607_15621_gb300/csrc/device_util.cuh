@@ -177,28 +177,31 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
   return *reinterpret_cast<uint32_t*>(&h);
 }
 
-// Cache values the kernels convert to fp16 are expected within +-65504. The
-// converters below saturate instead of overflowing to infinity (cvt .satfinite),
-// and `range` collects whether an input lay outside the fp16 range (a bf16
-// magnitude of 65536 or more, infinity or NaN; an fp32 magnitude that rounds
-// beyond 65504). flag_range() turns that into the FSX_ERR_RANGE error status, and
-// the tick is abandoned like any other device-side error.
-__device__ __forceinline__ uint32_t bf16x2_to_half2_sat(uint32_t v, uint32_t& range) {
-  const float lo = __uint_as_float(v << 16);
-  const float hi = __uint_as_float(v & 0xffff0000u);
-  range |= static_cast<uint32_t>((v & 0x7fffu) >= 0x4780u) | static_cast<uint32_t>(((v >> 16) & 0x7fffu) >= 0x4780u);
-  uint32_t r;
-  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
+// Cache values the kernels convert to fp16 are expected within +-65504. The converters
+// below keep in `peak` the largest magnitudes seen, as two packed fp16 (start at 0): a value
+// that rounds beyond 65504 became an infinity and a NaN stays one, so out_of_range(peak) tells
+// whether an input lay outside the fp16 range. flag_range() turns that into the FSX_ERR_RANGE
+// error status, and the tick is abandoned like any other device-side error: the infinity
+// reaches no caller. (One max per pair of values: the conversions bound the staging warps.)
+__device__ __forceinline__ uint32_t peak_of(uint32_t peak, uint32_t h) {
+  const __half2 m = __hmax2_nan(*reinterpret_cast<const __half2*>(&peak), __habs2(*reinterpret_cast<const __half2*>(&h)));
+  return *reinterpret_cast<const uint32_t*>(&m);
 }
-__device__ __forceinline__ uint32_t f32x2_to_half2_sat(float lo, float hi, uint32_t& range) {
-  range |= static_cast<uint32_t>(!(fabsf(lo) < 65520.f)) | static_cast<uint32_t>(!(fabsf(hi) < 65520.f));
-  uint32_t r;
-  asm("cvt.rn.satfinite.f16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
-  return r;
+__device__ __forceinline__ uint32_t bf16x2_to_half2_peak(uint32_t v, uint32_t& peak) {
+  const uint32_t h = pack_half2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
+  peak = peak_of(peak, h);
+  return h;
 }
-__device__ __forceinline__ void flag_range(int* status, uint32_t range) {
-  if (range) set_status(status, kStatusRange);
+__device__ __forceinline__ uint32_t f32x2_to_half2_peak(float lo, float hi, uint32_t& peak) {
+  const uint32_t h = pack_half2(lo, hi);
+  peak = peak_of(peak, h);
+  return h;
+}
+__device__ __forceinline__ bool out_of_range(uint32_t peak) {  // an infinity or a NaN in either half
+  return (peak & 0x7c00u) == 0x7c00u || (peak & 0x7c000000u) == 0x7c000000u;
+}
+__device__ __forceinline__ void flag_range(int* status, uint32_t peak) {
+  if (out_of_range(peak)) set_status(status, kStatusRange);
 }
 
 // Two bf16 (low half first) -> two fp16, via fp32 (bf16 -> fp32 is exact).

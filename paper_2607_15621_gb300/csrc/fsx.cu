@@ -201,6 +201,7 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
     pa.head_w = h->head_w;
     pa.head_b = h->head_b;
     pa.targs = h->d_args;
+    pa.cache_maps = h->d_cache_maps;
     pa.n_layers = c.n_layers;
     pa.d = d;
     pa.H = c.n_heads;

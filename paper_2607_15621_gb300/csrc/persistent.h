@@ -27,6 +27,7 @@ struct PersistArgs {
   const float* head_w;
   const float* head_b;
   const TickArgs* targs;
+  const CUtensorMap* cache_maps;  // bf16: [2 n_layers] maps of the K and V caches (AttnArgs), or NULL
   int n_layers, d, H, F, n_action, n_frame, n_waypoints;
   int n_b_clusters;             // F / 64
   int frame_dtype;

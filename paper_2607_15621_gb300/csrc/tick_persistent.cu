@@ -49,8 +49,14 @@
 // shared memory, and the accumulator rows that produces are never read. Every
 // GEMM is issued by four warps into four accumulators that the epilogue adds:
 // one issuing thread pays a fixed cost per MMA that four issuers overlap.
+//
+// The layer loop is straight-line code that every layer runs once, so its size counts: at 168 KB of
+// instructions for the kernel a layer of 224 rows took 22.2 us, at 192 KB 26.7 us, at 132 KB 21.9 us.
+// Loops whose order allows it are therefore rolled, and a body used twice is one loop turn more.
 #include <cooperative_groups.h>
 #include <math_constants.h>
+
+#include <type_traits>
 
 #include "device_util.cuh"
 #include "kernels.h"
@@ -81,6 +87,9 @@ constexpr uint32_t kTmemCols = kNAcc * kAccCols;
 constexpr uint32_t kIdesc = idesc_f16(128, kTokTile);
 constexpr int kRecvBytes = kRowsPerRank * kD * 4;  // merge partials one CTA sends another (fp32)
 constexpr int kRsBytes = 32 * kTokTile * 4;        // gate/up partials one CTA sends another (fp32)
+constexpr int kNB = 3;                             // cache-row staging buffers
+constexpr int kAttendWarps = 6;                    // warps 0-5 attend, warps 6 and 7 convert the next chunk
+constexpr int kCvtWarps = kThr / 32 - kAttendWarps;
 static_assert(kRecvBytes == kRsBytes, "the merge and the gate/up reduce-scatter share the receive buffer");
 
 struct Smem {
@@ -115,6 +124,38 @@ __device__ __forceinline__ void red_add_v4(float* addr, float4 v) {
                : "memory");
 }
 
+// Bounded wait (about one second) for phase `parity` of an mbarrier, acquiring at CTA or cluster scope;
+// false (and status set) when it runs out. Written for size: the kernel holds some thirty of them
+// and its layer loop has to stay in the instruction cache. The timer's low word wraps after 4.3 s.
+template <bool kCluster>
+__device__ __forceinline__ bool wait_phase(uint64_t* bar, uint32_t parity, int* status) {
+  const uint32_t addr = smem_addr(bar);
+  uint32_t t0 = 0;
+  for (;;) {
+    uint32_t done, now;
+    if (kCluster)
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.try_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, "
+          "0, p;\n}"
+          : "=r"(done)
+          : "r"(addr), "r"(parity)
+          : "memory");
+    else
+      asm volatile(
+          "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
+          : "=r"(done)
+          : "r"(addr), "r"(parity)
+          : "memory");
+    if (done) return true;
+    asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(now));
+    if (t0 == 0) t0 = now | 1u;
+    if (now - t0 > kWaitLimitNs && now - t0 < 0x80000000u) {
+      set_status(status, kStatusTimeout);
+      return false;
+    }
+  }
+}
+
 // Device-wide arrival counter: after the CTA barrier one thread adds 1 with
 // release semantics, which publishes the CTA's earlier global writes.
 __device__ __forceinline__ void arrive(int* counter) {
@@ -129,45 +170,65 @@ __device__ __forceinline__ uint32_t cluster_addr(const void* local, int rank) {
   return r;
 }
 
+// The same for the address `delta` away from this CTA's: what separates the two CTAs' shared memory
+// is the same for every offset.
+__device__ __forceinline__ uint32_t peer_at(const void* local, uint32_t delta) { return smem_addr(local) + delta; }
+
 // Arm an exchange barrier (count 1) for its next phase: the arrival plus the
 // bytes the partners will deliver by st.async.
 __device__ __forceinline__ void arm(uint64_t* bar, uint32_t bytes) { mbar_arrive_expect_tx(bar, bytes); }
 
-// tensor memory -> registers: N (16 or 32) consecutive fp32 columns of each of the four
-// accumulators, all loads in flight before one wait, added in accumulator order
-template <int N>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[N]);
-template <>
-__device__ __forceinline__ void tmem_ld_cols<16>(uint32_t taddr, uint32_t (&r)[16]) {
+// 2^x on the special-function unit (relative error about 2^-22; -inf -> +0)
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+// The running maximum of the attention moves only when a tile's exceeds it by more than this.
+constexpr float kLazyRescale = 8.f;
+
+// one 64-token x 64-dim box of a head of the cache (3-D map [rows, heads, 128], 128-byte swizzle)
+__device__ __forceinline__ void tma_load_cache(void* dst, const CUtensorMap* map, int x, int head, int row,
+                                               uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.3d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4}], "
+      "[%5];" ::"r"(smem_addr(dst)),
+      "l"(map), "r"(x), "r"(head), "r"(row), "r"(smem_addr(bar))
+      : "memory");
+}
+
+// tensor memory -> registers: 24 consecutive fp32 columns of each of the four accumulators, all
+// loads in flight before one wait, added in accumulator order
+constexpr int kHalfTok = kTokTile / 2;  // tokens a warp reads: warps 0-3 the first 24, warps 4-7 the rest
+__device__ __forceinline__ void tmem_ld24(uint32_t taddr, uint32_t (&r)[kHalfTok]) {
   asm volatile(
       "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0,%1,%2,%3,%4,%5,%6,%7,%8,%9,%10,%11,%12,%13,%14,%15}, [%16];"
       : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
         "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr));
-}
-template <>
-__device__ __forceinline__ void tmem_ld_cols<32>(uint32_t taddr, uint32_t (&r)[32]) {
-  tmem_ld32_issue(taddr, r);
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]), "=r"(r[22]), "=r"(r[23])
+               : "r"(taddr + 16u));
 }
 // the wait for every TMEM load of this thread; the registers are tied to it so that
 // no use of them is scheduled before it (the first wait completes all loads)
-__device__ __forceinline__ void tmem_wait_tied(uint32_t (&r)[16]) {
+__device__ __forceinline__ void tmem_wait_tied(uint32_t (&r)[kHalfTok]) {
   asm volatile("tcgen05.wait::ld.sync.aligned;"
                : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+                 "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]), "+r"(r[15]),
+                 "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]), "+r"(r[22]), "+r"(r[23])
                :
                : "memory");
 }
-__device__ __forceinline__ void tmem_wait_tied(uint32_t (&r)[32]) { tmem_wait_ld32(r); }
-template <int N>
-__device__ __forceinline__ void tmem_ld_sum4(uint32_t taddr, float (&v)[N]) {
-  uint32_t r[kNAcc][N];
+__device__ __forceinline__ void tmem_ld_sum4(uint32_t taddr, float (&v)[kHalfTok]) {
+  uint32_t r[kNAcc][kHalfTok];
 #pragma unroll
-  for (int a = 0; a < kNAcc; ++a) tmem_ld_cols<N>(taddr + static_cast<uint32_t>(a) * kAccCols, r[a]);
+  for (int a = 0; a < kNAcc; ++a) tmem_ld24(taddr + static_cast<uint32_t>(a) * kAccCols, r[a]);
 #pragma unroll
   for (int a = 0; a < kNAcc; ++a) tmem_wait_tied(r[a]);
 #pragma unroll
-  for (int i = 0; i < N; ++i)
+  for (int i = 0; i < kHalfTok; ++i)
     v[i] = ((__uint_as_float(r[0][i]) + __uint_as_float(r[1][i])) + __uint_as_float(r[2][i])) + __uint_as_float(r[3][i]);
 }
 
@@ -210,7 +271,10 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   uint64_t* bbar = agbar + 1;          // phase B: partial sums of x^2 and gate/up partials
   uint64_t* hbar = bbar + 1;           // phase B: the partners' SwiGLU columns
   uint64_t* drain_bar = hbar + 1;      // the four issuing threads' last MMAs (before TMEM is freed)
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(drain_bar + 1);
+  uint64_t* raw_bar = drain_bar + 1;   // [kNB] a cache chunk's raw rows have landed in their buffer
+  uint64_t* cvt_bar = raw_bar + kNB;   // [kNB] the buffer's rows are fp16 (both converting warps)
+  uint64_t* free_bar = cvt_bar + kNB;  // [kNB] the six attending warps are done with the buffer
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(free_bar + kNB);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);  // a wait of this CTA timed out
   float* gss = reinterpret_cast<float*>(smem + L.gss);
   float* rstd = reinterpret_cast<float*>(smem + L.rstd);
@@ -231,6 +295,9 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   const int lane = tid & 31;
   const int rank = static_cast<int>(cluster.block_rank());
   const int head = blockIdx.x / kCl;             // phase A: this cluster's head
+  uint32_t pdelta[kCl - 1];                      // shared-memory distance of partners rank + 1, + 2, + 3
+#pragma unroll
+  for (int i = 0; i < kCl - 1; ++i) pdelta[i] = cluster_addr(smem, (rank + 1 + i) & (kCl - 1)) - smem_addr(smem);
   const int G = gridDim.x;
   const int cta = blockIdx.x;
   const int d = p.d;                             // 512 (checked on the host)
@@ -254,10 +321,8 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     const int i = q % kLayerChunks;
     return i >= kPersistAChunks + (in_b ? kPersistBChunks : 0);
   };
-  int issued_upto = 0;  // thread 0: ring positions issued so far (in increasing order)
   auto issue = [&](int q) {  // one thread; an empty position just completes the slot's phase
     if (q >= total_chunks || *abort) return;  // after a timeout no new copy starts
-    issued_upto = q + 1;
     uint64_t* bar = full + (q % kSlots);
     if (is_empty(q)) {
       mbar_arrive(bar);
@@ -269,21 +334,21 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   // wait for position q; false after a timeout of this tick (no MMA then reads the slot)
   auto wait_chunk = [&](int q) -> bool {
     if (*abort) return false;
-    const bool ok = mbar_wait(full + (q % kSlots), static_cast<uint32_t>((q / kSlots) & 1), p.status);
+    const bool ok = wait_phase<false>(full + (q % kSlots), static_cast<uint32_t>((q / kSlots) & 1), p.status);
     if (!ok) *abort = 1;
     return ok;
   };
   // wait for phase `parity` of an exchange barrier; false after a timeout of this tick
   auto xwait = [&](uint64_t* bar, int parity) -> bool {
     if (*abort) return false;
-    const bool ok = mbar_wait_cluster(bar, static_cast<uint32_t>(parity & 1), p.status);
+    const bool ok = wait_phase<true>(bar, static_cast<uint32_t>(parity & 1), p.status);
     if (!ok) *abort = 1;
     return ok;
   };
   uint32_t n_mma = 0;  // completed MMA groups (phase of mma_bar)
   // all threads: wait for the MMA groups just committed, then order TMEM reads after them
   auto wait_mma = [&]() {  // this CTA's own MMAs always complete: waited even after a timeout
-    if (!mbar_wait(mma_bar, n_mma & 1u, p.status)) *abort = 1;
+    if (!wait_phase<false>(mma_bar, n_mma & 1u, p.status)) *abort = 1;
     ++n_mma;
     tc_fence_after();
   };
@@ -304,6 +369,12 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     mbar_init(mma_bar, kNAcc);
     for (int i = 0; i < kCl + 5; ++i) mbar_init(xbar + i, 1);
     mbar_init(drain_bar, kNAcc);
+    for (int i = 0; i < kNB; ++i) {
+      mbar_init(raw_bar + i, 64);
+      mbar_init(cvt_bar + i, 32 * kCvtWarps);
+      mbar_init(free_bar + i, kAttendWarps);
+    }
+#pragma unroll 1
     for (int q = 0; q < kSlots; ++q) issue(q);
   }
 
@@ -408,10 +479,9 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         if (xu == 0) gss[rank * kTokTile + r] = ss;
 #pragma unroll
         for (int pi = 1; pi < kCl; ++pi) {
-          const int peer = (rank + pi) & (kCl - 1);
-          const uint32_t pb = cluster_addr(peer_bar, peer);
-          if (send_x) st_async_v4(cluster_addr(dst, peer), h, pb);
-          if (xu == 0) st_async_b32(cluster_addr(gss + rank * kTokTile + r, peer), __float_as_uint(ss), pb);
+          const uint32_t dl = pdelta[pi - 1], pb = peer_at(peer_bar, dl);
+          if (send_x) st_async_v4(peer_at(dst, dl), h, pb);
+          if (xu == 0) st_async_b32(peer_at(gss + rank * kTokTile + r, dl), __float_as_uint(ss), pb);
         }
       }
     }
@@ -449,50 +519,44 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       res[i] = t < T ? ld_cg4(Xs + static_cast<size_t>(t) * d + col0 + lane * 4) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
-  // the four accumulators' sum (128 output columns x 48 tokens) -> dstT[token][column];
-  // warps 0-3 take tokens 0-31, warps 4-7 tokens 32-47 of their 32 TMEM lanes
+  // the four accumulators' sum (128 output columns x 48 tokens) -> dstT[token][column]
   auto tmem_to_dstT = [&]() {
-    const int col = (warp & 3) * 32 + lane;
-    const uint32_t taddr = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
-    if (warp < 4) {
-      float v[32];
-      tmem_ld_sum4<32>(taddr, v);
+    const int t0 = (warp >> 2) * kHalfTok;
+    float v[kHalfTok];
+    tmem_ld_sum4(tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + static_cast<uint32_t>(t0), v);
+    float* dst = dstT + t0 * kDS + (warp & 3) * 32 + lane;
 #pragma unroll
-      for (int j = 0; j < 32; ++j) dstT[j * kDS + col] = v[j];
-    } else {
-      float v[16];
-      tmem_ld_sum4<16>(taddr + 32u, v);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) dstT[(32 + j) * kDS + col] = v[j];
-    }
+    for (int j = 0; j < kHalfTok; ++j) dst[j * kDS] = v[j];
     tc_fence_before();
     __syncthreads();
   };
 
   // ---- this CTA's cache rows of a layer, staged in the shared memory that is idle
   // from the end of the QKV MMA to the end of the attention: ring slots 2-5 and
-  // the activation image behind them (112 KB, contiguous). It is cut into kNB
-  // buffers of kStageKeys keys (K rows then V rows, each row padded to kRowStride
-  // bytes so ldmatrix reads are conflict-free), so kNB - 1 chunks are in flight
-  // while one is consumed. Rows arrive raw (bf16 / fp32) by 16-byte cp.async
-  // copies and are converted to fp16 in place (at the start of the row). Thread
-  // t always handles 16-byte units t, t + 256, ... of a buffer (row = unit >> s,
-  // no division), and the weight copies of positions 8-11 of the layer (slots
-  // 2-5) are issued only once the attention is done with the region.
-  constexpr int kRowStride = sizeof(CT) == 2 ? kD * 2 + 16 : kD * 4 + 16;  // 272 / 528 bytes
-  constexpr int kNB = 3;                                                  // staging buffers
+  // the activation image behind them (112 KB, contiguous), cut into kNB buffers of kStageKeys keys.
+  // bf16: a buffer is the swizzled 128-byte-row layout that TMA writes ([K, V][2 blocks of 64
+  // dims][64 keys]; 16-byte unit u of key k at unit u ^ (k mod 8)), so ldmatrix reads are
+  // conflict-free and one thread loads a whole chunk with four boxes; a short last chunk comes by
+  // 16-byte cp.async of two warps (rows past the range are never read). fp32: rows of 512 bytes
+  // padded to kRowStride, by cp.async. The chunk's 64 arrivals (copies included) complete its
+  // buffer's raw_bar; rows are converted to fp16 in place (fp32: at the start of the row, whole
+  // rows by one warp). The first chunk of a layer is converted by all eight warps; from then on
+  // warps 6 and 7 convert chunk j + 1 and refill the buffer of chunk j - 1 while warps 0-5 attend
+  // over chunk j. With every thread copying, converting and meeting at three block barriers per
+  // chunk, a chunk of 64 keys took 2.3 us: 0.97 to attend, 0.64 to convert, 0.26 to issue copies, the
+  // rest waiting; now 1.7 us, 1.0 of them the two warps' conversion (4096 rows, 8 layers: 467 -> 393 us a
+  // tick). A bulk copy per row in place of the TMA boxes took 4.5 us a
+  // chunk: 128 of them hold two warps for longer than the rest of their work. The weight copies of
+  // positions 8-11 of the layer (slots 2-5) are issued only once the attention is done with the region.
+  constexpr bool kSw = sizeof(CT) == 2;                                   // swizzled buffers
+  constexpr int kRowStride = kD * 4 + 16;                                 // fp32: 528 bytes
+  constexpr int kBlockBytes = 64 * 128;                                   // bf16: 64 keys x 64 dims
   constexpr int kStageRegion = 4 * kSlotBytes + 8 * kActAtom;             // 112 KB (d = 512)
-  constexpr int kStageKeys = sizeof(CT) == 2 ? 64 : 36;                   // two whole key tiles (bf16)
-  constexpr int kBufBytes = 2 * kStageKeys * kRowStride;                  // 34 / 37.1 KB
-  constexpr int kUnitsPerRow = kD * static_cast<int>(sizeof(CT)) / 16;   // raw 16-byte units: 16 / 32
-  constexpr int kUnitShift = sizeof(CT) == 2 ? 4 : 5;
-  constexpr int kRawIters = (2 * kStageKeys * kUnitsPerRow + kThr - 1) / kThr;  // 8 / 9
-  constexpr int kCvtIters = (2 * kStageKeys * 16 + kThr - 1) / kThr;            // fp16 units: 8 / 5
+  constexpr int kStageKeys = kSw ? 64 : 36;                               // bf16: two whole key tiles
+  constexpr int kBufBytes = kSw ? 4 * kBlockBytes : 2 * kStageKeys * kRowStride;  // 32 / 37.1 KB
   static_assert(kSlots == 6 && kPersistAChunks == 8, "staging assumes slots 2-5 hold positions 8-11");
-  static_assert((1 << kUnitShift) == kUnitsPerRow, "unit shift");
-  static_assert(kBufBytes % 16 == 0 && (kStageKeys * kRowStride) % 16 == 0, "cp.async / ldmatrix alignment");
+  static_assert((kStageKeys * kRowStride) % 16 == 0 && kBlockBytes % 1024 == 0, "copy / swizzle alignment");
   static_assert(kNB * kBufBytes <= kStageRegion, "staging buffers exceed slots 2-5 + the activation image");
-  static_assert(sizeof(CT) == 4 || kStageKeys % (2 * kKeyTile) == 0, "an even number of key tiles per bf16 chunk");
   static_assert(3 * 2 * 8 * 32 * 16 + 3 * 2 * 32 * 16 <= 8 * kActAtom, "key-half merge scratch exceeds the activation image");
   unsigned char* const stage_base = ring + 2 * kSlotBytes;  // the activation image follows the ring
   // Keys of this CTA: the cache in whole staging chunks, split near-evenly over the
@@ -507,93 +571,101 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   const long long kbeg = cache_lo(rank);                                // first cache key of this CTA
   const int n_cache = static_cast<int>(cache_lo(rank + 1) - kbeg);      // cache keys of this CTA
   const int n_chunks = (n_cache + kStageKeys - 1) / kStageKeys;
-  const int own_lo = 0;                                                 // own keys of this CTA
   const int own_n = rank == own_rank ? T : 0;
   const size_t tok_bytes = static_cast<size_t>(p.H) * kD * sizeof(CT);  // one token row of all heads
   const size_t head_off = (static_cast<size_t>(o_lo + kbeg) * p.H + head) * kD * sizeof(CT);
-  // all threads: 16-byte cp.async copies of chunk j into buffer j % kNB (one commit group)
-  auto stage_issue = [&](int j, const unsigned char* kh, const unsigned char* vh) {
-    const int k0 = j * kStageKeys;
-    const int n = min(kStageKeys, n_cache - k0);
-    unsigned char* kb = stage_base + (j % kNB) * kBufBytes;
-#pragma unroll
-    for (int it = 0; it < kRawIters; ++it) {
-      const int i = tid + it * kThr;
-      const int r = i >> kUnitShift;  // row of [K rows ; V rows]
-      const int u = i & (kUnitsPerRow - 1);
-      const bool is_v = r >= kStageKeys;
-      const int key = is_v ? r - kStageKeys : r;
-      if (r < 2 * kStageKeys && key < n)
-        cp_async_16(smem_addr(kb + r * kRowStride + u * 16),
-                    (is_v ? vh : kh) + static_cast<size_t>(k0 + key) * tok_bytes + u * 16);
-    }
-    cp_async_commit();
+  // Chunk j of layer l is chunk g = l n_chunks + j of this CTA's stream; it uses buffer g mod kNB, as
+  // that buffer's (g / kNB)-th chunk.
+  auto chunk_keys = [&](int j) { return min(kStageKeys, n_cache - j * kStageKeys); };
+  auto stage_buf = [&](int g) { return stage_base + (g % kNB) * kBufBytes; };
+  auto stage_parity = [&](int g) { return static_cast<uint32_t>((g / kNB) & 1); };
+  // bounded wait for phase `parity` of a staging barrier
+  auto swait = [&](uint64_t* bar, uint32_t parity) {
+    if (*abort) return;
+    if (!wait_phase<false>(bar, parity, p.status)) *abort = 1;
   };
-  uint32_t range_seen = 0;  // a cache value outside the fp16 range was saturated
-  // all threads: wait for chunk j and convert it to fp16 in place
-  auto stage_ready = [&](int j) {
-    const int younger = min(n_chunks - 1 - j, kNB - 1);  // groups of later chunks still in flight
-    if (younger >= 2)
-      cp_async_wait<2>();
-    else if (younger == 1)
-      cp_async_wait<1>();
-    else
-      cp_async_wait<0>();
-    // bf16: a thread converts exactly the units it copied (same unit -> thread map), so
-    // its own wait suffices; fp32 units are regrouped and need every thread's copies
-    if (sizeof(CT) != 2) __syncthreads();
-    const int n = min(kStageKeys, n_cache - j * kStageKeys);
-    unsigned char* kb = stage_base + (j % kNB) * kBufBytes;
-    if (sizeof(CT) == 2) {
-      // two rounds of half the units, every load of a round before its first store
-      constexpr int kHalf = (kCvtIters + 1) / 2;
+  // 64 threads (t = 0 .. 63): the copies of chunk j; after a timeout no new copy starts
+  auto stage_issue = [&](int j, int g, int t, int layer, const unsigned char* kh, const unsigned char* vh) {
+    if (*abort) return;
+    const int n = chunk_keys(j);
+    uint64_t* bar = raw_bar + g % kNB;
+    unsigned char* kb = stage_buf(g);
+    if (kSw && p.cache_maps != nullptr && n == kStageKeys) {
+      if (t == 0) {
+        const CUtensorMap* maps = p.cache_maps + 2 * layer;
+        const int row = static_cast<int>(o_lo + kbeg) + j * kStageKeys;
+        // the buffer's last generic accesses (the barriers before this call) come before the async writes
+        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+        mbar_arrive_expect_tx(bar, kBufBytes);
 #pragma unroll
-      for (int r0 = 0; r0 < kCvtIters; r0 += kHalf) {
-        uint4 v[kHalf];
+        for (int e = 0; e < 4; ++e) tma_load_cache(kb + e * kBlockBytes, maps + (e >> 1), (e & 1) * 64, head, row, bar);
+      } else {
+        mbar_arrive(bar);
+      }
+      return;
+    }
+    constexpr int kUnits = kD * static_cast<int>(sizeof(CT)) / 16;  // raw 16-byte units of a row: 16 / 32
+    for (int i = t; i < 2 * n * kUnits; i += 64) {
+      const int r = i / kUnits, u = i % kUnits;
+      const bool is_v = r >= n;
+      const int key = is_v ? r - n : r;
+      const unsigned char* src = (is_v ? vh : kh) + static_cast<size_t>(j * kStageKeys + key) * tok_bytes + u * 16;
+      unsigned char* dst = kSw ? kb + ((is_v ? 2 : 0) + (u >> 3)) * kBlockBytes + key * 128 + (((u & 7) ^ (key & 7)) << 4)
+                               : kb + ((is_v ? kStageKeys : 0) + key) * kRowStride + u * 16;
+      cp_async_16(smem_addr(dst), src);
+    }
+    // this thread's arrival, once its copies have landed
+    asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
+  };
+  uint32_t range_seen = 0;  // largest magnitudes of this thread's converted cache values
+  // warp wi of nw: its share of chunk j's raw rows -> fp16 in place
+  auto convert = [&](int j, int g, int wi, int nw) {
+    const int n = chunk_keys(j);
+    unsigned char* kb = stage_buf(g);
+    if (kSw) {  // 16-byte units as they lie, 512 contiguous bytes a step: unit i is of key (i / 8) mod 64
+      constexpr int kBatch = 4;  // loads in flight
+#pragma unroll 1
+      for (int i0 = wi * 32 + lane; i0 < kBufBytes / 16; i0 += nw * 32 * kBatch) {
+        uint4 v[kBatch];
 #pragma unroll
-        for (int it = 0; it < kHalf; ++it) {
-          const int i = tid + (r0 + it) * kThr;
-          const int r = i >> 4;
-          const int key = r >= kStageKeys ? r - kStageKeys : r;
-          if (r0 + it < kCvtIters && r < 2 * kStageKeys && key < n)
-            v[it] = *reinterpret_cast<const uint4*>(kb + r * kRowStride + (i & 15) * 16);
-        }
+        for (int e = 0; e < kBatch; ++e) v[e] = *reinterpret_cast<const uint4*>(kb + (i0 + e * nw * 32) * 16);
 #pragma unroll
-        for (int it = 0; it < kHalf; ++it) {
-          const int i = tid + (r0 + it) * kThr;
-          const int r = i >> 4;
-          const int key = r >= kStageKeys ? r - kStageKeys : r;
-          if (r0 + it < kCvtIters && r < 2 * kStageKeys && key < n)
-            *reinterpret_cast<uint4*>(kb + r * kRowStride + (i & 15) * 16) =
-                make_uint4(bf16x2_to_half2_sat(v[it].x, range_seen), bf16x2_to_half2_sat(v[it].y, range_seen),
-                           bf16x2_to_half2_sat(v[it].z, range_seen), bf16x2_to_half2_sat(v[it].w, range_seen));
+        for (int e = 0; e < kBatch; ++e) {
+          const int i = i0 + e * nw * 32;
+          uint32_t range = 0;
+          *reinterpret_cast<uint4*>(kb + i * 16) =
+              make_uint4(bf16x2_to_half2_peak(v[e].x, range), bf16x2_to_half2_peak(v[e].y, range),
+                         bf16x2_to_half2_peak(v[e].z, range), bf16x2_to_half2_peak(v[e].w, range));
+          range_seen = peak_of(range_seen, ((i >> 3) & 63) < n ? range : 0u);  // rows past the range hold no cache value
         }
       }
     } else {
-      // 32-byte fp32 unit u of a row -> 16-byte fp16 unit u at the row start. A row's 16
-      // units fall in one round of 256, all reads of a round land before its writes, and
-      // a unit's input is never written by a later round.
+      // two rows a step, fp16 unit `lane mod 16` of each; a step's units are all read before the first is written
+      constexpr int kBatch = 2;
+      const int u = lane & 15;
 #pragma unroll 1
-      for (int it = 0; it < kCvtIters; ++it) {
-        const int i = tid + it * kThr;
-        const int r = i >> 4;
-        const int key = r >= kStageKeys ? r - kStageKeys : r;
-        const bool live = r < 2 * kStageKeys && key < n;
-        unsigned char* row = kb + r * kRowStride;
-        const int u = i & 15;
-        uint4 o = make_uint4(0u, 0u, 0u, 0u);
-        if (live) {
-          const float4 a = *reinterpret_cast<const float4*>(row + u * 32);
-          const float4 b = *reinterpret_cast<const float4*>(row + u * 32 + 16);
-          o = make_uint4(f32x2_to_half2_sat(a.x, a.y, range_seen), f32x2_to_half2_sat(a.z, a.w, range_seen),
-                         f32x2_to_half2_sat(b.x, b.y, range_seen), f32x2_to_half2_sat(b.z, b.w, range_seen));
+      for (int r0 = 2 * wi + (lane >> 4); r0 < 2 * kStageKeys + (lane >> 4); r0 += 2 * nw * kBatch) {
+        uint4 v[kBatch];
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) {
+          const int r = r0 + 2 * nw * e;
+          v[e] = make_uint4(0u, 0u, 0u, 0u);
+          if (r < 2 * kStageKeys && (r >= kStageKeys ? r - kStageKeys : r) < n) {
+            const float4 a = *reinterpret_cast<const float4*>(kb + r * kRowStride + u * 32);
+            const float4 b = *reinterpret_cast<const float4*>(kb + r * kRowStride + u * 32 + 16);
+            v[e] = make_uint4(f32x2_to_half2_peak(a.x, a.y, range_seen), f32x2_to_half2_peak(a.z, a.w, range_seen),
+                              f32x2_to_half2_peak(b.x, b.y, range_seen), f32x2_to_half2_peak(b.z, b.w, range_seen));
+          }
         }
-        __syncthreads();
-        if (live) *reinterpret_cast<uint4*>(row + u * 16) = o;
-        __syncthreads();
+        __syncwarp();
+#pragma unroll
+        for (int e = 0; e < kBatch; ++e) {
+          const int r = r0 + 2 * nw * e;
+          if (r < 2 * kStageKeys && (r >= kStageKeys ? r - kStageKeys : r) < n)
+            *reinterpret_cast<uint4*>(kb + r * kRowStride + u * 16) = v[e];
+        }
       }
     }
-    __syncthreads();
   };
 
   // ---- arm the exchange barriers for layer 0, then publish the token assembly
@@ -635,6 +707,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       float4 xv[3][2];
       load_x(Xc, rank * 128, xv);
       // zero the buffer phase B accumulates into (while the loads are in flight)
+#pragma unroll 1
       for (int e = zA0 + tid; e < zA1; e += kThr) __stcg(Xz + e, 0.f);
       // this rank's 128 columns of x -> fp16 image here and in the partners (K slices
       // 2 rank, 2 rank + 1), partial sums of x^2 to every rank
@@ -670,40 +743,39 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     compute_rstd();
     __syncthreads();
     wait_mma();
-    for (int j = 0; j < kNB && j < n_chunks; ++j)  // slots 2-5 and the activation image are free
-      stage_issue(j, kc, vc);
+    // slots 2-5 and the activation image are free: the warps without QKV rows start the cache copies
+    const int g0 = layer * n_chunks;
+    if ((warp & 3) == 3) {
+#pragma unroll 1
+      for (int j = 0; j < kNB && j < n_chunks; ++j) stage_issue(j, g0 + j, (warp >> 2) * 32 + lane, layer, kc, vc);
+    }
     // rows 32j..32j+31 of the accumulators are q, k, v dims 32 rank .. 32 rank + 31,
     // scaled by 1 / rms of their token
     if ((warp & 3) < 3) {
       const int kind = warp & 3;
       __half* b = kind == 0 ? qbuf : (kind == 1 ? ownk : ownv);
       const int dim = rank * 32 + lane;
-      const uint32_t taddr = tmem + (static_cast<uint32_t>(kind * 32) << 16);
-      const int c_lo = warp < 4 ? 0 : 32;
-      const int c_hi = warp < 4 ? 32 : 48;
-      if (warp < 4) {
-        float v[32];
-        tmem_ld_sum4<32>(taddr, v);
+      // q: padded rows; own k and v: swizzled blocks of 64 dims like the staged cache rows
+      auto at = [&](int row, int dm) {
+        return kind == 0 ? b + row * kQS + dm
+                         : b + (dm >> 6) * (kActAtom / 2) + row * 64 + ((((dm & 63) >> 3) ^ (row & 7)) << 3) + (dm & 7);
+      };
+      const int c_lo = (warp >> 2) * kHalfTok, c_hi = c_lo + kHalfTok;
+      float v[kHalfTok];
+      tmem_ld_sum4(tmem + (static_cast<uint32_t>(kind * 32) << 16) + static_cast<uint32_t>(c_lo), v);
 #pragma unroll
-        for (int j = 0; j < 32; ++j) b[j * kQS + dim] = __float2half_rn(v[j] * rstd[j]);
-      } else {
-        float v[16];
-        tmem_ld_sum4<16>(taddr + 32u, v);
-#pragma unroll
-        for (int j = 0; j < 16; ++j) b[(32 + j) * kQS + dim] = __float2half_rn(v[j] * rstd[32 + j]);
-      }
+      for (int j = 0; j < kHalfTok; ++j) *at(c_lo + j, dim) = __float2half_rn(v[j] * rstd[c_lo + j]);
       __syncwarp();
       // this warp's token rows below T (dims 32 rank .. + 31, four 16-byte units a row): q to
       // every partner, own k and v to the rank that attends over the own keys
       if (*abort == 0 && (kind == 0 || own_rank != rank)) {
         for (int i = lane; i < (min(c_hi, T) - c_lo) * 4; i += 32) {
-          const __half* src = b + (c_lo + (i >> 2)) * kQS + rank * 32 + (i & 3) * 8;
+          const __half* src = at(c_lo + (i >> 2), rank * 32 + (i & 3) * 8);
           const uint4 v = *reinterpret_cast<const uint4*>(src);
           if (kind == 0) {
 #pragma unroll
             for (int pi = 1; pi < kCl; ++pi) {
-              const int peer = (rank + pi) & (kCl - 1);
-              st_async_v4(cluster_addr(src, peer), v, cluster_addr(qbar, peer));
+              st_async_v4(peer_at(src, pdelta[pi - 1]), v, peer_at(qbar, pdelta[pi - 1]));
             }
           } else {
             st_async_v4(cluster_addr(src, own_rank), v, cluster_addr(qbar, own_rank));
@@ -714,6 +786,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     tc_fence_before();
     __syncthreads();
     if (tid == 0)  // slots 0, 1 are free: W_o of this layer (slots 2-5 stage the cache)
+#pragma unroll 1
       for (int i = kSlots; i < kPersistAChunks; ++i) issue(q0 + i);
     xwait(qbar, par);  // q (and on the own-key rank, own k / v) of every partner
     if (tid == 0 && *abort == 0) arm(qbar, FSX_Q_BYTES);
@@ -732,107 +805,159 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
 #pragma unroll
       for (int e = 0; e < 4; ++e) o_acc[nb][e] = 0.f;
     uint32_t qf[8][4];
-    if (warp < 6) {
+    if (warp < kAttendWarps) {
 #pragma unroll
       for (int kk = 0; kk < 8; ++kk) {
         const __half* src = qbuf + static_cast<size_t>(qt * 16 + (lane & 15)) * kQS + kk * 16 + (lane >> 4) * 8;
         ldsm_x4(qf[kk][0], qf[kk][1], qf[kk][2], qf[kk][3], smem_addr(src));
       }
     }
-    // this warp's key tiles of keys 0..n-1, K rows at kb and V rows at vb (fp16, `stride` bytes apart)
-    auto attend = [&](const unsigned char* kb, const unsigned char* vb, int stride, int n) {
+    // this warp's key tiles of keys 0..n-1, K rows at kb and V rows at vb (fp16, `stride` bytes
+    // apart). The four 8-key columns of S run as independent MMA chains; the running maximum
+    // moves only when a tile's exceeds it by more than 8 (log2 units; P <= 2^8 stays well inside
+    // fp16), so the accumulators are rarely rescaled.
+    // Swizzled rows (`sw`): blocks of 64 dims `stride` bytes apart, 128-byte rows; else rows `stride`
+    // bytes apart.
+    const uint32_t kx[2] = {static_cast<uint32_t>(((lane >> 3) ^ (lane & 7)) << 4),
+                            static_cast<uint32_t>(((4 + (lane >> 3)) ^ (lane & 7)) << 4)};
+    const uint32_t vx[4] = {static_cast<uint32_t>(((lane >> 4) ^ (lane & 7)) << 4),
+                            static_cast<uint32_t>(((2 + (lane >> 4)) ^ (lane & 7)) << 4),
+                            static_cast<uint32_t>(((4 + (lane >> 4)) ^ (lane & 7)) << 4),
+                            static_cast<uint32_t>(((6 + (lane >> 4)) ^ (lane & 7)) << 4)};
+    auto attend = [&](auto sw, uint32_t kb, uint32_t vb, uint32_t stride, int n) {
+      constexpr bool kSwizzled = decltype(sw)::value;
       for (int t0 = kh * kKeyTile; t0 < n; t0 += 2 * kKeyTile) {
         const int rows = min(kKeyTile, n - t0);
         float sc[4][4];
+        uint32_t krow[4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
 #pragma unroll
           for (int e = 0; e < 4; ++e) sc[j][e] = 0.f;
           int r = t0 + j * 8 + (lane & 7);
           r = r < n ? r : 0;  // masked below; any valid row keeps the products finite
-          const uint32_t krow = smem_addr(kb + r * stride);
+          krow[j] = kSwizzled ? kb + r * 128 : kb + r * stride + (lane >> 3) * 16;
+        }
 #pragma unroll
-          for (int dd = 0; dd < 4; ++dd) {
-            uint32_t b0, b1, b2, b3;
-            ldsm_x4(b0, b1, b2, b3, krow + (dd * 4 + (lane >> 3)) * 16);
-            mma_f16_16816(sc[j], qf[2 * dd][0], qf[2 * dd][1], qf[2 * dd][2], qf[2 * dd][3], b0, b1);
-            mma_f16_16816(sc[j], qf[2 * dd + 1][0], qf[2 * dd + 1][1], qf[2 * dd + 1][2], qf[2 * dd + 1][3], b2, b3);
+        for (int dd = 0; dd < 4; ++dd) {
+          uint32_t b[4][4];
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            ldsm_x4(b[j][0], b[j][1], b[j][2], b[j][3],
+                    kSwizzled ? krow[j] + (dd >> 1) * stride + kx[dd & 1] : krow[j] + dd * 64);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            mma_f16_16816(sc[j], qf[2 * dd][0], qf[2 * dd][1], qf[2 * dd][2], qf[2 * dd][3], b[j][0], b[j][1]);
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            mma_f16_16816(sc[j], qf[2 * dd + 1][0], qf[2 * dd + 1][1], qf[2 * dd + 1][2], qf[2 * dd + 1][3], b[j][2], b[j][3]);
+        }
+        if (rows < kKeyTile) {
+#pragma unroll
+          for (int j = 0; j < 4; ++j) {
+            const int key = j * 8 + 2 * (lane & 3);
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+              if (key + (e & 1) >= rows) sc[j][e] = -CUDART_INF_F;
           }
         }
         float mx[2] = {-CUDART_INF_F, -CUDART_INF_F};
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const int key = j * 8 + 2 * (lane & 3);
-#pragma unroll
-          for (int e = 0; e < 4; ++e) sc[j][e] = (key + (e & 1)) < rows ? sc[j][e] * scale_log2 : -CUDART_INF_F;
           mx[0] = fmaxf(mx[0], fmaxf(sc[j][0], sc[j][1]));
           mx[1] = fmaxf(mx[1], fmaxf(sc[j][2], sc[j][3]));
         }
-        float alpha[2], m_new[2], rs[2] = {0.f, 0.f};
 #pragma unroll
         for (int r = 0; r < 2; ++r) {
           mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 1));
           mx[r] = fmaxf(mx[r], __shfl_xor_sync(0xffffffffu, mx[r], 2));
-          m_new[r] = fmaxf(m_run[r], mx[r]);
-          alpha[r] = exp2f(m_run[r] - m_new[r]);
-          m_run[r] = m_new[r];
+          mx[r] *= scale_log2;
         }
+        if (__any_sync(0xffffffffu, mx[0] > m_run[0] + kLazyRescale || mx[1] > m_run[1] + kLazyRescale)) {
+          float alpha[2];
+#pragma unroll
+          for (int r = 0; r < 2; ++r) {
+            const float m_new = fmaxf(m_run[r], mx[r]);
+            alpha[r] = exp2f(m_run[r] - m_new);
+            m_run[r] = m_new;
+            l_run[r] *= alpha[r];
+          }
+#pragma unroll
+          for (int nb = 0; nb < 16; ++nb) {
+            o_acc[nb][0] *= alpha[0];
+            o_acc[nb][1] *= alpha[0];
+            o_acc[nb][2] *= alpha[1];
+            o_acc[nb][3] *= alpha[1];
+          }
+        }
+        float rs[2] = {0.f, 0.f};
         uint32_t pf[2][4];
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-          const float p0 = exp2f(sc[j][0] - m_new[0]);
-          const float p1 = exp2f(sc[j][1] - m_new[0]);
-          const float p2 = exp2f(sc[j][2] - m_new[1]);
-          const float p3 = exp2f(sc[j][3] - m_new[1]);
+          const float p0 = ex2_approx(fmaf(sc[j][0], scale_log2, -m_run[0]));
+          const float p1 = ex2_approx(fmaf(sc[j][1], scale_log2, -m_run[0]));
+          const float p2 = ex2_approx(fmaf(sc[j][2], scale_log2, -m_run[1]));
+          const float p3 = ex2_approx(fmaf(sc[j][3], scale_log2, -m_run[1]));
           rs[0] += p0 + p1;
           rs[1] += p2 + p3;
           pf[j >> 1][(j & 1) * 2 + 0] = pack_half2(p0, p1);
           pf[j >> 1][(j & 1) * 2 + 1] = pack_half2(p2, p3);
         }
-#pragma unroll
-        for (int r = 0; r < 2; ++r) {
-          rs[r] += __shfl_xor_sync(0xffffffffu, rs[r], 1);
-          rs[r] += __shfl_xor_sync(0xffffffffu, rs[r], 2);
-          l_run[r] = l_run[r] * alpha[r] + rs[r];
-        }
-#pragma unroll
-        for (int nb = 0; nb < 16; ++nb) {
-          o_acc[nb][0] *= alpha[0];
-          o_acc[nb][1] *= alpha[0];
-          o_acc[nb][2] *= alpha[1];
-          o_acc[nb][3] *= alpha[1];
-        }
+        l_run[0] += rs[0];  // this thread's keys; the quad's sums are added after the last tile
+        l_run[1] += rs[1];
 #pragma unroll
         for (int kk = 0; kk < 2; ++kk) {
           int r = t0 + kk * 16 + (lane & 7) + 8 * ((lane >> 3) & 1);
           r = r < n ? r : 0;
-          const uint32_t vrow = smem_addr(vb + r * stride);
+          const uint32_t vrow = kSwizzled ? vb + r * 128 : vb + r * stride + (lane >> 4) * 16;
 #pragma unroll
           for (int np = 0; np < 8; ++np) {
             uint32_t b0, b1, b2, b3;
-            ldsm_x4_trans(b0, b1, b2, b3, vrow + (np * 2 + (lane >> 4)) * 16);
+            ldsm_x4_trans(b0, b1, b2, b3, kSwizzled ? vrow + (np >> 2) * stride + vx[np & 3] : vrow + np * 32);
             mma_f16_16816(o_acc[2 * np], pf[kk][0], pf[kk][1], pf[kk][2], pf[kk][3], b0, b1);
             mma_f16_16816(o_acc[2 * np + 1], pf[kk][0], pf[kk][1], pf[kk][2], pf[kk][3], b2, b3);
           }
         }
       }
     };
-    for (int j = 0; j < n_chunks; ++j) {
-      stage_ready(j);
-      if (warp < 6) {
-        const unsigned char* kb = stage_base + (j % kNB) * kBufBytes;
-        attend(kb, kb + kStageKeys * kRowStride, kRowStride, min(kStageKeys, n_cache - j * kStageKeys));
+    // one loop for both roles, with the own keys as the attending warps' last turn (one copy of
+    // either body: the layer loop has to stay in the instruction cache)
+#pragma unroll 1
+    for (int j = 0; j < n_chunks + (own_n > 0 ? 1 : 0); ++j) {
+      const int g = g0 + j;
+      const bool own = j == n_chunks;
+      if (!own && (j == 0 || warp >= kAttendWarps)) {  // the layer's first chunk by all warps
+        swait(raw_bar + g % kNB, stage_parity(g));
+        convert(j, g, j == 0 ? warp : warp - kAttendWarps, j == 0 ? kThr / 32 : kCvtWarps);
       }
-      __syncthreads();  // buffer j % kNB consumed
-      if (j + kNB < n_chunks) stage_issue(j + kNB, kc, vc);
+      if (j == 0) __syncthreads();
+      if (warp < kAttendWarps) {
+        if (!own && j > 0) swait(cvt_bar + g % kNB, stage_parity(g));
+        if (kSw || !own) {
+          const uint32_t kb = smem_addr(own ? reinterpret_cast<unsigned char*>(ownk) : stage_buf(g));
+          const uint32_t vb = own ? smem_addr(ownv) : kb + (kSw ? 2 * kBlockBytes : kStageKeys * kRowStride);
+          attend(std::integral_constant<bool, kSw>{}, kb, vb, own ? kActAtom : (kSw ? kBlockBytes : kRowStride),
+                 own ? own_n : chunk_keys(j));
+        } else {
+          attend(std::true_type{}, smem_addr(ownk), smem_addr(ownv), kActAtom, own_n);
+        }
+        __syncwarp();
+        if (!own && lane == 0) mbar_arrive(free_bar + g % kNB);
+      } else if (!own) {
+        mbar_arrive(cvt_bar + g % kNB);  // the first chunk's too: every chunk is a phase of its buffer's barrier
+        const int jr = j - 1 + kNB;      // into the buffer of chunk j - 1
+        if (j > 0 && jr < n_chunks) {
+          swait(free_bar + (g - 1) % kNB, stage_parity(g - 1));
+          stage_issue(jr, g0 + jr, (warp - kAttendWarps) * 32 + lane, layer, kc, vc);
+        }
+      }
     }
-    if (tid == 0) {  // every staged row has landed and been read: gate/up, W_d into slots 2-5
+    __syncthreads();  // every staged row has landed and been read
+    if (tid == 0) {   // gate/up, W_d into slots 2-5
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+#pragma unroll 1
       for (int i = kPersistAChunks; i < kLayerChunks; ++i) issue(q0 + i);
     }
-    if (warp < 6 && own_n > 0)
-      attend(reinterpret_cast<const unsigned char*>(ownk + static_cast<size_t>(own_lo) * kQS),
-             reinterpret_cast<const unsigned char*>(ownv + static_cast<size_t>(own_lo) * kQS), kQS * 2, own_n);
 
     // --- merge the two key halves of each query tile: warp (qt, kh) keeps value dims
     // 64 kh .. 64 kh + 63. It hands the other 64 dims of its accumulator and its running
@@ -842,7 +967,12 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     {
       float4* xo = reinterpret_cast<float4*>(act);   // [3 qt][2 kh][8][32 lanes]
       float4* xml = xo + 3 * 2 * 8 * 32;              // [3 qt][2 kh][32 lanes]: m0, m1, l0, l1
-      if (warp < 6) {
+      if (warp < kAttendWarps) {
+#pragma unroll
+        for (int r = 0; r < 2; ++r) {
+          l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 1);
+          l_run[r] += __shfl_xor_sync(0xffffffffu, l_run[r], 2);
+        }
 #pragma unroll
         for (int nb = 0; nb < 8; ++nb) {
           const float* src = kh == 0 ? o_acc[8 + nb] : o_acc[nb];
@@ -851,7 +981,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         xml[(qt * 2 + kh) * 32 + lane] = make_float4(m_run[0], m_run[1], l_run[0], l_run[1]);
       }
       __syncthreads();
-      if (warp < 6) {
+      if (warp < kAttendWarps) {
         const int pk = 1 - kh;
         const float4 pml = xml[(qt * 2 + pk) * 32 + lane];
         const float pm[2] = {pml.x, pml.y};
@@ -879,7 +1009,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
 
     // --- merge the 4 splits: every row's normalised fp32 partial and log-sum-exp go
     // straight from the registers to the rank that owns the row (st.async to the partners)
-    if (warp < 6 && *abort == 0) {
+    if (warp < kAttendWarps && *abort == 0) {
       auto put4 = [&](float* ptr, int dst, float a, float b, float c, float e) {
         if (dst == rank)
           *reinterpret_cast<float4*>(ptr) = make_float4(a, b, c, e);
@@ -959,8 +1089,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         if (*abort == 0) {
 #pragma unroll
           for (int pi = 1; pi < kCl; ++pi) {
-            const int peer = (rank + pi) & (kCl - 1);
-            st_async_v2(cluster_addr(dst, peer), out.x, out.y, cluster_addr(agbar, peer));
+            st_async_v2(peer_at(dst, pdelta[pi - 1]), out.x, out.y, peer_at(agbar, pdelta[pi - 1]));
           }
         }
         if (p.attn_capture != nullptr && row < T)
@@ -989,6 +1118,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     tmem_to_dstT();
     if (tid == 0) {  // slots 0, 1 free (all of 0-5 for CTAs without phase B): next layer's QKV
       const int n = in_b ? 2 : kSlots;
+#pragma unroll 1
       for (int i = 0; i < n; ++i) issue(q0 + kLayerChunks + i);
     }
     scatter_add(Xm, rank * 128, res, head == 0);
@@ -1003,6 +1133,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         float4 xv[3][2];
         load_x(Xm, rank * 128, xv);
         // zero the buffer the next phase A accumulates into (this layer's input is consumed)
+#pragma unroll 1
         for (int e = zB0 + tid; e < zB1; e += kThr) __stcg(Xc + e, 0.f);
         // this rank's 128 columns of x -> fp16 K slices 0, 1 here (no exchange: each CTA runs
         // the gate/up MMAs over its own K quarter), partial sums of x^2 to every rank
@@ -1029,29 +1160,24 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         const int q = warp & 3;
         const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16);
         float* dst = recv + (rank * 32 + lane) * kTokTile;
-        auto put = [&](const float* v, int c0, int n) {
-          for (int j = 0; j < n; j += 4) {
-            const uint4 u = make_uint4(__float_as_uint(v[j]), __float_as_uint(v[j + 1]), __float_as_uint(v[j + 2]),
-                                       __float_as_uint(v[j + 3]));
-            if (q == rank)
-              *reinterpret_cast<uint4*>(dst + c0 + j) = u;
-            else if (*abort == 0)
-              st_async_v4(cluster_addr(dst + c0 + j, q), u, cluster_addr(bbar, q));
-          }
-        };
-        if (warp < 4) {
-          float v[32];
-          tmem_ld_sum4<32>(taddr, v);
-          put(v, 0, 32);
-        } else {
-          float v[16];
-          tmem_ld_sum4<16>(taddr + 32u, v);
-          put(v, 32, 16);
+        const int c0 = (warp >> 2) * kHalfTok;
+        float v[kHalfTok];
+        tmem_ld_sum4(taddr + static_cast<uint32_t>(c0), v);
+        const uint32_t peer = cluster_addr(dst + c0, q), peer_bar = cluster_addr(bbar, q);
+#pragma unroll
+        for (int j = 0; j < kHalfTok; j += 4) {
+          const uint4 u = make_uint4(__float_as_uint(v[j]), __float_as_uint(v[j + 1]), __float_as_uint(v[j + 2]),
+                                     __float_as_uint(v[j + 3]));
+          if (q == rank)
+            *reinterpret_cast<uint4*>(dst + c0 + j) = u;
+          else if (*abort == 0)
+            st_async_v4(peer + j * 4, u, peer_bar);
         }
       }
       tc_fence_before();
       __syncthreads();
       if (tid == 0)  // slots 2, 3 free: next layer's QKV
+#pragma unroll 1
         for (int i = 2; i < 4; ++i) issue(q0 + kLayerChunks + i);
       xwait(bbar, par);  // every partner's partial sums of x^2 and gate/up partials
       if (tid == 0 && *abort == 0) arm(bbar, FSX_B_BYTES);
@@ -1089,8 +1215,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         if (t < T && *abort == 0) {
 #pragma unroll
           for (int pi = 1; pi < kCl; ++pi) {
-            const int peer = (rank + pi) & (kCl - 1);
-            st_async_v4(cluster_addr(dst, peer), hv4, cluster_addr(hbar, peer));
+            st_async_v4(peer_at(dst, pdelta[pi - 1]), hv4, peer_at(hbar, pdelta[pi - 1]));
           }
         }
       }
@@ -1112,6 +1237,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       wait_mma();
       tmem_to_dstT();
       if (tid == 0)  // slots 4, 5 free: next layer's QKV
+#pragma unroll 1
         for (int i = 4; i < kSlots; ++i) issue(q0 + kLayerChunks + i);
       float* Xn = X0 + static_cast<size_t>((sA + 2) % 3) * xs;
       scatter_add(Xn, rank * 128, resb, c == 0);
@@ -1120,29 +1246,22 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   }
 
   // ---- leave nothing in flight. Every path reaches this point, a timed-out tick included
-  // (its waits on other CTAs return at once). In order: this thread's cache-row copies;
-  // the ring copies issued (a timed-out tick stops issuing, and may have skipped the waits
-  // of the last ones: wait, bounded, for the last position of every slot); the MMAs of the
+  // (its waits on other CTAs return at once). In order: the cache-row and weight copies (all waited
+  // for in the normal course; a timed-out tick stops issuing, may have skipped the waits of the last
+  // ones, and gives them 1 ms: they land within microseconds); the MMAs of the
   // four issuing threads (a last commit each on drain_bar); the partners' stores into this
   // CTA's shared memory (the cluster barrier below); then the tensor memory is freed.
   cp_async_wait<0>();
-  if (tid == 0)
-    for (int q = issued_upto - kSlots; q < issued_upto; ++q)
-      if (q >= 0 && !is_empty(q)) {
-        const unsigned long long t0 = global_timer_ns();
-        uint32_t done = 0;
-        while (!done && global_timer_ns() - t0 < 100000000ull)
-          asm volatile(
-              "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-              : "=r"(done)
-              : "r"(smem_addr(full + q % kSlots)), "r"(static_cast<uint32_t>((q / kSlots) & 1))
-              : "memory");
-      }
+  if (*abort) {
+    const unsigned long long t0 = global_timer_ns();
+    while (global_timer_ns() - t0 < 1000000ull) {
+    }
+  }
   if (warp < kNAcc) {
     if (lane == 0) umma_commit(drain_bar);
     __syncwarp();
   }
-  mbar_wait(drain_bar, 0u, p.status);
+  wait_phase<false>(drain_bar, 0u, p.status);
   tc_fence_after();
   // no CTA leaves while a partner may still write into its shared memory
   cluster.sync();
