@@ -88,6 +88,7 @@ constexpr uint32_t kIdesc = idesc_f16(128, kTokTile);
 constexpr int kRecvBytes = kRowsPerRank * kD * 4;  // merge partials one CTA sends another (fp32)
 constexpr int kRsBytes = 32 * kTokTile * 4;        // gate/up partials one CTA sends another (fp32)
 constexpr int kNB = 3;                             // cache-row staging buffers
+constexpr int kIssuer = kThr - 32;                 // thread that issues the weight copies: in a warp without attention rows
 constexpr int kAttendWarps = 6;                    // warps 0-5 attend, warps 6 and 7 convert the next chunk
 constexpr int kCvtWarps = kThr / 32 - kAttendWarps;
 static_assert(kRecvBytes == kRsBytes, "the merge and the gate/up reduce-scatter share the receive buffer");
@@ -321,6 +322,8 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     const int i = q % kLayerChunks;
     return i >= kPersistAChunks + (in_b ? kPersistBChunks : 0);
   };
+  // Issued off the critical steps: four of these calls on the thread that everyone then meets at a
+  // barrier cost 0.4 us, and before the last additions of a phase they held up every later CTA.
   auto issue = [&](int q) {  // one thread; an empty position just completes the slot's phase
     if (q >= total_chunks || *abort) return;  // after a timeout no new copy starts
     uint64_t* bar = full + (q % kSlots);
@@ -785,7 +788,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     }
     tc_fence_before();
     __syncthreads();
-    if (tid == 0)  // slots 0, 1 are free: W_o of this layer (slots 2-5 stage the cache)
+    if (tid == kIssuer)  // slots 0, 1 are free: W_o of this layer (slots 2-5 stage the cache)
 #pragma unroll 1
       for (int i = kSlots; i < kPersistAChunks; ++i) issue(q0 + i);
     xwait(qbar, par);  // q (and on the own-key rank, own k / v) of every partner
@@ -953,7 +956,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       }
     }
     __syncthreads();  // every staged row has landed and been read
-    if (tid == 0) {   // gate/up, W_d into slots 2-5
+    if (tid == kIssuer) {  // gate/up, W_d into slots 2-5
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
 #pragma unroll 1
       for (int i = kPersistAChunks; i < kLayerChunks; ++i) issue(q0 + i);
@@ -1116,14 +1119,14 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     if (head == 0) load_residual(Xc, rank * 128, res);  // cluster 0 adds the residual itself
     wait_mma();
     tmem_to_dstT();
-    if (tid == 0) {  // slots 0, 1 free (all of 0-5 for CTAs without phase B): next layer's QKV
+    scatter_add(Xm, rank * 128, res, head == 0);
+    flag_range(p.status, range_seen);  // every thread's own units; published by the arrival
+    arrive(p.counters + sA + 1);
+    if (tid == kIssuer) {  // slots 0, 1 free (all of 0-5 for CTAs without phase B): next layer's QKV
       const int n = in_b ? 2 : kSlots;
 #pragma unroll 1
       for (int i = 0; i < n; ++i) issue(q0 + kLayerChunks + i);
     }
-    scatter_add(Xm, rank * 128, res, head == 0);
-    flag_range(p.status, range_seen);  // every thread's own units; published by the arrival
-    arrive(p.counters + sA + 1);
 
     // =========================== phase B ===========================
     if (in_b) {
@@ -1176,13 +1179,13 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       }
       tc_fence_before();
       __syncthreads();
-      if (tid == 0)  // slots 2, 3 free: next layer's QKV
-#pragma unroll 1
-        for (int i = 2; i < 4; ++i) issue(q0 + kLayerChunks + i);
       xwait(bbar, par);  // every partner's partial sums of x^2 and gate/up partials
       if (tid == 0 && *abort == 0) arm(bbar, FSX_B_BYTES);
       compute_rstd();
       __syncthreads();
+      if (tid == kIssuer)  // slots 2, 3 free: next layer's QKV
+#pragma unroll 1
+        for (int i = 2; i < 4; ++i) issue(q0 + kLayerChunks + i);
       // h = silu(gate) * up for this rank's 16 SwiGLU columns: K partials summed in rank
       // order and scaled by 1 / rms; 8 columns a thread -> the swizzled slice here and in
       // every partner
@@ -1236,12 +1239,12 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       if (c == 0) load_residual(Xm, rank * 128, resb);  // cluster 0 adds the residual itself
       wait_mma();
       tmem_to_dstT();
-      if (tid == 0)  // slots 4, 5 free: next layer's QKV
-#pragma unroll 1
-        for (int i = 4; i < kSlots; ++i) issue(q0 + kLayerChunks + i);
       float* Xn = X0 + static_cast<size_t>((sA + 2) % 3) * xs;
       scatter_add(Xn, rank * 128, resb, c == 0);
       arrive(p.counters + sA + 2);
+      if (tid == kIssuer)  // slots 4, 5 free: next layer's QKV
+#pragma unroll 1
+        for (int i = 4; i < kSlots; ++i) issue(q0 + kLayerChunks + i);
     }
   }
 
