@@ -120,23 +120,24 @@ __global__ void __launch_bounds__(128) append_embed_kernel(const EmbedArgsA a) {
 // vehicle b, head h, in one launch. The CTA rotates the new queries and keys itself
 // (cos / sin from the embed kernel) and rounds the new keys and values to bf16 in shared
 // memory; rank 0 of the cluster writes them to the cache rows dst[b] + i. The keys are the
-// vehicle's cached rows (positions 0 .. L_b-1) in 16-key units, then one unit of its new
+// vehicle's cached rows (positions 0 .. L_b-1) in 8-key units, then one unit of its new
 // rows; new token i sees every cached row and new rows 0 .. i. Everything is fp32.
 //
 // The keys are few and every row is read once, so the kernel is bound by load latency:
-// a warp works on 16-key units, holds one unit's K and V rows (8 KB) in registers and issues
+// a warp works on 8-key units, holds one unit's K and V rows (4 KB) in registers and issues
 // the next unit's K loads as soon as the scores are formed and its V loads after P V; four
 // CTAs share an SM (16 units in flight), and the units go round robin over the 4 warps of
 // `cluster` CTAs (as many as keep four CTAs per SM for the batch). No key moves through
-// shared memory: in the score step 4 lanes share a key row (full 32-byte sectors), 2 keys per
-// lane, and a transposed reduction over the 4 lanes leaves lane 4 g + 2 t + i with half i of
-// the queries of key 8 t + g. Both products use packed fp32 FMAs. The CTAs of a cluster
-// exchange their (max, sum, output) through distributed shared memory, each merging its share
-// of the n_new x 128 outputs.
-// Measured per layer (ncu, 4 tokens a vehicle): one vehicle with 224 rows 8.9 us a launch, 16
-// vehicles with 96-480 rows 31 us; the separate rotary (fp64 pow and sincos per pair and layer)
-// and attention (a lane per key) launches before took 55 and 130 us, and 32-key units with two
-// CTAs per SM 12.3 and 41 us.
+// shared memory: 16 lanes share a row in both products (two whole rows an instruction), the
+// queries stay in registers, and a transposed reduction over the 16 lanes leaves lane
+// 16 h + 4 k + i of the warp with the scores of key 2 k + h for quarter i of the queries. Both
+// products use packed fp32 FMAs. The CTAs of a cluster exchange their (max, sum, output) through
+// distributed shared memory, each merging its share of the n_new x 128 outputs.
+// Measured: from the end of QKV to the last output 7.4 us for one vehicle with 224 rows, about 30 us for
+// 16 vehicles with 96-480 rows (issue-bound: 420 instructions per 8 keys); two-layer appends 210 -> 204
+// and 322 -> 302 us a call against 16-key units with 4 lanes a row and the queries in shared memory. The
+// separate rotary (fp64 pow and sincos per pair and layer) and attention (a lane per key) launches that
+// this kernel replaced took 55 and 130 us.
 struct AttnArgsA {
   const __half* qkv;   // [M, 3 HD]: q | k | v before the rotation
   int ld;
@@ -153,7 +154,7 @@ struct AttnArgsA {
 
 constexpr int kNewStride = kHeadDim + 8;  // bf16 row stride of the new keys / values in shared memory
 constexpr int kMaxSplit = 8;              // CTAs of a cluster
-constexpr int kUnit = 16;                 // keys of a warp's unit of work
+constexpr int kUnit = 8;                  // keys of a warp's unit of work
 static_assert(kMaxNew <= kUnit, "the new rows are one unit");
 
 // d += a * b on two packed fp32 values
@@ -178,12 +179,11 @@ __device__ __forceinline__ float2 unpack2(uint64_t v) {
 __device__ __forceinline__ uint64_t bf16x2_to_f32x2(uint32_t v) {
   return pack2(__uint_as_float(v << 16), __uint_as_float(v & 0xffff0000u));
 }
-// 16 bytes of shared memory, read where it stands: hoisted out of the loop over the units, the
-// query values would take 32 registers per query
-__device__ __forceinline__ ulonglong2 ld_shared2(uint32_t addr) {
-  ulonglong2 v;
-  asm volatile("ld.shared.v2.b64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "r"(addr));
-  return v;
+// 2^x on the special-function unit (relative error about 2^-22, as exp2f; -inf -> +0)
+__device__ __forceinline__ float ex2_approx(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
 }
 __device__ __forceinline__ uint32_t peer_addr(const void* local, int rank) {
   uint32_t r;
@@ -203,7 +203,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
   __shared__ __align__(16) float sm_o[kAttnWarps][NQ][kHeadDim];
   __shared__ float rv_o[NQ * kHeadDim];                       // [split][this rank's share of the outputs]
   __shared__ float rv_m[kMaxSplit][NQ], rv_l[kMaxSplit][NQ];  // every split's running maxima and sums
-  constexpr int NH = NQ / 2;  // queries whose scores a lane keeps
+  constexpr int NH = NQ / 4;  // queries whose scores a lane keeps
   fsx::pdl_launch_dependents();
   fsx::pdl_wait();
   const int S = gridDim.x, rank = blockIdx.x;  // the cluster spans the grid's x extent
@@ -216,34 +216,50 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
   const int L = static_cast<int>(hi - lo);
   const int n_units = (L + kUnit - 1) / kUnit + 1;  // the last one: the new rows
 
-  const int g = lane >> 2, j = lane & 3;    // scores: key within a group of 8, 16-byte unit
-  const int hv = lane >> 4, u = lane & 15;  // values: key parity, 16-byte unit
-  uint4 kraw[2][4], vraw[8];
-  // row loads of unit c (zeros past the vehicle's rows)
+  // this thread's operands of the rotation, requested ahead of the cache rows
+  constexpr int kRot = NQ * kRopePairs / (kAttnWarps * 32);
+  float2 cs[kRot];
+  __half rq[kRot][2], rk[kRot][2], rv[kRot][2];
+#pragma unroll
+  for (int t = 0; t < kRot; ++t) {
+    const int i = (t * kAttnWarps * 32 + tid) / kRopePairs, jj = tid % kRopePairs;
+    if (i < nq) {
+      const int m = b * nq + i;
+      const __half* q = a.qkv + static_cast<size_t>(m) * a.ld + h * kHeadDim + jj;
+      cs[t] = a.rot[static_cast<size_t>(m) * kRopePairs + jj];
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        rq[t][e] = q[e * kRopePairs];
+        rk[t][e] = q[a.HD + e * kRopePairs];
+        rv[t][e] = q[2 * a.HD + e * kRopePairs];
+      }
+    }
+  }
+
+  const int hv = lane >> 4, u = lane & 15;  // key parity, 16-byte unit of a row
+  uint4 kraw[4], vraw[4];
+  // row loads of unit c: lane's key 2 kk + hv, zeros past the vehicle's rows
   auto unit_keys = [&](int c) { return c == n_units - 1 ? nq : min(kUnit, L - kUnit * c); };
-  auto unit_base = [&](int c, const __nv_bfloat16* cache, const __nv_bfloat16* fresh) {
-    return c == n_units - 1 ? fresh : cache + (static_cast<size_t>(lo) + kUnit * static_cast<size_t>(c)) * a.HD + h * kHeadDim;
-  };
-  auto load_k = [&](int c) {
+  const size_t lane_off = static_cast<size_t>(hv) * a.HD + u * 8;  // of this lane's first row and dims, in values
+  const size_t unit0 = static_cast<size_t>(lo) * a.HD + h * kHeadDim + lane_off;
+  const size_t pair = 2 * static_cast<size_t>(a.HD);               // from key 2 kk + hv to key 2 kk + 2 + hv
+  auto load_rows = [&](int c, const __nv_bfloat16* cache, const __nv_bfloat16* fresh, uint4 (&raw)[4]) {
+    const __nv_bfloat16* row = cache + unit0 + static_cast<size_t>(c) * (kUnit / 2) * pair;
+    if (kUnit * c + kUnit <= L) {  // a whole unit of cached rows
+#pragma unroll
+      for (int kk = 0; kk < 4; ++kk) raw[kk] = *reinterpret_cast<const uint4*>(row + kk * pair);
+      return;
+    }
+    const bool own = c == n_units - 1;
     const int n = unit_keys(c);
-    const size_t stride = c == n_units - 1 ? kNewStride : static_cast<size_t>(a.HD);
-    const __nv_bfloat16* kb = unit_base(c, a.k_cache, &kn[0][0]);
+    if (own) row = fresh + hv * kNewStride + u * 8;
 #pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-      for (int i = 0; i < 4; ++i)
-        kraw[t][i] = 8 * t + g < n ? *reinterpret_cast<const uint4*>(kb + (8 * t + g) * stride + (4 * i + j) * 8)
-                                   : make_uint4(0u, 0u, 0u, 0u);
+    for (int kk = 0; kk < 4; ++kk)
+      raw[kk] = 2 * kk + hv < n ? *reinterpret_cast<const uint4*>(row + kk * (own ? 2 * static_cast<size_t>(kNewStride) : pair))
+                                : make_uint4(0u, 0u, 0u, 0u);
   };
-  auto load_v = [&](int c) {
-    const int n = unit_keys(c);
-    const size_t stride = c == n_units - 1 ? kNewStride : static_cast<size_t>(a.HD);
-    const __nv_bfloat16* vb = unit_base(c, a.v_cache, &vn[0][0]);
-#pragma unroll
-    for (int kk = 0; kk < 8; ++kk)
-      vraw[kk] = 2 * kk + hv < n ? *reinterpret_cast<const uint4*>(vb + (2 * kk + hv) * stride + u * 8)
-                                 : make_uint4(0u, 0u, 0u, 0u);
-  };
+  auto load_k = [&](int c) { load_rows(c, a.k_cache, &kn[0][0], kraw); };
+  auto load_v = [&](int c) { load_rows(c, a.v_cache, &vn[0][0], vraw); };
   const int step = S * kAttnWarps;
   int c = rank * kAttnWarps + warp;
   if (c < n_units - 1) {  // in flight while the new rows are rotated
@@ -253,23 +269,17 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
 
   const float scale = 1.4426950408889634f * rsqrtf(static_cast<float>(kHeadDim));  // log2(e) / sqrt(128)
 #pragma unroll
-  for (int t0 = 0; t0 < NQ * kRopePairs; t0 += kAttnWarps * 32) {
-    const int i = (t0 + tid) / kRopePairs, jj = tid % kRopePairs;
+  for (int t = 0; t < kRot; ++t) {
+    const int i = (t * kAttnWarps * 32 + tid) / kRopePairs, jj = tid % kRopePairs;
     if (i < nq) {
-      const int m = b * nq + i;
-      const float2 cs = a.rot[static_cast<size_t>(m) * kRopePairs + jj];
-      const __half* q = a.qkv + static_cast<size_t>(m) * a.ld + h * kHeadDim + jj;
-      const __half* k = q + a.HD;
-      const __half* v = q + 2 * a.HD;
-      const float q0 = __half2float(q[0]), q1 = __half2float(q[kRopePairs]);
-      const float k0 = __half2float(k[0]), k1 = __half2float(k[kRopePairs]);
-      const float v0 = __half2float(v[0]), v1 = __half2float(v[kRopePairs]);
-      qs[i][jj] = (q0 * cs.x - q1 * cs.y) * scale;
-      qs[i][jj + kRopePairs] = (q0 * cs.y + q1 * cs.x) * scale;
-      kn[i][jj] = __float2bfloat16_rn(k0 * cs.x - k1 * cs.y);
-      kn[i][jj + kRopePairs] = __float2bfloat16_rn(k0 * cs.y + k1 * cs.x);
-      vn[i][jj] = __float2bfloat16_rn(v0);
-      vn[i][jj + kRopePairs] = __float2bfloat16_rn(v1);
+      const float q0 = __half2float(rq[t][0]), q1 = __half2float(rq[t][1]);
+      const float k0 = __half2float(rk[t][0]), k1 = __half2float(rk[t][1]);
+      qs[i][jj] = (q0 * cs[t].x - q1 * cs[t].y) * scale;
+      qs[i][jj + kRopePairs] = (q0 * cs[t].y + q1 * cs[t].x) * scale;
+      kn[i][jj] = __float2bfloat16_rn(k0 * cs[t].x - k1 * cs[t].y);
+      kn[i][jj + kRopePairs] = __float2bfloat16_rn(k0 * cs[t].y + k1 * cs[t].x);
+      vn[i][jj] = __float2bfloat16_rn(__half2float(rv[t][0]));
+      vn[i][jj + kRopePairs] = __float2bfloat16_rn(__half2float(rv[t][1]));
     } else {
       qs[i][jj] = qs[i][jj + kRopePairs] = 0.f;
     }
@@ -283,8 +293,17 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
       *reinterpret_cast<uint4*>(a.v_cache + o) = *reinterpret_cast<const uint4*>(&vn[i][uu * 8]);
     }
 
-  const uint32_t q_addr = fsx::smem_addr(&qs[0][8 * j]);  // unit 4 i + j of query qi: 128 qi + 32 i values on
-  const int q_lane = (j & 1) * NH;  // this lane's queries q_lane .. q_lane + NH - 1
+  uint64_t q2[NQ][4];  // dims 8 u .. 8 u + 7 of every query
+#pragma unroll
+  for (int qi = 0; qi < NQ; ++qi) {
+    const ulonglong2 qa = *reinterpret_cast<const ulonglong2*>(&qs[qi][8 * u]);
+    const ulonglong2 qb = *reinterpret_cast<const ulonglong2*>(&qs[qi][8 * u + 4]);
+    q2[qi][0] = qa.x;
+    q2[qi][1] = qa.y;
+    q2[qi][2] = qb.x;
+    q2[qi][3] = qb.y;
+  }
+  const int q_lane = (u & 3) * NH;  // this lane's queries q_lane .. q_lane + NH - 1
   float m_run[NH], l_run[NH];       // l_run: this lane's keys only
   uint64_t o[NQ][4];                // this half warp's keys, value dims 8 u .. 8 u + 7
 #pragma unroll
@@ -305,48 +324,48 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
     const bool own = c == n_units - 1;
     const int n = unit_keys(c);
     const int next = c + step;
-    uint64_t acc[2][NQ];
+    // this lane's 8 dims of every score, then the transposed sum over the row's 16 lanes: key bits
+    // (lane bits 3, 2), then query quarter (lane bits 1, 0)
+    const bool up8 = (u & 8) != 0, up4 = (u & 4) != 0, up2 = (u & 2) != 0, up1 = (u & 1) != 0;
+    float r4[2][NQ];  // [key bit 0], key bit 1 by lane bit 3
 #pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-      for (int qi = 0; qi < NQ; ++qi) acc[t][qi] = 0ull;
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
+    for (int k0 = 0; k0 < 2; ++k0) {
       uint64_t kv[2][4];
 #pragma unroll
-      for (int t = 0; t < 2; ++t) {
-        kv[t][0] = bf16x2_to_f32x2(kraw[t][i].x);
-        kv[t][1] = bf16x2_to_f32x2(kraw[t][i].y);
-        kv[t][2] = bf16x2_to_f32x2(kraw[t][i].z);
-        kv[t][3] = bf16x2_to_f32x2(kraw[t][i].w);
+      for (int e = 0; e < 2; ++e) {
+        const uint4 w = kraw[k0 + 2 * e];
+        kv[e][0] = bf16x2_to_f32x2(w.x);
+        kv[e][1] = bf16x2_to_f32x2(w.y);
+        kv[e][2] = bf16x2_to_f32x2(w.z);
+        kv[e][3] = bf16x2_to_f32x2(w.w);
       }
 #pragma unroll
       for (int qi = 0; qi < NQ; ++qi) {
-        const ulonglong2 qa = ld_shared2(q_addr + (qi * kHeadDim + 32 * i) * 4);
-        const ulonglong2 qb = ld_shared2(q_addr + (qi * kHeadDim + 32 * i + 4) * 4);
+        float sum[2];
 #pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          fma2(acc[t][qi], kv[t][0], qa.x);
-          fma2(acc[t][qi], kv[t][1], qa.y);
-          fma2(acc[t][qi], kv[t][2], qb.x);
-          fma2(acc[t][qi], kv[t][3], qb.y);
+        for (int e = 0; e < 2; ++e) {
+          uint64_t acc = mul2(kv[e][0], q2[qi][0]);
+          fma2(acc, kv[e][1], q2[qi][1]);
+          fma2(acc, kv[e][2], q2[qi][2]);
+          fma2(acc, kv[e][3], q2[qi][3]);
+          const float2 f = unpack2(acc);
+          sum[e] = f.x + f.y;
         }
+        r4[k0][qi] = (up8 ? sum[1] : sum[0]) + __shfl_xor_sync(0xffffffffu, up8 ? sum[0] : sum[1], 8);
       }
     }
     if (next < n_units) load_k(next);
-    // transposed sum over the 4 lanes of a key row: first the key group, then the query half
-    const bool up2 = (j & 2) != 0, up1 = (j & 1) != 0;
-    float r[NQ], p[NH];
+    float r2[NQ], r1[NQ / 2], p[NH];
 #pragma unroll
-    for (int qi = 0; qi < NQ; ++qi) {
-      const float2 f0 = unpack2(acc[0][qi]), f1 = unpack2(acc[1][qi]);
-      const float a0 = f0.x + f0.y, a1 = f1.x + f1.y;
-      r[qi] = (up2 ? a1 : a0) + __shfl_xor_sync(0xffffffffu, up2 ? a0 : a1, 2);
-    }
+    for (int qi = 0; qi < NQ; ++qi)
+      r2[qi] = (up4 ? r4[1][qi] : r4[0][qi]) + __shfl_xor_sync(0xffffffffu, up4 ? r4[0][qi] : r4[1][qi], 4);
+#pragma unroll
+    for (int qi = 0; qi < NQ / 2; ++qi)
+      r1[qi] = (up2 ? r2[NQ / 2 + qi] : r2[qi]) + __shfl_xor_sync(0xffffffffu, up2 ? r2[qi] : r2[NQ / 2 + qi], 2);
 #pragma unroll
     for (int qq = 0; qq < NH; ++qq)
-      p[qq] = (up1 ? r[NH + qq] : r[qq]) + __shfl_xor_sync(0xffffffffu, up1 ? r[qq] : r[NH + qq], 1);
-    const int key = 8 * (j >> 1) + g;
+      p[qq] = (up1 ? r1[NH + qq] : r1[qq]) + __shfl_xor_sync(0xffffffffu, up1 ? r1[qq] : r1[NH + qq], 1);
+    const int key = 2 * (u >> 2) + hv;
     float alpha[NH];
     bool moved = false;
 #pragma unroll
@@ -355,13 +374,13 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
       const int qi = q_lane + qq;
       const bool vis = qi < nq && key < n && (!own || key <= qi);
       const float sv = vis ? p[qq] : -INFINITY;
-      float mx = sv;  // over the 16 keys: the lanes with this lane's query half
+      float mx = sv;  // over the 8 keys: the lanes with this lane's query quarter
 #pragma unroll
-      for (int sh = 16; sh > 1; sh >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, sh));
+      for (int sh = 16; sh > 2; sh >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, sh));
       const float m_new = fmaxf(m_run[qq], mx);
       const bool none = m_new == -INFINITY;  // an unused query slot
-      alpha[qq] = none ? 1.f : exp2f(m_run[qq] - m_new);
-      p[qq] = vis && !none ? exp2f(sv - m_new) : 0.f;
+      alpha[qq] = none ? 1.f : ex2_approx(m_run[qq] - m_new);
+      p[qq] = none ? 0.f : ex2_approx(sv - m_new);  // 0 where not visible
       l_run[qq] = l_run[qq] * alpha[qq] + p[qq];
       moved = moved || alpha[qq] != 1.f;
       m_run[qq] = m_new;
@@ -376,13 +395,12 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
       }
     }
 #pragma unroll
-    for (int kk = 0; kk < 8; ++kk) {
+    for (int kk = 0; kk < 4; ++kk) {
       const uint64_t v0 = bf16x2_to_f32x2(vraw[kk].x), v1 = bf16x2_to_f32x2(vraw[kk].y);
       const uint64_t v2 = bf16x2_to_f32x2(vraw[kk].z), v3 = bf16x2_to_f32x2(vraw[kk].w);
-      const int kv = 2 * kk + hv;  // its probabilities are with lanes 4 (kv mod 8) + 2 (kv / 8) + query half
 #pragma unroll
-      for (int qi = 0; qi < NQ; ++qi) {
-        const float pk = __shfl_sync(0xffffffffu, p[qi % NH], ((kv & 7) << 2) | ((kv >> 3) << 1) | (qi / NH));
+      for (int qi = 0; qi < NQ; ++qi) {  // key 2 kk + hv: its probabilities are in this half warp
+        const float pk = __shfl_sync(0xffffffffu, p[qi % NH], (lane & 16) | (kk << 2) | (qi / NH));
         const uint64_t pp = pack2(pk, pk);
         fma2(o[qi][0], pp, v0);
         fma2(o[qi][1], pp, v1);
@@ -408,8 +426,8 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
   for (int qq = 0; qq < NH; ++qq) {
     float l = l_run[qq];
 #pragma unroll
-    for (int sh = 16; sh > 1; sh >>= 1) l += __shfl_xor_sync(0xffffffffu, l, sh);
-    if (lane < 2) {
+    for (int sh = 16; sh > 2; sh >>= 1) l += __shfl_xor_sync(0xffffffffu, l, sh);
+    if (lane < 4) {
       sm_m[warp][q_lane + qq] = m_run[qq];
       sm_l[warp][q_lane + qq] = l;
     }
@@ -460,10 +478,11 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
 }
 
 // CTAs per (vehicle, head): the largest power of two up to 8 that keeps the batch's CTAs
-// within the four that share an SM
+// within two waves of the four that share an SM (16 vehicles: 325 us a call with one CTA each, the
+// longest history last to finish, 312 us with two)
 int append_attn_splits(int B, int n_heads, int sm_count) {
   int s = kMaxSplit;
-  while (s > 1 && static_cast<long long>(B) * n_heads * s > 4ll * sm_count) s >>= 1;
+  while (s > 1 && static_cast<long long>(B) * n_heads * s > 8ll * sm_count) s >>= 1;
   return s;
 }
 
