@@ -497,6 +497,7 @@ struct fsx_append_s {
   long long weight_bytes = 0;
   std::vector<const unsigned char*> w_qkv, w_o, w_gu, w_dn;
   CUtensorMap map_x16[fsx::kStreamTileCount], map_o[fsx::kStreamTileCount], map_h[fsx::kStreamTileCount];
+  CUtensorMap map_o_res[fsx::kResTileCount], map_h_res[fsx::kResTileCount];
   float* x = nullptr;
   __half* x16 = nullptr;
   float* ss = nullptr;
@@ -579,6 +580,7 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
   FSX_CUDA_H(cudaSetDevice(device));
   FSX_CUDA_H(cudaDeviceGetAttribute(&h->sm_count, cudaDevAttrMultiProcessorCount, device));
   FSX_CUDA_H(fsx::gemm_stream_set_attributes());
+  FSX_CUDA_H(fsx::gemm_res_set_attributes());
 
   // ---- weight tiles per layer [QKV | W_o | gate/up | W_d], 128-row x 64-K swizzled
   // images; RMSNorm gains folded into the K columns of QKV and gate/up; gate/up rows
@@ -668,6 +670,10 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
           !fsx::encode_act_map(&h->map_o[i], h->o, m_pad, HD, fsx::kStreamTiles[i]) ||
           !fsx::encode_act_map(&h->map_h[i], h->hbuf, m_pad, F, fsx::kStreamTiles[i]))
         return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
+    for (int i = 0; i < fsx::kResTileCount; ++i)
+      if (!fsx::encode_act_map(&h->map_o_res[i], h->o, m_pad, HD, fsx::kResTiles[i]) ||
+          !fsx::encode_act_map(&h->map_h_res[i], h->hbuf, m_pad, F, fsx::kResTiles[i]))
+        return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
   }
   {
     double inv_freq[kRopePairs];
@@ -727,6 +733,14 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
   append_embed_kernel<<<M, 128, 0, st>>>(ea);
   FSX_CUDA(cudaGetLastError());
 
+  // The residual projections' tiles are few (d / 128): K is cut over clusters where those fit the
+  // chip (gemm_res.cu), else the weight stream is cut evenly like the others'.
+  const fsx::ResPlan plan_o = fsx::gemm_res_plan(M, d, HD), plan_d = fsx::gemm_res_plan(M, d, F);
+  auto launch_residual = [&](const CUtensorMap* maps, const CUtensorMap* maps_res, const fsx::ResPlan& plan,
+                             const fsx::TcGemmArgs& g) {
+    if (plan.splits > 1) return fsx::launch_gemm_res(maps_res[plan.tile], g, plan, st, true);
+    return fsx::launch_gemm_stream(maps[bn_i], g, fsx::kEpiResidual, h->sm_count, st, true);
+  };
   const int attn_splits = append_attn_splits(B, c.n_heads, h->sm_count);
   for (int l = 0; l < c.n_layers; ++l) {
     fsx::TcGemmArgs g{};
@@ -775,7 +789,7 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     go.ss_stride = h->ss_stride;
     go.part = h->gemm_part;
     go.tile_count = h->tile_count;
-    FSX_CUDA(fsx::launch_gemm_stream(h->map_o[bn_i], go, fsx::kEpiResidual, h->sm_count, st, true));
+    FSX_CUDA(launch_residual(h->map_o, h->map_o_res, plan_o, go));
 
     fsx::TcGemmArgs gg{};
     gg.M = M;
@@ -806,7 +820,7 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     gd.part = h->gemm_part;
     gd.tile_count = h->tile_count;
     gd.x_copy = l == c.n_layers - 1 ? d_hidden : nullptr;  // the residual stream after the last layer
-    FSX_CUDA(fsx::launch_gemm_stream(h->map_h[bn_i], gd, fsx::kEpiResidual, h->sm_count, st, true));
+    FSX_CUDA(launch_residual(h->map_h, h->map_h_res, plan_d, gd));
   }
   return FSX_OK;
 }

@@ -45,18 +45,18 @@ __host__ __device__ constexpr int recv_bytes() {  // [split][own groups]: roundi
 }
 template <int BN>
 __host__ __device__ constexpr int n_stages() {
-  return BN <= 48 ? 8 : (BN <= 64 ? 7 : (BN <= 96 ? 5 : (BN <= 144 ? 4 : 3)));
+  return BN <= 16 ? 10 : BN <= 48 ? 8 : (BN <= 64 ? 7 : (BN <= 96 ? 5 : (BN <= 144 ? 4 : 3)));
 }
 template <int BN>
 __host__ __device__ constexpr int smem_bytes() {
   return 1024 /* alignment */ + 1024 /* barriers */ + recv_bytes<BN>() + n_stages<BN>() * stage_bytes<BN>();
 }
-static_assert(smem_bytes<48>() <= 232448 && smem_bytes<64>() <= 232448 && smem_bytes<96>() <= 232448 &&
+static_assert(smem_bytes<16>() <= 232448 && smem_bytes<48>() <= 232448 && smem_bytes<64>() <= 232448 && smem_bytes<96>() <= 232448 &&
                   smem_bytes<128>() <= 232448 && smem_bytes<144>() <= 232448 && smem_bytes<160>() <= 232448,
               "shared memory of a token tile exceeds the per-block limit");
 template <int BN>
 __host__ __device__ constexpr uint32_t tmem_cols() {
-  return BN <= 64 ? 64 : (BN <= 128 ? 128 : 256);
+  return BN <= 32 ? 32 : BN <= 64 ? 64 : (BN <= 128 ? 128 : 256);
 }
 
 __device__ __forceinline__ void tma_tokens(void* dst, const CUtensorMap* map, int k, int m, uint64_t* bar) {
@@ -300,8 +300,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
             p.xo[idx] = v;
             p.xo16[idx] = __float2half_rn(v);
           }
+          acc[i][t] = v;
           ss[t] += v * v;
         }
+      if (p.x_copy != nullptr) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+          for (int t = 0; t < 4; ++t)
+            if (m + t < p.M) p.x_copy[static_cast<size_t>(m + t) * p.ldxo + t_n * kRows + 32 * i + lane] = acc[i][t];
+      }
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
         const float s = warp_sum(ss[t]);
@@ -330,6 +338,7 @@ const void* res_fn(int bn, size_t* smem) {
     *smem = smem_bytes<BN_>();                                     \
     return reinterpret_cast<const void*>(&gemm_res_kernel<BN_>);   \
   }
+  FSX_RES(16)
   FSX_RES(48)
   FSX_RES(64)
   FSX_RES(96)
@@ -364,6 +373,7 @@ ResPlan gemm_res_plan(int M, int N, int K) {
   const int KT = K / kTcTileK;
   for (int i = 0; i < kResTileCount; ++i) {
     const int bn = kResTiles[i];
+    if (bn == 16 && M > 16) continue;  // several tiles of 16 reread the weights as often
     const int tiles = (N / kRows) * ((M + bn - 1) / bn);
     size_t smem = 0;
     const void* fn = res_fn(bn, &smem);

@@ -34,7 +34,7 @@ struct TcGemmArgs {
   // gemm_stream: fp32 partials of the tiles that several CTAs share, and arrivals per tile
   float* part;
   int* tile_count;
-  // gemm_stream, kEpiResidual: optional second copy of the updated rows (layout of xo)
+  // gemm_stream and gemm_res, kEpiResidual: optional second copy of the updated rows (layout of xo)
   float* x_copy;
   // pair variant: index of the tile at `w` in the weight map (tiles of 16 KB from the map's base)
   int w_tile0;
@@ -61,8 +61,8 @@ cudaError_t launch_gemm_stream(const CUtensorMap& map_a, const TcGemmArgs& args,
                                cudaStream_t stream, bool pdl);
 // ---- residual projections with K cut over the CTAs of a cluster (gemm_res.cu): takes w, N, K, M,
 // xo, xo16, ldxo, ss_out and ss_stride; map_a with a box of kResTiles[plan.tile] rows
-constexpr int kResTileCount = 6;
-constexpr int kResTiles[kResTileCount] = {48, 64, 96, 128, 144, 160};
+constexpr int kResTileCount = 7;
+constexpr int kResTiles[kResTileCount] = {16, 48, 64, 96, 128, 144, 160};
 struct ResPlan {
   int tile;    // index into kResTiles
   int splits;  // K splits = cluster size (1: not for this kernel)
