@@ -57,9 +57,10 @@ template <int BN>
 __host__ __device__ constexpr int n_stages() {  // as many as that share of the shared memory holds
   return BN <= 16 ? 6 : (BN <= 32 ? 10 : (BN <= 64 ? 9 : (BN <= 128 ? 6 : 4)));
 }
+constexpr int kBatch = 4;  // segments of a split tile in flight at once (QKV and gate/up have at most 3)
 template <int BN>
-__host__ __device__ constexpr int sum_batch() {  // segments of a split tile in flight at once
-  return ctas_per_sm<BN>() == 2 ? 4 : 8;
+__host__ __device__ constexpr int sum_chunks() {  // token chunks of a group summed at once
+  return BN <= 16 ? 1 : (BN <= 32 ? 2 : 4);
 }
 template <int BN>
 __host__ __device__ constexpr int smem_bytes() {
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
   extern __shared__ __align__(1024) unsigned char smem_raw[];
   constexpr int kStages = n_stages<BN>();
   constexpr int kStageBytes = stage_bytes<BN>();
-  constexpr int kBatch = sum_batch<BN>();
+  constexpr int kRound = sum_chunks<BN>();
   constexpr uint32_t kTmemCols = 2 * BN <= 32 ? 32 : 2 * BN;  // two accumulators of BN fp32 columns
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -329,32 +330,43 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
         if (*last) {
           __threadfence();
           if (etid == 0) p.tile_count[tile] = 0;  // zero between launches
-          for (int c0 = grp * kChunk; c0 < BN && c0 < p.M; c0 += kGroups * kChunk) {
-            float v[kChunk];
+          // kRound chunks of the group at a time, kBatch segments of each in flight, added in range order
+          for (int c0 = grp * kChunk; c0 < BN && c0 < p.M; c0 += kRound * kGroups * kChunk) {
+            float v[kRound][kChunk];
 #pragma unroll
-            for (int j = 0; j < kChunk; ++j) v[j] = 0.f;
-            for (int sg = 0; sg < n_seg; sg += kBatch) {  // in range order
-              float4 w4[kBatch][2];
+            for (int r = 0; r < kRound; ++r)
 #pragma unroll
-              for (int e = 0; e < kBatch; ++e) {
-                const int c = first + sg + e;
-                const float4* d = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(2 * c + (sg + e == 0 ? 1 : 0)) * kSlot) +
-                                  static_cast<size_t>(c0 / 4) * kRows + row;
+              for (int j = 0; j < kChunk; ++j) v[r][j] = 0.f;
+            for (int sg = 0; sg < n_seg; sg += kBatch) {
+              float4 w4[kRound][kBatch][2];
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh)
-                  w4[e][hh] = sg + e < n_seg ? __ldcg(d + hh * kRows) : make_float4(0.f, 0.f, 0.f, 0.f);
-              }
+              for (int r = 0; r < kRound; ++r)
 #pragma unroll
-              for (int e = 0; e < kBatch; ++e)
+                for (int e = 0; e < kBatch; ++e) {
+                  const int c = first + sg + e, cr = c0 + r * kGroups * kChunk;
+                  const float4* d = reinterpret_cast<const float4*>(p.part + static_cast<size_t>(2 * c + (sg + e == 0 ? 1 : 0)) * kSlot) +
+                                    static_cast<size_t>(cr / 4) * kRows + row;
 #pragma unroll
-                for (int hh = 0; hh < 2; ++hh) {
-                  v[4 * hh] += w4[e][hh].x;
-                  v[4 * hh + 1] += w4[e][hh].y;
-                  v[4 * hh + 2] += w4[e][hh].z;
-                  v[4 * hh + 3] += w4[e][hh].w;
+                  for (int hh = 0; hh < 2; ++hh)
+                    w4[r][e][hh] = sg + e < n_seg && cr < BN && cr < p.M ? __ldcg(d + hh * kRows) : make_float4(0.f, 0.f, 0.f, 0.f);
                 }
+#pragma unroll
+              for (int r = 0; r < kRound; ++r)
+#pragma unroll
+                for (int e = 0; e < kBatch; ++e)
+#pragma unroll
+                  for (int hh = 0; hh < 2; ++hh) {
+                    v[r][4 * hh] += w4[r][e][hh].x;
+                    v[r][4 * hh + 1] += w4[r][e][hh].y;
+                    v[r][4 * hh + 2] += w4[r][e][hh].z;
+                    v[r][4 * hh + 3] += w4[r][e][hh].w;
+                  }
             }
-            finish(tile, c0, v);
+#pragma unroll
+            for (int r = 0; r < kRound; ++r) {
+              const int cr = c0 + r * kGroups * kChunk;
+              if (cr < BN && cr < p.M) finish(tile, cr, v[r]);
+            }
           }
         }
       }
