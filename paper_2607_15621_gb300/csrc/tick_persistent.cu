@@ -5,10 +5,10 @@
 // attention head (H clusters, 4H CTAs, one CTA per SM, all co-resident).
 // Every layer runs two phases separated by device-wide counters:
 //   phase A (every cluster = one head h):
-//     each CTA reads its 128 columns of x, converts them to fp16 and sends them
-//     with the per-token partial sums of x^2 to the whole cluster; four warps
-//     each run the tensor-core MMAs (tcgen05, accumulators in tensor memory) of
-//     one K quarter as soon as that quarter has arrived, for the CTA's 96 rows
+//     each CTA reads all of x (86 KB from L2; a quarter each, exchanged in the cluster, took
+//     longer: 671 against 663 us a tick at 224 rows), converts it to fp16, a row's 1/rms with it;
+//     four warps each run the tensor-core MMAs (tcgen05, accumulators in tensor memory) of
+//     one K quarter, for the CTA's 96 rows
 //     of [W_q; W_k; W_v] of head h (32 q, 32 k, 32 v dims; the RMSNorm gain is
 //     folded into the weights and 1/rms is applied to the accumulator sum) ->
 //     q goes to all 4 CTAs, k_ae and v_ae to the CTA that attends over the own
@@ -79,6 +79,8 @@ constexpr int kKeyTile = 32;           // keys per staged attention tile
 constexpr int kQS = kD + 8;            // fp16 row stride of q / own k / own v (halves)
 constexpr int kDS = 128 + 4;           // fp32 row stride of the output transpose buffer
 constexpr int kRowsPerRank = kTokTile / kCl;  // 12
+constexpr int kDModel = 512;                  // expert width this kernel is built for
+constexpr int kRowsPerWarp = kTokTile / (kThr / 32);  // 6: token rows a warp converts in phase A
 constexpr int kQkvAtom = 3 * 32 * 128;        // one 64-wide K slice of the CTA's 96 QKV rows (12 KB)
 constexpr int kActAtom = kTokTile * 128;      // one K slice of the 48 token rows (6 KB)
 constexpr int kNAcc = 4;                      // accumulators: one per MMA-issuing warp
@@ -265,8 +267,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   const Smem L = smem_layout(p.d);
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + L.bars);  // [kSlots] weight ring
   uint64_t* mma_bar = full + kSlots;   // the four issuing warps' MMA groups
-  uint64_t* xbar = mma_bar + 1;        // [4] x quarter + partial sums of x^2 from rank s (phase A)
-  uint64_t* qbar = xbar + kCl;         // q (and own k / v) from the partners
+  uint64_t* qbar = mma_bar + 1;        // q (and own k / v) from the partners
   uint64_t* rsbar = qbar + 1;          // split partials of the rows this CTA merges
   uint64_t* agbar = rsbar + 1;         // merged o_h rows of the partners
   uint64_t* bbar = agbar + 1;          // phase B: partial sums of x^2 and gate/up partials
@@ -301,7 +302,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   for (int i = 0; i < kCl - 1; ++i) pdelta[i] = cluster_addr(smem, (rank + 1 + i) & (kCl - 1)) - smem_addr(smem);
   const int G = gridDim.x;
   const int cta = blockIdx.x;
-  const int d = p.d;                             // 512 (checked on the host)
+  constexpr int d = kDModel;                     // p.d (checked on the host): constant offsets keep the code small
   const int T = p.n_action + p.n_frame;
   const int HD = p.H * kD;
   const bool in_b = head < p.n_b_clusters;       // phase B participant (whole clusters)
@@ -359,7 +360,6 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   // ---- exchange byte counts, identical in every layer (recomputed at each use from the
   // launch parameters rather than held in registers across the attention)
 #define FSX_T (p.n_action + p.n_frame)
-#define FSX_X_BYTES static_cast<uint32_t>(FSX_T * (128 * 2 + 4))  // fp16 x quarter + partial sums, per partner
 #define FSX_RS_BYTES static_cast<uint32_t>((kCl - 1) * (kRecvBytes + kRowsPerRank * 4))
 #define FSX_AG_BYTES static_cast<uint32_t>((kCl - 1) * kRowsPerRank * kD * 2)
 #define FSX_B_BYTES static_cast<uint32_t>((kCl - 1) * (kRsBytes + FSX_T * 4))
@@ -370,7 +370,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     *abort = 0;
     for (int i = 0; i < kSlots; ++i) mbar_init(full + i, 1);
     mbar_init(mma_bar, kNAcc);
-    for (int i = 0; i < kCl + 5; ++i) mbar_init(xbar + i, 1);
+    for (int i = 0; i < 5; ++i) mbar_init(qbar + i, 1);
     mbar_init(drain_bar, kNAcc);
     for (int i = 0; i < kNB; ++i) {
       mbar_init(raw_bar + i, 64);
@@ -464,10 +464,9 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         xv[i][h] = r < T ? ld_cg4(Xs + static_cast<size_t>(r) * d + col0 + xu * 8 + 4 * h) : make_float4(0.f, 0.f, 0.f, 0.f);
     }
   };
-  // those columns -> fp16 x image (local, and the partners when `send_x`), per-token
-  // partial sums of x^2 -> gss[rank] here and in the partners; the partners'
-  // `peer_bar` counts the bytes
-  auto convert_send = [&](const float4 (&xv)[3][2], int k0, bool send_x, uint64_t* peer_bar) {
+  // those columns -> K slices 0, 1 of the fp16 x image; per-token partial sums of x^2 -> gss[rank]
+  // here and in the partners, whose `bbar` counts the bytes
+  auto convert_quarter = [&](const float4 (&xv)[3][2]) {
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
       const int r = xr0 + 16 * i;
@@ -476,15 +475,13 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
 #pragma unroll
       for (int o = 8; o > 0; o >>= 1) ss += __shfl_xor_sync(0xffffffffu, ss, o);  // the row's 16 threads
       if (r < T && *abort == 0) {
-        const uint4 h = make_uint4(pack_half2(a.x, a.y), pack_half2(a.z, a.w), pack_half2(b.x, b.y), pack_half2(b.z, b.w));
-        unsigned char* dst = act + sw128_offset(kTokTile, r, k0 + xu * 8);
-        *reinterpret_cast<uint4*>(dst) = h;
-        if (xu == 0) gss[rank * kTokTile + r] = ss;
+        *reinterpret_cast<uint4*>(act + sw128_offset(kTokTile, r, xu * 8)) =
+            make_uint4(pack_half2(a.x, a.y), pack_half2(a.z, a.w), pack_half2(b.x, b.y), pack_half2(b.z, b.w));
+        if (xu == 0) {
+          gss[rank * kTokTile + r] = ss;
 #pragma unroll
-        for (int pi = 1; pi < kCl; ++pi) {
-          const uint32_t dl = pdelta[pi - 1], pb = peer_at(peer_bar, dl);
-          if (send_x) st_async_v4(peer_at(dst, dl), h, pb);
-          if (xu == 0) st_async_b32(peer_at(gss + rank * kTokTile + r, dl), __float_as_uint(ss), pb);
+          for (int pi = 0; pi < kCl - 1; ++pi)
+            st_async_b32(peer_at(gss + rank * kTokTile + r, pdelta[pi]), __float_as_uint(ss), peer_at(bbar, pdelta[pi]));
         }
       }
     }
@@ -674,7 +671,6 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   // ---- arm the exchange barriers for layer 0, then publish the token assembly
   if (tid < kTokTile) rstd[tid] = 0.f;  // padding tokens T..47 stay at zero
   if (tid == 0) {
-    for (int s_ = 1; s_ < kCl; ++s_) arm(xbar + ((rank + s_) & (kCl - 1)), FSX_X_BYTES);
     arm(qbar, FSX_Q_BYTES);
     arm(rsbar, FSX_RS_BYTES);
     arm(agbar, FSX_AG_BYTES);
@@ -707,31 +703,48 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     // =========================== phase A ===========================
     wait_counter(p.counters + sA, sA == 0 ? G : n_b_ctas, p.status, abort, p.wait_limit_ns);
     {
-      float4 xv[3][2];
-      load_x(Xc, rank * 128, xv);
+      // warp w: token rows w, w + 8, ... whole (every load of a row contiguous, all in flight) -> fp16
+      // image of all of K and the row's 1 / rms
+      float4 xv[kRowsPerWarp][4];
+      const float* Xw = Xc + warp * d + lane * 4;
+#pragma unroll
+      for (int i = 0; i < kRowsPerWarp; ++i)
+#pragma unroll
+        for (int c = 0; c < 4; ++c)
+          xv[i][c] = warp + 8 * i < T ? ld_cg4(Xw + 8 * i * d + c * 128) : make_float4(0.f, 0.f, 0.f, 0.f);
       // zero the buffer phase B accumulates into (while the loads are in flight)
 #pragma unroll 1
       for (int e = zA0 + tid; e < zA1; e += kThr) __stcg(Xz + e, 0.f);
-      // this rank's 128 columns of x -> fp16 image here and in the partners (K slices
-      // 2 rank, 2 rank + 1), partial sums of x^2 to every rank
-      convert_send(xv, rank * 128, true, xbar + rank);
+      unsigned char* act_w = act + sw128_offset(kTokTile, warp, lane * 4);
+#pragma unroll
+      for (int i = 0; i < kRowsPerWarp; ++i) {
+        const int r = warp + 8 * i;
+        float ss = 0.f;
+#pragma unroll
+        for (int c = 0; c < 4; ++c) {
+          const float4 x = xv[i][c];
+          ss += x.x * x.x + x.y * x.y + x.z * x.z + x.w * x.w;
+          if (r < T)  // row warp + 8 i: the 8-row group i of each K slice
+            *reinterpret_cast<uint2*>(act_w + c * 2 * kActAtom + i * 1024) =
+                make_uint2(pack_half2(x.x, x.y), pack_half2(x.z, x.w));
+        }
+        ss = warp_sum(ss);
+        if (lane == 0 && r < T) rstd[r] = rsqrtf(ss / static_cast<float>(d) + 1e-6f);
+      }
     }
-    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the local quarter -> tensor core
+    asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // x -> tensor core
     __syncthreads();
 
     // --- QKV: D[96 (+32 unused) rows x 48 tokens] over K = 512. Warp w < 4 runs K quarter w
-    // (slices 2w, 2w + 1: rank w's columns of x) into accumulator w as soon as rank w's
-    // columns and the weight slots under them have arrived; the 12 KB K slices lie back
-    // to back in slots 0-5
+    // (slices 2w, 2w + 1) into accumulator w as soon as the weight slots under it have arrived; the
+    // 12 KB K slices lie back to back in slots 0-5
     if (warp < kNAcc) {
       tc_fence_after();
       const int a0 = 2 * warp;
       bool ok = true;
       for (int sl = (a0 * kQkvAtom) / kSlotBytes; sl <= ((a0 + 2) * kQkvAtom - 1) / kSlotBytes; ++sl)
         ok = wait_chunk(q0 + sl) && ok;
-      if (warp != rank) ok = xwait(xbar + warp, par) && ok;
       if (ok && lane == 0) {
-        asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // the partner's columns -> tensor core
         mma_k(warp, ring_a + a0 * kQkvAtom, act_a + a0 * kActAtom, 0, 4, true);
         mma_k(warp, ring_a + (a0 + 1) * kQkvAtom, act_a + (a0 + 1) * kActAtom, 0, 4, false);
       }
@@ -739,12 +752,6 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       if (lane == 0) umma_commit(mma_bar);
       __syncwarp();
     }
-    // every partner's partial sums of x^2 have arrived: 1 / rms per token; re-arm for the next layer
-    for (int s_ = 1; s_ < kCl; ++s_) xwait(xbar + ((rank + s_) & (kCl - 1)), par);
-    if (tid == 0 && *abort == 0)
-      for (int s_ = 1; s_ < kCl; ++s_) arm(xbar + ((rank + s_) & (kCl - 1)), FSX_X_BYTES);
-    compute_rstd();
-    __syncthreads();
     wait_mma();
     // slots 2-5 and the activation image are free: the warps without QKV rows start the cache copies
     const int g0 = layer * n_chunks;
@@ -1140,7 +1147,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         for (int e = zB0 + tid; e < zB1; e += kThr) __stcg(Xc + e, 0.f);
         // this rank's 128 columns of x -> fp16 K slices 0, 1 here (no exchange: each CTA runs
         // the gate/up MMAs over its own K quarter), partial sums of x^2 to every rank
-        convert_send(xv, 0, false, bbar);
+        convert_quarter(xv);
       }
       asm volatile("fence.proxy.async.shared::cta;" ::: "memory");  // visible to the tensor core
       __syncthreads();
@@ -1304,7 +1311,6 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   }
 }
 #undef FSX_T
-#undef FSX_X_BYTES
 #undef FSX_RS_BYTES
 #undef FSX_AG_BYTES
 #undef FSX_B_BYTES
