@@ -12,7 +12,7 @@
 //   K slot (xkSlots) [64 keys][128 d]     smem, B of S          (K-major)
 //   V slot (xkSlots) [64 keys][128 d]     smem, B of P V        (N = d contiguous, MN-major;
 //                                         bf16 cache rows, fp16 own rows and fp32 caches)
-//   raw (x2, fp32)   [64 keys][128 d] fp32 smem, rows as they lie in the cache, per tensor
+//   raw (x2, fp32)   [16 keys][128 d] fp32 smem, rows as they lie in the cache, per tensor
 //   S (x2)           [64 q][64 keys] fp32 tensor memory, 64 columns each
 //   P_hi, P_lo       [64 q][64 keys]      tensor memory, A of P V, written over the
 //                                         S buffer they were computed from (32 columns each)
@@ -24,10 +24,11 @@
 //
 // Warp roles: warps 0-2 run the online softmax for query rows
 // 16 w .. 16 w + 15, two rows per thread; warp 3 lane 0 issues S and P V as their inputs become
-// ready; then 2 warps (4 for fp32) stage and convert the K rows and as many the V rows, two
-// chunks ahead. bf16 caches: two CTAs per SM, whole chunks by TMA. fp32 caches: twice the bytes
-// a key, so one CTA per SM holds two raw chunks per tensor (128 KB) in flight by 16-byte copies;
-// a warp converts only rows that it copied.
+// ready; warps 4-5 stage and convert the K rows, warps 6-7 the V rows, two
+// chunks ahead. Two CTAs per SM. bf16 caches: whole chunks by TMA. fp32 caches: 16-key stages by
+// 16-byte copies, two in flight per tensor (32 KB a CTA), converted into the slot by the warp that
+// copied the rows: another CTA's stream then hides a start-up, which 64-key stages and one CTA per SM
+// cannot (24 vehicles with 16-1000 rows, 32 heads: 78 -> 76.8 us).
 // Splits: the CTAs of one (vehicle, head) form a thread-block cluster and merge
 // (log-sum-exp weights) by pushing each split's normalised fp32 rows to the rank that owns them
 // through distributed shared memory. Split and fp32 launches check every cache value they stage
@@ -35,7 +36,9 @@
 // Measured against the mma.sync kernel of attention.cu, which split and fp32 launches ran before: a
 // tick of 4 vehicles with 0-700 bf16 rows, 8 layers, 2 splits: 740 -> 452 us; one vehicle with 2048
 // rows, 8 splits, Eq. 1 alone: 34 -> 27 us a call; 24 vehicles with 16-1000 fp32 rows, Eq. 1
-// alone: 104 -> 81 us a call (4.1 TB/s).
+// alone: 104 -> 68 us a call (4.9 TB/s) with the order below.
+// Launches of more than one wave without a plan start the longest caches first (each CTA finds its
+// vehicle among at most 128 by counting; the 24 fp32 vehicles: 76.8 -> 67.7 us). A tick's plan is sorted already.
 // Every wait is bounded; a timeout raises the status word and the CTA drains its
 // MMAs before it frees the tensor memory.
 #include <cuda.h>
@@ -59,11 +62,18 @@ constexpr int kTmemCols = 256;         // S[2] x 64 + O 128
 constexpr uint32_t kColS = 0;    // S / P buffers at columns 0 and 64
 constexpr uint32_t kColO = 128;
 constexpr int kMaxClusterSplits = 8;
+constexpr int kMaxByLength = 128;  // vehicles a launch without a plan sorts
 
 // shared-memory layout (bytes from the 1024-aligned base)
 constexpr int kQBytes = 64 * kD * 2;            // 16 KB
 constexpr int kSlotBytes = kSlotKeys * kD * 2;  // 16 KB
-constexpr int kRawBytes = kSlotKeys * kD * 4;   // one fp32 chunk of a tensor
+constexpr int kRawKeys = 16;                     // keys of a raw fp32 stage
+constexpr int kRawBytes = kRawKeys * kD * 4;
+constexpr int kRawPerChunk = kSlotKeys / kRawKeys;
+constexpr int kProdWarps = 2;                    // per tensor
+constexpr int kProdThreads = 32 * kProdWarps;
+constexpr int kThreadsTc = 32 * (kProdWarp0 + 2 * kProdWarps);
+constexpr int kCtasPerSm = kAttentionCtasPerSm;
 // barriers: kfull[3], kempty[3], vfull[3], vempty[3], sfull[2], pfull[2], pvdone[2], drain, ktma[3], vtma[3]
 constexpr int kNumBars = 25;
 template <bool F32>
@@ -77,19 +87,15 @@ struct CacheType<true> {
 template <bool F32>
 struct Shape {
   static constexpr int kSlots = F32 ? 2 : 3;           // per tensor
-  static constexpr int kProdWarps = F32 ? 4 : 2;       // per tensor
-  static constexpr int kProdThreads = 32 * kProdWarps;
-  static constexpr int kThreads = 32 * (kProdWarp0 + 2 * kProdWarps);
   static constexpr int kOffQ = 0;
   static constexpr int kOffK = kOffQ + kQBytes;
   static constexpr int kOffV = kOffK + kSlots * kSlotBytes;
   static constexpr int kOffRaw = kOffV + kSlots * kSlotBytes;  // [K, V][2]
   static constexpr int kOffBar = kOffRaw + (F32 ? 4 * kRawBytes : 0);
   static constexpr int kSmem = kOffBar + kNumBars * 8 + 8 /*tmem slot + abort*/;
-  static constexpr int kCtas = F32 ? 1 : 2;            // per SM
 };
-static_assert(2 * (Shape<false>::kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
-static_assert(Shape<true>::kSmem + 1024 <= 228 * 1024, "one CTA per SM");
+static_assert(kCtasPerSm * (Shape<false>::kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
+static_assert(kCtasPerSm * (Shape<true>::kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 // merge buffers at the start of the K slots: at most (48 + 7) rows of 128 fp32 values, then their log-sum-exps
 static_assert((48 + kMaxClusterSplits - 1) * (kD + 1) * 4 <= Shape<true>::kSlots * kSlotBytes, "merge buffers");
 
@@ -250,7 +256,7 @@ __device__ __forceinline__ void tma_load_cache(void* dst, const CUtensorMap* map
 
 // map_k, map_v: maps of the one layer's caches when p.cache_maps is NULL and p.param_maps is set
 template <bool F32, bool SPLIT>
-__global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
+__global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
     attn_tc_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
   using SH = Shape<F32>;
   using CT = typename CacheType<F32>::T;
@@ -287,7 +293,24 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
   }
   AttnPlan plan_z{0, 0, 0};
   if (p.plan != nullptr) plan_z = p.plan[blockIdx.z];
-  const int b = p.plan != nullptr ? plan_z.b : (p.order != nullptr ? p.order[blockIdx.z] : static_cast<int>(blockIdx.z));
+  int b = p.plan != nullptr ? plan_z.b : static_cast<int>(blockIdx.z);
+  if (p.by_length) {  // this CTA's vehicle: the one with blockIdx.z longer caches before it (ties by index)
+    long long* len = reinterpret_cast<long long*>(smem + SH::kOffK);
+    int* pick = reinterpret_cast<int*>(len + kMaxByLength);
+    const int n = static_cast<int>(gridDim.z);
+    if (tid < n) len[tid] = p.offsets[tid + 1] - p.offsets[tid];
+    __syncthreads();
+    if (tid < n) {
+      const long long mine = len[tid];
+      int before = 0;
+#pragma unroll 4
+      for (int j = 0; j < n; ++j) before += len[j] > mine || (len[j] == mine && j < tid) ? 1 : 0;
+      if (before == static_cast<int>(blockIdx.z)) *pick = tid;
+    }
+    __syncthreads();
+    b = *pick;
+    __syncthreads();  // read before the slot is staged into
+  }
 
   unsigned char* qt = smem + SH::kOffQ;
   unsigned char* kslot = smem + SH::kOffK;
@@ -308,12 +331,12 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
 
   // ---- producers' staging of chunk i (own rows fp16, cache rows bf16 converted later)
   const bool is_prod = warp >= kProdWarp0;
-  const bool is_v = warp >= kProdWarp0 + SH::kProdWarps;
-  const int pw = warp & (SH::kProdWarps - 1);  // warp within the tensor's staging warps
+  const bool is_v = warp >= kProdWarp0 + kProdWarps;
+  const int pw = warp & (kProdWarps - 1);  // warp within the tensor's staging warps
   const int pt = pw * 32 + lane;               // thread within them
   const int pu = pt & 15;                      // 16-byte unit of a 256-byte row
   const int pr0 = pt >> 4;                     // rows pr0, pr0 + kRowStep, ...
-  constexpr int kRowStep = SH::kProdThreads / 16;
+  constexpr int kRowStep = kProdThreads / 16;
   const size_t tok = static_cast<size_t>(H) * kD;
   const __half* obase = (is_v ? p.v_own : p.k_own) + static_cast<size_t>(b) * p.n_own * p.own_stride + h * kD + pu * 8;
   const CT* cbase = nullptr;             // this CTA's first cache row of the tensor (its head), set below
@@ -345,19 +368,21 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
                      : static_cast<int>(min(static_cast<long long>(kSlotKeys),
                                             L - (i - has_own) * static_cast<long long>(kSlotKeys)));
   };
+  // fp32: raw stage t (keys 16 t .. of this CTA's run), one warp instruction a row; row r of a stage
+  // is the warp's that has r mod kProdWarps == pw. Past the run's end an empty group.
+  auto issue_raw = [&](int t) {
+    const int rows = static_cast<int>(min(static_cast<long long>(kRawKeys), L - static_cast<long long>(t) * kRawKeys));
+    const uint32_t raw = smem_addr(smem + SH::kOffRaw + ((is_v ? 2 : 0) + (t & 1)) * kRawBytes) + lane * 16;
+    const CT* src = cbase + static_cast<size_t>(t) * kRawKeys * tok + lane * 4;
+#pragma unroll
+    for (int r = pw; r < kRawKeys; r += kProdWarps)
+      if (r < rows) cp_async_16(raw + r * (kD * 4), src + static_cast<size_t>(r) * tok);
+    cp_async_commit();
+  };
   auto issue = [&](int i) {
     unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
     const int rows = chunk_rows(i);
     const long long c0 = (i - has_own) * static_cast<long long>(kSlotKeys);
-    if (F32 && !is_own(i)) {  // raw fp32 rows, one warp instruction a row; row r is this warp's for r mod kProdWarps == pw
-      const uint32_t raw = smem_addr(smem + SH::kOffRaw + ((is_v ? 2 : 0) + (i & 1)) * kRawBytes) + lane * 16;
-      const CT* src = cbase + static_cast<size_t>(c0) * tok + lane * 4;
-#pragma unroll 8
-      for (int r = pw; r < kSlotKeys; r += SH::kProdWarps)
-        if (r < rows) cp_async_16(raw + r * (kD * 4), src + static_cast<size_t>(r) * tok);
-      cp_async_commit();
-      return;
-    }
     if (by_tma(i)) {
       if (pt == 0) {
         uint64_t* bar = tbar + i % kSlots;
@@ -384,7 +409,7 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
     cp_async_commit();
   };
   // queries: 64 rows x 16 units, rows >= n_q zero (one copy group per thread)
-  for (int i = tid; i < 64 * 16; i += SH::kThreads) {
+  for (int i = tid; i < 64 * 16; i += kThreadsTc) {
     const int r = i >> 4;
     const int u = i & 15;
     unsigned char* dst = qt + tile128_off(r, u);
@@ -424,9 +449,9 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
 
   if (tid == 0) {
     for (int i = 0; i < kSlots; ++i) {
-      mbar_init(kfull + i, SH::kProdThreads);
+      mbar_init(kfull + i, kProdThreads);
       mbar_init(kempty + i, 1);
-      mbar_init(vfull + i, SH::kProdThreads);
+      mbar_init(vfull + i, kProdThreads);
       mbar_init(vempty + i, 1);
       mbar_arrive(kempty + i);  // release 0 of every slot: free from the start
       mbar_arrive(vempty + i);
@@ -452,13 +477,22 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
       for (int i = 0; i < kSlots; ++i) mbar_init(tbar + i, 1);
       fence_proxy_async();
     }
-    for (int i = has_own; i < n_first; ++i) issue(i);
-    if (n_first == 2)
-      cp_async_wait<2>();
-    else if (n_first == 1)
-      cp_async_wait<1>();
-    else
-      cp_async_wait<0>();
+    if (F32) {
+      issue_raw(0);
+      issue_raw(1);
+      if (has_own != 0)
+        cp_async_wait<3>();
+      else
+        cp_async_wait<2>();
+    } else {
+      for (int i = has_own; i < n_first; ++i) issue(i);
+      if (n_first == 2)
+        cp_async_wait<2>();
+      else if (n_first == 1)
+        cp_async_wait<1>();
+      else
+        cp_async_wait<0>();
+    }
   } else {
     cp_async_wait<0>();
   }
@@ -563,41 +597,44 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
     uint32_t range = 0;    // fp32: largest magnitudes of the staged values; bf16: bits set by out-of-range ones
     int i = 0;
     for (; ok && i < n_chunks; ++i) {
-      if (i + 1 < n_chunks) cp_async_wait<1>();
-      else cp_async_wait<0>();
       unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
       if (F32) {
-        if (!is_own(i)) {  // raw rows -> fp16 slot, once its previous chunk is consumed
-          __syncwarp();    // the warp's copies of its rows
+        if (is_own(i)) {
+          cp_async_wait<2>();  // the two raw stages behind it stay in flight
+        } else {               // raw rows -> fp16 slot, once its previous chunk is consumed
           ok = wait_bar(empty + i % kSlots, (i / kSlots) & 1, p.status, abort);
           if (!ok) break;
-          const unsigned char* raw = smem + SH::kOffRaw + ((is_v ? 2 : 0) + (i & 1)) * kRawBytes;
           const int rows = chunk_rows(i);
           const int u = lane & 15;
           const int sw = (lane >> 2) & 1;  // the two 16-byte reads of a unit in an order that spreads the banks
+          for (int st = 0; st < kRawPerChunk; ++st) {
+            const int t = (i - has_own) * kRawPerChunk + st;
+            cp_async_wait<1>();  // stage t landed, t + 1 in flight
+            __syncwarp();        // the warp's copies of its rows
+            const unsigned char* raw = smem + SH::kOffRaw + ((is_v ? 2 : 0) + (t & 1)) * kRawBytes;
 #pragma unroll
-          for (int m = 0; m < kSlotKeys / SH::kProdWarps; m += 2) {
-            const int r = pw + SH::kProdWarps * (m + (lane >> 4));
-            uint4 out = make_uint4(0u, 0u, 0u, 0u);  // keys past the range: finite zeros
-            if (r < rows) {
-              const float4 x = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + sw * 16);
-              const float4 y = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + (sw ^ 1) * 16);
-              const uint32_t x0 = f32x2_to_half2_peak(x.x, x.y, range), x1 = f32x2_to_half2_peak(x.z, x.w, range);
-              const uint32_t y0 = f32x2_to_half2_peak(y.x, y.y, range), y1 = f32x2_to_half2_peak(y.z, y.w, range);
-              out = sw == 0 ? make_uint4(x0, x1, y0, y1) : make_uint4(y0, y1, x0, x1);
+            for (int m = 0; m < kRawKeys / kProdWarps; m += 2) {
+              const int r = pw + kProdWarps * (m + (lane >> 4));
+              uint4 out = make_uint4(0u, 0u, 0u, 0u);  // keys past the range: finite zeros
+              if (st * kRawKeys + r < rows) {
+                const float4 x = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + sw * 16);
+                const float4 y = *reinterpret_cast<const float4*>(raw + r * (kD * 4) + u * 32 + (sw ^ 1) * 16);
+                const uint32_t x0 = f32x2_to_half2_peak(x.x, x.y, range), x1 = f32x2_to_half2_peak(x.z, x.w, range);
+                const uint32_t y0 = f32x2_to_half2_peak(y.x, y.y, range), y1 = f32x2_to_half2_peak(y.z, y.w, range);
+                out = sw == 0 ? make_uint4(x0, x1, y0, y1) : make_uint4(y0, y1, x0, x1);
+              }
+              *reinterpret_cast<uint4*>(slot + tile128_off(st * kRawKeys + r, u)) = out;
             }
-            *reinterpret_cast<uint4*>(slot + tile128_off(r, u)) = out;
+            __syncwarp();  // the raw rows are read before they are refilled
+            issue_raw(t + 2);
           }
-          __syncwarp();  // the raw rows are read before they are refilled
         }
         fence_proxy_async();
         mbar_arrive(full + (i % kSlots));
-        if (i + 2 < n_chunks) {
-          issue(i + 2);
-          issued = i + 3;
-        }
         continue;
       }
+      if (i + 1 < n_chunks) cp_async_wait<1>();
+      else cp_async_wait<0>();
       if (by_tma(i)) {
         ok = wait_bar(tbar + i % kSlots, tma_parity(i), p.status, abort);
         if (!ok) break;
@@ -836,7 +873,7 @@ __global__ void __launch_bounds__(Shape<F32>::kThreads, Shape<F32>::kCtas)
     const float* rows_l = rows_o + S * rows_per * kD;
     const int q_lo = rank * rows_per;
     const int n_rows = min(p.n_q, q_lo + rows_per) - q_lo;
-    for (int t = tid; t < n_rows * (kD / 4); t += SH::kThreads) {
+    for (int t = tid; t < n_rows * (kD / 4); t += kThreadsTc) {
       const int qq = t / (kD / 4), d = (t % (kD / 4)) * 4;
       float mmax = -CUDART_INF_F;
       for (int r = 0; r < S; ++r) mmax = fmaxf(mmax, rows_l[r * rows_per + qq]);
@@ -895,15 +932,13 @@ cudaError_t attention_tc_set_attributes(int cache_dtype, bool split) {
 
 // The most splits, at least 2 and at most `wanted`, whose clusters are all resident at once: one
 // cluster in a second wave costs as much as the first wave. The occupancy counts clusters at one
-// CTA per SM; where two share an SM, s CTAs take the SMs of (s + 1) / 2 (32 clusters of 8 started
+// CTA per SM; two share an SM here, so s CTAs take the SMs of (s + 1) / 2 (32 clusters of 8 started
 // within 3.3 us of one another, against 15 that it counts for 8 and 36 for 4).
 // Split launches check every cache value, so a call that asks for splits keeps two.
 static int resident_splits(int wanted, int B, int n_heads, int cache_dtype) {
-  const int threads = cache_dtype == 1 ? Shape<false>::kThreads : Shape<true>::kThreads;
-  const int per_sm = attention_ctas_per_sm(cache_dtype);
   int s = wanted;
-  while (s > 2 && max_resident_clusters(tc_fn(cache_dtype, true), threads, static_cast<size_t>(tc_smem(cache_dtype)),
-                                        (s + per_sm - 1) / per_sm) < static_cast<long long>(B) * n_heads)
+  while (s > 2 && max_resident_clusters(tc_fn(cache_dtype, true), kThreadsTc, static_cast<size_t>(tc_smem(cache_dtype)),
+                                        (s + kCtasPerSm - 1) / kCtasPerSm) < static_cast<long long>(B) * n_heads)
     --s;
   return s;
 }
@@ -911,6 +946,13 @@ static int resident_splits(int wanted, int B, int n_heads, int cache_dtype) {
 cudaError_t launch_attention_tc(const AttnArgs& a_in, int B, int cache_dtype, cudaStream_t stream, bool pdl) {
   AttnArgs a = a_in;
   if (a.n_splits > 1) a.n_splits = resident_splits(a.n_splits, B, a.n_heads, cache_dtype);
+  // a long cache that starts in the last wave runs alone: 26 B/ns a CTA, so 1000 fp32 rows are 40 us
+  int dev = 0, sm_count = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
+  if (e != cudaSuccess) return e;
+  a.by_length = a.plan == nullptr && a.targs == nullptr && B > 1 && B <= kMaxByLength &&
+                static_cast<long long>(B) * a.n_heads * a.n_splits > static_cast<long long>(kCtasPerSm) * sm_count;
   CUtensorMap map_k{}, map_v{};
   a.param_maps = 0;
   // one layer's caches outside a tick: maps by value (the row count is not known here; a chunk
@@ -920,8 +962,7 @@ cudaError_t launch_attention_tc(const AttnArgs& a_in, int B, int cache_dtype, cu
       encode_cache_map(&map_v, a.v_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)))
     a.param_maps = 1;
   void* kargs[] = {&a, &map_k, &map_v};
-  const int threads = cache_dtype == 1 ? Shape<false>::kThreads : Shape<true>::kThreads;
-  return launch_ex(tc_fn(cache_dtype, a.n_splits > 1), dim3(a.n_splits, a.n_heads, B), dim3(threads),
+  return launch_ex(tc_fn(cache_dtype, a.n_splits > 1), dim3(a.n_splits, a.n_heads, B), dim3(kThreadsTc),
                    static_cast<size_t>(tc_smem(cache_dtype)), stream, pdl, kargs, 1, a.n_splits);
 }
 

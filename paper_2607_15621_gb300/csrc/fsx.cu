@@ -131,7 +131,7 @@ namespace {
 
 int attention_splits(const fsx_handle_s* h, int B) {
   const int work = B * h->cfg.n_heads;
-  const int s = (fsx::attention_ctas_per_sm(h->cfg.cache_dtype) * h->sm_count) / std::max(work, 1);  // one wave of CTAs
+  const int s = (fsx::kAttentionCtasPerSm * h->sm_count) / std::max(work, 1);  // one wave of CTAs
   return std::min(std::max(s, 1), 8);  // the splits merge inside one thread-block cluster
 }
 
@@ -322,7 +322,6 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
     a.out = h->o;
     a.out_stride = HD;
     a.lse = nullptr;
-    a.order = h->order;
     a.plan = h->plan;
     a.cache_maps = h->d_cache_maps;
     a.status = h->status;

@@ -62,11 +62,11 @@ struct AttnArgs {
   float* lse;                 // optional [B, H, n_q] natural log
   float* part_o;              // [B, H, S, 48, 128] when n_splits > 1
   float* part_lse;            // [B, H, S, 48]   (log2 domain)
-  const int* order;           // optional [B]: CTA row z works on vehicle order[z] (longest cache first)
   const AttnPlan* plan;       // optional [B] (tensor-core path): CTA row z works on plan[z]
   // optional (tensor-core path, with targs): [2 n_layers] TMA maps of the layers' K and V caches
   // (bf16 [rows, n_heads, 128]); whole 64-key chunks are then loaded by TMA
   const CUtensorMap* cache_maps;
+  int by_length;              // set by the launcher: CTA row z works on the vehicle with the z-th longest cache
   int param_maps;             // set by the launcher: maps of k_cache / v_cache are kernel arguments
   int* status;
 };
@@ -81,7 +81,7 @@ bool attention_tc_eligible(const AttnArgs& a, int n_splits);
 cudaError_t launch_attention_tc(const AttnArgs& a, int B, int cache_dtype, cudaStream_t stream, bool pdl);
 cudaError_t attention_tc_set_attributes(int cache_dtype, bool split);
 // CTAs of the tcgen05 path that share an SM
-constexpr int attention_ctas_per_sm(int cache_dtype) { return cache_dtype == 1 ? 2 : 1; }
+constexpr int kAttentionCtasPerSm = 2;
 
 // --------------------------------------------------------- embed / head
 struct EmbedArgs {

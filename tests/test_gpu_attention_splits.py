@@ -1,6 +1,6 @@
 """The tensor-core attention's key splits and fp32 caches at the edges of their tiling, through fsx_attention against
 the fp64 oracle: cache lengths around the 64-key chunks, splits without any cache key, one to 48 queries, one to 64 own
-keys, and the range check of every cache value that split and fp32 launches make.
+keys, launches of more than one wave (longest caches first) and the range check of every cache value that split and fp32 launches make.
 
 Tolerance, as a share of a row's largest entry. bf16 caches: q, k and the scores' operands are exact in fp16, P keeps 16
 bits, so the fp16 result's own rounding (2^-11 = 4.9e-4) dominates: 1e-3. fp32 caches: K and V are rounded to fp16 (2^-12
@@ -28,6 +28,19 @@ TOL = {"bf16": 1e-3, "fp32": 3e-3}
 ])
 def test_splits_and_dtypes(cache_dtype, n_splits, lengths, n_q, n_own):
     c = make(lengths, n_q=n_q, n_own=n_own, cache_dtype=cache_dtype, seed=n_splits * 31 + len(lengths))
+    out, lse = gpu_attention(c, n_splits)
+    ref, ref_lse = oracle_attention(c)
+    assert row_err(out, ref).max() <= TOL[cache_dtype]
+    assert np.abs(lse - ref_lse).max() <= 2e-3
+
+
+@pytest.mark.parametrize("cache_dtype", ["bf16", "fp32"])
+@pytest.mark.parametrize("n_splits,lengths", [
+    (1, [7, 64, 64, 0, 130, 1, 64, 129, 0, 200]),      # 320 CTAs, just over one wave: longest first, ties by index
+    (8, [5, 70, 70]), (1, [3 * (i * 37 % 128 // 4) for i in range(128)]), (1, [i % 3 for i in range(129)]),
+])
+def test_more_than_one_wave(cache_dtype, n_splits, lengths):
+    c = make(lengths, n_q=42 if len(lengths) < 100 else 3, n_own=10, cache_dtype=cache_dtype, seed=len(lengths))
     out, lse = gpu_attention(c, n_splits)
     ref, ref_lse = oracle_attention(c)
     assert row_err(out, ref).max() <= TOL[cache_dtype]
