@@ -1,6 +1,7 @@
 """The tensor-core attention's key splits and fp32 caches at the edges of their tiling, through fsx_attention against
 the fp64 oracle: cache lengths around the 64-key chunks, splits without any cache key, one to 48 queries, one to 64 own
-keys, launches of more than one wave (longest caches first) and the range check of every cache value that split and fp32 launches make.
+keys, launches of more than one wave (longest caches first), and the range check of every cache value that split and fp32
+launches make.
 
 Tolerance, as a share of a row's largest entry. bf16 caches: q, k and the scores' operands are exact in fp16, P keeps 16
 bits, so the fp16 result's own rounding (2^-11 = 4.9e-4) dominates: 1e-3. fp32 caches: K and V are rounded to fp16 (2^-12
