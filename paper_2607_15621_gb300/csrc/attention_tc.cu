@@ -1,4 +1,4 @@
-// Eq. 1 of Sec. 3.1 on the 5th-generation tensor cores: one CTA per (vehicle, head, key split)
+// Eq. 1 of Sec. 3.1 on the 5th-generation tensor cores: per (vehicle, head, key split) a CTA
 // computes softmax(Q [K_vlm ; K_ae]^T / sqrt(128)) [V_vlm ; V_ae] for the
 // expert's queries (at most 48, padded to an M = 64 tile) with a bf16 or fp32 backbone
 // cache, fp32 accumulation. S = Q K^T in fp16: the cache K rows are
@@ -20,15 +20,24 @@
 //   Row q of an M = 64 tile lives in lane (q mod 16) + 32 (q / 16).
 // The vehicle's cache keys are cut into 64-key chunks and the chunks into near-equal runs, one
 // per split; split 0 (never the longest run) takes the expert's own keys (fp16 as produced) as
-// its chunk 0 before its cache chunks. Chunk i sits in K / V slot i mod kSlots.
+// its chunk 0 before its cache chunks. The g-th chunk of a CTA sits in K / V slot g mod kSlots.
+//
+// Items: without splits a CTA works through up to 32 (vehicle, head) items, two CTAs per SM, one wave.
+// The chunks of its items are one stream for every warp role: the next item's first loads, queries and
+// S run under the softmax and the output of the one before. A CTA per item paid for start-up, output
+// and launch 4.9 of the 9.2 us of a 3-chunk item; with the smaller code below, 8 layers, before -> now:
+// a 40-frame clip (64-224 rows) 812 -> 730 us, 128 vehicles with 64-2048 rows 3996 -> 3800 (3985 where
+// such long items kept a CTA each), 16 with 96-480 rows 483 -> 480.
 //
 // Warp roles: warps 0-2 run the online softmax for query rows
-// 16 w .. 16 w + 15, two rows per thread; warp 3 lane 0 issues S and P V as their inputs become
-// ready; warps 4-5 stage and convert the K rows, warps 6-7 the V rows, two
-// chunks ahead. Two CTAs per SM. bf16 caches: whole chunks by TMA. fp32 caches: 16-key stages by
-// 16-byte copies, two in flight per tensor (32 KB a CTA), converted into the slot by the warp that
-// copied the rows: another CTA's stream then hides a start-up, which 64-key stages and one CTA per SM
-// cannot (24 vehicles with 16-1000 rows, 32 heads: 78 -> 76.8 us).
+// 16 w .. 16 w + 15, two rows per thread; warp 3 lane 0 loads the queries and issues S and P V as their
+// inputs become ready; warps 4-5 stage and convert the K rows, warps 6-7 the V rows, two
+// chunks ahead. Queries, own rows and whole bf16 chunks come by TMA; a short last bf16 chunk by 16-byte
+// copies; fp32 rows in 16-key stages by 16-byte copies, two in flight per tensor (32 KB a CTA), converted
+// into the slot by the warp that copied the rows.
+// Code size: the kernel is cold when a layer starts, its instructions come through a memory system
+// that the first chunks' loads keep busy, and every CTA waits for the same lines: at 92 KB the first
+// softmax chunk took 4.5 us on every SM at once (40-frame clip 769 us), at 43 KB 0.7 us (728).
 // Splits: the CTAs of one (vehicle, head) form a thread-block cluster and merge
 // (log-sum-exp weights) by pushing each split's normalised fp32 rows to the rank that owns them
 // through distributed shared memory. Split and fp32 launches check every cache value they stage
@@ -36,9 +45,9 @@
 // Measured against the mma.sync kernel of attention.cu, which split and fp32 launches ran before: a
 // tick of 4 vehicles with 0-700 bf16 rows, 8 layers, 2 splits: 740 -> 452 us; one vehicle with 2048
 // rows, 8 splits, Eq. 1 alone: 34 -> 27 us a call; 24 vehicles with 16-1000 fp32 rows, Eq. 1
-// alone: 104 -> 68 us a call (4.9 TB/s) with the order below.
-// Launches of more than one wave without a plan start the longest caches first (each CTA finds its
-// vehicle among at most 128 by counting; the 24 fp32 vehicles: 76.8 -> 67.7 us). A tick's plan is sorted already.
+// alone: 104 -> 66 us a call (5.0 TB/s) with the order below.
+// Launches of more than one wave without a plan take the longest caches first (each CTA sorts at most
+// 128 vehicles by counting; the 24 fp32 vehicles: 76.8 -> 67.7 us). A tick's plan is sorted already.
 // Every wait is bounded; a timeout raises the status word and the CTA drains its
 // MMAs before it frees the tensor memory.
 #include <cuda.h>
@@ -62,7 +71,9 @@ constexpr int kTmemCols = 256;         // S[2] x 64 + O 128
 constexpr uint32_t kColS = 0;    // S / P buffers at columns 0 and 64
 constexpr uint32_t kColO = 128;
 constexpr int kMaxClusterSplits = 8;
+constexpr int kMaxRounds = 32;     // items a CTA works on, at most (one lane prepares each)
 constexpr int kMaxByLength = 128;  // vehicles a launch without a plan sorts
+constexpr int kBoxBytes = kSlotKeys * 64 * 2;  // a TMA box: 64 rows of 64 values
 
 // shared-memory layout (bytes from the 1024-aligned base)
 constexpr int kQBytes = 64 * kD * 2;            // 16 KB
@@ -74,8 +85,9 @@ constexpr int kProdWarps = 2;                    // per tensor
 constexpr int kProdThreads = 32 * kProdWarps;
 constexpr int kThreadsTc = 32 * (kProdWarp0 + 2 * kProdWarps);
 constexpr int kCtasPerSm = kAttentionCtasPerSm;
-// barriers: kfull[3], kempty[3], vfull[3], vempty[3], sfull[2], pfull[2], pvdone[2], drain, ktma[3], vtma[3]
-constexpr int kNumBars = 25;
+// barriers: kfull[3], kempty[3], vfull[3], vempty[3], sfull[2], pfull[2], pvdone[2], drain, ktma[3], vtma[3],
+// qfull, qempty, oread
+constexpr int kNumBars = 28;
 template <bool F32>
 struct CacheType {
   using T = __nv_bfloat16;
@@ -92,7 +104,8 @@ struct Shape {
   static constexpr int kOffV = kOffK + kSlots * kSlotBytes;
   static constexpr int kOffRaw = kOffV + kSlots * kSlotBytes;  // [K, V][2]
   static constexpr int kOffBar = kOffRaw + (F32 ? 4 * kRawBytes : 0);
-  static constexpr int kSmem = kOffBar + kNumBars * 8 + 8 /*tmem slot + abort*/;
+  static constexpr int kOffItems = kOffBar + kNumBars * 8 + 16 /*tmem slot, abort, items*/;
+  static constexpr int kSmem = kOffItems + kMaxRounds * 16;
 };
 static_assert(kCtasPerSm * (Shape<false>::kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
 static_assert(kCtasPerSm * (Shape<true>::kSmem + 1024) <= 228 * 1024, "two CTAs per SM");
@@ -150,28 +163,27 @@ __device__ __forceinline__ void umma_f16_ta(uint32_t tmem_d, uint32_t tmem_a, ui
 
 __device__ __forceinline__ void fence_proxy_async() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
-// bounded wait that also gives up once another thread of the CTA gave up
+// bounded wait that also gives up once another thread of the CTA gave up. Written for size, as the
+// rest of the kernel is: its code is cold when a layer starts and arrives through a memory system
+// that the first chunks' loads keep busy. The timer's low word wraps after 4.3 s.
 __device__ __forceinline__ bool wait_bar(uint64_t* bar, uint32_t parity, int* status, volatile int* abort) {
   const uint32_t addr = smem_addr(bar);
-  unsigned long long t0 = 0;
-  for (uint32_t it = 0;; ++it) {
-    uint32_t done;
+  uint32_t t0 = 0;
+  for (;;) {
+    uint32_t done, now;
     asm volatile(
         "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
         : "=r"(done)
         : "r"(addr), "r"(parity)
         : "memory");
     if (done) return true;
-    if ((it & 63u) == 63u) {
-      if (*abort) return false;
-      const unsigned long long now = global_timer_ns();
-      if (t0 == 0) {
-        t0 = now;
-      } else if (now - t0 > kWaitLimitNs) {
-        set_status(status, kStatusTimeout);
-        *abort = 1;
-        return false;
-      }
+    if (*abort) return false;
+    asm volatile("mov.u32 %0, %%globaltimer_lo;" : "=r"(now));
+    if (t0 == 0) t0 = now | 1u;
+    if (now - t0 > kWaitLimitNs && now - t0 < 0x80000000u) {
+      set_status(status, kStatusTimeout);
+      *abort = 1;
+      return false;
     }
   }
 }
@@ -254,10 +266,33 @@ __device__ __forceinline__ void tma_load_cache(void* dst, const CUtensorMap* map
       : "memory");
 }
 
-// map_k, map_v: maps of the one layer's caches when p.cache_maps is NULL and p.param_maps is set
+// one 64-row x 64-dim box of a vehicle's queries or own rows (4-D map [B, rows, heads, 128]; rows past the
+// vehicle's are filled with zeros)
+__device__ __forceinline__ void tma_load_rows(void* dst, const CUtensorMap* map, int x, int head, int b,
+                                              uint64_t* bar) {
+  asm volatile(
+      "cp.async.bulk.tensor.4d.shared::cluster.global.tile.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], "
+      "[%6];" ::"r"(smem_addr(dst)),
+      "l"(map), "r"(x), "r"(head), "r"(0), "r"(b), "r"(smem_addr(bar))
+      : "memory");
+}
+__device__ __forceinline__ void tma_load_rows_pair(void* dst, const CUtensorMap* map, int head, int b, uint64_t* bar) {
+  mbar_arrive_expect_tx(bar, 2 * kBoxBytes);
+  tma_load_rows(dst, map, 0, head, b, bar);
+  tma_load_rows(static_cast<unsigned char*>(dst) + kBoxBytes, map, 64, head, b, bar);
+}
+
+__device__ __forceinline__ void prefetch_map(const CUtensorMap* map) {
+  asm volatile("prefetch.tensormap [%0];" ::"l"(map) : "memory");
+}
+
+// maps.k, maps.v: maps of the one layer's caches when p.cache_maps is NULL and p.param_maps is set
+struct AttnMaps {
+  CUtensorMap q, k_own, v_own, k, v;
+};
 template <bool F32, bool SPLIT>
 __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
-    attn_tc_kernel(const AttnArgs p, const __grid_constant__ CUtensorMap map_k, const __grid_constant__ CUtensorMap map_v) {
+    attn_tc_kernel(const AttnArgs p, const int n_vehicles, const __grid_constant__ AttnMaps maps) {
   using SH = Shape<F32>;
   using CT = typename CacheType<F32>::T;
   constexpr int kSlots = SH::kSlots;
@@ -266,22 +301,20 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
   const int tid = threadIdx.x;
   const int warp = tid >> 5;
   const int lane = tid & 31;
-  const int h = blockIdx.y;
   const int H = p.n_heads;
   const int S = SPLIT ? static_cast<int>(gridDim.x) : 1;     // the cluster spans the grid's x extent
   const int rank = SPLIT ? static_cast<int>(blockIdx.x) : 0;
-  const int has_own = rank == 0 ? 1 : 0;                     // chunk 0 holds the own keys
+  const int has_own = rank == 0 ? 1 : 0;                     // an item's chunk 0 holds the own keys
 
   pdl_launch_dependents();
+  if (tid == kMmaWarp * 32) prefetch_map(&maps.q);
+  if (tid == kProdWarp0 * 32) prefetch_map(&maps.k_own);
+  if (tid == (kProdWarp0 + kProdWarps) * 32) prefetch_map(&maps.v_own);
   pdl_wait();
   if ((smem_addr(smem) & 1023u) != 0u) {  // the swizzled operands need a 1024-byte aligned base
     if (tid == 0) set_status(p.status, kStatusDeviceArg);
     return;
   }
-  // Start-up is a chain of dependent global loads (vehicle, offsets, queries, own rows),
-  // each at the latency of a loaded memory system. The batched tick hands every CTA row
-  // its schedule entry (vehicle, first cache row, length: one load); the copies of the
-  // vehicle's queries and own keys / values are then in flight while the rest is read.
   const CT* kc;
   const CT* vc;
   if (p.targs != nullptr) {
@@ -290,26 +323,6 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
   } else {
     kc = static_cast<const CT*>(p.k_cache);
     vc = static_cast<const CT*>(p.v_cache);
-  }
-  AttnPlan plan_z{0, 0, 0};
-  if (p.plan != nullptr) plan_z = p.plan[blockIdx.z];
-  int b = p.plan != nullptr ? plan_z.b : static_cast<int>(blockIdx.z);
-  if (p.by_length) {  // this CTA's vehicle: the one with blockIdx.z longer caches before it (ties by index)
-    long long* len = reinterpret_cast<long long*>(smem + SH::kOffK);
-    int* pick = reinterpret_cast<int*>(len + kMaxByLength);
-    const int n = static_cast<int>(gridDim.z);
-    if (tid < n) len[tid] = p.offsets[tid + 1] - p.offsets[tid];
-    __syncthreads();
-    if (tid < n) {
-      const long long mine = len[tid];
-      int before = 0;
-#pragma unroll 4
-      for (int j = 0; j < n; ++j) before += len[j] > mine || (len[j] == mine && j < tid) ? 1 : 0;
-      if (before == static_cast<int>(blockIdx.z)) *pick = tid;
-    }
-    __syncthreads();
-    b = *pick;
-    __syncthreads();  // read before the slot is staged into
   }
 
   unsigned char* qt = smem + SH::kOffQ;
@@ -324,128 +337,169 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
   uint64_t* pfull = bars + 14;   // [2] P of a chunk written over its S
   uint64_t* pvdone = bars + 16;  // [2] P V of a chunk done (one per buffer)
   uint64_t* drain = bars + 18;   // every MMA of the CTA done
-  uint64_t* ktma = bars + 19;    // [3] a whole cache chunk's K rows landed by TMA
+  uint64_t* ktma = bars + 19;    // [3] a chunk's K rows landed by TMA
   uint64_t* vtma = bars + 22;    // [3] the same for V
+  uint64_t* qfull = bars + 25;   // an item's queries landed
+  uint64_t* qempty = bars + 26;  // every S of an item done with them
+  uint64_t* oread = bars + 27;   // an item's O read
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + kNumBars);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  volatile int* n_work = reinterpret_cast<volatile int*>(tmem_slot + 2);
+  struct Packed {  // an item as it lies in the table
+    long long row0;
+    int L;
+    uint32_t bh;
+  };
+  struct Item {
+    long long row0;  // this CTA's first cache row of the vehicle
+    int L, b, h, n;  // its number of cache keys; vehicle; head; chunks
+    int last;        // rows of the last cache chunk
+  };
+  Packed* table = reinterpret_cast<Packed*>(smem + SH::kOffItems);
+  static_assert(sizeof(Packed) == 16, "item table");
+  auto item = [&](int k) {
+    const Packed w = table[k];
+    const int n_cc = (w.L + kSlotKeys - 1) / kSlotKeys;
+    return Item{w.row0, w.L, static_cast<int>(w.bh >> 16), static_cast<int>(w.bh & 0xffffu), has_own + n_cc,
+                w.L - (n_cc - 1) * kSlotKeys};
+  };
 
-  // ---- producers' staging of chunk i (own rows fp16, cache rows bf16 converted later)
+  // ---- items: (vehicle, head) pairs, the vehicle's place in the schedule major. A CTA works on item
+  // k gridDim + (k even ? its index : its mirror image), k = 0, 1, ...: with the longest caches
+  // first the CTA of the longest item of a round gets the shortest of the next.
+  int* order = reinterpret_cast<int*>(smem + SH::kOffK);  // before a slot is staged into
+  if (p.by_length) {  // order[z]: the vehicle with z longer caches before it (ties by index)
+    long long* len = reinterpret_cast<long long*>(order + kMaxByLength);
+    if (tid < n_vehicles) len[tid] = p.offsets[tid + 1] - p.offsets[tid];
+    __syncthreads();
+    if (tid < n_vehicles) {
+      const long long mine = len[tid];
+      int before = 0;
+#pragma unroll 1
+      for (int j = 0; j < n_vehicles; ++j) before += len[j] > mine || (len[j] == mine && j < tid) ? 1 : 0;
+      order[before] = tid;
+    }
+    __syncthreads();
+  }
+  if (warp == 0) {  // lane k: the k-th item
+    const long long n_items = static_cast<long long>(n_vehicles) * H;
+    const int G = static_cast<int>(gridDim.x), c = static_cast<int>(blockIdx.x);
+    long long j = static_cast<long long>(lane) * G + ((lane & 1) ? G - 1 - c : c);
+    if (SPLIT) j = lane == 0 ? static_cast<long long>(blockIdx.z) * H + blockIdx.y : n_items;
+    bool valid = lane < kMaxRounds && j < n_items;
+    long long row0 = 0, len = 0;
+    int b = 0, h = 0;
+    if (valid) {
+      const int z = static_cast<int>(j) / H;
+      h = static_cast<int>(j) % H;
+      if (p.plan != nullptr) {  // written by the tick's first kernel: one 16-byte entry
+        const AttnPlan w = p.plan[z];
+        b = w.b;
+        row0 = w.lo;
+        len = w.len;
+      } else {
+        b = p.by_length ? order[z] : z;
+        row0 = p.offsets[b];
+        len = p.offsets[b + 1] - row0;
+      }
+      // never read outside the caller's cache: such a vehicle is reported and passed over
+      valid = row0 >= 0 && len >= 0 && row0 <= p.max_total && len <= p.max_total - row0 &&
+              len <= INT32_MAX - kSlotKeys && (len == 0 || (kc != nullptr && vc != nullptr));
+      if (!valid) set_status(p.status, kStatusDeviceArg);
+    }
+    if (SPLIT) {  // this split's run of whole chunks
+      const uint32_t n_cc = static_cast<uint32_t>((len + kSlotKeys - 1) / kSlotKeys);
+      const long long k_lo = n_cc * rank / S * static_cast<long long>(kSlotKeys);
+      const long long k_hi = min(len, n_cc * (rank + 1) / S * static_cast<long long>(kSlotKeys));
+      row0 += k_lo;
+      len = k_hi > k_lo ? k_hi - k_lo : 0;
+    }
+    const uint32_t mask = __ballot_sync(0xffffffffu, valid);
+    if (valid)
+      table[__popc(mask & ((1u << lane) - 1u))] =
+          Packed{row0, static_cast<int>(len), static_cast<uint32_t>(b) << 16 | static_cast<uint32_t>(h)};
+    if (lane == 0) *n_work = __popc(mask);
+  }
+  if (p.by_length) fence_proxy_async();  // the order lies where a slot is staged into
+
+  // ---- producers' staging
   const bool is_prod = warp >= kProdWarp0;
   const bool is_v = warp >= kProdWarp0 + kProdWarps;
   const int pw = warp & (kProdWarps - 1);  // warp within the tensor's staging warps
-  const int pt = pw * 32 + lane;               // thread within them
-  const int pu = pt & 15;                      // 16-byte unit of a 256-byte row
-  const int pr0 = pt >> 4;                     // rows pr0, pr0 + kRowStep, ...
+  const int pt = pw * 32 + lane;           // thread within them
+  const int pu = pt & 15;                  // 16-byte unit of a 256-byte row
+  const int pr0 = pt >> 4;                 // rows pr0, pr0 + kRowStep, ...
   constexpr int kRowStep = kProdThreads / 16;
   const size_t tok = static_cast<size_t>(H) * kD;
-  const __half* obase = (is_v ? p.v_own : p.k_own) + static_cast<size_t>(b) * p.n_own * p.own_stride + h * kD + pu * 8;
-  const CT* cbase = nullptr;             // this CTA's first cache row of the tensor (its head), set below
-  long long L = 0;                       // cache keys of this CTA
-  long long row0 = 0;                    // this CTA's first cache row, set below
   unsigned char* pslots = is_v ? vslot : kslot;
-  // Whole cache chunks (every cache chunk but a short last one) come by two TMA box loads
-  // issued by one thread of the tensor's warps (when the batched tick supplies the cache
-  // maps); the own keys and a short last chunk by 16-byte copies of every thread.
+  uint64_t* tbar = is_v ? vtma : ktma;
+  const CUtensorMap* omap = is_v ? &maps.v_own : &maps.k_own;
+  // Own keys and whole cache chunks (every cache chunk but a short last one) come by two TMA box
+  // loads issued by one thread of the tensor's warps; a short last chunk by 16-byte copies of every
+  // thread, zeros behind it.
   const CUtensorMap* tmap = nullptr;
   if (!F32) {
     if (p.cache_maps != nullptr && p.targs != nullptr)
       tmap = p.cache_maps + 2 * p.layer + (is_v ? 1 : 0);
     else if (p.param_maps)
-      tmap = is_v ? &map_v : &map_k;
+      tmap = is_v ? &maps.v : &maps.k;
   }
-  uint64_t* tbar = is_v ? vtma : ktma;
-  auto is_own = [&](int i) { return i < has_own; };
-  auto by_tma = [&](int i) {
-    return tmap != nullptr && i >= has_own && static_cast<long long>(i - has_own + 1) * kSlotKeys <= L;
+  // the producers' next chunk to issue: chunk ci of item ck
+  int ci = 0, ck = 0;
+  // bf16: stage chunk g of the CTA; returns its rows, bit 8 own keys, bit 9 by TMA
+  auto issue = [&](int g) {
+    unsigned char* slot = pslots + (g % kSlots) * kSlotBytes;
+    uint64_t* bar = tbar + g % kSlots;
+    const Item cur = item(ck);
+    int desc;
+    if (ci < has_own) {
+      desc = p.n_own | 0x300;
+      if (pt == 0) tma_load_rows_pair(slot, omap, cur.h, cur.b, bar);
+    } else {
+      const long long c0 = (ci - has_own) * static_cast<long long>(kSlotKeys);
+      const int rows = ci + 1 < cur.n ? kSlotKeys : cur.last;
+      desc = rows;
+      if (tmap != nullptr && rows == kSlotKeys) {
+        desc |= 0x200;
+        if (pt == 0) {
+          const int y = static_cast<int>(cur.row0 + c0);
+          mbar_arrive_expect_tx(bar, kSlotBytes);
+          tma_load_cache(slot, tmap, 0, cur.h, y, bar);
+          tma_load_cache(slot + kSlotBytes / 2, tmap, 64, cur.h, y, bar);
+        }
+      } else {
+        const CT* src = (is_v ? vc : kc) + (static_cast<size_t>(cur.row0 + c0) * H + cur.h) * kD + pu * 8;
+#pragma unroll 2
+        for (int m = 0; m < kSlotKeys / kRowStep; ++m) {
+          const int r = pr0 + kRowStep * m;
+          unsigned char* dst = slot + tile128_off(r, pu);
+          if (r < rows)
+            cp_async_16(smem_addr(dst), src + static_cast<size_t>(r) * tok);
+          else
+            *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);  // keys past the range: finite zeros
+        }
+      }
+    }
+    cp_async_commit();  // one group per chunk, empty behind a TMA load
+    if (++ci == cur.n) {
+      ci = 0;
+      ++ck;
+    }
+    return desc;
   };
-  // the TMA chunks follow the own chunk, so slot s = i mod kSlots sees them in order from its
-  // first one (i = kSlots for slot 0 behind an own chunk): the phase of chunk i on its slot's barrier
-  auto tma_parity = [&](int i) {
-    return static_cast<uint32_t>((i / kSlots - (has_own != 0 && i % kSlots == 0 ? 1 : 0)) & 1);
-  };
-  auto chunk_rows = [&](int i) {
-    return is_own(i) ? p.n_own
-                     : static_cast<int>(min(static_cast<long long>(kSlotKeys),
-                                            L - (i - has_own) * static_cast<long long>(kSlotKeys)));
-  };
-  // fp32: raw stage t (keys 16 t .. of this CTA's run), one warp instruction a row; row r of a stage
-  // is the warp's that has r mod kProdWarps == pw. Past the run's end an empty group.
-  auto issue_raw = [&](int t) {
-    const int rows = static_cast<int>(min(static_cast<long long>(kRawKeys), L - static_cast<long long>(t) * kRawKeys));
+  // fp32: raw stage t of an item (keys 16 t .. of its cache rows), one warp instruction a row; row r of a
+  // stage is the warp's that has r mod kProdWarps == pw. Past the item's end an empty group.
+  auto issue_raw = [&](const Item& cur, int t) {
+    const int rows = static_cast<int>(
+        min(static_cast<long long>(kRawKeys), cur.L - static_cast<long long>(t) * kRawKeys));
     const uint32_t raw = smem_addr(smem + SH::kOffRaw + ((is_v ? 2 : 0) + (t & 1)) * kRawBytes) + lane * 16;
-    const CT* src = cbase + static_cast<size_t>(t) * kRawKeys * tok + lane * 4;
+    const size_t row = static_cast<size_t>(cur.row0 + t * static_cast<long long>(kRawKeys));
+    const CT* src = (is_v ? vc : kc) + (row * H + cur.h) * kD + lane * 4;
 #pragma unroll
     for (int r = pw; r < kRawKeys; r += kProdWarps)
       if (r < rows) cp_async_16(raw + r * (kD * 4), src + static_cast<size_t>(r) * tok);
     cp_async_commit();
   };
-  auto issue = [&](int i) {
-    unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
-    const int rows = chunk_rows(i);
-    const long long c0 = (i - has_own) * static_cast<long long>(kSlotKeys);
-    if (by_tma(i)) {
-      if (pt == 0) {
-        uint64_t* bar = tbar + i % kSlots;
-        const int y = static_cast<int>(row0 + c0);
-        mbar_arrive_expect_tx(bar, kSlotBytes);
-        tma_load_cache(slot, tmap, 0, h, y, bar);
-        tma_load_cache(slot + kSlotBytes / 2, tmap, 64, h, y, bar);
-      }
-      cp_async_commit();  // an empty group keeps one group per chunk
-      return;
-    }
-#pragma unroll 8
-    for (int m = 0; m < kSlotKeys / kRowStep; ++m) {
-      const int r = pr0 + kRowStep * m;
-      unsigned char* dst = slot + tile128_off(r, pu);
-      if (r < rows) {
-        const void* src = is_own(i) ? static_cast<const void*>(obase + static_cast<size_t>(r) * p.own_stride)
-                                    : static_cast<const void*>(cbase + static_cast<size_t>(c0 + r) * tok + pu * 8);
-        cp_async_16(smem_addr(dst), src);
-      } else {
-        *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);  // keys past the range: finite zeros
-      }
-    }
-    cp_async_commit();
-  };
-  // queries: 64 rows x 16 units, rows >= n_q zero (one copy group per thread)
-  for (int i = tid; i < 64 * 16; i += kThreadsTc) {
-    const int r = i >> 4;
-    const int u = i & 15;
-    unsigned char* dst = qt + tile128_off(r, u);
-    if (r < p.n_q)
-      cp_async_16(smem_addr(dst), p.q + (static_cast<size_t>(b) * p.n_q + r) * p.q_stride + h * kD + u * 8);
-    else
-      *reinterpret_cast<uint4*>(dst) = make_uint4(0u, 0u, 0u, 0u);
-  }
-  cp_async_commit();
-  if (is_prod && has_own != 0) issue(0);  // own keys / values
-
-  long long o_lo, o_hi;
-  if (p.plan != nullptr) {
-    o_lo = plan_z.lo;
-    o_hi = o_lo + plan_z.len;  // a length of -1 fails the check below
-  } else {
-    const int64_t* offs = p.targs != nullptr ? p.targs->offsets : p.offsets;
-    const int64_t* starts = p.targs != nullptr ? p.targs->starts : nullptr;
-    o_lo = starts != nullptr ? starts[b] : offs[b];
-    o_hi = o_lo + (offs[b + 1] - offs[b]);
-  }
-  if (o_lo < 0 || o_hi < o_lo || o_hi > p.max_total || (o_hi > o_lo && (kc == nullptr || vc == nullptr))) {
-    cp_async_wait<0>();  // the query / own-row copies land before the CTA leaves
-    set_status(p.status, kStatusDeviceArg);  // never read outside the caller's cache
-    return;
-  }
-  L = o_hi - o_lo;
-  row0 = o_lo;
-  if (SPLIT) {  // this split's run of whole chunks
-    const long long n_cc = (L + kSlotKeys - 1) / kSlotKeys;
-    const long long k_lo = n_cc * rank / S * kSlotKeys, k_hi = min(L, n_cc * (rank + 1) / S * kSlotKeys);
-    row0 = o_lo + k_lo;
-    L = k_hi > k_lo ? k_hi - k_lo : 0;
-  }
-  const int n_chunks = has_own + static_cast<int>((L + kSlotKeys - 1) / kSlotKeys);  // 0: a split without keys
-  cbase = (is_v ? vc : kc) + (static_cast<size_t>(row0) * H + h) * kD;
 
   if (tid == 0) {
     for (int i = 0; i < kSlots; ++i) {
@@ -462,56 +516,37 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
       mbar_init(pvdone + i, 1);
     }
     mbar_init(drain, 1);
-    // a kernel before this one has already abandoned the tick: this CTA stops below
-    *abort = *reinterpret_cast<volatile int*>(p.status) != 0 ? 1 : 0;
+    mbar_init(qempty, 1);
+    mbar_init(oread, kSoftmaxWarps * 32);
+    // a kernel before this one has already abandoned the tick: this CTA stops below (outside a tick only
+    // this launch sets the word, and the other vehicles' rows are still written)
+    *abort = p.targs != nullptr && *reinterpret_cast<volatile int*>(p.status) != 0 ? 1 : 0;
   }
   if (warp == kMmaWarp) {
+    if (lane == 0) mbar_init(qfull, 1);
+    __syncwarp();
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
                  "r"(kTmemCols)
                  : "memory");
     asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
-  }
-  const int n_first = min(n_chunks, 2);  // chunks whose loads are issued up front
-  if (is_prod) {  // the first cache chunks; then wait for this thread's query copies
-    if (pt == 0 && tmap != nullptr) {  // the TMA barriers, before the first TMA chunk; read after the CTA barrier
-      for (int i = 0; i < kSlots; ++i) mbar_init(tbar + i, 1);
-      fence_proxy_async();
-    }
-    if (F32) {
-      issue_raw(0);
-      issue_raw(1);
-      if (has_own != 0)
-        cp_async_wait<3>();
-      else
-        cp_async_wait<2>();
-    } else {
-      for (int i = has_own; i < n_first; ++i) issue(i);
-      if (n_first == 2)
-        cp_async_wait<2>();
-      else if (n_first == 1)
-        cp_async_wait<1>();
-      else
-        cp_async_wait<0>();
-    }
-  } else {
-    cp_async_wait<0>();
+  } else if (is_prod && pt < kSlots) {
+    mbar_init(tbar + pt, 1);
   }
   fence_proxy_async();
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *reinterpret_cast<volatile uint32_t*>(tmem_slot);
-  if (*abort) {  // the tick was abandoned before this kernel: no MMA was issued
-    cp_async_wait<0>();
-    if (is_prod && pt == 0)
-      for (int i = has_own; i < n_first; ++i)  // the first chunks landed
-        if (by_tma(i)) mbar_wait(tbar + i % kSlots, tma_parity(i), p.status);
+  const int n_my = *n_work;
+  if (*abort || n_my == 0) {  // the tick was abandoned before this kernel, or no vehicle is valid: nothing was issued
     if (SPLIT) {  // the other splits may not have seen the status yet: they push their rows here
       cluster_barrier();
       cluster_barrier();
     }
-    if (warp == kMmaWarp)
+    if (warp == kMmaWarp) {
+      __syncwarp();
       asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" ::"r"(tmem), "r"(kTmemCols) : "memory");
+    }
     return;
   }
 
@@ -522,54 +557,74 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
       const uint32_t id_pv_own = idesc_f16_mn(64, kD, true);       // fp16 P, fp16 own V
       const uint32_t id_pv = idesc_f16_mn(64, kD, true) | (1u << 7) | (1u << 10);  // bf16 P, bf16 cache V
       const uint32_t aq = smem_addr(qt);
-      auto issue_s = [&](int i) {  // S of chunk i into buffer i & 1
-        const uint32_t d = tmem + kColS + (i & 1) * kSlotKeys;
-        const uint32_t kb = smem_addr(kslot + (i % kSlots) * kSlotBytes);
+      auto issue_s = [&](int g) {  // S of chunk g of the CTA into buffer g & 1
+        const uint32_t d = tmem + kColS + (g & 1) * kSlotKeys;
+        const uint32_t kb = smem_addr(kslot + (g % kSlots) * kSlotBytes);
 #pragma unroll
         for (int kk = 0; kk < 8; ++kk) {
           const uint32_t off = (kk >> 2) * 8192 + (kk & 3) * 32;
           umma_f16(d, sw128_desc(aq + off), sw128_desc(kb + off), id_s, kk > 0 ? 1u : 0u);
         }
-        umma_commit(kempty + (i % kSlots));
-        umma_commit(sfull + (i & 1));
+        umma_commit(kempty + (g % kSlots));
+        umma_commit(sfull + (g & 1));
       };
-      auto issue_pv = [&](int i) {  // O (+)= P V of chunk i, P from tensor memory
-        const uint32_t pa = tmem + kColS + (i & 1) * kSlotKeys;
-        const uint32_t vb = smem_addr(vslot + (i % kSlots) * kSlotBytes);
-        const uint32_t idv = F32 || is_own(i) ? id_pv_own : id_pv;
+      auto issue_pv = [&](int g, bool first) {  // O (+)= P V of chunk g, P from tensor memory
+        const uint32_t pa = tmem + kColS + (g & 1) * kSlotKeys;
+        const uint32_t vb = smem_addr(vslot + (g % kSlots) * kSlotBytes);
+        const uint32_t idv = F32 || (first && has_own != 0) ? id_pv_own : id_pv;
 #pragma unroll
         for (int kk = 0; kk < 4; ++kk) {  // 16 keys = 8 columns of packed fp16 pairs
           const uint64_t bd = sw128_desc_mn(vb + kk * 2048, 8192, 1024);
-          umma_f16_ta(tmem + kColO, pa + kk * 8, bd, idv, (i > 0 || kk > 0) ? 1u : 0u);  // P_hi
-          umma_f16_ta(tmem + kColO, pa + kSlotKeys / 2 + kk * 8, bd, idv, 1u);          // P_lo
+          umma_f16_ta(tmem + kColO, pa + kk * 8, bd, idv, (!first || kk > 0) ? 1u : 0u);  // P_hi
+          umma_f16_ta(tmem + kColO, pa + kSlotKeys / 2 + kk * 8, bd, idv, 1u);            // P_lo
         }
-        umma_commit(vempty + (i % kSlots));
-        umma_commit(pvdone + (i & 1));
+        umma_commit(vempty + (g % kSlots));
+        umma_commit(pvdone + (g & 1));
       };
-      // S(ns) and P V(npv) are issued as soon as their inputs are ready: S(ns) needs
-      // its K rows and P V(ns - 2) done with the buffer it overwrites, P V(npv) needs
-      // P(npv) and its V rows. Each test is at most one phase behind its barrier.
-      int ns = 0, npv = 0;
+      // S(gs) and P V(gp) are issued as soon as their inputs are ready: S(gs) needs its item's
+      // queries, its K rows and P V(gs - 2) done with the buffer it overwrites; P V(gp) needs P(gp),
+      // its V rows and, as an item's first, the O of the item before read. An item's queries are
+      // loaded once the last S of the item before is done with theirs. Each test is at most one
+      // phase behind its barrier.
+      int k = 0, i = 0, kq = -1;        // S(gs) is chunk i of item k; queries loaded up to item kq
+      int n = item(0).n;
+      int gs = 0, gp = 0, kp = -1;      // P V(gp - 1) is of item kp
+      uint32_t firsts = 0;              // bit g & 31: chunk g is an item's first
       unsigned long long t_idle = 0;
-      for (uint32_t it = 0; npv < n_chunks; ++it) {
+      for (uint32_t spin = 0; i < n || gp < gs; ++spin) {
         bool progressed = false;
-        if (ns < n_chunks && (ns < 2 || npv >= ns - 1) && test_bar(kfull + (ns % kSlots), (ns / kSlots) & 1) &&
-            (ns < 2 || test_bar(pvdone + (ns & 1), ((ns - 2) >> 1) & 1))) {
-          tc_fence_after();
-          issue_s(ns);
-          ++ns;
+        if (kq < k && i < n && (k == 0 || test_bar(qempty, (k - 1) & 1))) {
+          tma_load_rows_pair(qt, &maps.q, item(k).h, item(k).b, qfull);
+          kq = k;
           progressed = true;
         }
-        if (npv < ns && test_bar(pfull + (npv & 1), (npv >> 1) & 1) &&
-            test_bar(vfull + (npv % kSlots), (npv / kSlots) & 1)) {
+        if (i < n && kq == k && (gs < 2 || gp >= gs - 1) && test_bar(kfull + (gs % kSlots), (gs / kSlots) & 1) &&
+            (gs < 2 || test_bar(pvdone + (gs & 1), ((gs - 2) >> 1) & 1)) && (i > 0 || test_bar(qfull, k & 1))) {
           tc_fence_after();
-          issue_pv(npv);
-          ++npv;
+          issue_s(gs);
+          firsts = (firsts & ~(1u << (gs & 31))) | ((i == 0 ? 1u : 0u) << (gs & 31));
+          ++gs;
+          if (++i == n) {
+            umma_commit(qempty);
+            i = 0;
+            n = ++k < n_my ? item(k).n : 0;
+          }
           progressed = true;
+        }
+        if (gp < gs && test_bar(pfull + (gp & 1), (gp >> 1) & 1) &&
+            test_bar(vfull + (gp % kSlots), (gp / kSlots) & 1)) {
+          const bool first = ((firsts >> (gp & 31)) & 1u) != 0u;
+          if (!first || kp < 0 || test_bar(oread, kp & 1)) {
+            tc_fence_after();
+            issue_pv(gp, first);
+            kp += first ? 1 : 0;
+            ++gp;
+            progressed = true;
+          }
         }
         if (progressed) {
           t_idle = 0;
-        } else if ((it & 63u) == 63u) {
+        } else if ((spin & 63u) == 63u) {
           if (*abort) break;
           const unsigned long long now = global_timer_ns();
           if (t_idle == 0) {
@@ -583,32 +638,47 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
       }
       umma_commit(drain);  // completes once every MMA issued above has (waited on even after an abort)
       mbar_wait(drain, 0, p.status);
+      if (kq >= 0) mbar_wait(qfull, kq & 1, p.status);  // after an abort the last queries may still be on their way
     }
     __syncwarp();
   } else if (is_prod) {
     // ---------------------------------------------------------------- producers
-    // per chunk i: wait for its rows, convert cache rows bf16 -> fp16 in place (each
-    // thread the units it copied), signal, then refill the slot of chunk i - 1 with
-    // chunk i + 2 once the MMAs released it
     uint64_t* full = is_v ? vfull : kfull;
     uint64_t* empty = is_v ? vempty : kempty;
     bool ok = true;
-    int issued = n_first;  // chunks whose loads were issued
     uint32_t range = 0;    // fp32: largest magnitudes of the staged values; bf16: bits set by out-of-range ones
-    int i = 0;
-    for (; ok && i < n_chunks; ++i) {
-      unsigned char* slot = pslots + (i % kSlots) * kSlotBytes;
-      if (F32) {
-        if (is_own(i)) {
-          cp_async_wait<2>();  // the two raw stages behind it stay in flight
-        } else {               // raw rows -> fp16 slot, once its previous chunk is consumed
-          ok = wait_bar(empty + i % kSlots, (i / kSlots) & 1, p.status, abort);
+    uint32_t tphase = 0;   // bit s: parity of slot s's next TMA chunk
+    if (F32) {
+      // per item: own keys by TMA, then per cache chunk four raw stages converted into the slot
+      int g = 0;
+      for (int k = 0; k < n_my; ++k) {
+        const Item cur = item(k);
+#pragma unroll 1
+        for (int t = 0; t < 2; ++t) issue_raw(cur, t);
+        if (has_own != 0) {
+          ok = wait_bar(empty + g % kSlots, (g / kSlots) & 1, p.status, abort);
           if (!ok) break;
-          const int rows = chunk_rows(i);
+          if (pt == 0) tma_load_rows_pair(pslots + (g % kSlots) * kSlotBytes, omap, cur.h, cur.b, tbar + g % kSlots);
+          ok = wait_bar(tbar + g % kSlots, (tphase >> (g % kSlots)) & 1u, p.status, abort);
+          if (!ok) {
+            if (pt == 0) mbar_wait(tbar + g % kSlots, (tphase >> (g % kSlots)) & 1u, p.status);
+            break;
+          }
+          tphase ^= 1u << (g % kSlots);
+          mbar_arrive(full + (g % kSlots));
+          ++g;
+        }
+        const int n_cc = cur.n - has_own;
+        for (int c = 0; c < n_cc; ++c, ++g) {  // raw rows -> fp16 slot, once its previous chunk is consumed
+          unsigned char* slot = pslots + (g % kSlots) * kSlotBytes;
+          ok = wait_bar(empty + g % kSlots, (g / kSlots) & 1, p.status, abort);
+          if (!ok) break;
+          const int rows = c + 1 < n_cc ? kSlotKeys : cur.last;
           const int u = lane & 15;
           const int sw = (lane >> 2) & 1;  // the two 16-byte reads of a unit in an order that spreads the banks
+#pragma unroll 1
           for (int st = 0; st < kRawPerChunk; ++st) {
-            const int t = (i - has_own) * kRawPerChunk + st;
+            const int t = c * kRawPerChunk + st;
             cp_async_wait<1>();  // stage t landed, t + 1 in flight
             __syncwarp();        // the warp's copies of its rows
             const unsigned char* raw = smem + SH::kOffRaw + ((is_v ? 2 : 0) + (t & 1)) * kRawBytes;
@@ -626,64 +696,91 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
               *reinterpret_cast<uint4*>(slot + tile128_off(st * kRawKeys + r, u)) = out;
             }
             __syncwarp();  // the raw rows are read before they are refilled
-            issue_raw(t + 2);
+            issue_raw(cur, t + 2);
+          }
+          fence_proxy_async();
+          mbar_arrive(full + (g % kSlots));
+        }
+        if (!ok) break;
+      }
+      flag_range(p.status, range);
+      cp_async_wait<0>();
+    } else {
+      // per chunk g: wait for its rows, convert cache K rows bf16 -> fp16 in place (each thread the
+      // units it copied), signal. Up to two chunks behind it, of this item or the next, are staged:
+      // g + 1 before g is waited for, g + 2 once the MMAs have released the slot of g - 1.
+      int g = 0, staged = 0;
+      int d0 = -1, d1 = -1, d2 = -1;  // chunks g, g + 1, g + 2 as staged; -1: not staged
+      for (;;) {
+        if (ck < n_my && item(ck).n > 0 && staged < g + 3) {
+          uint64_t* bar = empty + staged % kSlots;
+          const uint32_t parity = (staged / kSlots) & 1;
+          bool free;
+          if (staged < g + 2) {
+            free = ok = wait_bar(bar, parity, p.status, abort);
+            if (!ok) break;
+          } else {
+            free = __all_sync(0xffffffffu, test_bar(bar, parity));
+          }
+          if (free) {
+            const int d = issue(staged);
+            if (staged == g) d0 = d;
+            else if (staged == g + 1) d1 = d;
+            else d2 = d;
+            ++staged;
+            if (staged < g + 3) continue;
+          }
+        }
+        if (d0 < 0) break;
+        if (d2 >= 0) cp_async_wait<2>();
+        else if (d1 >= 0) cp_async_wait<1>();
+        else cp_async_wait<0>();
+        unsigned char* slot = pslots + (g % kSlots) * kSlotBytes;
+        if (d0 & 0x200) {
+          ok = wait_bar(tbar + g % kSlots, (tphase >> (g % kSlots)) & 1u, p.status, abort);
+          if (!ok) break;
+          tphase ^= 1u << (g % kSlots);
+        }
+        if (!(d0 & 0x100) && (!is_v || kCheck)) {  // a cache chunk: K rows -> fp16 (V stays bf16)
+#pragma unroll 1
+          for (int m0 = 0; m0 < kSlotKeys / kRowStep; m0 += 8) {
+            uint4 v[8];
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+              v[m] = *reinterpret_cast<const uint4*>(slot + tile128_off(pr0 + kRowStep * (m0 + m), pu));
+            if (kCheck) {
+#pragma unroll
+              for (int m = 0; m < 8; ++m)
+                range |= bf16x2_out_of_range(v[m].x) | bf16x2_out_of_range(v[m].y) | bf16x2_out_of_range(v[m].z) |
+                         bf16x2_out_of_range(v[m].w);
+            }
+            if (!is_v) {
+#pragma unroll
+              for (int m = 0; m < 8; ++m)
+                *reinterpret_cast<uint4*>(slot + tile128_off(pr0 + kRowStep * (m0 + m), pu)) =
+                    make_uint4(bf16x2_to_half2(v[m].x), bf16x2_to_half2(v[m].y), bf16x2_to_half2(v[m].z),
+                               bf16x2_to_half2(v[m].w));
+            }
           }
         }
         fence_proxy_async();
-        mbar_arrive(full + (i % kSlots));
-        continue;
+        mbar_arrive(full + (g % kSlots));
+        d0 = d1;
+        d1 = d2;
+        d2 = -1;
+        ++g;
       }
-      if (i + 1 < n_chunks) cp_async_wait<1>();
-      else cp_async_wait<0>();
-      if (by_tma(i)) {
-        ok = wait_bar(tbar + i % kSlots, tma_parity(i), p.status, abort);
-        if (!ok) break;
-      }
-      // refill first when the slot of chunk i - 1 is already free (the warp agrees on it)
-      bool refilled = false;
-      if (i + 2 < n_chunks) {
-        refilled = __all_sync(0xffffffffu, test_bar(empty + ((i + 2) % kSlots), ((i + 2) / kSlots) & 1));
-        if (refilled) {
-          issue(i + 2);
-          issued = i + 3;
+      if (!ok && pt == 0) {  // after an abort: the TMA chunks issued but not consumed land before the CTA leaves
+#pragma unroll 1
+        for (int j = 0; j < 3; ++j) {
+          const int d = j == 0 ? d0 : (j == 1 ? d1 : d2);
+          const int sl = (g + j) % kSlots;
+          if (d >= 0 && (d & 0x200)) mbar_wait(tbar + sl, (tphase >> sl) & 1u, p.status);
         }
       }
-      if (!is_own(i) && (!is_v || kCheck)) {  // cache K rows -> fp16 (V stays bf16): every read before the first write
-        uint4 v[kSlotKeys / kRowStep];
-#pragma unroll
-        for (int m = 0; m < kSlotKeys / kRowStep; ++m)
-          v[m] = *reinterpret_cast<const uint4*>(slot + tile128_off(pr0 + kRowStep * m, pu));
-        if (kCheck) {
-#pragma unroll
-          for (int m = 0; m < kSlotKeys / kRowStep; ++m)
-            range |= bf16x2_out_of_range(v[m].x) | bf16x2_out_of_range(v[m].y) | bf16x2_out_of_range(v[m].z) |
-                     bf16x2_out_of_range(v[m].w);
-        }
-        if (!is_v) {
-#pragma unroll
-          for (int m = 0; m < kSlotKeys / kRowStep; ++m)
-            *reinterpret_cast<uint4*>(slot + tile128_off(pr0 + kRowStep * m, pu)) =
-                make_uint4(bf16x2_to_half2(v[m].x), bf16x2_to_half2(v[m].y), bf16x2_to_half2(v[m].z),
-                           bf16x2_to_half2(v[m].w));
-        }
-      }
-      fence_proxy_async();
-      mbar_arrive(full + (i % kSlots));
-      if (i + 2 < n_chunks && !refilled) {
-        ok = wait_bar(empty + ((i + 2) % kSlots), ((i + 2) / kSlots) & 1, p.status, abort);
-        if (ok) {
-          issue(i + 2);
-          issued = i + 3;
-        }
-      }
+      if (SPLIT && range != 0) set_status(p.status, kStatusRange);
+      cp_async_wait<0>();
     }
-    if (F32) flag_range(p.status, range);
-    else if (SPLIT && range != 0) set_status(p.status, kStatusRange);
-    cp_async_wait<0>();
-    // after an abort: the TMA chunks issued but not consumed land before the CTA leaves
-    if (pt == 0)
-      for (int j = i; j < issued; ++j)
-        if (by_tma(j)) mbar_wait(tbar + j % kSlots, tma_parity(j), p.status);
     __syncwarp();
   } else {
     // ---------------------------------------------------------------- softmax rows
@@ -698,15 +795,24 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
     const int rbw = ra + 8;
     const uint32_t lane_base = static_cast<uint32_t>(warp * 32) << 16;
     const float scale_log2 = 1.4426950408889634f * rsqrtf(static_cast<float>(kD));
+    const bool va = ra < p.n_q;
+    const bool vb = rbw < p.n_q;
+    bool ok = true;
+    int g0 = 0;  // item k starts with chunk g0 of the CTA
+#pragma unroll 1
+    for (int k = 0; k < n_my; ++k) {
+    const int n = item(k).n;
     float m_run[2] = {-CUDART_INF_F, -CUDART_INF_F};
     float l_run[2] = {0.f, 0.f};
-    bool ok = true;
-    for (int i = 0; i < n_chunks; ++i) {
-      const int valid = chunk_rows(i);
-      ok = wait_bar(sfull + (i & 1), (i >> 1) & 1, p.status, abort);
+#pragma unroll 1
+    for (int i = 0; i < n; ++i) {
+      const int g = g0 + i;
+      const bool own = i < has_own;
+      const int valid = own ? p.n_own : (i + 1 < n ? kSlotKeys : item(k).last);
+      ok = wait_bar(sfull + (g & 1), (g >> 1) & 1, p.status, abort);
       if (!ok) break;
       tc_fence_after();
-      const uint32_t sbuf = tmem + lane_base + kColS + (i & 1) * kSlotKeys;
+      const uint32_t sbuf = tmem + lane_base + kColS + (g & 1) * kSlotKeys;
       uint32_t sv[32];  // [g][row a: 2 keys, row b: 2 keys]
       tmem_ld_16x256b_x8(sbuf, sv);
       float s[2][16];   // [row][g * 2 + e] for key 8 g + 2 t4 + e
@@ -756,29 +862,34 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
         float r4[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
-          const float p0 = ex2_approx(fmaf(s[r][2 * g], scale_log2, nm));
-          const float p1 = ex2_approx(fmaf(s[r][2 * g + 1], scale_log2, nm));
-          r4[g & 3] += p0 + p1;
-          uint32_t hi, lo;
-          if (F32 || is_own(i)) {  // fp16 like the V rows
-            hi = pack_half2(p0, p1);
-            const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&hi));
-            lo = pack_half2(p0 - f.x, p1 - f.y);
-          } else {  // bf16 cache chunks: bf16 like the V rows
-            hi = pack_bf16x2(p0, p1);
-            lo = pack_bf16x2(p0 - __uint_as_float(hi << 16), p1 - __uint_as_float(hi & 0xffff0000u));
-          }
-          ph[2 * g + r] = hi;
-          pl[2 * g + r] = lo;
+          s[r][2 * g] = ex2_approx(fmaf(s[r][2 * g], scale_log2, nm));
+          s[r][2 * g + 1] = ex2_approx(fmaf(s[r][2 * g + 1], scale_log2, nm));
+          r4[g & 3] += s[r][2 * g] + s[r][2 * g + 1];
         }
         float rs = (r4[0] + r4[1]) + (r4[2] + r4[3]);
         rs += __shfl_xor_sync(0xffffffffu, rs, 1);
         rs += __shfl_xor_sync(0xffffffffu, rs, 2);
         l_run[r] = l_run[r] * alpha[r] + rs;
       }
+      if (F32 || own) {  // fp16 like the V rows
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const float p0 = s[e & 1][e & ~1], p1 = s[e & 1][e | 1];
+          ph[e] = pack_half2(p0, p1);
+          const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&ph[e]));
+          pl[e] = pack_half2(p0 - f.x, p1 - f.y);
+        }
+      } else {  // bf16 cache chunks: bf16 like the V rows
+#pragma unroll
+        for (int e = 0; e < 16; ++e) {
+          const float p0 = s[e & 1][e & ~1], p1 = s[e & 1][e | 1];
+          ph[e] = pack_bf16x2(p0, p1);
+          pl[e] = pack_bf16x2(p0 - __uint_as_float(ph[e] << 16), p1 - __uint_as_float(ph[e] & 0xffff0000u));
+        }
+      }
       if (any_grow && i > 0) {
         // rescale this warp's O rows once P V of the previous chunk is done
-        ok = wait_bar(pvdone + ((i - 1) & 1), ((i - 1) >> 1) & 1, p.status, abort);
+        ok = wait_bar(pvdone + ((g - 1) & 1), ((g - 1) >> 1) & 1, p.status, abort);
         if (!ok) break;
         tc_fence_after();
 #pragma unroll 1
@@ -797,17 +908,19 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
       tmem_st_16x128b_x8(sbuf + kSlotKeys / 2, pl);
       asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
       tc_fence_before();
-      mbar_arrive(pfull + (i & 1));
+      mbar_arrive(pfull + (g & 1));
     }
-    ok = ok && wait_bar(drain, 0, p.status, abort);  // every P V done
+    if (!ok) break;
+    g0 += n;
+    // the item's last P V done, and with it those before
+    if (n > 0) ok = wait_bar(pvdone + ((g0 - 1) & 1), ((g0 - 1) >> 1) & 1, p.status, abort);
+    if (!ok) break;
     tc_fence_after();
     const float inv[2] = {l_run[0] > 0.f ? 1.f / l_run[0] : 0.f, l_run[1] > 0.f ? 1.f / l_run[1] : 0.f};
-    const bool va = ra < p.n_q;
-    const bool vb = rbw < p.n_q;
     // A cache key beyond the fp16 range became an infinity here; where it raised a
     // score to +inf (or NaN) the row's sum is NaN: report it, the tick is abandoned.
     // (A key whose scores all fell to -inf carries weight 0, as the exact value would.)
-    if (ok && ((va && !(l_run[0] == l_run[0])) || (vb && !(l_run[1] == l_run[1])))) set_status(p.status, kStatusRange);
+    if (((va && !(l_run[0] == l_run[0])) || (vb && !(l_run[1] == l_run[1])))) set_status(p.status, kStatusRange);
     if (SPLIT) {
       // every CTA of the cluster is done with its slots; rows go to their owners' K slots
       __syncwarp();
@@ -819,47 +932,55 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
       const int ia = rank * rows_per + ra - own_a * rows_per, ib = rank * rows_per + rbw - own_b * rows_per;
       const uint32_t da = peer_addr(rows_o + ia * kD + 2 * t4, va ? own_a : 0);
       const uint32_t db = peer_addr(rows_o + ib * kD + 2 * t4, vb ? own_b : 0);
-      if (ok) {
-#pragma unroll 1
-        for (int c = 0; c < kD; c += 64) {
-          uint32_t o[32];
-          __syncwarp();
-          tmem_ld_16x256b_x8(tmem + lane_base + kColO + c, o);
-          const bool any = n_chunks > 0;  // a split without keys pushes zeros (its accumulator was never written)
-#pragma unroll
-          for (int g = 0; g < 8; ++g) {
-            if (va) st_peer2(da + (c + 8 * g) * 4, any ? __uint_as_float(o[4 * g]) * inv[0] : 0.f,
-                             any ? __uint_as_float(o[4 * g + 1]) * inv[0] : 0.f);
-            if (vb) st_peer2(db + (c + 8 * g) * 4, any ? __uint_as_float(o[4 * g + 2]) * inv[1] : 0.f,
-                             any ? __uint_as_float(o[4 * g + 3]) * inv[1] : 0.f);
-          }
-        }
-        if (t4 == 0) {
-          if (va) st_peer(peer_addr(rows_l + ia, own_a), l_run[0] > 0.f ? m_run[0] + log2f(l_run[0]) : -CUDART_INF_F);
-          if (vb) st_peer(peer_addr(rows_l + ib, own_b), l_run[1] > 0.f ? m_run[1] + log2f(l_run[1]) : -CUDART_INF_F);
-        }
-      }
-      __syncwarp();
-    } else if (ok) {
-      __half* oa = p.out + (static_cast<size_t>(b) * p.n_q + (va ? ra : 0)) * p.out_stride + h * kD + 2 * t4;
-      __half* ob = p.out + (static_cast<size_t>(b) * p.n_q + (vb ? rbw : 0)) * p.out_stride + h * kD + 2 * t4;
 #pragma unroll 1
       for (int c = 0; c < kD; c += 64) {
         uint32_t o[32];
+        __syncwarp();
         tmem_ld_16x256b_x8(tmem + lane_base + kColO + c, o);
+        const bool any = n > 0;  // a split without keys pushes zeros (its accumulator was never written)
 #pragma unroll
         for (int g = 0; g < 8; ++g) {
-          if (va) *reinterpret_cast<uint32_t*>(oa + c + 8 * g) =
-              pack_half2(__uint_as_float(o[4 * g]) * inv[0], __uint_as_float(o[4 * g + 1]) * inv[0]);
-          if (vb) *reinterpret_cast<uint32_t*>(ob + c + 8 * g) =
-              pack_half2(__uint_as_float(o[4 * g + 2]) * inv[1], __uint_as_float(o[4 * g + 3]) * inv[1]);
+          if (va) st_peer2(da + (c + 8 * g) * 4, any ? __uint_as_float(o[4 * g]) * inv[0] : 0.f,
+                           any ? __uint_as_float(o[4 * g + 1]) * inv[0] : 0.f);
+          if (vb) st_peer2(db + (c + 8 * g) * 4, any ? __uint_as_float(o[4 * g + 2]) * inv[1] : 0.f,
+                           any ? __uint_as_float(o[4 * g + 3]) * inv[1] : 0.f);
         }
       }
-      if (p.lse != nullptr && t4 == 0) {
-        float* lrow = p.lse + (static_cast<size_t>(b) * H + h) * p.n_q;
-        if (va) lrow[ra] = l_run[0] > 0.f ? (m_run[0] + log2f(l_run[0])) * 0.6931471805599453f : -CUDART_INF_F;
-        if (vb) lrow[rbw] = l_run[1] > 0.f ? (m_run[1] + log2f(l_run[1])) * 0.6931471805599453f : -CUDART_INF_F;
+      if (t4 == 0) {
+        if (va) st_peer(peer_addr(rows_l + ia, own_a), l_run[0] > 0.f ? m_run[0] + log2f(l_run[0]) : -CUDART_INF_F);
+        if (vb) st_peer(peer_addr(rows_l + ib, own_b), l_run[1] > 0.f ? m_run[1] + log2f(l_run[1]) : -CUDART_INF_F);
       }
+      __syncwarp();
+      break;
+    }
+    const int b = item(k).b, h = item(k).h;
+    __half* oa = p.out + (static_cast<size_t>(b) * p.n_q + (va ? ra : 0)) * p.out_stride + h * kD + 2 * t4;
+    __half* ob = p.out + (static_cast<size_t>(b) * p.n_q + (vb ? rbw : 0)) * p.out_stride + h * kD + 2 * t4;
+#pragma unroll 1
+    for (int c = 0; c < kD; c += 64) {
+      uint32_t o[32];
+      tmem_ld_16x256b_x8(tmem + lane_base + kColO + c, o);
+      if (c + 64 == kD) {  // O is read: the next item's first P V may overwrite it
+        tc_fence_before();
+        mbar_arrive(oread);
+      }
+#pragma unroll
+      for (int g = 0; g < 8; ++g) {
+        if (va) *reinterpret_cast<uint32_t*>(oa + c + 8 * g) =
+            pack_half2(__uint_as_float(o[4 * g]) * inv[0], __uint_as_float(o[4 * g + 1]) * inv[0]);
+        if (vb) *reinterpret_cast<uint32_t*>(ob + c + 8 * g) =
+            pack_half2(__uint_as_float(o[4 * g + 2]) * inv[1], __uint_as_float(o[4 * g + 3]) * inv[1]);
+      }
+    }
+    if (p.lse != nullptr && t4 == 0) {
+      float* lrow = p.lse + (static_cast<size_t>(b) * H + h) * p.n_q;
+      if (va) lrow[ra] = l_run[0] > 0.f ? (m_run[0] + log2f(l_run[0])) * 0.6931471805599453f : -CUDART_INF_F;
+      if (vb) lrow[rbw] = l_run[1] > 0.f ? (m_run[1] + log2f(l_run[1])) * 0.6931471805599453f : -CUDART_INF_F;
+    }
+    }
+    if (SPLIT && !ok) {  // aborted: meet the cluster without pushing
+      __syncwarp();
+      cluster_barrier();
     }
   }
   if (SPLIT) {
@@ -872,14 +993,18 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
     const float* rows_o = reinterpret_cast<const float*>(smem + SH::kOffK);
     const float* rows_l = rows_o + S * rows_per * kD;
     const int q_lo = rank * rows_per;
+    const int b = item(0).b, h = item(0).h;
     const int n_rows = min(p.n_q, q_lo + rows_per) - q_lo;
+#pragma unroll 1
     for (int t = tid; t < n_rows * (kD / 4); t += kThreadsTc) {
       const int qq = t / (kD / 4), d = (t % (kD / 4)) * 4;
       float mmax = -CUDART_INF_F;
+#pragma unroll 1
       for (int r = 0; r < S; ++r) mmax = fmaxf(mmax, rows_l[r * rows_per + qq]);
       float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
       float wsum = 0.f;
       if (mmax != -CUDART_INF_F)
+#pragma unroll 2
         for (int r = 0; r < S; ++r) {  // in split order
           const float w = exp2f(rows_l[r * rows_per + qq] - mmax);
           const float4 v = *reinterpret_cast<const float4*>(rows_o + (r * rows_per + qq) * kD + d);
@@ -946,23 +1071,34 @@ static int resident_splits(int wanted, int B, int n_heads, int cache_dtype) {
 cudaError_t launch_attention_tc(const AttnArgs& a_in, int B, int cache_dtype, cudaStream_t stream, bool pdl) {
   AttnArgs a = a_in;
   if (a.n_splits > 1) a.n_splits = resident_splits(a.n_splits, B, a.n_heads, cache_dtype);
-  // a long cache that starts in the last wave runs alone: 26 B/ns a CTA, so 1000 fp32 rows are 40 us
+  // a long cache begun last runs alone: 26 B/ns a CTA, so 1000 fp32 rows are 40 us
   int dev = 0, sm_count = 0;
   cudaError_t e = cudaGetDevice(&dev);
   if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sm_count, cudaDevAttrMultiProcessorCount, dev);
   if (e != cudaSuccess) return e;
   a.by_length = a.plan == nullptr && a.targs == nullptr && B > 1 && B <= kMaxByLength &&
                 static_cast<long long>(B) * a.n_heads * a.n_splits > static_cast<long long>(kCtasPerSm) * sm_count;
-  CUtensorMap map_k{}, map_v{};
+  AttnMaps maps{};
+  if (!encode_rows_map(&maps.q, a.q, B, a.n_q, a.q_stride, a.n_heads) ||
+      !encode_rows_map(&maps.k_own, a.k_own, B, a.n_own, a.own_stride, a.n_heads) ||
+      !encode_rows_map(&maps.v_own, a.v_own, B, a.n_own, a.own_stride, a.n_heads))
+    return cudaErrorInvalidValue;
   a.param_maps = 0;
   // one layer's caches outside a tick: maps by value (the row count is not known here; a chunk
   // is loaded by TMA only when all of its rows are the vehicle's)
   if (cache_dtype == 1 && a.targs == nullptr && a.k_cache != nullptr && a.v_cache != nullptr &&
-      encode_cache_map(&map_k, a.k_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)) &&
-      encode_cache_map(&map_v, a.v_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)))
+      encode_cache_map(&maps.k, a.k_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)) &&
+      encode_cache_map(&maps.v, a.v_cache, INT32_MAX, static_cast<uint32_t>(a.n_heads)))
     a.param_maps = 1;
-  void* kargs[] = {&a, &map_k, &map_v};
-  return launch_ex(tc_fn(cache_dtype, a.n_splits > 1), dim3(a.n_splits, a.n_heads, B), dim3(kThreadsTc),
+  const long long items = static_cast<long long>(B) * a.n_heads;
+  if (B > 65535 || a.n_heads > 65535 || items > INT32_MAX) return cudaErrorInvalidConfiguration;
+  // one wave of CTAs, each with up to kMaxRounds items; more items: as many waves as that takes
+  const long long wave = static_cast<long long>(kCtasPerSm) * sm_count;
+  const long long waves = (items + wave * kMaxRounds - 1) / (wave * kMaxRounds);
+  const dim3 grid = a.n_splits > 1 ? dim3(a.n_splits, a.n_heads, B)
+                                   : dim3(static_cast<unsigned>(items < waves * wave ? items : waves * wave));
+  void* kargs[] = {&a, &B, &maps};
+  return launch_ex(tc_fn(cache_dtype, a.n_splits > 1), grid, dim3(kThreadsTc),
                    static_cast<size_t>(tc_smem(cache_dtype)), stream, pdl, kargs, 1, a.n_splits);
 }
 

@@ -789,4 +789,18 @@ bool encode_cache_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_
             CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+bool encode_rows_map(CUtensorMap* map, const void* base, int n_vehicles, int rows, long long row_stride, int n_heads) {
+  const EncodeTiledFn fn = encode_fn();
+  if (fn == nullptr) return false;
+  const cuuint64_t dims[4] = {128, static_cast<cuuint64_t>(n_heads), static_cast<cuuint64_t>(rows),
+                              static_cast<cuuint64_t>(n_vehicles)};
+  const cuuint64_t row_bytes = static_cast<cuuint64_t>(row_stride) * 2;
+  const cuuint64_t strides[3] = {256, row_bytes, static_cast<cuuint64_t>(rows) * row_bytes};
+  const cuuint32_t box[4] = {64, 1, 64, 1};
+  const cuuint32_t estr[4] = {1, 1, 1, 1};
+  return fn(map, CU_TENSOR_MAP_DATA_TYPE_FLOAT16, 4, const_cast<void*>(base), dims, strides, box, estr,
+            CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+            CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
+}
+
 }  // namespace fsx

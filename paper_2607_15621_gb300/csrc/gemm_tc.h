@@ -78,6 +78,9 @@ bool encode_act_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t 
 // 3-D bf16 tensor map over a token-major KV cache [rows, n_heads, 128]: a box is 64 tokens of one
 // head and 64 of its 128 dims, 128-byte swizzle (the attention's operand layout).
 bool encode_cache_map(CUtensorMap* map, const void* base, uint64_t rows, uint32_t n_heads);
+// TMA map of n_vehicles x rows fp16 rows of n_heads x 128 values, 64-row boxes of one head and vehicle
+// (rows past a vehicle's are filled with zeros)
+bool encode_rows_map(CUtensorMap* map, const void* base, int n_vehicles, int rows, long long row_stride, int n_heads);
 // 2-D fp16 tensor map over an output y[rows, cols] with row stride `ld` elements, 64-column x
 // 32-row boxes, 128-byte swizzle (the store / SwiGLU epilogues' TMA stores)
 bool encode_out_map(CUtensorMap* map, const void* base, uint64_t rows, uint64_t cols, uint64_t ld);

@@ -39,6 +39,7 @@ def test_splits_and_dtypes(cache_dtype, n_splits, lengths, n_q, n_own):
 @pytest.mark.parametrize("n_splits,lengths", [
     (1, [7, 64, 64, 0, 130, 1, 64, 129, 0, 200]),      # 320 CTAs, just over one wave: longest first, ties by index
     (8, [5, 70, 70]), (1, [3 * (i * 37 % 128 // 4) for i in range(128)]), (1, [i % 3 for i in range(129)]),
+    (1, [65 * (i % 5 == 0) for i in range(310)]),      # more items than one wave of CTAs takes
 ])
 def test_more_than_one_wave(cache_dtype, n_splits, lengths):
     c = make(lengths, n_q=42 if len(lengths) < 100 else 3, n_own=10, cache_dtype=cache_dtype, seed=len(lengths))
@@ -46,6 +47,33 @@ def test_more_than_one_wave(cache_dtype, n_splits, lengths):
     ref, ref_lse = oracle_attention(c)
     assert row_err(out, ref).max() <= TOL[cache_dtype]
     assert np.abs(lse - ref_lse).max() <= 2e-3
+
+
+@pytest.mark.parametrize("cache_dtype", ["bf16", "fp32"])
+def test_vehicles_without_valid_offsets_are_passed_over(cache_dtype):
+    """Two vehicles of negative length among sixteen (512 items): reported, their rows untouched, the rest right."""
+    lengths = [70 - 4 * i for i in range(16)]
+    c = make(lengths, n_q=10, n_own=10, cache_dtype=cache_dtype, seed=3)
+    ref, _ = oracle_attention(c)
+    bad = (5, 14)
+    off = c["off"].copy()
+    off[6] = off[5] - 1     # vehicle 5: length -1; vehicle 6 starts one row early
+    off[15] = off[14] - 1   # vehicle 14: length -1; vehicle 15 starts one row early
+    dev = lambda t: t.to("cuda").contiguous()
+    n_q = n_own = 10
+    out = torch.full((16 * n_q, H * D), -7.0, device="cuda", dtype=torch.float16)
+    ws = torch.empty(fsx.attention_workspace_bytes(16, H, n_q, 1), device="cuda", dtype=torch.uint8)
+    fsx.attention(dev(c["q"]), H * D, dev(c["ko"]), dev(c["vo"]), H * D, n_q, n_own, dev(c["kc"]), dev(c["vc"]),
+                  c["dtype"], torch.as_tensor(off, device="cuda"), 16, H, 1, out, None, ws)
+    torch.cuda.synchronize()
+    out = out.cpu().double().numpy()
+    assert int(ws[:4].cpu().view(torch.int32)[0]) != 0
+    for b in range(16):
+        rows = slice(b * n_q, (b + 1) * n_q)
+        if b in bad:
+            assert (out[rows] == -7.0).all()
+        elif b - 1 not in bad:
+            assert row_err(out[rows], ref[rows]).max() <= TOL[cache_dtype]
 
 
 @pytest.mark.parametrize("cache_dtype,n_splits", [("bf16", 2), ("bf16", 8), ("fp32", 1), ("fp32", 3)])
