@@ -5,12 +5,16 @@
 // Each CTA runs its K steps into one accumulator in tensor memory, then the cluster
 // reduce-scatters the partial tiles through distributed shared memory: every CTA owns a run of
 // the tile's 4-token groups, the others send it their fp32 partials of those groups by st.async
-// stores that complete on its mbarrier, and it adds them in split order (deterministic), updates
+// stores that complete on its mbarrier (its own partials too), and it adds them in split order (deterministic), updates
 // x, its fp16 copy and the per-token sums of x^2. The partials never pass through L2 and no CTA
 // polls global memory. Measured against that path (write the partial tile, fence, counter, poll,
 // read back), ticks of 8 layers: 4 vehicles 441 -> 404 us, 16 vehicles 512 -> 484 us, 40 clip blocks
-// 848 -> 818 us. In a launch of W_o for 672 tokens (96-token tiles, 4 splits) the K steps take 3.4 us,
-// the exchange 3.4 us and the update 1.3 us (device timer, steps of 0.26 us).
+// 848 -> 818 us. In a launch of W_o for 672 tokens (96-token tiles, 4 splits) the K steps took 3.4 us,
+// the exchange 3.4 us and the update 1.3 us (device timer, steps of 0.26 us). The last two were long
+// for their code: a launch finds its instructions evicted by the layer's other kernels, and 42 KB of
+// them, most in this epilogue, came in on its critical path. At 27 KB (destinations from a table made
+// before the wait on the previous kernel, one site of the push, one address per token): 4 vehicles
+// 405 -> 374 us, 16 vehicles 480 -> 459, the clip 731 -> 724, a two-layer append of 4 tokens 199 -> 194.
 //   warp 0: producer (one bulk copy of a packed 16 KB weight image and one 2-D TMA token box per
 //           64-wide K step; the first weights before the wait on the previous kernel);
 //   warp 1: MMA issue (M = 128, N = BN, K = 16);
@@ -105,6 +109,9 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
   uint64_t* rx = tmem_full + 1;           // the other splits' partials of this CTA's groups
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(rx + 1);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  // [n_groups]: where in the cluster this CTA's partials of a 4-token group go, and the barrier they complete on
+  uint2* route = reinterpret_cast<uint2*>(base + 256);
+  static_assert(256 + BN / 4 * 8 <= 1024 && 2 * kStages * 8 + 24 <= 256, "header");
   unsigned char* recv = base + 1024;
   unsigned char* stages = recv + recv_bytes<BN>();
   static_assert(recv_bytes<BN>() % 1024 == 0, "the stages must stay 1024-byte aligned");
@@ -133,8 +140,16 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
     }
     mbar_init(tmem_full, 1);
     mbar_init(rx, 1);
-    mbar_arrive_expect_tx(rx, static_cast<uint32_t>((KS - 1) * (g_hi - g_lo) * kGroupBytes));
+    mbar_arrive_expect_tx(rx, static_cast<uint32_t>(KS * (g_hi - g_lo) * kGroupBytes));
     asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
+  }
+  if (tid >= 64 && tid - 64 < n_groups) {
+    const int g = tid - 64;
+    int o = 0;
+    while (g >= group_lo(o + 1)) ++o;
+    const int o_lo = group_lo(o), slot = rank * (group_lo(o + 1) - o_lo) + g - o_lo;
+    route[g] = make_uint2(peer_addr(smem_addr(recv) + static_cast<uint32_t>(slot * kGroupBytes), o),
+                          peer_addr(smem_addr(rx), o));
   }
   if (warp == 1) {
     asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;" ::"r"(smem_addr(tmem_slot)),
@@ -215,68 +230,58 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
     auto load_x = [&](int gl) {
       const int m = m0 + 4 * (g_lo + gl);
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int t = 0; t < 4; ++t) {  // a token's address once, its rows at constant distances
+        const float* src = p.xo + static_cast<size_t>(m + t) * p.ldxo + t_n * kRows + lane;
 #pragma unroll
-        for (int t = 0; t < 4; ++t)
-          x[i][t] = m + t < p.M ? __ldcg(p.xo + static_cast<size_t>(m + t) * p.ldxo + t_n * kRows + 32 * i + lane) : 0.f;
-    };
-    const int n_own = g_hi - g_lo;
-    if (ew < n_own) load_x(ew);
-    wait(tmem_full, 0u);
-    tc_fence_after();
-    const uint32_t recv_a = smem_addr(recv), rx_a = smem_addr(rx);
-    const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16);
-    const bool send = *abort == 0;
-    int owner = -1, o_lo = 0, o_hi = 0;  // owner of the current group and its run
-    uint32_t dst = 0, bar = 0;           // its receive buffer (group 0 of the tile, this row) and barrier
-    auto push = [&](const uint32_t (&r)[16], int g0) {  // groups g0 .. g0 + 3
-#pragma unroll
-      for (int e = 0; e < 4; ++e) {
-        const int g = g0 + e;
-        if (g >= n_groups) break;
-        while (g >= o_hi) {
-          ++owner;
-          o_lo = group_lo(owner);
-          o_hi = group_lo(owner + 1);
-          dst = peer_addr(recv_a, owner) + static_cast<uint32_t>((rank * (o_hi - o_lo) - o_lo) * kGroupBytes + row * 16);
-          bar = peer_addr(rx_a, owner);
-        }
-        const uint4 v = make_uint4(r[4 * e], r[4 * e + 1], r[4 * e + 2], r[4 * e + 3]);
-        if (owner == rank)
-          *reinterpret_cast<uint4*>(recv + (rank * (o_hi - o_lo) + g - o_lo) * kGroupBytes + row * 16) = v;
-        else if (send)
-          st_async_v4(dst + static_cast<uint32_t>(g * kGroupBytes), v, bar);
+        for (int i = 0; i < 4; ++i) x[i][t] = m + t < p.M ? __ldcg(src + 32 * i) : 0.f;
       }
     };
-    // 16-token chunks grp, grp + 2, ... of the tile (BN is a multiple of 16), the next one on its way
-    uint32_t ra[16], rb[16];
-    int c = grp;
-    __syncwarp();
-    if (4 * c < n_groups) tmem_ld16_issue(taddr + 16u * c, ra);
-    while (4 * c < n_groups) {
-      tmem_wait16(ra);
-      if (4 * (c + 2) < n_groups) tmem_ld16_issue(taddr + 16u * (c + 2), rb);
-      push(ra, 4 * c);
-      __syncwarp();
-      c += 2;
-      if (4 * c >= n_groups) break;
-      tmem_wait16(rb);
-      if (4 * (c + 2) < n_groups) tmem_ld16_issue(taddr + 16u * (c + 2), ra);
-      push(rb, 4 * c);
-      __syncwarp();
-      c += 2;
-    }
-    __syncwarp();
-    cluster_arrive();  // this thread sends nothing more
-    asm volatile("bar.sync 1, %0;" ::"n"(32 * kEpiWarps) : "memory");  // this CTA's own partials
-    if (*abort == 0 && !mbar_wait_cluster(rx, 0u, p.status)) *abort = 1;
-    for (int gl = ew; gl < n_own; gl += kEpiWarps) {
-      if (gl != ew) load_x(gl);
+    const int n_own = g_hi - g_lo;
+#pragma unroll 1
+    for (int it = 0, gl = ew; it == 0 || gl < n_own; ++it, gl += kEpiWarps) {
+      if (gl < n_own) load_x(gl);
+      if (it == 0) {  // the exchange
+        wait(tmem_full, 0u);
+        tc_fence_after();
+        const uint32_t taddr = tmem + (static_cast<uint32_t>(q * 32) << 16);
+        const bool send = *abort == 0;
+        // 16-token chunks grp, grp + 2, ... of the tile (BN is a multiple of 16), the next one on its way
+        uint32_t ra[16], rb[16];
+        int c = grp;
+        __syncwarp();
+        if (4 * c < n_groups) {
+          tmem_ld16_issue(taddr + 16u * c, ra);
+          tmem_wait16(ra);
+        }
+#pragma unroll 1
+        for (; 4 * c < n_groups; c += 2) {
+          const bool more = 4 * (c + 2) < n_groups;
+          if (more) tmem_ld16_issue(taddr + 16u * (c + 2), rb);
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            if (4 * c + e < n_groups && send) {
+              const uint2 to = route[4 * c + e];
+              st_async_v4(to.x + row * 16, make_uint4(ra[4 * e], ra[4 * e + 1], ra[4 * e + 2], ra[4 * e + 3]), to.y);
+            }
+          }
+          __syncwarp();
+          if (more) {
+            tmem_wait16(rb);
+#pragma unroll
+            for (int e = 0; e < 16; ++e) ra[e] = rb[e];
+          }
+        }
+        __syncwarp();
+        cluster_arrive();  // this thread sends nothing more
+        if (*abort == 0 && !mbar_wait_cluster(rx, 0u, p.status)) *abort = 1;
+      }
+      if (gl >= n_own) break;
       float acc[4][4];
 #pragma unroll
       for (int i = 0; i < 4; ++i)
 #pragma unroll
         for (int t = 0; t < 4; ++t) acc[i][t] = 0.f;
+#pragma unroll 2
       for (int s = 0; s < KS; ++s) {  // in split order
         const unsigned char* src = recv + (s * n_own + gl) * kGroupBytes + lane * 16;
 #pragma unroll
@@ -291,24 +296,24 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
       const int m = m0 + 4 * (g_lo + gl);
       float ss[4] = {0.f, 0.f, 0.f, 0.f};
 #pragma unroll
-      for (int i = 0; i < 4; ++i)
+      for (int t = 0; t < 4; ++t) {
+        const size_t idx = static_cast<size_t>(m + t) * p.ldxo + t_n * kRows + lane;
 #pragma unroll
-        for (int t = 0; t < 4; ++t) {
-          const float v = x[i][t] + acc[i][t];
-          if (m + t < p.M) {
-            const size_t idx = static_cast<size_t>(m + t) * p.ldxo + t_n * kRows + 32 * i + lane;
-            p.xo[idx] = v;
-            p.xo16[idx] = __float2half_rn(v);
-          }
-          acc[i][t] = v;
-          ss[t] += v * v;
+        for (int i = 0; i < 4; ++i) {
+          acc[i][t] += x[i][t];
+          ss[t] += acc[i][t] * acc[i][t];
         }
-      if (p.x_copy != nullptr) {
+        if (m + t < p.M) {
 #pragma unroll
-        for (int i = 0; i < 4; ++i)
+          for (int i = 0; i < 4; ++i) {
+            p.xo[idx + 32 * i] = acc[i][t];
+            p.xo16[idx + 32 * i] = __float2half_rn(acc[i][t]);
+          }
+          if (p.x_copy != nullptr) {
 #pragma unroll
-          for (int t = 0; t < 4; ++t)
-            if (m + t < p.M) p.x_copy[static_cast<size_t>(m + t) * p.ldxo + t_n * kRows + 32 * i + lane] = acc[i][t];
+            for (int i = 0; i < 4; ++i) p.x_copy[idx + 32 * i] = acc[i][t];
+          }
+        }
       }
 #pragma unroll
       for (int t = 0; t < 4; ++t) {
