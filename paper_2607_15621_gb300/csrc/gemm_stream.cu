@@ -21,6 +21,9 @@
 // 128-token tiles, waiting K splits and no dependent launch: 4 tokens 311 -> 237 us a call (QKV
 // 30.1 -> 23.7 us a launch, gate/up 55.8 -> 35.3, W_o and W_d together 42.6 -> 36.9), 64 tokens
 // 370 -> 339 us (QKV 30.2 -> 26.7, gate/up 56.4 -> 42.0, W_o and W_d 45.5 -> 50.4).
+// Code size: a launch finds its instructions evicted by the layer's other kernels. One copy of the
+// epilogue instead of one per chunk in flight and 32-bit step arithmetic (gate/up at 64 tokens
+// 73 -> 49 KB, QKV at 16 tokens 33 -> 28): 4 tokens 193.5 -> 187.3 us a call, 64 tokens 266 -> 261.
 #include <cuda.h>
 
 #include "device_util.cuh"
@@ -124,9 +127,10 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int KT = p.K / kTcTileK;
-  const long long total = static_cast<long long>(p.N / kRows) * KT;  // K steps of the matrix
+  // K steps of the matrix; times the CTAs they fit 32 bits (2^32 / 152 steps are 460 GB of weights)
+  const uint32_t total = static_cast<uint32_t>(p.N / kRows) * KT;
   const int G = gridDim.x;
-  const long long s0 = total * blockIdx.x / G, s1 = total * (blockIdx.x + 1) / G;  // this CTA's steps
+  const uint32_t s0 = total * blockIdx.x / G, s1 = total * (blockIdx.x + 1) / G;  // this CTA's steps
   auto wait = [&](uint64_t* bar, uint32_t parity) {
     if (*abort) return;
     if (!mbar_wait(bar, parity, p.status)) *abort = 1;
@@ -201,8 +205,8 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
     pdl_wait();
     constexpr uint32_t idesc = idesc_f16(kRows, BN);
     int g = 0, i = 0;
-    for (long long t = s0; t < s1; ++i) {
-      const long long end = min(s1, (t / KT + 1) * KT);
+    for (uint32_t t = s0; t < s1; ++i) {
+      const uint32_t end = min(s1, (t / KT + 1) * KT);
       const int acc = i & 1;
       if (i >= 2) wait(tmem_empty + acc, static_cast<uint32_t>(((i >> 1) - 1) & 1));
       tc_fence_after();
@@ -295,12 +299,12 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
     // segment of CTA c in a tile it shares: slot 2 c + 1 when the tile starts in its range,
     // else 2 c; [8-token chunk][2][128 rows] groups of 4 tokens
     constexpr size_t kSlot = static_cast<size_t>(BN) * kRows;
-    auto cta_of = [&](long long s) { return static_cast<int>(((s + 1) * G - 1) / total); };
+    auto cta_of = [&](uint32_t step) { return static_cast<int>(((step + 1) * G - 1) / total); };
     int i = 0;
-    for (long long t = s0; t < s1; ++i) {
+    for (uint32_t t = s0; t < s1; ++i) {
       const int tile = static_cast<int>(t / KT);
-      const long long t_lo = static_cast<long long>(tile) * KT, t_hi = t_lo + KT;
-      const long long end = min(s1, t_hi);
+      const uint32_t t_lo = tile * KT, t_hi = t_lo + KT;
+      const uint32_t end = min(s1, t_hi);
       const int acc = i & 1;
       const bool whole = t == t_lo && end == t_hi;
       wait(tmem_full + acc, static_cast<uint32_t>((i >> 1) & 1));
@@ -362,10 +366,15 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
                     v[r][4 * hh + 3] += w4[r][e][hh].w;
                   }
             }
-#pragma unroll
-            for (int r = 0; r < kRound; ++r) {
+#pragma unroll 1
+            for (int r = 0; r < kRound; ++r) {  // one copy of the code: the chunks move up
               const int cr = c0 + r * kGroups * kChunk;
-              if (cr < BN && cr < p.M) finish(tile, cr, v[r]);
+              if (cr >= BN || cr >= p.M) break;
+              finish(tile, cr, v[0]);
+#pragma unroll
+              for (int e = 1; e < kRound; ++e)
+#pragma unroll
+                for (int j = 0; j < kChunk; ++j) v[e - 1][j] = v[e][j];
             }
           }
         }
