@@ -210,7 +210,8 @@ fsx_status fsx_kernel_time(fsx_handle h, float* ms, int* launches);
  *              + (b*n_own+j)*own_stride (same column layout).
  *   d_k_cache, d_v_cache, d_offsets : as one layer of fsx_tick.
  *   n_q in 1..48, n_own >= 0, n_splits in 1..64 (keys of vehicle b are cut
- *   into n_splits near-equal ranges), head_dim == 128.
+ *   into at most n_splits near-equal ranges: with 2..8 as many as are resident at
+ *   once), head_dim == 128.
  *   d_out    : DEVICE fp16 [B*n_q, n_heads*head_dim].
  *   d_lse    : DEVICE fp32 [B, n_heads, n_q] natural-log log-sum-exp of the
  *              scaled scores, or NULL.
