@@ -10,7 +10,7 @@
 //     as one 16 KB bulk copy of a pre-swizzled image (packed at fsx_create in
 //     the 128-byte swizzle layout the MMA reads), the token tile by a 2-D TMA
 //     load with the same swizzle (rows past M read as zeros), through a
-//     4-stage ring that runs on across tile boundaries;
+//     ring of 4 to 8 stages that runs on across tile boundaries;
 //   warp 1 (one lane): issues tcgen05.mma (M=128, N=BN, K=16) x4 per stage,
 //     releases each stage to the producer, and alternates between two
 //     accumulators in tensor memory, so the MMAs of tile i+1 run while the
@@ -20,7 +20,7 @@
 //     chunk is read from TMEM in the 16x256b shape (mma accumulator fragments),
 //     scaled, packed to fp16 (SwiGLU: each thread holds a gate value beside its
 //     up value) and written transposed into a token-major staging tile by
-//     stmatrix, then stored as 16-byte row pieces; the fp32 residual update
+//     stmatrix, then stored by TMA; the fp32 residual update
 //     reads its 32 lanes in the 32x32b shape (each element owned by one thread)
 //     and also emits each token's sum of x^2 over its 128 columns.
 // Pair variant (opt-in for QKV at 256-token tiles and 2048 tokens or more): a cluster of two CTAs on an SM
