@@ -96,3 +96,10 @@ def test_values_beyond_fp16_are_reported(cache_dtype, n_splits, which, row, dim)
     for bad in (65536.0, -1e30, float("inf"), float("nan")):
         c[which][row, 7, dim] = bad
         assert status() == fsx.FSX_ERR_RANGE, bad
+
+
+def test_default_stream_of_a_call_is_the_current_one():
+    side = torch.cuda.Stream()
+    for s in (torch.cuda.default_stream(), side):
+        with torch.cuda.stream(s):
+            assert fsx._stream(None) == torch.cuda.current_stream().cuda_stream == s.cuda_stream
