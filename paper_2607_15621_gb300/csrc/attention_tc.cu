@@ -439,9 +439,10 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
   // thread, zeros behind it.
   const CUtensorMap* tmap = nullptr;
   if (!F32) {
-    if (p.cache_maps != nullptr && p.targs != nullptr)
+    if (p.cache_maps != nullptr && p.targs != nullptr) {
       tmap = p.cache_maps + 2 * p.layer + (is_v ? 1 : 0);
-    else if (p.param_maps)
+      if (is_prod && pt == 0) tensormap_acquire(tmap);  // the thread that issues this tensor's loads
+    } else if (p.param_maps)
       tmap = is_v ? &maps.v : &maps.k;
   }
   // the producers' next chunk to issue: chunk ci of item ck

@@ -166,6 +166,13 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, uint32_t by
       : "memory");
 }
 
+// Before the first TMA load of a CTA through a tensor map that lies in global memory, by the thread
+// that issues its loads: the map may have been rewritten at the same address (by a host copy, hence
+// the system scope) since an earlier kernel loaded through it, and TMA reads maps by a proxy of its own.
+__device__ __forceinline__ void tensormap_acquire(const void* map) {
+  asm volatile("fence.proxy.tensormap::generic.acquire.sys [%0], 128;" ::"l"(map) : "memory");
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);

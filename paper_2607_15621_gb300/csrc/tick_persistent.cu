@@ -701,6 +701,12 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     const unsigned char* vc = n_chunks > 0 ? static_cast<const unsigned char*>(p.targs->v_cache[layer]) + head_off : nullptr;
 
     // =========================== phase A ===========================
+    // the two threads that issue TMA loads of cache chunks (stage_issue's t = 0), this layer's maps;
+    // before the wait on the other CTAs, which hides it
+    if (kSw && p.cache_maps != nullptr && n_cache >= kStageKeys && (tid == 3 * 32 || tid == kAttendWarps * 32)) {
+      tensormap_acquire(p.cache_maps + 2 * layer);
+      tensormap_acquire(p.cache_maps + 2 * layer + 1);
+    }
     wait_counter(p.counters + sA, sA == 0 ? G : n_b_ctas, p.status, abort, p.wait_limit_ns);
     {
       // warp w: token rows w, w + 8, ... whole (every load of a row contiguous, all in flight) -> fp16
