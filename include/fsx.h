@@ -220,7 +220,11 @@ fsx_status fsx_kernel_time(fsx_handle h, float* ms, int* launches);
  *              call's kernels touch it; it must not be shared by calls that
  *              overlap on the GPU. Asynchronous on `stream`; cache offsets
  *              outside [0, ...] non-decreasing order make the kernels write
- *              nothing. */
+ *              nothing.
+ * A cache value outside the fp16 range sets the status word to FSX_ERR_RANGE. With
+ * fp32 caches or 2..8 splits the rows are then those of the cache clipped to +-65504
+ * (NaN values stay NaN); with one split of a bf16 cache they may hold infinities or
+ * NaN, and with more than 8 splits they may be left unwritten. */
 size_t fsx_attention_workspace_bytes(int B, int n_heads, int n_q, int n_splits);
 fsx_status fsx_attention(const void* d_q, long long q_stride,
                          const void* d_k_own, const void* d_v_own, long long own_stride,

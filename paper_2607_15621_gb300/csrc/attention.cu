@@ -92,7 +92,7 @@ __device__ __forceinline__ void cp_async_wait_n(int n) {
 template <typename CT>
 __device__ __forceinline__ void convert_unit(const unsigned char* raw, uint4* dst, bool own, uint32_t& range);
 
-// bf16 cache rows: 16 raw bytes = 8 values -> 8 fp16 (their largest magnitudes kept)
+// bf16 cache rows: 16 raw bytes = 8 values -> 8 fp16 (saturated, their largest magnitudes kept)
 template <>
 __device__ __forceinline__ void convert_unit<__nv_bfloat16>(const unsigned char* raw, uint4* dst, bool own,
                                                             uint32_t& range) {
@@ -100,8 +100,9 @@ __device__ __forceinline__ void convert_unit<__nv_bfloat16>(const unsigned char*
   if (own) {
     *dst = v;
   } else {
-    *dst = make_uint4(bf16x2_to_half2_peak(v.x, range), bf16x2_to_half2_peak(v.y, range),
-                      bf16x2_to_half2_peak(v.z, range), bf16x2_to_half2_peak(v.w, range));
+    const uint4 h = make_uint4(bf16x2_to_half2_peak(v.x, range), bf16x2_to_half2_peak(v.y, range),
+                               bf16x2_to_half2_peak(v.z, range), bf16x2_to_half2_peak(v.w, range));
+    *dst = out_of_range(range) ? saturate_half8(h) : h;
   }
 }
 
@@ -113,8 +114,9 @@ __device__ __forceinline__ void convert_unit<float>(const unsigned char* raw, ui
   } else {
     const float4 a = *reinterpret_cast<const float4*>(raw);
     const float4 b = *reinterpret_cast<const float4*>(raw + 16);
-    *dst = make_uint4(f32x2_to_half2_peak(a.x, a.y, range), f32x2_to_half2_peak(a.z, a.w, range),
-                      f32x2_to_half2_peak(b.x, b.y, range), f32x2_to_half2_peak(b.z, b.w, range));
+    const uint4 h = make_uint4(f32x2_to_half2_peak(a.x, a.y, range), f32x2_to_half2_peak(a.z, a.w, range),
+                               f32x2_to_half2_peak(b.x, b.y, range), f32x2_to_half2_peak(b.z, b.w, range));
+    *dst = out_of_range(range) ? saturate_half8(h) : h;
   }
 }
 

@@ -41,7 +41,8 @@
 // Splits: the CTAs of one (vehicle, head) form a thread-block cluster and merge
 // (log-sum-exp weights) by pushing each split's normalised fp32 rows to the rank that owns them
 // through distributed shared memory. Split and fp32 launches check every cache value they stage
-// against the fp16 range.
+// against the fp16 range and go on with it clipped to +-65504 (bf16 values of V to +-65536, the
+// nearest bf16).
 // Measured against the mma.sync kernel of attention.cu, which split and fp32 launches ran before: a
 // tick of 4 vehicles with 0-700 bf16 rows, 8 layers, 2 splits: 740 -> 452 us; one vehicle with 2048
 // rows, 8 splits, Eq. 1 alone: 34 -> 27 us a call; 24 vehicles with 16-1000 fp32 rows, Eq. 1
@@ -238,6 +239,18 @@ constexpr float kLazyRescale = 8.f;  // log2 units; P <= 2^8 between rescales
 // bits 15 / 31 set where a bf16 value lies outside the fp16 range (magnitude bits >= 0x4780)
 __device__ __forceinline__ uint32_t bf16x2_out_of_range(uint32_t v) {
   return ((v & 0x7fff7fffu) + 0x38803880u) & 0x80008000u;
+}
+
+// the same values clipped to +-65536 (0x4780, the smallest bf16 magnitude out of range); a NaN stays
+__device__ __forceinline__ uint32_t clip_bf16x2(uint32_t v) {
+  const uint32_t lo = v & 0x7fffu, hi = v & 0x7fff0000u;
+  if (lo > 0x4780u && lo <= 0x7f80u) v = (v & 0xffff8000u) | 0x4780u;
+  if (hi > 0x47800000u && hi <= 0x7f800000u) v = (v & 0x8000ffffu) | 0x47800000u;
+  return v;
+}
+// a finite value clipped to the fp16 range
+__device__ __forceinline__ float clip_finite(float x) {
+  return fabsf(x) < CUDART_INF_F ? fminf(fmaxf(x, -65504.f), 65504.f) : x;
 }
 
 // arrive at and wait for the cluster's barrier (threads of a warp may come apart)
@@ -693,6 +706,7 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
                 const uint32_t x0 = f32x2_to_half2_peak(x.x, x.y, range), x1 = f32x2_to_half2_peak(x.z, x.w, range);
                 const uint32_t y0 = f32x2_to_half2_peak(y.x, y.y, range), y1 = f32x2_to_half2_peak(y.z, y.w, range);
                 out = sw == 0 ? make_uint4(x0, x1, y0, y1) : make_uint4(y0, y1, x0, x1);
+                if (out_of_range(range)) out = saturate_half8(out);
               }
               *reinterpret_cast<uint4*>(slot + tile128_off(st * kRawKeys + r, u)) = out;
             }
@@ -761,6 +775,15 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
                 *reinterpret_cast<uint4*>(slot + tile128_off(pr0 + kRowStep * (m0 + m), pu)) =
                     make_uint4(bf16x2_to_half2(v[m].x), bf16x2_to_half2(v[m].y), bf16x2_to_half2(v[m].z),
                                bf16x2_to_half2(v[m].w));
+            }
+            if (kCheck && range != 0) {  // an error: this thread's units in place, clipped
+#pragma unroll 1
+              for (int m = m0; m < m0 + 8; ++m) {
+                uint4* u = reinterpret_cast<uint4*>(slot + tile128_off(pr0 + kRowStep * m, pu));
+                const uint4 w = *u;
+                *u = is_v ? make_uint4(clip_bf16x2(w.x), clip_bf16x2(w.y), clip_bf16x2(w.z), clip_bf16x2(w.w))
+                          : saturate_half8(w);
+              }
             }
           }
         }
@@ -1017,8 +1040,12 @@ __global__ void __launch_bounds__(kThreadsTc, kCtasPerSm)
         }
       const float iw = wsum > 0.f ? 1.f / wsum : 0.f;
       const int q = q_lo + qq;
+      float o[4] = {acc.x * iw, acc.y * iw, acc.z * iw, acc.w * iw};
+      if (!F32)  // values clipped to +-65536 may leave the fp16 range
+#pragma unroll
+        for (int e = 0; e < 4; ++e) o[e] = clip_finite(o[e]);
       *reinterpret_cast<uint2*>(p.out + (static_cast<size_t>(b) * p.n_q + q) * p.out_stride + h * kD + d) =
-          make_uint2(pack_half2(acc.x * iw, acc.y * iw), pack_half2(acc.z * iw, acc.w * iw));
+          make_uint2(pack_half2(o[0], o[1]), pack_half2(o[2], o[3]));
       if (p.lse != nullptr && d == 0)
         p.lse[(static_cast<size_t>(b) * H + h) * p.n_q + q] =
             wsum > 0.f ? (mmax + log2f(wsum)) * 0.6931471805599453f : -CUDART_INF_F;

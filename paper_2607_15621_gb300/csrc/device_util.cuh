@@ -188,8 +188,11 @@ __device__ __forceinline__ uint32_t pack_half2(float lo, float hi) {
 // below keep in `peak` the largest magnitudes seen, as two packed fp16 (start at 0): a value
 // that rounds beyond 65504 became an infinity and a NaN stays one, so out_of_range(peak) tells
 // whether an input lay outside the fp16 range. flag_range() turns that into the FSX_ERR_RANGE
-// error status, and the tick is abandoned like any other device-side error: the infinity
-// reaches no caller. (One max per pair of values: the conversions bound the staging warps.)
+// error status: a tick is abandoned like on any other device-side error, and Eq. 1 alone still
+// writes its rows, so once out_of_range(peak) its callers put saturate_half8() between the
+// conversion and the operand tile and the rows are those of the cache clipped to +-65504.
+// (One max per pair of values and one test per unit, against a saturating conversion and two
+// compares per value: the conversions bound the staging warps.)
 __device__ __forceinline__ uint32_t peak_of(uint32_t peak, uint32_t h) {
   const __half2 m = __hmax2_nan(*reinterpret_cast<const __half2*>(&peak), __habs2(*reinterpret_cast<const __half2*>(&h)));
   return *reinterpret_cast<const uint32_t*>(&m);
@@ -205,7 +208,15 @@ __device__ __forceinline__ uint32_t f32x2_to_half2_peak(float lo, float hi, uint
   return h;
 }
 __device__ __forceinline__ bool out_of_range(uint32_t peak) {  // an infinity or a NaN in either half
-  return (peak & 0x7c00u) == 0x7c00u || (peak & 0x7c000000u) == 0x7c000000u;
+  return ((peak + 0x04000400u) & 0x80008000u) != 0u;           // magnitudes: no carry between the halves
+}
+__device__ __forceinline__ uint32_t saturate_half2(uint32_t h) {  // infinities -> +-65504, a NaN stays
+  const __half2 lim = __float2half2_rn(65504.f);
+  const __half2 v = __hmax2_nan(__hmin2_nan(*reinterpret_cast<const __half2*>(&h), lim), __hneg2(lim));
+  return *reinterpret_cast<const uint32_t*>(&v);
+}
+__device__ __forceinline__ uint4 saturate_half8(uint4 h) {
+  return make_uint4(saturate_half2(h.x), saturate_half2(h.y), saturate_half2(h.z), saturate_half2(h.w));
 }
 __device__ __forceinline__ void flag_range(int* status, uint32_t peak) {
   if (out_of_range(peak)) set_status(status, kStatusRange);

@@ -98,6 +98,28 @@ def test_values_beyond_fp16_are_reported(cache_dtype, n_splits, which, row, dim)
         assert status() == fsx.FSX_ERR_RANGE, bad
 
 
+@pytest.mark.parametrize("cache_dtype,n_splits,n_own", [
+    ("bf16", 2, 42), ("bf16", 8, 42), ("fp32", 1, 42), ("fp32", 3, 42), ("bf16", 3, 70), ("fp32", 2, 70)])
+@pytest.mark.parametrize("which,bad", [("kc", 1.0e6), ("kc", float("-inf")), ("vc", -3.0e5), ("vc", float("inf"))])
+def test_rows_beside_a_range_error_are_those_of_the_clipped_cache(cache_dtype, n_splits, n_own, which, bad):
+    """70 own keys: the mma.sync kernel, which rounds P to fp16.
+
+    Tolerance, as a share of a row's largest entry, where a value of 65504 carries nearly the whole row: 2^-11 for the
+    fp16 result; bf16 V is clipped to 65536, another 2^-11; together 1e-3 and the usual 1e-3: 2e-3. P in fp16 has units
+    of 2^-24 below 2^-14: 2^-25 * 65504 = 2e-3 of an entry, over rows whose largest is at least 0.4, and 3e-3 as usual:
+    8e-3. The log-sum-exp of scores up to 3e5 is an fp32 sum: 1e-5 of it."""
+    c = make([201], n_own=n_own, cache_dtype=cache_dtype, seed=10)
+    clipped = dict(c)
+    for row, head, dim in ((3, 5, 7), (130, 5, 70), (200, 17, 127)):
+        c[which][row, head, dim] = bad
+    clipped[which] = c[which].double().clamp(-65504.0, 65504.0)
+    ref, ref_lse = oracle_attention(clipped)
+    out, lse = gpu_attention(c, n_splits)
+    assert np.isfinite(out).all() and np.isfinite(lse).all()
+    assert row_err(out, ref).max() <= (2e-3 if cache_dtype == "bf16" and n_own <= 64 else 8e-3)
+    assert (np.abs(lse - ref_lse) <= 2e-3 + 1e-5 * np.abs(ref_lse)).all()
+
+
 def test_default_stream_of_a_call_is_the_current_one():
     side = torch.cuda.Stream()
     for s in (torch.cuda.default_stream(), side):
