@@ -468,9 +468,11 @@ fsx_status prepare_tick(fsx_handle_s* h, const void* const* k_cache, const void*
   if (!h->args_valid || std::memcmp(&a, &h->h_args, sizeof(TickArgs)) != 0) {
     const bool caches_changed = !h->args_valid || std::memcmp(a.k_cache, h->h_args.k_cache, sizeof(a.k_cache)) != 0 ||
                                 std::memcmp(a.v_cache, h->h_args.v_cache, sizeof(a.v_cache)) != 0;
-    h->h_args = a;
-    FSX_CUDA(cudaMemcpyAsync(h->d_args, &h->h_args, sizeof(TickArgs), cudaMemcpyHostToDevice, st));
-    if (caches_changed && h->d_cache_maps != nullptr) {
+    const bool new_maps = caches_changed && h->d_cache_maps != nullptr;
+    // until all of it is enqueued the device holds no complete set: a call that fails below leaves the
+    // next one to start over, also with the same pointers
+    h->args_valid = false;
+    if (new_maps) {
       // the map of a NULL pointer stays zero: a layer without cache rows never loads through it
       std::memset(h->h_cache_maps.data(), 0, h->h_cache_maps.size() * sizeof(CUtensorMap));
       for (int l = 0; l < h->cfg.n_layers; ++l)
@@ -481,9 +483,12 @@ fsx_status prepare_tick(fsx_handle_s* h, const void* const* k_cache, const void*
                                      static_cast<uint64_t>(h->cfg.max_total_cache_tokens), h->cfg.n_heads))
             return fail(FSX_ERR_INVALID_ARG, "a cache pointer is not 16-byte aligned (tensor map encoding failed)");
         }
+    }
+    h->h_args = a;
+    FSX_CUDA(cudaMemcpyAsync(h->d_args, &h->h_args, sizeof(TickArgs), cudaMemcpyHostToDevice, st));
+    if (new_maps)
       FSX_CUDA(cudaMemcpyAsync(h->d_cache_maps, h->h_cache_maps.data(), h->h_cache_maps.size() * sizeof(CUtensorMap),
                                cudaMemcpyHostToDevice, st));
-    }
     h->args_valid = true;
   }
   return FSX_OK;
