@@ -382,8 +382,8 @@ fsx_status fsx_append_create(const fsx_append_config* cfg, const fsx_append_weig
 /* Append n_new tokens for each of B vehicles.
  *   k_cache, v_cache : HOST arrays of n_layers DEVICE pointers, none NULL; layer
  *                      l points to bf16 [max_cache_rows, n_heads, head_dim]
- *                      rows, token-major. Read, and written only at the rows
- *                      named by d_dst_rows.
+ *                      rows, token-major, the keys 16-byte and the values 8-byte
+ *                      aligned. Read, and written only at the rows named by d_dst_rows.
  *   d_offsets        : DEVICE int64 [B+1], non-decreasing, offsets[0] >= 0,
  *                      offsets[B] <= max_cache_rows: vehicle b's cached tokens
  *                      0 .. L_b-1 are rows offsets[b] .. offsets[b+1]-1 (L_b may be 0).

@@ -21,6 +21,7 @@
 #include <cstdarg>
 #include <cstdio>
 #include <thread>
+#include <type_traits>
 #include <vector>
 
 #include "../../include/fsx.h"
@@ -194,8 +195,26 @@ __device__ __forceinline__ void st_peer(uint32_t addr, float v) {
   asm volatile("st.shared::cluster.f32 [%0], %1;" ::"r"(addr), "f"(v) : "memory");
 }
 
-// NQ: query slots (4 or 8) for n_new <= NQ new tokens
-template <int NQ>
+// Two 8-byte accesses in place of one of 16, for a cache that is only 8-byte aligned
+template <bool WIDE>
+__device__ __forceinline__ uint4 ld_unit(const __nv_bfloat16* p) {
+  if (WIDE) return *reinterpret_cast<const uint4*>(p);
+  const uint2 a = reinterpret_cast<const uint2*>(p)[0], b = reinterpret_cast<const uint2*>(p)[1];
+  return make_uint4(a.x, a.y, b.x, b.y);
+}
+template <bool WIDE>
+__device__ __forceinline__ void st_unit(__nv_bfloat16* p, uint4 v) {
+  if (WIDE) {
+    *reinterpret_cast<uint4*>(p) = v;
+  } else {
+    reinterpret_cast<uint2*>(p)[0] = make_uint2(v.x, v.y);
+    reinterpret_cast<uint2*>(p)[1] = make_uint2(v.z, v.w);
+  }
+}
+
+// NQ: query slots (4 or 8) for n_new <= NQ new tokens; VWIDE: the values' cache is 16-byte aligned
+// (the keys' always is, the values' needs 8 bytes only)
+template <int NQ, bool VWIDE>
 __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_kernel(const AttnArgsA a) {
   __shared__ __align__(16) float qs[NQ][kHeadDim];
   __shared__ __align__(16) __nv_bfloat16 kn[kMaxNew][kNewStride], vn[kMaxNew][kNewStride];
@@ -243,11 +262,12 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
   const size_t lane_off = static_cast<size_t>(hv) * a.HD + u * 8;  // of this lane's first row and dims, in values
   const size_t unit0 = static_cast<size_t>(lo) * a.HD + h * kHeadDim + lane_off;
   const size_t pair = 2 * static_cast<size_t>(a.HD);               // from key 2 kk + hv to key 2 kk + 2 + hv
-  auto load_rows = [&](int c, const __nv_bfloat16* cache, const __nv_bfloat16* fresh, uint4 (&raw)[4]) {
+  auto load_rows = [&](auto wide, int c, const __nv_bfloat16* cache, const __nv_bfloat16* fresh, uint4 (&raw)[4]) {
+    constexpr bool kWide = decltype(wide)::value;
     const __nv_bfloat16* row = cache + unit0 + static_cast<size_t>(c) * (kUnit / 2) * pair;
     if (kUnit * c + kUnit <= L) {  // a whole unit of cached rows
 #pragma unroll
-      for (int kk = 0; kk < 4; ++kk) raw[kk] = *reinterpret_cast<const uint4*>(row + kk * pair);
+      for (int kk = 0; kk < 4; ++kk) raw[kk] = ld_unit<kWide>(row + kk * pair);
       return;
     }
     const bool own = c == n_units - 1;
@@ -255,11 +275,11 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
     if (own) row = fresh + hv * kNewStride + u * 8;
 #pragma unroll
     for (int kk = 0; kk < 4; ++kk)
-      raw[kk] = 2 * kk + hv < n ? *reinterpret_cast<const uint4*>(row + kk * (own ? 2 * static_cast<size_t>(kNewStride) : pair))
+      raw[kk] = 2 * kk + hv < n ? ld_unit<kWide>(row + kk * (own ? 2 * static_cast<size_t>(kNewStride) : pair))
                                 : make_uint4(0u, 0u, 0u, 0u);
   };
-  auto load_k = [&](int c) { load_rows(c, a.k_cache, &kn[0][0], kraw); };
-  auto load_v = [&](int c) { load_rows(c, a.v_cache, &vn[0][0], vraw); };
+  auto load_k = [&](int c) { load_rows(std::true_type{}, c, a.k_cache, &kn[0][0], kraw); };
+  auto load_v = [&](int c) { load_rows(std::integral_constant<bool, VWIDE>{}, c, a.v_cache, &vn[0][0], vraw); };
   const int step = S * kAttnWarps;
   int c = rank * kAttnWarps + warp;
   if (c < n_units - 1) {  // in flight while the new rows are rotated
@@ -290,7 +310,7 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
       const int i = t / (kHeadDim / 8), uu = t - i * (kHeadDim / 8);
       const size_t o = static_cast<size_t>(d0 + i) * a.HD + h * kHeadDim + uu * 8;
       *reinterpret_cast<uint4*>(a.k_cache + o) = *reinterpret_cast<const uint4*>(&kn[i][uu * 8]);
-      *reinterpret_cast<uint4*>(a.v_cache + o) = *reinterpret_cast<const uint4*>(&vn[i][uu * 8]);
+      st_unit<VWIDE>(a.v_cache + o, *reinterpret_cast<const uint4*>(&vn[i][uu * 8]));
     }
 
   uint64_t q2[NQ][4];  // dims 8 u .. 8 u + 7 of every query
@@ -475,6 +495,14 @@ __global__ void __launch_bounds__(kAttnWarps * 32, NQ == 4 ? 4 : 2) append_attn_
     }
     a.out[static_cast<size_t>(b * nq + qi) * a.HD + h * kHeadDim + dd] = __float2half_rn(den > 0.f ? num / den : 0.f);
   }
+}
+
+const void* append_attn_fn(int n_new, bool v_wide) {
+  if (n_new <= 4)
+    return v_wide ? reinterpret_cast<const void*>(&append_attn_kernel<4, true>)
+                  : reinterpret_cast<const void*>(&append_attn_kernel<4, false>);
+  return v_wide ? reinterpret_cast<const void*>(&append_attn_kernel<kMaxNew, true>)
+                : reinterpret_cast<const void*>(&append_attn_kernel<kMaxNew, false>);
 }
 
 // CTAs per (vehicle, head): the largest power of two up to 8 that keeps the batch's CTAs
@@ -707,8 +735,11 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
   if (!k_cache || !v_cache || !d_offsets || !d_dst_rows || !d_x_new || !d_hidden)
     return fail(FSX_ERR_INVALID_ARG, "a pointer argument is NULL");
   if (B < 1 || B > c.max_batch) return fail(FSX_ERR_INVALID_ARG, "B=%d outside 1..max_batch=%d", B, c.max_batch);
-  for (int l = 0; l < c.n_layers; ++l)
+  for (int l = 0; l < c.n_layers; ++l) {
     if (!k_cache[l] || !v_cache[l]) return fail(FSX_ERR_INVALID_ARG, "cache layer %d pointer is NULL", l);
+    if (reinterpret_cast<uintptr_t>(k_cache[l]) % 16 != 0 || reinterpret_cast<uintptr_t>(v_cache[l]) % 8 != 0)
+      return fail(FSX_ERR_INVALID_ARG, "cache layer %d pointer is not aligned (keys 16 bytes, values 8)", l);
+  }
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   FSX_CUDA(cudaSetDevice(h->device));
   const int d = c.d_model, HD = h->HD, F = c.d_ff;
@@ -771,8 +802,7 @@ fsx_status fsx_append(fsx_append_handle h, void* const* k_cache, void* const* v_
     aa.out = h->o;
     aa.status = h->status;
     void* attn_args[] = {&aa};
-    FSX_CUDA(fsx::launch_ex(c.n_new <= 4 ? reinterpret_cast<const void*>(&append_attn_kernel<4>)
-                                         : reinterpret_cast<const void*>(&append_attn_kernel<kMaxNew>),
+    FSX_CUDA(fsx::launch_ex(append_attn_fn(c.n_new, reinterpret_cast<uintptr_t>(v_cache[l]) % 16 == 0),
                             dim3(attn_splits, c.n_heads, B), dim3(kAttnWarps * 32), 0, st, true, attn_args, 1,
                             attn_splits));
 

@@ -25,11 +25,11 @@ def row_err(got, ref):
     return (np.abs(got - ref).max(-1) / np.maximum(np.abs(ref).max(-1), 1e-30)).max()
 
 
-@pytest.mark.parametrize("n_new,lengths", [
+@pytest.mark.parametrize("n_new,lengths,v_offset", [(n, l, 0) for n, l in (
     (4, [0]), (4, [31]), (1, [32]), (3, [33]), (8, [128]), (5, [1025]),
     (4, [127, 0]), (8, [129, 32, 257]), (4, [1, 64, 31, 300, 0]), (7, [5, 0, 97, 128, 33]),
-])
-def test_append_attention_edges(n_new, lengths):
+)] + [(4, [127, 0, 9], 4), (8, [33, 70], 4)])  # values' cache aligned to 8 bytes only
+def test_append_attention_edges(n_new, lengths, v_offset):
     dims = synth.BackboneDims(n_layers=1, d_model=256, d_ff=256, n_new=n_new)
     H, D, B = dims.n_heads, dims.head_dim, len(lengths)
     w = synth.make_backbone_weights(dims, 5, "bf16")
@@ -41,7 +41,10 @@ def test_append_attention_edges(n_new, lengths):
     kc = (torch.randn(rows, H, D, generator=g) * torch.exp(0.5 * torch.randn(H, D, generator=g))).bfloat16()
     vc = torch.randn(rows, H, D, generator=g).bfloat16()
     x = synth.make_append_tokens(dims, B, seed=6)
-    kg, vg = kc.cuda(), vc.cuda()
+    kg = kc.cuda()
+    vg = torch.empty(vc.numel() + v_offset, dtype=vc.dtype, device="cuda")[v_offset:].view_as(vc)
+    vg.copy_(vc)
+    assert vg.data_ptr() % 16 == 2 * v_offset
     hidden = torch.empty(B, n_new, dims.d_model, device="cuda")
     ap = fsx.Append(dims, w, B, rows)
     try:
@@ -59,3 +62,20 @@ def test_append_attention_edges(n_new, lengths):
                        np.asarray(ref[0]).reshape(B * n_new, -1)) <= TOL
         keep = np.setdiff1d(np.arange(rows), written)
         assert torch.equal(got[keep], was[keep])
+
+
+def test_misaligned_caches_are_refused_on_the_host():
+    dims = synth.BackboneDims(n_layers=1, d_model=256, d_ff=256)
+    flat = torch.zeros(24 * dims.n_heads * dims.head_dim + 8, dtype=torch.bfloat16, device="cuda")
+    x = synth.make_append_tokens(dims, 1, seed=6).cuda()
+    hidden = torch.empty(1, dims.n_new, dims.d_model, device="cuda")
+    off, dst = torch.tensor([0, 8]).cuda(), torch.tensor([8]).cuda()
+    ap = fsx.Append(dims, synth.make_backbone_weights(dims, 5, "bf16"), 1, 20)
+    try:
+        for k0, v0 in ((4, 0), (0, 2)):
+            with pytest.raises(fsx.FsxError) as e:
+                ap.append([flat[k0:]], [flat[v0:]], off, dst, x, hidden)
+            assert e.value.status == fsx.FSX_ERR_INVALID_ARG
+        assert ap.status() == fsx.FSX_OK
+    finally:
+        ap.close()
