@@ -278,6 +278,10 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   uint64_t* free_bar = cvt_bar + kNB;  // [kNB] the six attending warps are done with the buffer
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(free_bar + kNB);
   volatile int* abort = reinterpret_cast<volatile int*>(tmem_slot + 1);  // a wait of this CTA timed out
+  // after a timeout: the first ring position and the first cache chunk that were not issued (both are
+  // issued in order); recorded when one is skipped, so that the normal course writes nothing
+  volatile int* ring_end = abort + 1;
+  volatile int* chunk_end = abort + 2;
   float* gss = reinterpret_cast<float*>(smem + L.gss);
   float* rstd = reinterpret_cast<float*>(smem + L.rstd);
   unsigned char* ring = smem + L.ring;
@@ -326,7 +330,11 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   // Issued off the critical steps: four of these calls on the thread that everyone then meets at a
   // barrier cost 0.4 us, and before the last additions of a phase they held up every later CTA.
   auto issue = [&](int q) {  // one thread; an empty position just completes the slot's phase
-    if (q >= total_chunks || *abort) return;  // after a timeout no new copy starts
+    if (q >= total_chunks) return;
+    if (*abort) {  // after a timeout no new copy starts
+      atomicMin(const_cast<int*>(ring_end), q);
+      return;
+    }
     uint64_t* bar = full + (q % kSlots);
     if (is_empty(q)) {
       mbar_arrive(bar);
@@ -368,6 +376,8 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
 
   if (tid == 0) {
     *abort = 0;
+    *ring_end = total_chunks;
+    *chunk_end = 0x7fffffff;
     for (int i = 0; i < kSlots; ++i) mbar_init(full + i, 1);
     mbar_init(mma_bar, kNAcc);
     for (int i = 0; i < 5; ++i) mbar_init(qbar + i, 1);
@@ -584,13 +594,19 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     if (*abort) return;
     if (!wait_phase<false>(bar, parity, p.status)) *abort = 1;
   };
-  // 64 threads (t = 0 .. 63): the copies of chunk j; after a timeout no new copy starts
+  auto by_tma = [&](int n) { return kSw && p.cache_maps != nullptr && n == kStageKeys; };
+  // 64 threads (t = 0 .. 63): the copies of chunk j; after a timeout no new copy starts. A TMA chunk
+  // is one thread's alone, its arrivals too, so that its phase completes whatever the others have seen.
+  // (t = 0 in warp 7 in place of warps 3 and 6, one thread for all copies, took 0.4 % longer a tick.)
   auto stage_issue = [&](int j, int g, int t, int layer, const unsigned char* kh, const unsigned char* vh) {
-    if (*abort) return;
+    if (*abort) {
+      if (t == 0) atomicMin(const_cast<int*>(chunk_end), g);
+      return;
+    }
     const int n = chunk_keys(j);
     uint64_t* bar = raw_bar + g % kNB;
     unsigned char* kb = stage_buf(g);
-    if (kSw && p.cache_maps != nullptr && n == kStageKeys) {
+    if (by_tma(n)) {
       if (t == 0) {
         const CUtensorMap* maps = p.cache_maps + 2 * layer;
         const int row = static_cast<int>(o_lo + kbeg) + j * kStageKeys;
@@ -599,8 +615,7 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
         mbar_arrive_expect_tx(bar, kBufBytes);
 #pragma unroll
         for (int e = 0; e < 4; ++e) tma_load_cache(kb + e * kBlockBytes, maps + (e >> 1), (e & 1) * 64, head, row, bar);
-      } else {
-        mbar_arrive(bar);
+        mbar_arrive_n(bar, 63);
       }
       return;
     }
@@ -1263,12 +1278,23 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
 
   // ---- leave nothing in flight. Every path reaches this point, a timed-out tick included
   // (its waits on other CTAs return at once). In order: the cache-row and weight copies (all waited
-  // for in the normal course; a timed-out tick stops issuing, may have skipped the waits of the last
-  // ones, and gives them 1 ms: they land within microseconds); the MMAs of the
-  // four issuing threads (a last commit each on drain_bar); the partners' stores into this
-  // CTA's shared memory (the cluster barrier below); then the tensor memory is freed.
+  // for in the normal course; a timed-out tick stops issuing and may have skipped the waits of the last
+  // ones, so one thread waits, bounded, for the last position of every ring slot and the last TMA
+  // chunk of every staging buffer); st.async stores already on their way, here or to a partner (1 ms:
+  // they land within microseconds); the MMAs of the four issuing threads (a last commit each on
+  // drain_bar); the partners' other accesses to this CTA's shared memory (the cluster barrier below);
+  // then the tensor memory is freed.
   cp_async_wait<0>();
   if (*abort) {
+    if (tid == kIssuer) {
+#pragma unroll 1
+      for (int q = max(*ring_end - kSlots, 0); q < *ring_end; ++q)
+        wait_phase<false>(full + q % kSlots, static_cast<uint32_t>((q / kSlots) & 1), p.status);
+      const int g_end = min(*chunk_end, p.n_layers * n_chunks);
+#pragma unroll 1
+      for (int g = max(g_end - kNB, 0); g < g_end; ++g)
+        if (by_tma(chunk_keys(g % n_chunks))) wait_phase<false>(raw_bar + g % kNB, stage_parity(g), p.status);
+    }
     const unsigned long long t0 = global_timer_ns();
     while (global_timer_ns() - t0 < 1000000ull) {
     }

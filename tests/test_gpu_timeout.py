@@ -1,8 +1,8 @@
 """The bounded-wait timeout path of the single-launch tick, exercised without breaking
 any kernel: a test hook lowers the limit of the tick's device-wide counter waits to
 1 ns, so the first wait that finds its counter incomplete gives up at once. The tick
-must end (every CTA drains what it has in flight: its cache-row copies, the weight
-copies it issued, its MMAs, its partners' stores), report FSX_ERR_TIMEOUT and write no
+must end (every CTA drains what it has in flight: its cache-row copies, by TMA where whole
+64-key chunks are loaded, the weight copies it issued, its MMAs, its partners' stores), report FSX_ERR_TIMEOUT and write no
 waypoint; with the default limit restored, the next tick on the same handle must match
 the oracle."""
 from __future__ import annotations
@@ -20,8 +20,9 @@ import fsx_cases as fc
 pytestmark = pytest.mark.gpu
 
 
-def test_wait_timeout_is_reported_and_the_next_tick_is_clean():
-    case = fc.Case(synth.Dims(n_layers=4), [100], "bf16", seed=12)
+@pytest.mark.parametrize("rows,dtype", [(100, "bf16"), (1500, "bf16"), (1500, "fp32")])
+def test_wait_timeout_is_reported_and_the_next_tick_is_clean(rows, dtype):
+    case = fc.Case(synth.Dims(n_layers=4), [rows], dtype, seed=12)
     ex = case.expert()
     try:
         assert ex.launches(1) == 1  # the single-launch tick
