@@ -48,7 +48,6 @@ __global__ void __launch_bounds__(kEmbedWarps * 32) embed_kernel(const EmbedArgs
     }
     for (int o = 16; o > 0; o >>= 1) cnt += __shfl_xor_sync(0xffffffffu, cnt, o);
     if (lane == 0) {
-      a.order[cnt] = row;
       AttnPlan e;
       e.lo = st != nullptr ? st[row] : off[row];
       e.b = row;

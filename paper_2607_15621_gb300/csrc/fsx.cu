@@ -84,8 +84,7 @@ struct fsx_handle_s {
   __half* qkv = nullptr;
   __half* o = nullptr;
   __half* hbuf = nullptr;
-  int* order = nullptr;         // [max_batch] vehicles by decreasing cache length (attention schedule)
-  fsx::AttnPlan* plan = nullptr;  // [max_batch] the same schedule with each vehicle's cache range
+  fsx::AttnPlan* plan = nullptr;  // [max_batch] attention schedule: vehicles by decreasing cache length, with their ranges
   int* status = nullptr;
   TickArgs* d_args = nullptr;
   TickArgs h_args{};
@@ -253,7 +252,6 @@ fsx_status enqueue_tick(fsx_handle_s* h, int B, cudaStream_t st, __half* attn_ca
   ea.x16 = h->x16;
   ea.ss = h->ss;
   ea.ss_stride = h->ss_stride;
-  ea.order = h->order;
   ea.plan = h->plan;
   ea.status = h->status;
   FSX_CUDA(fsx::launch_embed(ea, st, pdl));
@@ -513,7 +511,7 @@ void free_handle(fsx_handle_s* h) {
   if (h->paper_params) cudaFree(h->paper_params);
   if (h->paper_frames) cudaFree(h->paper_frames);
   void* bufs[] = {h->p_arena, h->p_x, h->p_counters, h->w_arena, h->params, h->x, h->x16, h->ss, h->qkv, h->o, h->hbuf,
-                  h->order, h->plan, h->status, h->d_args, h->d_cache_maps,
+                  h->plan, h->status, h->d_args, h->d_cache_maps,
                   h->st_offsets, h->st_frames, h->st_waypoints};
   for (void* p : bufs)
     if (p) cudaFree(p);
@@ -791,7 +789,6 @@ fsx_status fsx_create(const fsx_config* cfg, const fsx_weights* w, int device, f
           !fsx::encode_act_map(&h->map_h_res[i], h->hbuf, m_pad, F, fsx::kResTiles[i]))
         return bail(fail(FSX_ERR_CUDA, "tensor map encoding of the activation buffers failed"));
   }
-  FSX_CUDA_H(cudaMalloc(&h->order, sizeof(int) * cfg->max_batch));
   FSX_CUDA_H(cudaMalloc(&h->plan, sizeof(fsx::AttnPlan) * cfg->max_batch));
   FSX_CUDA_H(cudaMalloc(&h->status, sizeof(int)));
   FSX_CUDA_H(cudaMemset(h->status, 0, sizeof(int)));

@@ -96,8 +96,7 @@ struct EmbedArgs {
   __half* x16;            // fp16 copy of x
   float* ss;              // per-row sums of x^2 over 128-column groups, [d/128][ss_stride]
   int ss_stride;
-  int* order;             // [B]: vehicles by decreasing cache length (ties by index)
-  AttnPlan* plan;         // [B]: the same order with each vehicle's cache range
+  AttnPlan* plan;         // [B]: vehicles by decreasing cache length (ties by index), each with its cache range
   int* status;
 };
 cudaError_t launch_embed(const EmbedArgs& a, cudaStream_t stream, bool pdl);
