@@ -535,6 +535,7 @@ fsx_status paper_attach(fsx_handle h, float* d_params, const float* d_head, floa
 float* paper_frames(fsx_handle h) { return h->paper_frames; }
 const float* paper_state_weights(fsx_handle h) { return h->paper_state_w; }
 int paper_device(fsx_handle h) { return h->device; }
+int paper_sm_count(fsx_handle h) { return h->sm_count; }
 int paper_max_batch(fsx_handle h) { return h->cfg.max_batch; }
 int paper_d(fsx_handle h) { return h->cfg.d_model; }
 int paper_visual_dtype(fsx_handle h) { return h->paper_visual_dtype; }

@@ -136,7 +136,7 @@ struct StateArgs {
   float* frames;           // [B, 5, d]
   int d, B;
 };
-cudaError_t launch_state_tokens(const StateArgs& a, cudaStream_t stream);
+cudaError_t launch_state_tokens(const StateArgs& a, int sm_count, cudaStream_t stream);
 
 // Launch helper: cudaLaunchKernelEx with the programmatic-stream-serialisation
 // attribute when `pdl` is set and a (cluster_x, cluster_y, 1) cluster when either exceeds 1.

@@ -33,6 +33,7 @@ float* paper_frames(fsx_handle h);
 const float* paper_state_weights(fsx_handle h);
 cudaError_t paper_order_after_last_tick(fsx_handle h, cudaStream_t st);
 int paper_device(fsx_handle h);
+int paper_sm_count(fsx_handle h);
 int paper_max_batch(fsx_handle h);
 int paper_d(fsx_handle h);
 int paper_visual_dtype(fsx_handle h);
@@ -221,11 +222,11 @@ __global__ void __launch_bounds__(kMlpThreads) head2_kernel(const Head2Args a) {
   }
 }
 
-cudaError_t launch_state_tokens(const StateArgs& a_in, cudaStream_t stream) {
+cudaError_t launch_state_tokens(const StateArgs& a_in, int sm_count, cudaStream_t stream) {
   StateArgs a = a_in;
   void* kargs[] = {&a};
   // one pass of 32 rows a block for few vehicles, about two blocks per SM for many
-  int slices = 304 / a.B;
+  int slices = 2 * sm_count / a.B;
   slices = slices > a.d / 32 ? a.d / 32 : (slices < 1 ? 1 : slices);
   return launch_ex(reinterpret_cast<const void*>(&state_tokens_kernel), dim3(slices, a.B), dim3(kMlpThreads), 0, stream,
                    false, kargs);
@@ -357,7 +358,7 @@ fsx_status fsx_paper_tick(fsx_handle h, const void* const* k_cache, const void* 
   a.frames = fsx::paper_frames(h);
   a.d = fsx::paper_d(h);
   a.B = B;
-  if (e == cudaSuccess) e = fsx::launch_state_tokens(a, st);
+  if (e == cudaSuccess) e = fsx::launch_state_tokens(a, fsx::paper_sm_count(h), st);
   if (e != cudaSuccess) return pfail(FSX_ERR_CUDA, cudaGetErrorString(e));
   return fsx_tick(h, k_cache, v_cache, d_offsets, B, fsx::paper_frames(h), d_waypoints, stream);
 }
