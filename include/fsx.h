@@ -218,9 +218,10 @@ fsx_status fsx_kernel_time(fsx_handle h, float* ms, int* launches);
  *   d_workspace : DEVICE scratch of fsx_attention_workspace_bytes(...) bytes:
  *              a status word, then the per-split partial outputs. Only this
  *              call's kernels touch it; it must not be shared by calls that
- *              overlap on the GPU. Asynchronous on `stream`; cache offsets
- *              outside [0, ...] non-decreasing order make the kernels write
- *              nothing.
+ *              overlap on the GPU. Asynchronous on `stream`.
+ * A vehicle whose offsets are negative or decrease sets the status word to
+ * FSX_ERR_DEVICE_ARG and its rows stay unwritten. The other vehicles' rows are written
+ * (with more than 8 splits, no own keys or more than 64, they may stay unwritten too).
  * A cache value outside the fp16 range sets the status word to FSX_ERR_RANGE. With
  * fp32 caches or 2..8 splits the rows are then those of the cache clipped to +-65504
  * (NaN values stay NaN); with one split of a bf16 cache they may hold infinities or
@@ -411,8 +412,9 @@ fsx_status fsx_append_get_status(fsx_append_handle h, void* stream);
 /* enable = 1: later appends on this handle run no kernel that waits on other CTAs,
  * so an append can share the GPU with a tick whose single-launch kernel needs all of
  * its CTAs resident (the concurrent schedule of fsx_session). The append's kernels
- * hold to that under either setting (split sums are completed by whichever CTA
- * arrives last), so both run the same code at the same speed. */
+ * hold to that under either setting (sums over several CTAs are made inside a cluster,
+ * whose CTAs are scheduled together, or by whichever CTA arrives last), so both run the
+ * same code at the same speed. */
 fsx_status fsx_append_set_concurrent(fsx_append_handle h, int enable);
 
 /* Bytes of the handle's fp16 weight arena (algorithmic weight bytes per call). */

@@ -7,9 +7,11 @@
 //            embedding, cache-row writes and causal attention over
 //            [cached rows ; new rows] -> W_o + residual -> RMSNorm+gate/up+SiLU
 //            -> W_d + residual ] -> residual stream out.
-// The four projections run on the few-token tensor-core GEMM (gemm_stream.cu): norm
-// gains folded into the packed weights, 1/rms applied in the epilogue from
-// per-128-column sums of x^2, the weight stream cut evenly over the SMs. The token
+// QKV and gate/up run on the few-token tensor-core GEMM (gemm_stream.cu): norm gains
+// folded into the packed weights, 1/rms applied in the epilogue from per-128-column
+// sums of x^2, the weight stream cut evenly over the SMs. W_o and W_d, whose tiles are
+// few, run with K cut over clusters (gemm_res.cu) where gemm_res_plan finds a split (at
+// the 7B shape for every token count), else on the streaming GEMM too. The token
 // count is n_new * B (4 for one vehicle), so the call streams every backbone
 // weight once and is bound by HBM. No kernel of a call waits on other CTAs of its
 // grid (those of a cluster are scheduled together).

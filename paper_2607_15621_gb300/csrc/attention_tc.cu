@@ -73,7 +73,9 @@ constexpr uint32_t kColS = 0;    // S / P buffers at columns 0 and 64
 constexpr uint32_t kColO = 128;
 constexpr int kMaxClusterSplits = 8;
 constexpr int kMaxRounds = 32;     // items a CTA works on, at most (one lane prepares each)
-constexpr int kMaxByLength = 128;  // vehicles a launch without a plan sorts
+// vehicles a launch without a plan sorts: each of its CTAs compares every pair, and 128 is the largest
+// batch that was measured; larger ones run in the given order
+constexpr int kMaxByLength = 128;
 constexpr int kBoxBytes = kSlotKeys * 64 * 2;  // a TMA box: 64 rows of 64 values
 
 // shared-memory layout (bytes from the 1024-aligned base)

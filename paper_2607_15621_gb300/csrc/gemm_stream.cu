@@ -18,9 +18,13 @@
 //   warps 2-9: epilogue, two groups of four warps (one per tensor-memory lane quadrant)
 //           taking 8-token chunks in turn.
 // Measured on the two-layer append (405 MB of weights a layer), against whole-tile CTAs with
-// 128-token tiles, waiting K splits and no dependent launch: 4 tokens 311 -> 237 us a call (QKV
-// 30.1 -> 23.7 us a launch, gate/up 55.8 -> 35.3, W_o and W_d together 42.6 -> 36.9), 64 tokens
-// 370 -> 339 us (QKV 30.2 -> 26.7, gate/up 56.4 -> 42.0, W_o and W_d 45.5 -> 50.4).
+// 128-token tiles, waiting K splits and no dependent launch, when W_o and W_d still ran here too:
+// 4 tokens 311 -> 237 us a call (QKV 30.1 -> 23.7 us a launch, gate/up 55.8 -> 35.3, W_o and W_d
+// together 42.6 -> 36.9), 64 tokens 370 -> 339 us (QKV 30.2 -> 26.7, gate/up 56.4 -> 42.0, W_o and
+// W_d 45.5 -> 50.4; they have moved to gemm_res.cu where it has a split for them).
+// More tokens, a whole one-layer append with 96-480 cached rows, before this kernel and the fused
+// attention -> now: 64 tokens 286 -> 136 us, 96 of 12 vehicles 307 -> 152, 128 of 16 330 -> 174,
+// 160 of 20 394 -> 182, 192 of 48 523 -> 234, 256 of 32 495 -> 239.
 // Code size: a launch finds its instructions evicted by the layer's other kernels. One copy of the
 // epilogue instead of one per chunk in flight and 32-bit step arithmetic (gate/up at 64 tokens
 // 73 -> 49 KB, QKV at 16 tokens 33 -> 28): 4 tokens 193.5 -> 187.3 us a call, 64 tokens 266 -> 261.

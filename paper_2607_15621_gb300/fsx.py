@@ -173,7 +173,8 @@ def _ptr(t) -> int:
 
 
 def _stream(stream) -> int:
-    if stream is None:  # torch.cuda.current_stream().cuda_stream without the Stream object (2.8 -> 0.4 us a call)
+    if stream is None:  # torch.cuda.current_stream().cuda_stream without the Stream object: 3.0 -> 0.4 us
+        # a call, and of Eq. 1 for one vehicle, back to back, 24-26 -> 20.5 us
         import torch
         torch.cuda.init()
         return torch._C._cuda_getCurrentRawStream(torch._C._cuda_getDevice())

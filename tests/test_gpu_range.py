@@ -1,5 +1,6 @@
 """Cache values beyond the fp16 range. The kernels convert cache keys (and, except in
-the bf16 tensor-core attention, values) to fp16; a finite bf16 or fp32 value beyond
+the bf16 tensor-core attention, values) to fp16, and the launches with key splits check the
+values they keep in bf16 as well; a finite bf16 or fp32 value beyond
 +-65504 would become an infinity there and turn the softmax of its rows into NaN.
 Such a value is a device-side error instead: the status becomes FSX_ERR_RANGE and the
 tick writes no waypoint, like a tick over bad offsets; the next tick over an
@@ -20,8 +21,8 @@ SMALL = synth.Dims(n_layers=4)
 PLANTED = [(3, 5, 7), (10, 5, 70), (20, 17, 1)]  # (row, head, dim) of vehicle 0's layer-2 keys
 
 
-# B = 1: the single-launch tick; B = 2: the mma.sync split-KV attention; B = 6 (bf16):
-# the tensor-core attention
+# B = 1: the single-launch tick; B = 2: the tensor-core attention with key splits; B = 6
+# (bf16): the same without splits
 @pytest.mark.parametrize("B,dtype", [(1, "bf16"), (2, "bf16"), (6, "bf16"), (1, "fp32"), (2, "fp32")])
 def test_out_of_range_cache_keys_abandon_the_tick(B, dtype):
     lengths = [40 + 13 * b for b in range(B)]
@@ -47,8 +48,8 @@ def test_out_of_range_cache_keys_abandon_the_tick(B, dtype):
 
 
 def test_out_of_range_cache_values_are_caught_where_converted():
-    """Values are converted to fp16 by the split-KV attention (B = 2 here) and the
-    single-launch tick (B = 1)."""
+    """Values are converted to fp16 by the single-launch tick (B = 1) and checked by the
+    attention with key splits (B = 2 here)."""
     for lengths in ([30, 50], [50]):
         case = fc.Case(SMALL, lengths, "bf16", seed=8)
         case.v[1][len(lengths) * 17 % sum(lengths), 2, 9] = -3.0e5

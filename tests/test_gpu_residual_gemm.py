@@ -1,5 +1,6 @@
-"""The residual projections with K cut over a cluster, at the edges of their token tiles (48, 128, 144), with ragged
-4-token groups, one to eight splits and K too short to cut, through one-layer ticks against the fp64 oracle. Every token
+"""The residual projections with K cut over a cluster, at the edges of their token tiles (48, 64, 96, 128, 144 and
+160 tokens; the 16-token tile runs in the append's tests), with ragged 4-token groups, two to eight splits and K too
+short or tokens too many to cut, through one-layer ticks against the fp64 oracle. Every token
 is decoded as a waypoint, so every updated row is compared.
 
 Tolerance (relative L2 per vehicle): operands are rounded to fp16 (2^-11 each) at six points of a layer (x, q/k/v, P V,
