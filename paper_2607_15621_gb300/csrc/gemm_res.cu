@@ -126,9 +126,11 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
   const int n_groups = min(BN, p.M - m0 + 3) / 4;
   auto group_lo = [&](int r) { return n_groups * r / KS; };
   const int g_lo = group_lo(rank), g_hi = group_lo(rank + 1);
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (*abort) return;
-    if (!mbar_wait(bar, parity, p.status)) *abort = 1;
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (*abort) return false;
+    const bool ok = mbar_wait(bar, parity, p.status);
+    if (!ok) *abort = 1;
+    return ok;
   };
 
   pdl_launch_dependents();
@@ -174,10 +176,12 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
   pdl_wait();
 
   if (warp == 0) {
-    for (int g = 0; g < n; ++g) {
+    int g = 0;
+    for (; g < n; ++g) {
       const int s = g % kStages;
       unsigned char* st = stages + s * kStageBytes;
-      if (g >= kStages) wait(empty + s, static_cast<uint32_t>(((g / kStages) - 1) & 1));
+      // after a timeout no further copy is issued: its stage's last one may still be on its way
+      if (g >= kStages && __any_sync(0xffffffffu, !wait(empty + s, static_cast<uint32_t>(((g / kStages) - 1) & 1)))) break;
       if (lane == 0) {
         if (g >= kStages) {
           mbar_arrive_expect_tx(full + s, kStageBytes);
@@ -190,14 +194,14 @@ __global__ void __launch_bounds__(kThreads, 1) gemm_res_kernel(const __grid_cons
     // after a timeout the MMA warp may have skipped its waits: the copies still in
     // flight land (bounded) before the shared memory is released
     if (*abort && lane == 0)
-      for (int g = n > kStages ? n - kStages : 0; g < n; ++g) {
+      for (int i = g > kStages ? g - kStages : 0; i < g; ++i) {
         const unsigned long long t0 = global_timer_ns();
         uint32_t done = 0;
         while (!done && global_timer_ns() - t0 < 100000000ull)
           asm volatile(
               "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
               : "=r"(done)
-              : "r"(smem_addr(full + g % kStages)), "r"(static_cast<uint32_t>((g / kStages) & 1))
+              : "r"(smem_addr(full + i % kStages)), "r"(static_cast<uint32_t>((i / kStages) & 1))
               : "memory");
       }
     __syncwarp();

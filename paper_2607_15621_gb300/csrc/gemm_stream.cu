@@ -135,9 +135,11 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
   const uint32_t total = static_cast<uint32_t>(p.N / kRows) * KT;
   const int G = gridDim.x;
   const uint32_t s0 = total * blockIdx.x / G, s1 = total * (blockIdx.x + 1) / G;  // this CTA's steps
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (*abort) return;
-    if (!mbar_wait(bar, parity, p.status)) *abort = 1;
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (*abort) return false;
+    const bool ok = mbar_wait(bar, parity, p.status);
+    if (!ok) *abort = 1;
+    return ok;
   };
 
   pdl_launch_dependents();
@@ -177,10 +179,12 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
       }
     __syncwarp();
     pdl_wait();
-    for (int g = 0; g < n; ++g) {
+    int g = 0;
+    for (; g < n; ++g) {
       const int s = g % kStages;
       unsigned char* st = stages + s * kStageBytes;
-      if (g >= kStages) wait(empty + s, static_cast<uint32_t>(((g / kStages) - 1) & 1));
+      // after a timeout no further copy is issued: its stage's last one may still be on its way
+      if (g >= kStages && __any_sync(0xffffffffu, !wait(empty + s, static_cast<uint32_t>(((g / kStages) - 1) & 1)))) break;
       if (lane == 0) {
         if (g >= kStages) {
           mbar_arrive_expect_tx(full + s, kStageBytes);
@@ -193,14 +197,14 @@ __global__ void __launch_bounds__(kThreads, ctas_per_sm<BN>()) gemm_stream_kerne
     // after a timeout the MMA warp may have skipped its waits: the copies still in
     // flight land (bounded) before the shared memory is released
     if (*abort && lane == 0)
-      for (int g = n > kStages ? n - kStages : 0; g < n; ++g) {
+      for (int i = g > kStages ? g - kStages : 0; i < g; ++i) {
         const unsigned long long t0 = global_timer_ns();
         uint32_t done = 0;
         while (!done && global_timer_ns() - t0 < 100000000ull)
           asm volatile(
               "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
               : "=r"(done)
-              : "r"(smem_addr(full + g % kStages)), "r"(static_cast<uint32_t>((g / kStages) & 1))
+              : "r"(smem_addr(full + i % kStages)), "r"(static_cast<uint32_t>((i / kStages) & 1))
               : "memory");
       }
     __syncwarp();

@@ -229,9 +229,11 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
   constexpr int kAbytes = (PAIR ? BN / 2 : BN) * kTileK * 2;
   constexpr uint32_t kTmemCols = tc_tmem_cols<BN>();
   // bounded wait that gives up at once after an earlier timeout of this CTA
-  auto wait = [&](uint64_t* bar, uint32_t parity) {
-    if (*abort) return;
-    if (!mbar_wait(bar, parity, p.status)) *abort = 1;
+  auto wait = [&](uint64_t* bar, uint32_t parity) -> bool {
+    if (*abort) return false;
+    const bool ok = mbar_wait(bar, parity, p.status);
+    if (!ok) *abort = 1;
+    return ok;
   };
 
   pdl_launch_dependents();
@@ -295,14 +297,18 @@ __global__ void __launch_bounds__(kTcThreads, 1) gemm_tc_kernel(const __grid_con
     __syncwarp();
     pdl_wait();
     int total = 0;
-    for (int u = u_first; u < n_units; u += u_step) {
+    bool go = true;  // after a timeout no further copy is issued: its stage's last one may still be on its way
+    for (int u = u_first; u < n_units && go; u += u_step) {
       const int m_tile = tile_of(u) / tiles_n;
       for (int kt = 0; kt < KT; ++kt, ++total) {
         const int g = total;
         const int s = g % kStages;
         unsigned char* st = stages + s * kStageBytes;
-        if (g >= kStages) wait(empty + s, static_cast<uint32_t>(((g / kStages) - 1) & 1));
-        if (PAIR) {  // after a timeout of this CTA no further copy is issued
+        if (g >= kStages) {
+          go = __all_sync(0xffffffffu, wait(empty + s, static_cast<uint32_t>(((g / kStages) - 1) & 1)));
+          if (!PAIR && !go) break;
+        }
+        if (PAIR) {
           if (lane == 0 && *abort == 0) {
             if (g >= kStages) {
               if (crank == 0) mbar_arrive_expect_tx(full + s, kPairTx);
