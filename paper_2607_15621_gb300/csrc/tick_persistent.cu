@@ -550,13 +550,17 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
   // 16-byte cp.async of two warps (rows past the range are never read). fp32: rows of 512 bytes
   // padded to kRowStride, by cp.async. The chunk's 64 arrivals (copies included) complete its
   // buffer's raw_bar; rows are converted to fp16 in place (fp32: at the start of the row, whole
-  // rows by one warp). The first chunk of a layer is converted by all eight warps; from then on
+  // rows by one warp). The first chunk of a layer is converted by all eight warps; from then on, bf16,
   // warps 6 and 7 convert chunk j + 1 and refill the buffer of chunk j - 1 while warps 0-5 attend
   // over chunk j. With every thread copying, converting and meeting at three block barriers per
   // chunk, a chunk of 64 keys took 2.3 us: 0.97 to attend, 0.64 to convert, 0.26 to issue copies, the
   // rest waiting; now 1.7 us, 1.0 of them the two warps' conversion (4096 rows, 8 layers: 467 -> 393 us a
   // tick). A bulk copy per row in place of the TMA boxes took 4.5 us a
-  // chunk: 128 of them hold two warps for longer than the rest of their work. The weight copies of
+  // chunk: 128 of them hold two warps for longer than the rest of their work. fp32 chunks are
+  // twice the bytes for fewer keys and have to be copied row by row, too much for two warps: there all
+  // eight convert each chunk, a block barrier a chunk, and warps 6 and 7 refill under the attention
+  // (4 layers, converting in two warps -> now: 480 rows 135 -> 113 us a tick, 1000 rows 174 -> 130, 4096
+  // rows 463 -> 254; in two orders of the 16-byte reads, without bank conflicts, 273). The weight copies of
   // positions 8-11 of the layer (slots 2-5) are issued only once the attention is done with the region.
   constexpr bool kSw = sizeof(CT) == 2;                                   // swizzled buffers
   constexpr int kRowStride = kD * 4 + 16;                                 // fp32: 528 bytes
@@ -619,15 +623,29 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
       }
       return;
     }
-    constexpr int kUnits = kD * static_cast<int>(sizeof(CT)) / 16;  // raw 16-byte units of a row: 16 / 32
-    for (int i = t; i < 2 * n * kUnits; i += 64) {
-      const int r = i / kUnits, u = i % kUnits;
-      const bool is_v = r >= n;
-      const int key = is_v ? r - n : r;
-      const unsigned char* src = (is_v ? vh : kh) + static_cast<size_t>(j * kStageKeys + key) * tok_bytes + u * 16;
-      unsigned char* dst = kSw ? kb + ((is_v ? 2 : 0) + (u >> 3)) * kBlockBytes + key * 128 + (((u & 7) ^ (key & 7)) << 4)
-                               : kb + ((is_v ? kStageKeys : 0) + key) * kRowStride + u * 16;
-      cp_async_16(smem_addr(dst), src);
+    if (kSw) {
+      constexpr int kUnits = kD * 2 / 16;  // 16-byte units of a row
+      for (int i = t; i < 2 * n * kUnits; i += 64) {
+        const int r = i / kUnits, u = i % kUnits;
+        const bool is_v = r >= n;
+        const int key = is_v ? r - n : r;
+        const unsigned char* src = (is_v ? vh : kh) + static_cast<size_t>(j * kStageKeys + key) * tok_bytes + u * 16;
+        unsigned char* dst = kb + ((is_v ? 2 : 0) + (u >> 3)) * kBlockBytes + key * 128 + (((u & 7) ^ (key & 7)) << 4);
+        cp_async_16(smem_addr(dst), src);
+      }
+    } else {  // a row a warp instruction, keys t / 32, t / 32 + 2, ... of K and of V
+      const size_t first = static_cast<size_t>(j * kStageKeys + (t >> 5)) * tok_bytes + (t & 31) * 16;
+      const unsigned char* ks = kh + first;
+      const unsigned char* vs = vh + first;
+      uint32_t dst = smem_addr(kb) + (t >> 5) * kRowStride + (t & 31) * 16;
+#pragma unroll 2
+      for (int key = t >> 5; key < n; key += 2) {
+        cp_async_16(dst, ks);
+        cp_async_16(dst + kStageKeys * kRowStride, vs);
+        ks += 2 * tok_bytes;
+        vs += 2 * tok_bytes;
+        dst += 2 * kRowStride;
+      }
     }
     // this thread's arrival, once its copies have landed
     asm volatile("cp.async.mbarrier.arrive.noinc.shared.b64 [%0];" ::"r"(smem_addr(bar)) : "memory");
@@ -957,13 +975,13 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
     for (int j = 0; j < n_chunks + (own_n > 0 ? 1 : 0); ++j) {
       const int g = g0 + j;
       const bool own = j == n_chunks;
-      if (!own && (j == 0 || warp >= kAttendWarps)) {  // the layer's first chunk by all warps
+      if (!own && (j == 0 || !kSw || warp >= kAttendWarps)) {  // every warp: the layer's first chunk, and fp32
         swait(raw_bar + g % kNB, stage_parity(g));
-        convert(j, g, j == 0 ? warp : warp - kAttendWarps, j == 0 ? kThr / 32 : kCvtWarps);
+        convert(j, g, j == 0 || !kSw ? warp : warp - kAttendWarps, j == 0 || !kSw ? kThr / 32 : kCvtWarps);
       }
-      if (j == 0) __syncthreads();
+      if (j == 0 || (!kSw && !own)) __syncthreads();  // converted; and the chunk before it is attended
       if (warp < kAttendWarps) {
-        if (!own && j > 0) swait(cvt_bar + g % kNB, stage_parity(g));
+        if (kSw && !own && j > 0) swait(cvt_bar + g % kNB, stage_parity(g));
         if (kSw || !own) {
           const uint32_t kb = smem_addr(own ? reinterpret_cast<unsigned char*>(ownk) : stage_buf(g));
           const uint32_t vb = own ? smem_addr(ownv) : kb + (kSw ? 2 * kBlockBytes : kStageKeys * kRowStride);
@@ -973,12 +991,12 @@ __global__ void __cluster_dims__(kCl, 1, 1) __launch_bounds__(kThr, 1) persisten
           attend(std::true_type{}, smem_addr(ownk), smem_addr(ownv), kActAtom, own_n);
         }
         __syncwarp();
-        if (!own && lane == 0) mbar_arrive(free_bar + g % kNB);
+        if (kSw && !own && lane == 0) mbar_arrive(free_bar + g % kNB);
       } else if (!own) {
-        mbar_arrive(cvt_bar + g % kNB);  // the first chunk's too: every chunk is a phase of its buffer's barrier
-        const int jr = j - 1 + kNB;      // into the buffer of chunk j - 1
+        if (kSw) mbar_arrive(cvt_bar + g % kNB);  // the first chunk's too: every chunk is a phase of its buffer's barrier
+        const int jr = j - 1 + kNB;               // into the buffer of chunk j - 1
         if (j > 0 && jr < n_chunks) {
-          swait(free_bar + (g - 1) % kNB, stage_parity(g - 1));
+          if (kSw) swait(free_bar + (g - 1) % kNB, stage_parity(g - 1));
           stage_issue(jr, g0 + jr, (warp - kAttendWarps) * 32 + lane, layer, kc, vc);
         }
       }
